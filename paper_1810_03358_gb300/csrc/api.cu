@@ -107,6 +107,9 @@ struct ffmin_system {
     int n_items64 = 0, grid_sym = 0;
     Item *d_items64 = nullptr;
     int2 *d_sys_items64 = nullptr;
+    Item *d_items32 = nullptr;
+    int2 *d_sys_items32 = nullptr;
+    int sms = 0;
     std::vector<int32_t> term_off[4];  // per-system offsets of bonds, angles, dihedrals, corrections
     int nb_total = 0, na_total = 0, nd_total = 0;
 };
@@ -143,7 +146,16 @@ static void bonded_items(const ffmin_system *sys, int b, std::vector<Item> &item
     }
 }
 
-// Work items for a given density, system by system: the system's bonded
+// Blocks per SM that the layouts of the FP32 lists reckon with: the FP32
+// partial sums end where a chunk ends, so these stay what they are when a
+// kernel's occupancy changes (a minimization amplifies another rounding)
+constexpr int LAYOUT_ROW_BLOCKS[2] = {6, 12};  // row list, by i-atoms per thread
+constexpr int LAYOUT_SYM_BLOCKS = 7;           // energy-only list
+
+// some evaluation of the object runs on the row list
+static bool needs_row_list(const ffmin_system *sys) { return !sys->c.sym64 || sys->prec == FFMIN_MIXED; }
+
+// Work items of the row list for a given density, system by system: the system's bonded
 // items (latency-bound FP64 work that overlaps the FP32 pair items), then its
 // (tile, j-chunk) pair items; every system's items are contiguous so that
 // the pair kernels can run over the active systems only.
@@ -152,7 +164,8 @@ static void build_items(ffmin_system *sys, int density, std::vector<Item> &items
     items.clear();
     tiles = sys->tiles_h;
     sys_items.assign(sys->n_sys, make_int2(0, 0));
-    const int chunk_grid = sys->prec == FFMIN_MIXED ? sys->grid32_max : sys->grid64_max;
+    const int chunk_grid =
+        sys->prec == FFMIN_MIXED ? LAYOUT_ROW_BLOCKS[sys->c.f32_ipt - 1] * sys->sms : sys->grid64_max;
     const int64_t total_tiles = (int64_t)tiles.size();
     size_t t = 0;
     for (int b = 0; b < sys->n_sys; b++) {
@@ -181,22 +194,16 @@ static void build_items(ffmin_system *sys, int density, std::vector<Item> &items
     }
 }
 
-// Symmetric FP64 list: per system its bonded items, then for every i-tile I
-// the chunks of `chunk` j-tiles covering tiles [I, nT) of the system (the
-// first chunk starts with the diagonal tile).  Item slots: the i-side rows,
-// then one row block per j-tile of the chunk.  chunk is chosen so that the
-// batch exposes about `want` items; tiles get row64 / chunk64 / tloc.
-static void build_items64(ffmin_system *sys, int64_t want, std::vector<Item> &items,
-                          std::vector<int2> &sys_items, int64_t *n_slots) {
+// Symmetric list: per system its bonded items, then for every i-tile I the
+// chunks of `chunk` j-tiles covering the tiles [I, nT) of the system, or,
+// split > 1 (then chunk == 1), the parts of 128 / split j-atoms of each
+// j-tile.  Partial rows: per item its i-side row, and with jrows one j-side
+// row per j-tile (see SymRow).  Fills the tiles' rows (member `row`).
+static void build_items_sym(ffmin_system *sys, int chunk, int split, bool jrows, SymRow Tile::*row,
+                            std::vector<Item> &items, std::vector<int2> &sys_items, int64_t *n_slots) {
     items.clear();
     sys_items.assign(sys->n_sys, make_int2(0, 0));
     std::vector<Tile> &tiles = sys->tiles_h;
-    int64_t pairs = 0;
-    for (int b = 0; b < sys->n_sys; b++) {
-        const int64_t nT = (sys->sys_natoms[b] + TI - 1) / TI;
-        pairs += nT * (nT + 1) / 2;
-    }
-    const int chunk = (int)std::max<int64_t>(1, pairs / std::max<int64_t>(want, 1));
     int64_t slots = 0;
     size_t t = 0;
     for (int b = 0; b < sys->n_sys; b++) {
@@ -206,22 +213,23 @@ static void build_items64(ffmin_system *sys, int64_t want, std::vector<Item> &it
         while (t < tiles.size() && tiles[t].sys == b) t++;
         const int nT = (int)(t - t0);
         for (int I = 0; I < nT; I++) {
-            Tile &tl = tiles[t0 + I];
-            tl.row64 = (int)items.size();
-            tl.chunk64 = chunk;
-            tl.tloc = I;
-            tl.slot64 = (int)slots;
+            tiles[t0 + I].tloc = I;
+            tiles[t0 + I].*row = SymRow{(int32_t)slots, chunk, split, 0};
             for (int J = I; J < nT; J += chunk) {
                 const int nJ = std::min(chunk, nT - J);
-                const Tile &last = tiles[t0 + J + nJ - 1];
-                Item it{};
-                it.tile = (int)(t0 + I);
-                it.j0 = tiles[t0 + J].a0;
-                it.nj = last.a0 + last.na - it.j0;
-                it.diag = J == I ? 1 : 0;
-                it.slot = (int)slots;
-                slots += 1 + nJ;
-                items.push_back(it);
+                const Tile &jf = tiles[t0 + J], &jl = tiles[t0 + J + nJ - 1];
+                for (int p = 0; p < split; p++) {
+                    Item it{};
+                    it.tile = (int)(t0 + I);
+                    it.joff = p * (TJ / split);
+                    it.j0 = jf.a0 + it.joff;
+                    it.nj = (split > 1 ? jf.a0 + std::min(jf.na, it.joff + TJ / split) : jl.a0 + jl.na) - it.j0;
+                    it.diag = J == I ? 1 : 0;
+                    it.slot = (int)(slots + p);
+                    it.jslot = (int)(slots + split);
+                    items.push_back(it);
+                }
+                slots += split + (jrows ? nJ : 0);
             }
         }
         sys_items[b] = make_int2(first, (int)items.size() - first);
@@ -229,8 +237,31 @@ static void build_items64(ffmin_system *sys, int64_t want, std::vector<Item> &it
     *n_slots = slots;
 }
 
-// FP64 partial rows of the symmetric list above this size fall back to the
-// row sweep (its partial rows grow as the square of the atom count)
+// pairs of tiles I <= J over the batch
+static int64_t tile_pairs(const ffmin_system *sys) {
+    int64_t pairs = 0;
+    for (int b = 0; b < sys->n_sys; b++) {
+        const int64_t nT = (sys->sys_natoms[b] + TI - 1) / TI;
+        pairs += nT * (nT + 1) / 2;
+    }
+    return pairs;
+}
+
+static void build_list32e(ffmin_system *sys, int dens, std::vector<Item> &items, std::vector<int2> &sys_items,
+                          int64_t *slots) {
+    const int64_t want = (int64_t)dens * LAYOUT_SYM_BLOCKS * sys->sms;
+    build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, false, &Tile::r32, items, sys_items,
+                    slots);
+}
+static void build_list64(ffmin_system *sys, int dens, std::vector<Item> &items, std::vector<int2> &sys_items,
+                         int64_t *slots) {
+    const int64_t want = (int64_t)dens * sys->grid_sym;
+    build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, true, &Tile::r64, items, sys_items,
+                    slots);
+}
+
+// a symmetric list whose partial rows (which grow as the square of the atom
+// count) would exceed this size gives way to the row sweep
 static const int64_t SYM64_MAX_BYTES = 4LL << 30;
 
 static void set_item_counts(ffmin_system *sys, int n_items) {
@@ -239,7 +270,7 @@ static void set_item_counts(ffmin_system *sys, int n_items) {
     // no more resident blocks than work items: idle blocks would only pay
     // for queue atomics
     sys->grid32 = std::max(1, std::min(sys->grid32_max, n_items));
-    sys->grid32e = std::max(1, std::min(sys->grid32e_max, sys->c.sym64 ? sys->n_items64 : n_items));
+    sys->grid32e = std::max(1, std::min(sys->grid32e_max, sys->c.sym32 ? sys->c.n_items32 : n_items));
     sys->grid64 = std::max(1, std::min(sys->grid64_max, sys->c.sym64 ? sys->n_items64 : n_items));
 }
 
@@ -571,39 +602,52 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     std::vector<int2> sys_items;
     sys->sys_natoms.resize(n_sys);
     for (int b = 0; b < n_sys; b++) sys->sys_natoms[b] = tops[b].n_atoms;
+    const bool mixed = precision == FFMIN_MIXED;
+    {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sys->sms, cudaDevAttrMultiProcessorCount, dev);
+    }
+    sys->grid_sym = pair_grid_size(2);
     for (int k = 0; k < 2; k++) {
         sys->grid32_max_s[k] = pair_grid_size(0, k + 1);
         sys->grid32e_max_s[k] = pair_grid_size(3, k + 1);
     }
-    sys->c.f32_ipt = 2;
-    // the row list's capacity below takes the FP32 shape with more
-    // resident blocks (more items at a given density)
-    sys->grid32_max = std::max(sys->grid32_max_s[0], sys->grid32_max_s[1]);
-    sys->grid32e_max = sys->grid32e_max_s[1];
-    sys->grid64_max = sys->grid64;
-    // symmetric list: `density` items per resident block of the symmetric
-    // FP64 kernel (the autotuner rebuilds it with the row list); capacity
-    // from the densest layout the autotuner may choose.  It also fills the
-    // tiles' row64 / chunk64 / tloc, which build_items copies
-    std::vector<Item> items64;
-    std::vector<int2> sys_items64;
-    const int grid_sym = pair_grid_size(2);
-    sys->grid_sym = grid_sym;
-    int64_t slots_cap = 0;
-    build_items64(sys, (int64_t)AUTOTUNE_DENSITIES[AUTOTUNE_N - 1] * grid_sym, items64, sys_items64, &slots_cap);
+    // capacities: the densest layout the autotuner may choose, in the FP32
+    // shape with more items
+    const int dmax = AUTOTUNE_DENSITIES[AUTOTUNE_N - 1];
+    std::vector<Item> items64, items32;
+    std::vector<int2> sys_items64, sys_items32;
+    int64_t slots64_cap = 0, slots32_cap = 0, slots = 0;
+    build_list64(sys, dmax, items64, sys_items64, &slots64_cap);
     const size_t items64_cap = items64.size();
-    build_items64(sys, (int64_t)sys->density * grid_sym, items64, sys_items64, &sys->n_slots64);
-    sys->n_items64 = (int)items64.size();
-    const bool sym64 = slots_cap * TI * (int64_t)sizeof(double4_32a) <= SYM64_MAX_BYTES;
-    if (sym64) sys->grid64_max = grid_sym;
+    build_list64(sys, sys->density, items64, sys_items64, &slots);
+    size_t items32_cap = 0;
+    if (mixed) {
+        build_list32e(sys, dmax, items32, sys_items32, &slots32_cap);
+        items32_cap = items32.size();
+        build_list32e(sys, sys->density, items32, sys_items32, &slots);
+    }
+    const bool sym64 = slots64_cap * TI * (int64_t)sizeof(double4_32a) <= SYM64_MAX_BYTES;
+    const bool sym32 = mixed && slots32_cap * TI * (int64_t)sizeof(float) <= SYM64_MAX_BYTES;
     sys->c.sym64 = sym64 ? 1 : 0;
+    sys->c.sym32 = sym32 ? 1 : 0;
+    sys->n_items64 = (int)items64.size();
     sys->c.n_items64 = sym64 ? sys->n_items64 : 0;
-    sys->n_slots64 = slots_cap;  // allocation size of the partial rows
-    // capacity: the densest layout the autotuner may choose
-    build_items(sys, AUTOTUNE_DENSITIES[AUTOTUNE_N - 1], items, tiles, sys_items);
-    sys->items_cap = (int64_t)items.size();
+    sys->c.n_items32 = sym32 ? (int)items32.size() : 0;
+    sys->n_slots64 = slots64_cap;  // allocation size of the partial rows
+    sys->grid64_max = sym64 ? sys->grid_sym : sys->grid64;
+    tiles = sys->tiles_h;
+    sys_items.assign(n_sys, make_int2(0, 0));
+    if (needs_row_list(sys)) {
+        sys->c.f32_ipt = 2;
+        build_items(sys, dmax, items, tiles, sys_items);
+        sys->items_cap = (int64_t)items.size();
+        build_items(sys, sys->density, items, tiles, sys_items);
+    }
+    sys->c.f32_ipt = 2;
     sys->grid32_max = sys->grid32_max_s[1];
-    build_items(sys, sys->density, items, tiles, sys_items);
+    sys->grid32e_max = sys->grid32e_max_s[1];
     std::vector<int32_t> inc_off(total + 1, 0);
     std::vector<int2> inc;
     for (int64_t a = 0; a < total; a++) {
@@ -657,6 +701,14 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
         c.items64 = sys->d_items64;
         c.sys_items64 = sys->d_sys_items64;
     }
+    if (sym32) {
+        CKC(dalloc(sys, &sys->d_items32, items32_cap));
+        CKC(cudaMemcpyAsync(sys->d_items32, items32.data(), items32.size() * sizeof(Item), cudaMemcpyHostToDevice,
+                            sys->stream));
+        CKC(upload(sys, &sys->d_sys_items32, sys_items32));
+        c.items32 = sys->d_items32;
+        c.sys_items32 = sys->d_sys_items32;
+    }
     CKC(dalloc(sys, &c.act, N_LISTS * (2 * (size_t)n_sys + 2)));
     SysState *d_st;
     CKC(dalloc(sys, &d_st, n_sys));
@@ -680,7 +732,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
             CKC(upload(sys, &d_parf, parf));
             c.parf = d_parf;
             CKC(dalloc(sys, &c.gpf, (size_t)sys->items_cap * TI));
-            if (sym64) CKC(dalloc(sys, &c.gpf_sym, (size_t)sys->n_slots64 * TI));
+            if (sym32) CKC(dalloc(sys, &c.gpf_sym, (size_t)slots32_cap * TI));
         }
     }
     int32_t *d_inc_off; int2 *d_inc, *d_bidx; double2 *d_bpar, *d_apar; int4 *d_aidx, *d_didx; double4_32a *d_dpar;
@@ -727,6 +779,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     CKC(dalloc(sys, &c.te, std::max(n_terms, 1)));
     CKC(dalloc(sys, &c.tg, 3 * (2 * bidx.size() + 3 * aidx.size() + 4 * didx.size() + 2 * xidx.size()) + 3));
     CKC(dalloc(sys, &c.red, (size_t)c.n_tiles * NRED));
+    CKC(dalloc(sys, &c.redf, (size_t)c.n_tiles * 4 * 8));
     CKC(dalloc(sys, &c.counters, CNT_N));
     CKC(dalloc(sys, &c.nactive, 1));
     CKC(dalloc(sys, &c.nmode, 2));
@@ -911,7 +964,6 @@ static ffmin_status ensure_loop(ffmin_system *sys) {
 // pair energy of the last E + grad evaluation (at `slot`), bonded terms in FP64
 static ffmin_status eval_slot(ffmin_system *sys, int slot, int kind, int dir = -1, double h = 0.0,
                               int delta = 0) {
-    const Ctx &c = sys->c;
     for (int b = 0; b < sys->n_sys; b++) {
         SysState &S = sys->hst[b];
         S.active = 1;
@@ -1334,28 +1386,42 @@ ffmin_status ffmin_neighbour_counts(ffmin_system *sys, const double *x_dev, int3
 // rebuilt at the next minimization.
 static ffmin_status install_layout(ffmin_system *sys, int dens, int ipt) {
     sys->c.f32_ipt = ipt;
+    std::vector<Item> items, list;
+    std::vector<Tile> tiles;
+    std::vector<int2> sys_items, sys_list;
+    int64_t slots = 0;
+    // the symmetric lists first: they set the rows of tiles_h
     sys->grid32_max = sys->grid32_max_s[ipt - 1];
     sys->grid32e_max = sys->grid32e_max_s[ipt - 1];
-    std::vector<Item> items, items64;
-    std::vector<Tile> tiles;
-    std::vector<int2> sys_items, sys_items64;
-    if (sys->c.sym64) {  // the symmetric list first: it sets the tiles' row64 / chunk64 / slot64
-        int64_t slots = 0;
-        build_items64(sys, (int64_t)dens * sys->grid_sym, items64, sys_items64, &slots);
-        CK(cudaMemcpyAsync(sys->d_items64, items64.data(), items64.size() * sizeof(Item), cudaMemcpyHostToDevice,
+    if (sys->c.sym32) {
+        build_list32e(sys, dens, list, sys_list, &slots);
+        CK(cudaMemcpyAsync(sys->d_items32, list.data(), list.size() * sizeof(Item), cudaMemcpyHostToDevice,
                            sys->stream));
-        CK(cudaMemcpyAsync(sys->d_sys_items64, sys_items64.data(), sys_items64.size() * sizeof(int2),
+        CK(cudaMemcpyAsync(sys->d_sys_items32, sys_list.data(), sys_list.size() * sizeof(int2),
                            cudaMemcpyHostToDevice, sys->stream));
-        sys->n_items64 = (int)items64.size();
+        sys->c.n_items32 = (int)list.size();
+        CK(cudaStreamSynchronize(sys->stream));  // the vectors are reused below
+    }
+    if (sys->c.sym64) {
+        build_list64(sys, dens, list, sys_list, &slots);
+        CK(cudaMemcpyAsync(sys->d_items64, list.data(), list.size() * sizeof(Item), cudaMemcpyHostToDevice,
+                           sys->stream));
+        CK(cudaMemcpyAsync(sys->d_sys_items64, sys_list.data(), sys_list.size() * sizeof(int2),
+                           cudaMemcpyHostToDevice, sys->stream));
+        sys->n_items64 = (int)list.size();
         sys->c.n_items64 = sys->n_items64;
     }
-    build_items(sys, dens, items, tiles, sys_items);
-    CK(cudaMemcpyAsync(sys->d_items, items.data(), items.size() * sizeof(Item), cudaMemcpyHostToDevice,
-                       sys->stream));
-    CK(cudaMemcpyAsync(sys->d_sys_items, sys_items.data(), sys_items.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                       sys->stream));
+    tiles = sys->tiles_h;
+    if (needs_row_list(sys)) {
+        build_items(sys, dens, items, tiles, sys_items);
+        CK(cudaMemcpyAsync(sys->d_items, items.data(), items.size() * sizeof(Item), cudaMemcpyHostToDevice,
+                           sys->stream));
+        CK(cudaMemcpyAsync(sys->d_sys_items, sys_items.data(), sys_items.size() * sizeof(int2),
+                           cudaMemcpyHostToDevice, sys->stream));
+    }
     CK(cudaMemcpyAsync(sys->d_tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice,
                        sys->stream));
+    CK(cudaStreamSynchronize(sys->stream));  // before the vectors go
     set_item_counts(sys, (int)items.size());
     sys->density = dens;
     if (sys->graph) {  // kernel parameters (item count, grid, shape) changed

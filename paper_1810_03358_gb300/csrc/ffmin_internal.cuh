@@ -8,8 +8,9 @@
 //   - pair-kernel inputs rewritten for every evaluation: per atom float4 or
 //     double4_32a (x, y, z, q*sqrt(C)) and constant float2 / double2
 //     (sigma, sqrt(24 eps));
-//   - per-(tile, j-chunk) partial row sums of the pair kernel
-//     ([n_items][TI] float4 or double4_32a: gx, gy, gz, row energy);
+//   - partial rows of the pair kernels, [slot][TI] float4 or double4_32a
+//     (gx, gy, gz, row energy): per work item its i-side rows, and on the
+//     symmetric lists its j-side rows;
 //   - bonded terms (FP64) with a per-atom incidence list, so that every
 //     atom gathers its own bonded gradient without atomics;
 //   - per-system control state (SysState) driven by the last block of the
@@ -55,24 +56,30 @@ enum Phase : int {
     PH_OGM_UPD, PH_OGM_Y, PH_HB
 };
 
-// a pair item (i-tile, j-chunk); tile < 0 marks a bonded item whose j0, nj
-// is a range of bonded terms (of one type and one system, diag = system).
-// Row-sweep lists (FP32, and FP64 when the symmetric list would not fit):
-// every j of the system's row, slot unused.  Symmetric FP64 list: j-chunks
-// of whole tiles at or right of the i-tile; the item writes its i-side
-// partial rows to slot and the j-side rows of its q-th j-tile to slot + 1 + q.
-struct Item { int32_t tile, j0, nj, diag, slot, pad0, pad1, pad2; };
+// A pair item; tile < 0 marks a bonded item whose j0, nj is a range of bonded
+// terms (of one type and one system, diag = system).
+// Row list (FP32 E + grad, and FP64 terms whose symmetric rows would not
+// fit): the j-chunk [j0, j0 + nj) of the row of i-tile `tile`; diag: the chunk
+// holds the i-tile; slot and below unused.
+// Symmetric lists (FP64 terms; FP32 energy only): a chunk of whole j-tiles at
+// or right of the i-tile (diag: it starts with the i-tile), or one part of a
+// single j-tile (see SymRow; nj <= 0 for a part beyond a ragged tile).  slot:
+// the item's i-side slot, jslot: the j-side slot of its first j-tile, joff:
+// offset of j0 inside its j-tile.
+struct Item { int32_t tile, j0, nj, diag, slot, jslot, joff, pad; };
 constexpr int BONDED_ITEM_TERMS = 64;
 
-// item0 / nitem: the tile's items in the row-sweep list; row64: its first
-// item in the symmetric list (row of tile pairs (tile, J >= tile)), chunk64:
-// j-tiles per symmetric item of its system, tloc: index inside its system;
-// slot64: the partial-row slot of its row's first symmetric item (the row's
-// items hold consecutive slots, 1 + chunk64 per item, so the q-th item of
-// the row starts at slot64 + q * (1 + chunk64));
-// xlo / xhi: the smallest and largest scaled partner (exclusion variant) of
-// its atoms, xlo > xhi when there is none
-struct Tile { int32_t sys, a0, na, item0, nitem, row64, chunk64, tloc, xlo, xhi, slot64, pad1; };
+// Row of a symmetric list: the items of one i-tile, by j.  Every `chunk`
+// j-tiles take split + chunk slots from `slot` on: the i-side rows of each
+// part, then one j-side row per j-tile.  split > 1 (parts of 128 / split
+// j-atoms, for objects with few tiles) only with chunk == 1.
+struct SymRow { int32_t slot, chunk, split, pad; };
+
+// item0 / nitem: the tile's items in the row list; tloc: index inside its
+// system; r64 / r32: its row in the FP64 and in the FP32 energy-only
+// symmetric list; xlo / xhi: the smallest and largest scaled partner
+// (exclusion variant) of its atoms, xlo > xhi when there is none
+struct Tile { int32_t sys, a0, na, item0, nitem, tloc, xlo, xhi; SymRow r64, r32; };
 
 struct DirOp {
     int32_t on, use_d, dots;  // dots: 1 -> |R|^2, <G,R>; 2 -> <Y_j, R> for the Y list
@@ -172,7 +179,7 @@ struct Ctx {
     const double2 *pard;
     const double *qs;       // q * sqrt(C) per atom (FP64)
     float4 *gpf;            // [n_items][TI]
-    float4 *gpf_sym;        // [slots of items64][TI]: FP32 energy-only rows (i-side) on the symmetric list
+    float *gpf_sym;         // [slots of items32][TI]: FP32 energy-only rows
     double4_32a *gpd;
     // bonded terms
     const int32_t *inc_off; // [n_atoms + 1]
@@ -194,18 +201,19 @@ struct Ctx {
     const float *xs_val;
     const int32_t *term_sys;  // [n_terms] system of each bonded term
     const int2 *sys_items;  // [n_sys] (first, count) of each system's work items (contiguous)
-    // FP64 pair terms: sym64 = 1 evaluates each unordered pair once
-    // (symmetric tiles, list items64 / sys_items64, partial rows gpd
-    // [slots][TI]); 0 uses the row sweep over items / sys_items
-    int32_t sym64, n_items64;
-    const Item *items64;
-    const int2 *sys_items64;
+    // sym64 / sym32 = 1: the FP64 terms / the FP32 energy-only evaluations run
+    // on a symmetric list (each unordered pair once; items64 / items32,
+    // partial rows gpd / gpf_sym); 0: the row list
+    int32_t sym64, n_items64, sym32, n_items32;
+    const Item *items64, *items32;
+    const int2 *sys_items64, *sys_items32;
     int32_t *act;           // per work queue L: [L * (2 n_sys + 2)]: active systems, their items,
                             // item prefix [n_sys], system ids [n_sys] (rebuilt every launch)
     double *te;             // [n_terms] energy of each bonded term
     double *tg;             // [2 nb + 3 na + 4 nd][3] gradient of each term at each position
     // reductions
     double *red;            // [n_tiles][NRED]
+    double *redf;           // finalize: [value][4 n_tiles]
     unsigned int *counters; // one per kernel kind, reset by the last block
     int32_t *nactive;       // systems still minimizing
     int32_t *nmode;         // [2] active systems per pair-kernel precision mode

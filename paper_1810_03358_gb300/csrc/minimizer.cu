@@ -65,153 +65,215 @@ __global__ void __launch_bounds__(TI) k_prepare(Ctx c) {
 }
 
 // ---------------------------------------------------------------- finalize
-// sum over q < n of f(q) (a double4; only .x .y .z when XYZ, only .w when
-// W) in four interleaved strands (q mod 4), combined as (s0 + s1) + (s2 + s3):
-// every group of four loads is issued together and no dependent chain of
-// FP64 adds is longer than n / 4 + 2
+// Bound: latency and the FP64 pipe (16 cycles per warp operation and SM).
+// Four blocks per tile, 32 atoms each: lane = atom, warp = strand, so an
+// atom's partial rows and bonded terms are summed by four threads (rows
+// q mod 4, combined in strand order through shared memory), and a small
+// system's sums spread over four times the SMs.  One thread per atom took
+// 25 us for 500 atoms and 31 us for 3,334 (cold caches).
+constexpr int FIN_SUB = TI / 32;  // blocks per tile
+
+// exact FP32 -> FP64 on the integer pipe (the conversion instruction runs at
+// the FP64 rate); the FP32 kernels flush denormals, which read as zero
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    unsigned hi = m >= 0x7f800000u ? (m >> 3) | 0x70000000u : (m >> 3) + 0x38000000u;  // inf, NaN : normal
+    const bool zero = m < 0x00800000u;
+    hi = zero ? 0u : hi;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), zero ? 0 : (int)(u << 29));
+}
+
+struct Row4 {
+    double x, y, z, w;
+};
+__device__ __forceinline__ Row4 row_at(const float4 *rows, int64_t slot, int i) {
+    const float4 p = rows[slot * TI + i];
+    return Row4{widen(p.x), widen(p.y), widen(p.z), widen(p.w)};
+}
+__device__ __forceinline__ Row4 row_at(const double4_32a *rows, int64_t slot, int i) {
+    const double4_32a p = rows[slot * TI + i];
+    return Row4{p.x, p.y, p.z, p.w};
+}
+
+// this strand's share (w, w + 4, ...) of the sum over q < n of f(q), added to
+// a; XYZ / W: the components that count
 template <bool XYZ, bool W, typename F>
-__device__ __forceinline__ double4 strand_sum(int n, F f) {
-    double ax[4] = {0.0, 0.0, 0.0, 0.0}, ay[4] = {0.0, 0.0, 0.0, 0.0};
-    double az[4] = {0.0, 0.0, 0.0, 0.0}, aw[4] = {0.0, 0.0, 0.0, 0.0};
-    int q = 0;
-    for (; q + 4 <= n; q += 4) {
-        double4 p[4];
+__device__ __forceinline__ void strand_sum(int n, int w, Row4 &a, F f) {
+    int q = w;
+    for (; q + 12 < n; q += 16) {  // four loads in flight
+        Row4 p[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) p[u] = f(q + u);
+        for (int u = 0; u < 4; u++) p[u] = f(q + 4 * u);
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            if (XYZ) { ax[u] += p[u].x; ay[u] += p[u].y; az[u] += p[u].z; }
-            if (W) aw[u] += p[u].w;
+            if (XYZ) { a.x += p[u].x; a.y += p[u].y; a.z += p[u].z; }
+            if (W) a.w += p[u].w;
         }
+    }
+    for (; q < n; q += 4) {
+        const Row4 p = f(q);
+        if (XYZ) { a.x += p.x; a.y += p.y; a.z += p.z; }
+        if (W) a.w += p.w;
+    }
+}
+
+// FP64 rows of atom i of tile t on the symmetric list: the j-side rows the
+// tile received from the rows of the tiles at or left of it, then its own
+// row's i-side rows (every part of every item)
+template <bool GRAD>
+__device__ __forceinline__ void sym_rows(const Ctx &c, const Tile &t, int tile0, int ntile, int i, int w, Row4 &a) {
+    const int T = t.tloc, C = t.r64.chunk, P = t.r64.split;
+    if (GRAD)
+        strand_sum<true, false>(T + 1, w, a, [&](int I) {
+            const int q = T - I;
+            return row_at(c.gpd, (int64_t)c.tiles[tile0 + I].r64.slot + (int64_t)(q / C) * (P + C) + P + q % C, i);
+        });
+    strand_sum<GRAD, true>((ntile - T + C - 1) / C * P, w, a, [&](int m) {
+        return row_at(c.gpd, (int64_t)t.r64.slot + (int64_t)(m / P) * (P + C) + m % P, i);
+    });
+}
+
+// sum (or max) of finalize value k over a system's blocks, fixed order, by a
+// whole warp; the result is valid on every lane
+__device__ double fin_sys_sum(const Ctx &c, const SysState &S, int k, int nb, bool mx) {
+    const int lane = threadIdx.x & 31, b1 = FIN_SUB * (S.tile0 + S.ntile);
+    const double *r = c.redf + (int64_t)k * nb;
+    double x = 0.0;
+#pragma unroll 4
+    for (int b = FIN_SUB * S.tile0 + lane; b < b1; b += 32) {
+        const double y = __ldcg(&r[b]);
+        x = mx ? fmax(x, y) : x + y;
     }
 #pragma unroll
-    for (int u = 0; u < 3; u++) {
-        if (q + u < n) {
-            const double4 p = f(q + u);
-            if (XYZ) { ax[u] += p.x; ay[u] += p.y; az[u] += p.z; }
-            if (W) aw[u] += p.w;
-        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = mx ? fmax(x, y) : x + y;
     }
-    return make_double4(XYZ ? (ax[0] + ax[1]) + (ax[2] + ax[3]) : 0.0, XYZ ? (ay[0] + ay[1]) + (ay[2] + ay[3]) : 0.0,
-                        XYZ ? (az[0] + az[1]) + (az[2] + az[3]) : 0.0, W ? (aw[0] + aw[1]) + (aw[2] + aw[3]) : 0.0);
+    return x;
 }
 
 __global__ void __launch_bounds__(TI) k_finalize(Ctx c) {
-    const Tile t = c.tiles[blockIdx.x];
-    const int kind = c.st[t.sys].ev_kind;
-    const int mode = c.st[t.sys].mode;
-    double v[RF_N];
-#pragma unroll
-    for (int k = 0; k < RF_N; k++) v[k] = 0.0;
-    const int i = threadIdx.x;
-    if (kind != EV_NONE && i < t.na) {
+    const Tile &t = c.tiles[blockIdx.x / FIN_SUB];
+    const SysState &S = c.st[t.sys];
+    const int kind = S.ev_kind, mode = S.mode;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nb = gridDim.x;
+    __shared__ Row4 part[2][NW][32];  // pair rows, bonded terms
+    __shared__ double val[RF_N][32];
+    const unsigned maxmask = (1u << RF_GINF) | (1u << RF_BAD);
+    if (kind != EV_NONE) {
+        const int i = (blockIdx.x % FIN_SUB) * 32 + lane;
+        const bool real = i < t.na, grad = kind == EV_EG;
         const int a = t.a0 + i;
-        double e, g0 = 0.0, g1 = 0.0, g2 = 0.0;
-        if (mode == 0 && c.sym64 && kind == EV_E) {
-            // FP32 energy only on the symmetric list: the i-side rows of the
-            // tile's own row of items (consecutive slots, 1 + C apart), each
-            // pair counted once
-            const SysState &S = c.st[t.sys];
-            const int T = t.tloc, C = t.chunk64;
-            const int nch = (S.ntile - T + C - 1) / C;
-            e = strand_sum<false, true>(nch, [&](int q) {
-                    const float4 p = c.gpf_sym[((int64_t)t.slot64 + (int64_t)q * (1 + C)) * TI + i];
-                    return make_double4(0.0, 0.0, 0.0, (double)p.w);
-                }).w;
-        } else if (mode == 0) {
-            const double4 r = strand_sum<true, true>(t.nitem, [&](int it) {
-                const float4 p = c.gpf[(int64_t)(t.item0 + it) * TI + i];
-                return make_double4((double)p.x, (double)p.y, (double)p.z, (double)p.w);
-            });
-            e = 0.5 * r.w;  // every pair was counted in both of its rows
-            g0 = r.x; g1 = r.y; g2 = r.z;
-        } else if (c.sym64) {
-            // symmetric tiles: the j-side rows this tile received from the
-            // items of rows I <= T, then its own row's i-side rows; each
-            // pair's energy was counted once (the slot of row I's item u is
-            // tiles[I].slot64 + u * (1 + C))
-            const SysState &S = c.st[t.sys];
-            const int T = t.tloc, C = t.chunk64;
-            double4 rj = make_double4(0.0, 0.0, 0.0, 0.0);
-            if (kind == EV_EG)
-                rj = strand_sum<true, false>(T + 1, [&](int I) {
-                    const int q = T - I;
-                    const int64_t slot = (int64_t)c.tiles[S.tile0 + I].slot64 + (int64_t)(q / C) * (1 + C) + 1 + q % C;
-                    const double4_32a p = c.gpd[slot * TI + i];
-                    return make_double4(p.x, p.y, p.z, 0.0);
+        Row4 r = Row4{0.0, 0.0, 0.0, 0.0}, bo = r;
+        if (real) {
+            if (mode == 0 && c.sym32 && !grad) {
+                // energies on the symmetric list, each pair counted once
+                const int C = t.r32.chunk;
+                strand_sum<false, true>((S.ntile - t.tloc + C - 1) / C, w, r, [&](int q) {
+                    const int64_t slot = (int64_t)t.r32.slot + (int64_t)q;
+                    return Row4{0.0, 0.0, 0.0, widen(c.gpf_sym[slot * TI + i])};
                 });
-            const int nch = (S.ntile - T + C - 1) / C;
-            const double4 ri = strand_sum<true, true>(nch, [&](int q) {
-                const double4_32a p = c.gpd[((int64_t)t.slot64 + (int64_t)q * (1 + C)) * TI + i];
-                return make_double4(p.x, p.y, p.z, p.w);
-            });
-            e = ri.w;
-            g0 = rj.x + ri.x; g1 = rj.y + ri.y; g2 = rj.z + ri.z;
-        } else {
-            const double4 r = strand_sum<true, true>(t.nitem, [&](int it) {
-                const double4_32a p = c.gpd[(int64_t)(t.item0 + it) * TI + i];
-                return make_double4(p.x, p.y, p.z, p.w);
-            });
-            e = 0.5 * r.w;  // every pair was counted in both of its rows
-            g0 = r.x; g1 = r.y; g2 = r.z;
-        }
-        v[RF_EPAIR] = e;
-        // bonded terms: evaluated once per term by the pair kernel's bonded
-        // items; every atom gathers its terms' energies (as owner) and
-        // position gradients through its incidence list (four entries'
-        // loads issued together; entry u of each group to strand u mod 2)
-        const bool grad = kind == EV_EG;
-        double be[2] = {0.0, 0.0}, bg[2][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
-        const int k1 = c.inc_off[a + 1];
-        for (int k = c.inc_off[a]; k < k1; k += 4) {
-            int2 in[4];
-            double te[4], gb[4][3];
-#pragma unroll
-            for (int u = 0; u < 4; u++) in[u] = k + u < k1 ? c.inc[k + u] : make_int2(-1, 0);
-#pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int type = in[u].x >> 2, pos = in[u].x & 3;
-                te[u] = in[u].x >= 0 && pos == 0 ? c.te[bonded_index(c, type, in[u].y)] : 0.0;
-                if (grad && in[u].x >= 0) {
-                    const double *g = c.tg + 3 * bonded_grad_slot(c, type, in[u].y, pos);
-                    gb[u][0] = g[0]; gb[u][1] = g[1]; gb[u][2] = g[2];
+            } else if (mode == 0) {
+                strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpf, t.item0 + it, i); });
+                r.w *= 0.5;  // every pair was counted in both of its rows
+            } else if (c.sym64) {
+                if (grad) sym_rows<true>(c, t, S.tile0, S.ntile, i, w, r);
+                else sym_rows<false>(c, t, S.tile0, S.ntile, i, w, r);
+            } else {
+                strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpd, t.item0 + it, i); });
+                r.w *= 0.5;
+            }
+            // bonded terms: evaluated once per term by the pair kernel's
+            // bonded items; every atom gathers its terms' energies (as owner)
+            // and position gradients through its incidence list
+            const int k1 = c.inc_off[a + 1];
+            for (int k = c.inc_off[a] + w; k < k1; k += NW) {
+                const int2 in = c.inc[k];
+                const int type = in.x >> 2, pos = in.x & 3;
+                if (pos == 0) bo.w += c.te[bonded_index(c, type, in.y)];
+                if (grad) {
+                    const double *g = c.tg + 3 * bonded_grad_slot(c, type, in.y, pos);
+                    bo.x += g[0]; bo.y += g[1]; bo.z += g[2];
                 }
             }
+        }
+        part[0][w][lane] = r;
+        part[1][w][lane] = bo;
+        __syncthreads();
+        if (w == 0) {
+            double v[RF_N];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                if (in[u].x < 0) break;
-                if ((in[u].x & 3) == 0) be[u & 1] += te[u];
-                if (grad) { bg[u & 1][0] += gb[u][0]; bg[u & 1][1] += gb[u][1]; bg[u & 1][2] += gb[u][2]; }
+            for (int k = 0; k < RF_N; k++) v[k] = 0.0;
+            if (real) {
+                const Row4 r1 = part[0][1][lane], r2 = part[0][2][lane], r3 = part[0][3][lane];
+                const Row4 b1 = part[1][1][lane], b2 = part[1][2][lane], b3 = part[1][3][lane];
+                r.w = (r.w + r1.w) + (r2.w + r3.w);
+                bo.w = (bo.w + b1.w) + (b2.w + b3.w);
+                if (grad) {
+                    r.x = (r.x + r1.x) + (r2.x + r3.x);
+                    r.y = (r.y + r1.y) + (r2.y + r3.y);
+                    r.z = (r.z + r1.z) + (r2.z + r3.z);
+                    bo.x = (bo.x + b1.x) + (b2.x + b3.x);
+                    bo.y = (bo.y + b1.y) + (b2.y + b3.y);
+                    bo.z = (bo.z + b1.z) + (b2.z + b3.z);
+                }
+                const double e = r.w + bo.w;
+                v[RF_EPAIR] = r.w;
+                v[RF_E] = e;
+                bool bad = !isfinite(e);
+                if (grad) {
+                    const double g0 = r.x + bo.x, g1 = r.y + bo.y, g2 = r.z + bo.z;
+                    double *gt = vslot(c, V_GT) + 3 * a;
+                    gt[0] = g0; gt[1] = g1; gt[2] = g2;
+                    const double *G = vslot(c, V_G) + 3 * a;
+                    const double *R = vslot(c, V_R) + 3 * a;
+                    v[RF_GG] = fma(g0, g0, fma(g1, g1, g2 * g2));
+                    v[RF_GINF] = fmax(fabs(g0), fmax(fabs(g1), fabs(g2)));
+                    v[RF_GTG] = fma(g0, G[0], fma(g1, G[1], g2 * G[2]));
+                    v[RF_GTR] = fma(g0, R[0], fma(g1, R[1], g2 * R[2]));
+                    bad = bad || !isfinite(g0) || !isfinite(g1) || !isfinite(g2);
+                }
+                v[RF_BAD] = bad ? 1.0 : 0.0;
             }
+#pragma unroll
+            for (int k = 0; k < RF_N; k++) val[k][lane] = v[k];
         }
-        e += be[0] + be[1];
-        if (grad) {
-            g0 += bg[0][0] + bg[1][0];
-            g1 += bg[0][1] + bg[1][1];
-            g2 += bg[0][2] + bg[1][2];
+        __syncthreads();
+        for (int k = w; k < RF_N; k += NW) {  // value k over the block's atoms (butterfly)
+            const bool mx = (maxmask >> k) & 1u;
+            double x = val[k][lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double y = __shfl_xor_sync(0xffffffffu, x, o);
+                x = mx ? fmax(x, y) : x + y;
+            }
+            if (lane == 0) c.redf[(int64_t)k * nb + blockIdx.x] = x;
         }
-        v[RF_E] = e;
-        bool bad = !isfinite(e);
-        if (grad) {
-            double *gt = vslot(c, V_GT) + 3 * a;
-            gt[0] = g0; gt[1] = g1; gt[2] = g2;
-            const double *G = vslot(c, V_G) + 3 * a;
-            const double *R = vslot(c, V_R) + 3 * a;
-            v[RF_GG] = fma(g0, g0, fma(g1, g1, g2 * g2));
-            v[RF_GINF] = fmax(fabs(g0), fmax(fabs(g1), fabs(g2)));
-            v[RF_GTG] = fma(g0, G[0], fma(g1, G[1], g2 * G[2]));
-            v[RF_GTR] = fma(g0, R[0], fma(g1, R[1], g2 * R[2]));
-            bad = bad || !isfinite(g0) || !isfinite(g1) || !isfinite(g2);
-        }
-        v[RF_BAD] = bad ? 1.0 : 0.0;
     }
-    const unsigned maxmask = (1u << RF_GINF) | (1u << RF_BAD);
-    block_reduce_columns<RF_N>(v, RF_N, maxmask, &c.red[(int64_t)blockIdx.x * NRED]);
     if (c.sep_reduce || !last_block(&c.counters[CNT_FIN])) return;
-    last_block_systems<RF_N>(
-        c, RF_N, maxmask, [](const SysState &S) { return S.ev_kind != EV_NONE; },
-        [&](SysState &S, const double *tot) { on_eval_done(c, S, tot); }, nullptr);
+    // fewer than 8 systems: the last block sums every system's blocks, one
+    // (system, value) per warp at a time, then warp 0 runs the control steps
+    // in system order on a shared-memory copy of the state
+    __shared__ double tot[LB_MAX_SYS][RF_N];
+    __shared__ SysState sS;
+    const int n = c.n_sys < LB_MAX_SYS ? c.n_sys : LB_MAX_SYS;
+    for (int u = w; u < n * RF_N; u += NW) {
+        const SysState &Sb = c.st[u / RF_N];
+        if (Sb.ev_kind == EV_NONE) continue;
+        const double x = fin_sys_sum(c, Sb, u % RF_N, nb, (maxmask >> (u % RF_N)) & 1u);
+        if (lane == 0) tot[u / RF_N][u % RF_N] = x;
+    }
     __syncthreads();
+    if (w == 0) {
+        for (int b = 0; b < n; b++) {
+            if (c.st[b].ev_kind == EV_NONE) continue;
+            warp_copy_state(&sS, &c.st[b]);
+            if (lane == 0) on_eval_done(c, sS, tot[b]);
+            __syncwarp();
+            warp_copy_state(&c.st[b], &sS);
+        }
+    }
     if (threadIdx.x == 0) c.counters[CNT_FIN] = 0;
 }
 
@@ -448,7 +510,8 @@ __global__ void __launch_bounds__(TI) k_sysreduce(Ctx c) {
     __shared__ SysState sS;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int k = w; k < nv; k += NW) {
-        const double x = warp_sys_sum(c, S, k, (maxmask >> k) & 1u);
+        const double x = STAGE == 3 ? fin_sys_sum(c, S, k, FIN_SUB * c.n_tiles, (maxmask >> k) & 1u)
+                                    : warp_sys_sum(c, S, k, (maxmask >> k) & 1u);
         if (lane == 0) tot[k] = x;
     }
     __syncthreads();
@@ -536,7 +599,7 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s) {
-    k_finalize<<<c.n_tiles, TI, 0, s>>>(c);
+    k_finalize<<<FIN_SUB * c.n_tiles, TI, 0, s>>>(c);
     return cudaGetLastError();
 }
 cudaError_t launch_update(const Ctx &c, cudaStream_t s) {

@@ -223,18 +223,169 @@ __device__ __forceinline__ void sweep_delta_factored(const float4 *__restrict__ 
     }
 }
 
+// Packed forms of the unmasked FP32 sweeps for two i-atoms per thread (i-atom
+// u in lane u of every packed register): fma.rn.f32x2 and its kin take one
+// issue slot for two lanes of the FMA pipe, which takes issue (25 scalar
+// instructions a pair with forces, 39 for a difference trial) off the list of
+// bounds.  What bounds them now is the register file: an fma2 of three
+// different registers takes 3 cycles of a partition and not 2 (measured in
+// isolation), 51 cycles for the two pairs of a step with forces where the FMA
+// pipe alone would take 44.  30,000 atoms: E + grad 0.737 -> 0.682 ms, difference
+// trial 0.568 -> 0.506 ms, energy 0.237 -> 0.227 ms.  Every lane performs the
+// operations of the scalar sweep in its order with its roundings, fused
+// multiply-adds included: a minimization amplifies any other rounding of
+// these sums (1e-7 in a gradient is 1e-3 A ten steps later), so both forms
+// give the same bits.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void upk(f2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// a j-atom staged with both lanes equal, so that a packed operand is what a
+// 128-bit load returns: building the pairs by moves puts scalar instructions
+// between the packed ones, which stalls the FMA pipe (78 % busy instead of
+// the 90s, measured)
+struct J2 {
+    ulonglong2 xy, zq, c;  // (x x, y y), (z z, q' q'), (c6 c6, c12 c12)
+};
+
+// r^-1 of a packed r^2; DM as in sweep()
+template <int DM>
+__device__ __forceinline__ f2 rsqrt2(f2 r2, int k, const int (&dk)[2]) {
+    float a, b;
+    upk(r2, a, b);
+    a = rsqrt_approx(a);
+    b = rsqrt_approx(b);
+    if (DM == 1) { a = k == dk[0] ? 0.f : a; b = k == dk[1] ? 0.f : b; }
+    if (DM == 2) { a = k <= dk[0] ? 0.f : a; b = k <= dk[1] ? 0.f : b; }
+    return pk(a, b);
+}
+
+// the i-atoms of a thread: negated coordinates, (q', -c6, c12)
+struct IPair {
+    f2 nx, ny, nz, q, nc6, c12;
+};
+
+template <int DM>
+__device__ __forceinline__ void sweep2(const J2 *__restrict__ sj, const IPair &A, const int (&dk)[2],
+                                       f2 &gx, f2 &gy, f2 &gz, f2 &ec, f2 &lj) {
+#pragma unroll 8
+    for (int k = 0; k < TJ; k++) {
+        const ulonglong2 xy = sj[k].xy, zq = sj[k].zq, cj = sj[k].c;
+        const f2 dx = add2(xy.x, A.nx), dy = add2(xy.y, A.ny), dz = add2(zq.x, A.nz);
+        const f2 r2 = fma2(dz, dz, fma2(dx, dx, mul2(dy, dy)));
+        const f2 ri = rsqrt2<DM>(r2, k, dk);
+        const f2 ri2 = mul2(ri, ri);
+        const f2 qq = mul2(A.q, zq.y);
+        const f2 ri6 = mul2(mul2(ri2, ri2), ri2);
+        const f2 p12 = mul2(mul2(A.c12, cj.y), ri6);
+        const f2 t1 = fma2(A.nc6, cj.x, p12);
+        ec = fma2(qq, ri, ec);
+        lj = fma2(ri6, t1, lj);
+        const f2 f = mul2(fma2(qq, ri, mul2(ri6, add2(p12, t1))), ri2);
+        gx = fma2(f, dx, gx);
+        gy = fma2(f, dy, gy);
+        gz = fma2(f, dz, gz);
+    }
+}
+
+template <int DM>
+__device__ __forceinline__ void sweep2_e(const J2 *__restrict__ sj, const IPair &A, const int (&dk)[2], f2 &fa, f2 &f6, f2 &f12) {
+#pragma unroll 8
+    for (int k = 0; k < TJ; k++) {
+        const ulonglong2 xy = sj[k].xy, zq = sj[k].zq, cj = sj[k].c;
+        const f2 dx = add2(xy.x, A.nx), dy = add2(xy.y, A.ny), dz = add2(zq.x, A.nz);
+        const f2 r2 = fma2(dz, dz, fma2(dx, dx, mul2(dy, dy)));
+        const f2 ri = rsqrt2<DM>(r2, k, dk);
+        const f2 ri2 = mul2(ri, ri);
+        const f2 ri6 = mul2(mul2(ri2, ri2), ri2);
+        fa = fma2(zq.y, ri, fa);
+        f6 = fma2(cj.x, ri6, f6);
+        f12 = fma2(cj.y, mul2(ri6, ri6), f12);
+    }
+}
+
+// the i-atoms' displacements are negated like their coordinates.  The scalar
+// form negates D before it multiplies; here the last sums change sign instead
+// (exact), so fa, f6, f12 hold the opposite of its sums
+template <int DM>
+__device__ __forceinline__ void sweep2_delta(const J2 *__restrict__ sj, const ulonglong2 *__restrict__ sexy,
+                                             const f2 *__restrict__ sez, const IPair &A, f2 nex, f2 ney, f2 nez,
+                                             const int (&dk)[2], f2 &fa, f2 &f6, f2 &f12) {
+    const f2 two = pk(2.f, 2.f);
+#pragma unroll 4
+    for (int k = 0; k < TJ; k++) {
+        const ulonglong2 xy = sj[k].xy, zq = sj[k].zq, cj = sj[k].c;
+        const ulonglong2 exy = sexy[k];
+        const f2 dx = add2(xy.x, A.nx), dy = add2(xy.y, A.ny), dz = add2(zq.x, A.nz);
+        const f2 ex = add2(exy.x, nex), ey = add2(exy.y, ney), ez = add2(sez[k], nez);
+        f2 r2 = fma2(dz, dz, fma2(dx, dx, mul2(dy, dy)));
+        f2 D = fma2(ez, fma2(two, dz, ez), fma2(ex, fma2(two, dx, ex), mul2(ey, fma2(two, dy, ey))));
+        float a, b, u, v;
+        upk(r2, a, b);
+        if (DM != 0) {  // j == i: r = 1 and no displacement, every difference vanishes
+            a = k == dk[0] ? 1.f : a;
+            b = k == dk[1] ? 1.f : b;
+            r2 = pk(a, b);
+        }
+        if (DM == 2) {  // each pair once: j < i contributes nothing
+            upk(D, u, v);
+            u = k <= dk[0] ? 0.f : u;
+            v = k <= dk[1] ? 0.f : v;
+            D = pk(u, v);
+        }
+        upk(add2(r2, D), u, v);
+        const f2 ri = pk(rsqrt_approx(a), rsqrt_approx(b)), rp = pk(rsqrt_approx(u), rsqrt_approx(v));
+        upk(add2(ri, rp), a, b);
+        const f2 inv = pk(rcp_approx(a), rcp_approx(b));
+        const f2 ri2 = mul2(ri, ri), rp2 = mul2(rp, rp);
+        const f2 X = mul2(mul2(D, ri2), rp2);
+        const f2 ri4 = mul2(ri2, ri2), rp4 = mul2(rp2, rp2);
+        const f2 d6 = mul2(X, add2(fma2(rp2, ri2, rp4), ri4));
+        const f2 d12 = mul2(d6, fma2(ri4, ri2, mul2(rp4, rp2)));
+        fa = fma2(zq.y, mul2(X, inv), fa);
+        f6 = fma2(cj.x, d6, f6);
+        f12 = fma2(cj.y, d12, f12);
+    }
+}
+
 // NT threads per block, IPT i-atoms per thread, NT * IPT == TI (one tile).
 // FP32 shapes: two i-atoms per thread (64-thread blocks: every j load from
 // shared memory serves two pairs) or one (128-thread blocks: twice the warps
 // per work item, which pays when an object has few items); the autotuner
-// picks one per object.  Register caps: FP32 kernels run 768 threads per SM
-// (12 blocks of 64 or 6 of 128, 80 registers; measured on GB300 faster than
-// 1,024 threads at 64 registers and than 4 i-atoms per thread), the FP64
-// kernel 8 blocks of 128 (64 registers); the rarely-run bonded items may
-// spill.  FFMIN_F32_THREADS_PER_SM overrides the FP32 cap (registers per
-// thread follow: 65536 / threads).
+// picks one per object.  Register caps: FP32 kernels run 640 threads per SM
+// (10 blocks of 64 or 5 of 128, 96 registers; 768 at 80 registers: difference
+// trials 2 % slower at 30,000 atoms and 13 % at 3,334, 512: E + grad 8 %
+// slower), the FP64 kernel 8 blocks of 128 (64 registers); the rarely-run
+// bonded items may spill.  FFMIN_F32_THREADS_PER_SM overrides the FP32 cap
+// (registers per thread follow: 65536 / threads).
 #ifndef FFMIN_F32_THREADS_PER_SM
-#define FFMIN_F32_THREADS_PER_SM 768
+#define FFMIN_F32_THREADS_PER_SM 640
 #endif
 // XS: the object carries the exclusion variant (FP32 sweeps scale the listed
 // pairs); a separate instantiation keeps the masked code out of the kernel
@@ -250,9 +401,14 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
     static_assert(NT * IPT == TI, "a block covers one i-tile");
     using V4 = typename VT<T>::V4;
     using V2 = typename VT<T>::V2;
-    __shared__ V4 sp[TJ];
-    __shared__ V2 sq[TJ];
-    __shared__ float4 sd[sizeof(T) == 4 ? TJ : 1];  // displacements (FP32 difference trials)
+    constexpr bool PACKED = sizeof(T) == 4 && IPT == 2;  // unmasked tiles
+    constexpr bool SCALAR = !PACKED || XS;               // masked tiles and the other shapes
+    __shared__ V4 sp[SCALAR ? TJ : 1];
+    __shared__ V2 sq[SCALAR ? TJ : 1];
+    __shared__ float4 sd[SCALAR && EONLY ? TJ : 1];  // displacements (FP32 difference trials)
+    __shared__ J2 sj[PACKED ? TJ : 1];
+    __shared__ ulonglong2 sexy[PACKED && EONLY ? TJ : 1];
+    __shared__ f2 sez[PACKED && EONLY ? TJ : 1];
     __shared__ int s_item;
     const V4 *__restrict__ pos;
     const V2 *__restrict__ par;
@@ -286,8 +442,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
                 // FP32 energy-only evaluations (plain or difference trials)
                 // run on the symmetric list: each pair once, no forces
                 const int b = asys[lo];
-                const int sym = MODE == 0 && EONLY && c.sym64;
-                s_item = (sym ? c.sys_items64 : c.sys_items)[b].x + (q - aoff[lo]);
+                const int sym = MODE == 0 && EONLY && c.sym32;
+                s_item = (sym ? c.sys_items32 : c.sys_items)[b].x + (q - aoff[lo]);
                 s_sym = sym;
             } else {
                 s_item = -1;
@@ -298,7 +454,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
         const bool sym = MODE == 0 && s_sym;
         __syncthreads();
         if (it < 0) break;
-        const Item I = sym ? c.items64[it] : c.items[it];
+        const Item I = sym ? c.items32[it] : c.items[it];
         if (I.tile < 0) {  // bonded terms (FP64), overlapping the pair items of other warps
             bonded_item(c, I.j0, I.nj, MODE);
             continue;
@@ -312,6 +468,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
         V2 ci[IPT];
         int ig[IPT];
         T gx[IPT], gy[IPT], gz[IPT], ec[IPT], lj[IPT];
+        f2 p0 = 0, p1 = 0, p2 = 0, p3 = 0, p4 = 0;  // packed sums
 #pragma unroll
         for (int u = 0; u < IPT; u++) {
             const int li = tid + u * NT;
@@ -331,22 +488,44 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
             for (int u = 0; u < IPT; u++)
                 di[u] = (delta && tid + u * NT < tl.na) ? c.dispf[ig[u]] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        IPair A{};
+        f2 nex = 0, ney = 0, nez = 0;
+        if constexpr (PACKED) {
+            A.nx = pk(-pi[0].x, -pi[1].x); A.ny = pk(-pi[0].y, -pi[1].y); A.nz = pk(-pi[0].z, -pi[1].z);
+            A.q = pk(pi[0].w, pi[1].w);
+            A.nc6 = pk(-ci[0].x, -ci[1].x);
+            A.c12 = pk(ci[0].y, ci[1].y);
+            nex = pk(-di[0].x, -di[1].x); ney = pk(-di[0].y, -di[1].y); nez = pk(-di[0].z, -di[1].z);
+        }
         const int jend = I.j0 + I.nj;
         for (int jt = I.j0; jt < jend; jt += TJ) {
 #pragma unroll
             for (int q = tid; q < TJ; q += NT) {
                 const int jl = jt + q;
-                if constexpr (MODE == 0) {
-                    if (delta) sd[q] = jl < jend ? c.dispf[jl] : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                V4 pj;
+                V2 cj;
                 if (jl < jend) {
-                    sp[q] = pos[jl];
-                    sq[q] = par[jl];
+                    pj = pos[jl];
+                    cj = par[jl];
                 } else {
-                    V4 d; d.x = T(1e6); d.y = T(1e6); d.z = T(1e6); d.w = T(0);
-                    V2 z; z.x = T(0); z.y = T(0);
-                    sp[q] = d;
-                    sq[q] = z;
+                    pj.x = pj.y = pj.z = T(1e6); pj.w = T(0);
+                    cj.x = cj.y = T(0);
+                }
+                if constexpr (SCALAR) { sp[q] = pj; sq[q] = cj; }
+                if constexpr (PACKED) {
+                    sj[q].xy = make_ulonglong2(pk(pj.x, pj.x), pk(pj.y, pj.y));
+                    sj[q].zq = make_ulonglong2(pk(pj.z, pj.z), pk(pj.w, pj.w));
+                    sj[q].c = make_ulonglong2(pk(cj.x, cj.x), pk(cj.y, cj.y));
+                }
+                if constexpr (MODE == 0 && EONLY) {
+                    if (delta) {
+                        const float4 d = jl < jend ? c.dispf[jl] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        if constexpr (SCALAR) sd[q] = d;
+                        if constexpr (PACKED) {
+                            sexy[q] = make_ulonglong2(pk(d.x, d.x), pk(d.y, d.y));
+                            sez[q] = pk(d.z, d.z);
+                        }
+                    }
                 }
             }
             __syncthreads();
@@ -364,7 +543,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
 #pragma unroll
                 for (int u = 0; u < IPT; u++) igm[u] = tid + u * NT < tl.na ? ig[u] : -1;
                 if constexpr (EONLY) {  // energy only: plain or difference trial
-                    if (masked) {
+                    if (XS && masked) {
                         if (delta) {
                             if (diag && sym) sweep_delta<IPT, 2, true>(sp, sq, sd, pi, ci, di, dk, ec, lj, &c, igm, jt);
                             else if (diag) sweep_delta<IPT, 1, true>(sp, sq, sd, pi, ci, di, dk, ec, lj, &c, igm, jt);
@@ -373,6 +552,16 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
                             if (diag && sym) sweep<T, IPT, false, 2, true>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj, &c, igm, jt);
                             else if (diag) sweep<T, IPT, false, 1, true>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj, &c, igm, jt);
                             else sweep<T, IPT, false, 0, true>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj, &c, igm, jt);
+                        }
+                    } else if constexpr (PACKED) {
+                        if (delta) {
+                            if (diag && sym) sweep2_delta<2>(sj, sexy, sez, A, nex, ney, nez, dk, p0, p1, p2);
+                            else if (diag) sweep2_delta<1>(sj, sexy, sez, A, nex, ney, nez, dk, p0, p1, p2);
+                            else sweep2_delta<0>(sj, sexy, sez, A, nex, ney, nez, dk, p0, p1, p2);
+                        } else {
+                            if (diag && sym) sweep2_e<2>(sj, A, dk, p0, p1, p2);
+                            else if (diag) sweep2_e<1>(sj, A, dk, p0, p1, p2);
+                            else sweep2_e<0>(sj, A, dk, p0, p1, p2);
                         }
                     } else if (delta) {  // factored sums in the (idle) gradient registers
                         if (diag && sym) sweep_delta_factored<IPT, 2>(sp, sq, sd, pi, di, dk, gx, gy, gz);
@@ -384,9 +573,18 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
                         else sweep_e_factored<IPT, 0>(sp, sq, pi, dk, gx, gy, gz);
                     }
                 } else {  // E + grad row sweep
-                    if (masked) {
+                    if (XS && masked) {
                         if (diag) sweep<T, IPT, true, 1, true>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj, &c, igm, jt);
                         else sweep<T, IPT, true, 0, true>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj, &c, igm, jt);
+                    } else if constexpr (PACKED) {
+                        // masked tiles add to the scalar sums in between: both
+                        // forms continue the same running sums
+                        p0 = pk(gx[0], gx[1]); p1 = pk(gy[0], gy[1]); p2 = pk(gz[0], gz[1]);
+                        p3 = pk(ec[0], ec[1]); p4 = pk(lj[0], lj[1]);
+                        if (diag) sweep2<1>(sj, A, dk, p0, p1, p2, p3, p4);
+                        else sweep2<0>(sj, A, dk, p0, p1, p2, p3, p4);
+                        upk(p0, gx[0], gx[1]); upk(p1, gy[0], gy[1]); upk(p2, gz[0], gz[1]);
+                        upk(p3, ec[0], ec[1]); upk(p4, lj[0], lj[1]);
                     } else {
                         if (diag) sweep<T, IPT, true, 1>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj);
                         else sweep<T, IPT, true, 0>(sp, sq, pi, ci, dk, gx, gy, gz, ec, lj);
@@ -401,14 +599,14 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
             }
             __syncthreads();
         }
-        // symmetric list (FP32 energy only): the i-side rows of the item's slot
         V4 *dst = out + (int64_t)it * TI;
-        if constexpr (MODE == 0) {
-            if (sym) dst = c.gpf_sym + (int64_t)I.slot * TI;
-        }
         // FP32 energy only: masked tiles summed the pair terms into ec / lj,
         // the others the factored sums into gx, gy, gz
         constexpr bool factored = MODE == 0 && EONLY;
+        if constexpr (factored && PACKED) {
+            const f2 sg = delta ? pk(-1.f, -1.f) : pk(1.f, 1.f);
+            upk(mul2(p0, sg), gx[0], gx[1]); upk(mul2(p1, sg), gy[0], gy[1]); upk(mul2(p2, sg), gz[0], gz[1]);
+        }
 #pragma unroll
         for (int u = 0; u < IPT; u++) {
             V4 o;
@@ -420,7 +618,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
                 o.x = gx[u]; o.y = gy[u]; o.z = gz[u];
                 o.w = ec[u] + lj[u] * T(1.0 / 6.0);
             }
-            dst[tid + u * NT] = o;
+            // symmetric list (FP32 energy only): energies alone
+            if (MODE == 0 && EONLY && sym) c.gpf_sym[(int64_t)I.slot * TI + tid + u * NT] = (float)o.w;
+            else dst[tid + u * NT] = o;
         }
     }
 }
@@ -566,7 +766,7 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
 #pragma unroll
                 for (int v = 1; v < NT_SYM / 32; v++) { o.x += jfx[v][tid]; o.y += jfy[v][tid]; o.z += jfz[v][tid]; }
                 o.w = 0.0;
-                c.gpd[(int64_t)(I.slot + 1 + (jt - I.j0) / TJ) * TI + tid] = o;
+                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + tid] = o;
             }
             __syncthreads();
         }
@@ -643,7 +843,9 @@ __global__ void __launch_bounds__(256) k_activelist(Ctx c) {
                 // object has one)
                 const int mine = S.ev_kind == EV_NONE ? -1
                                  : (S.mode == 1 ? LIST_F64 : (S.ev_kind == EV_E ? LIST_F32_E : LIST_F32_EG));
-                if (mine == L) n = (c.sym64 && L != LIST_F32_EG ? c.sys_items64 : c.sys_items)[b].y;
+                if (mine == L)
+                    n = (L == LIST_F64 ? (c.sym64 ? c.sys_items64 : c.sys_items)
+                                       : (L == LIST_F32_E && c.sym32 ? c.sys_items32 : c.sys_items))[b].y;
             }
             const int f = n > 0 ? 1 : 0;
             int si = n, ss = f;  // inclusive scans within the warp
