@@ -152,6 +152,9 @@ static void bonded_items(const ffmin_system *sys, int b, std::vector<Item> &item
 constexpr int LAYOUT_ROW_BLOCKS[2] = {6, 12};  // row list, by i-atoms per thread
 constexpr int LAYOUT_SYM_BLOCKS = 7;           // energy-only list
 
+// FP64 list: tile pairs are cut into parts below this many items per SM
+constexpr int SPLIT_ITEMS_PER_SM = 8;
+
 // some evaluation of the object runs on the row list
 static bool needs_row_list(const ffmin_system *sys) { return !sys->c.sym64 || sys->prec == FFMIN_MIXED; }
 
@@ -253,11 +256,16 @@ static void build_list32e(ffmin_system *sys, int dens, std::vector<Item> &items,
     build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, false, &Tile::r32, items, sys_items,
                     slots);
 }
+// the FP64 list: chunks of several j-tiles, or, for a batch with fewer tile
+// pairs than wanted items, parts of 64 or 32 j-atoms (a lone tile pair keeps
+// one SM busy for 128 steps while the others idle)
 static void build_list64(ffmin_system *sys, int dens, std::vector<Item> &items, std::vector<int2> &sys_items,
                          int64_t *slots) {
-    const int64_t want = (int64_t)dens * sys->grid_sym;
-    build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, true, &Tile::r64, items, sys_items,
-                    slots);
+    const int64_t want = (int64_t)dens * sys->grid_sym, pairs = tile_pairs(sys);
+    const int chunk = (int)std::max<int64_t>(1, pairs / want);
+    int split = 1;
+    while (chunk == 1 && split < 4 && pairs * split < SPLIT_ITEMS_PER_SM * sys->sms) split *= 2;
+    build_items_sym(sys, chunk, split, true, &Tile::r64, items, sys_items, slots);
 }
 
 // a symmetric list whose partial rows (which grow as the square of the atom
@@ -779,7 +787,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     CKC(dalloc(sys, &c.te, std::max(n_terms, 1)));
     CKC(dalloc(sys, &c.tg, 3 * (2 * bidx.size() + 3 * aidx.size() + 4 * didx.size() + 2 * xidx.size()) + 3));
     CKC(dalloc(sys, &c.red, (size_t)c.n_tiles * NRED));
-    CKC(dalloc(sys, &c.redf, (size_t)c.n_tiles * 4 * 8));
+    CKC(dalloc(sys, &c.redf, (size_t)c.n_tiles * 8));
     CKC(dalloc(sys, &c.counters, CNT_N));
     CKC(dalloc(sys, &c.nactive, 1));
     CKC(dalloc(sys, &c.nmode, 2));

@@ -213,7 +213,7 @@ struct Ctx {
     double *tg;             // [2 nb + 3 na + 4 nd][3] gradient of each term at each position
     // reductions
     double *red;            // [n_tiles][NRED]
-    double *redf;           // finalize: [value][4 n_tiles]
+    double *redf;           // finalize: [value][n_tiles]
     unsigned int *counters; // one per kernel kind, reset by the last block
     int32_t *nactive;       // systems still minimizing
     int32_t *nmode;         // [2] active systems per pair-kernel precision mode

@@ -66,12 +66,14 @@ __global__ void __launch_bounds__(TI) k_prepare(Ctx c) {
 
 // ---------------------------------------------------------------- finalize
 // Bound: latency and the FP64 pipe (16 cycles per warp operation and SM).
-// Four blocks per tile, 32 atoms each: lane = atom, warp = strand, so an
-// atom's partial rows and bonded terms are summed by four threads (rows
-// q mod 4, combined in strand order through shared memory), and a small
-// system's sums spread over four times the SMs.  One thread per atom took
-// 25 us for 500 atoms and 31 us for 3,334 (cold caches).
-constexpr int FIN_SUB = TI / 32;  // blocks per tile
+// One block per tile, four threads per atom: strand s of an atom sums its
+// partial rows s, s + 4, ..., the strands are combined through shared memory
+// as (0 + 1) + (2 + 3).  One thread per atom took 25 us for 500 atoms and 31 us
+// for 3,334 (cold caches).  The sums keep one order in every version of this
+// kernel (strands, then the columns of block_reduce_columns, then the tiles):
+// a MIXED minimization amplifies any other rounding.
+constexpr int FIN_STRANDS = 4;
+constexpr int FIN_NT = TI * FIN_STRANDS;
 
 // exact FP32 -> FP64 on the integer pipe (the conversion instruction runs at
 // the FP64 rate); the FP32 kernels flush denormals, which read as zero
@@ -133,15 +135,15 @@ __device__ __forceinline__ void sym_rows(const Ctx &c, const Tile &t, int tile0,
     });
 }
 
-// sum (or max) of finalize value k over a system's blocks, fixed order, by a
+// sum (or max) of finalize value k over a system's tiles, fixed order, by a
 // whole warp; the result is valid on every lane
-__device__ double fin_sys_sum(const Ctx &c, const SysState &S, int k, int nb, bool mx) {
-    const int lane = threadIdx.x & 31, b1 = FIN_SUB * (S.tile0 + S.ntile);
-    const double *r = c.redf + (int64_t)k * nb;
+__device__ double fin_sys_sum(const Ctx &c, const SysState &S, int k, bool mx) {
+    const int lane = threadIdx.x & 31, t1 = S.tile0 + S.ntile;
+    const double *r = c.redf + (int64_t)k * c.n_tiles;
     double x = 0.0;
 #pragma unroll 4
-    for (int b = FIN_SUB * S.tile0 + lane; b < b1; b += 32) {
-        const double y = __ldcg(&r[b]);
+    for (int t = S.tile0 + lane; t < t1; t += 32) {
+        const double y = __ldcg(&r[t]);
         x = mx ? fmax(x, y) : x + y;
     }
 #pragma unroll
@@ -152,17 +154,18 @@ __device__ double fin_sys_sum(const Ctx &c, const SysState &S, int k, int nb, bo
     return x;
 }
 
-__global__ void __launch_bounds__(TI) k_finalize(Ctx c) {
-    const Tile &t = c.tiles[blockIdx.x / FIN_SUB];
+__global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c) {
+    const Tile &t = c.tiles[blockIdx.x];
     const SysState &S = c.st[t.sys];
     const int kind = S.ev_kind, mode = S.mode;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nb = gridDim.x;
-    __shared__ Row4 part[2][NW][32];  // pair rows, bonded terms
-    __shared__ double val[RF_N][32];
+    const int i = threadIdx.x % TI, w = threadIdx.x / TI;  // atom, strand
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ Row4 part[FIN_STRANDS][TI];
+    __shared__ Row4 bond[TI];
+    __shared__ double val[RF_N][TI + 1];
+    __shared__ double strands[RF_N][RSTRANDS];
     const unsigned maxmask = (1u << RF_GINF) | (1u << RF_BAD);
     if (kind != EV_NONE) {
-        const int i = (blockIdx.x % FIN_SUB) * 32 + lane;
         const bool real = i < t.na, grad = kind == EV_EG;
         const int a = t.a0 + i;
         Row4 r = Row4{0.0, 0.0, 0.0, 0.0}, bo = r;
@@ -171,8 +174,7 @@ __global__ void __launch_bounds__(TI) k_finalize(Ctx c) {
                 // energies on the symmetric list, each pair counted once
                 const int C = t.r32.chunk;
                 strand_sum<false, true>((S.ntile - t.tloc + C - 1) / C, w, r, [&](int q) {
-                    const int64_t slot = (int64_t)t.r32.slot + (int64_t)q;
-                    return Row4{0.0, 0.0, 0.0, widen(c.gpf_sym[slot * TI + i])};
+                    return Row4{0.0, 0.0, 0.0, widen(c.gpf_sym[((int64_t)t.r32.slot + q) * TI + i])};
                 });
             } else if (mode == 0) {
                 strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpf, t.item0 + it, i); });
@@ -186,44 +188,40 @@ __global__ void __launch_bounds__(TI) k_finalize(Ctx c) {
             }
             // bonded terms: evaluated once per term by the pair kernel's
             // bonded items; every atom gathers its terms' energies (as owner)
-            // and position gradients through its incidence list
-            const int k1 = c.inc_off[a + 1];
-            for (int k = c.inc_off[a] + w; k < k1; k += NW) {
-                const int2 in = c.inc[k];
-                const int type = in.x >> 2, pos = in.x & 3;
-                if (pos == 0) bo.w += c.te[bonded_index(c, type, in.y)];
-                if (grad) {
-                    const double *g = c.tg + 3 * bonded_grad_slot(c, type, in.y, pos);
-                    bo.x += g[0]; bo.y += g[1]; bo.z += g[2];
+            // and position gradients through its incidence list, the even
+            // entries in strand 2, the odd ones in strand 3
+            if (w >= 2) {
+                const int k1 = c.inc_off[a + 1];
+#pragma unroll 2
+                for (int k = c.inc_off[a] + w - 2; k < k1; k += 2) {
+                    const int2 in = c.inc[k];
+                    const int type = in.x >> 2, pos = in.x & 3;
+                    if (pos == 0) bo.w += c.te[bonded_index(c, type, in.y)];
+                    if (grad) {
+                        const double *g = c.tg + 3 * bonded_grad_slot(c, type, in.y, pos);
+                        bo.x += g[0]; bo.y += g[1]; bo.z += g[2];
+                    }
                 }
             }
         }
-        part[0][w][lane] = r;
-        part[1][w][lane] = bo;
+        part[w][i] = r;
+        if (w == 3) bond[i] = bo;
         __syncthreads();
-        if (w == 0) {
+        if (w == 2) {  // the whole atom
             double v[RF_N];
 #pragma unroll
             for (int k = 0; k < RF_N; k++) v[k] = 0.0;
             if (real) {
-                const Row4 r1 = part[0][1][lane], r2 = part[0][2][lane], r3 = part[0][3][lane];
-                const Row4 b1 = part[1][1][lane], b2 = part[1][2][lane], b3 = part[1][3][lane];
-                r.w = (r.w + r1.w) + (r2.w + r3.w);
-                bo.w = (bo.w + b1.w) + (b2.w + b3.w);
-                if (grad) {
-                    r.x = (r.x + r1.x) + (r2.x + r3.x);
-                    r.y = (r.y + r1.y) + (r2.y + r3.y);
-                    r.z = (r.z + r1.z) + (r2.z + r3.z);
-                    bo.x = (bo.x + b1.x) + (b2.x + b3.x);
-                    bo.y = (bo.y + b1.y) + (b2.y + b3.y);
-                    bo.z = (bo.z + b1.z) + (b2.z + b3.z);
-                }
-                const double e = r.w + bo.w;
-                v[RF_EPAIR] = r.w;
+                const Row4 r0 = part[0][i], r1 = part[1][i], r3 = part[3][i], b1 = bond[i];
+                const double ep = (r0.w + r1.w) + (r.w + r3.w);
+                const double e = ep + (bo.w + b1.w);
+                v[RF_EPAIR] = ep;
                 v[RF_E] = e;
                 bool bad = !isfinite(e);
                 if (grad) {
-                    const double g0 = r.x + bo.x, g1 = r.y + bo.y, g2 = r.z + bo.z;
+                    const double g0 = ((r0.x + r1.x) + (r.x + r3.x)) + (bo.x + b1.x);
+                    const double g1 = ((r0.y + r1.y) + (r.y + r3.y)) + (bo.y + b1.y);
+                    const double g2 = ((r0.z + r1.z) + (r.z + r3.z)) + (bo.z + b1.z);
                     double *gt = vslot(c, V_GT) + 3 * a;
                     gt[0] = g0; gt[1] = g1; gt[2] = g2;
                     const double *G = vslot(c, V_G) + 3 * a;
@@ -237,35 +235,43 @@ __global__ void __launch_bounds__(TI) k_finalize(Ctx c) {
                 v[RF_BAD] = bad ? 1.0 : 0.0;
             }
 #pragma unroll
-            for (int k = 0; k < RF_N; k++) val[k][lane] = v[k];
+            for (int k = 0; k < RF_N; k++) val[k][i] = v[k];
         }
         __syncthreads();
-        for (int k = w; k < RF_N; k += NW) {  // value k over the block's atoms (butterfly)
+        // the tile's sums, in the order of block_reduce_columns
+        if (threadIdx.x < RF_N * RSTRANDS) {
+            const int k = threadIdx.x / RSTRANDS, s = threadIdx.x % RSTRANDS;
             const bool mx = (maxmask >> k) & 1u;
-            double x = val[k][lane];
+            double x = val[k][s];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double y = __shfl_xor_sync(0xffffffffu, x, o);
-                x = mx ? fmax(x, y) : x + y;
-            }
-            if (lane == 0) c.redf[(int64_t)k * nb + blockIdx.x] = x;
+            for (int u = s + RSTRANDS; u < TI; u += RSTRANDS) x = mx ? fmax(x, val[k][u]) : x + val[k][u];
+            strands[k][s] = x;
+        }
+        __syncthreads();
+        if (threadIdx.x < RF_N) {
+            const int k = threadIdx.x;
+            const bool mx = (maxmask >> k) & 1u;
+            double x = strands[k][0];
+#pragma unroll
+            for (int s = 1; s < RSTRANDS; s++) x = mx ? fmax(x, strands[k][s]) : x + strands[k][s];
+            c.redf[(int64_t)k * c.n_tiles + blockIdx.x] = x;
         }
     }
     if (c.sep_reduce || !last_block(&c.counters[CNT_FIN])) return;
-    // fewer than 8 systems: the last block sums every system's blocks, one
+    // fewer than 8 systems: the last block sums every system's tiles, one
     // (system, value) per warp at a time, then warp 0 runs the control steps
     // in system order on a shared-memory copy of the state
     __shared__ double tot[LB_MAX_SYS][RF_N];
     __shared__ SysState sS;
     const int n = c.n_sys < LB_MAX_SYS ? c.n_sys : LB_MAX_SYS;
-    for (int u = w; u < n * RF_N; u += NW) {
+    for (int u = warp; u < n * RF_N; u += FIN_NT / 32) {
         const SysState &Sb = c.st[u / RF_N];
         if (Sb.ev_kind == EV_NONE) continue;
-        const double x = fin_sys_sum(c, Sb, u % RF_N, nb, (maxmask >> (u % RF_N)) & 1u);
+        const double x = fin_sys_sum(c, Sb, u % RF_N, (maxmask >> (u % RF_N)) & 1u);
         if (lane == 0) tot[u / RF_N][u % RF_N] = x;
     }
     __syncthreads();
-    if (w == 0) {
+    if (warp == 0) {
         for (int b = 0; b < n; b++) {
             if (c.st[b].ev_kind == EV_NONE) continue;
             warp_copy_state(&sS, &c.st[b]);
@@ -510,7 +516,7 @@ __global__ void __launch_bounds__(TI) k_sysreduce(Ctx c) {
     __shared__ SysState sS;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int k = w; k < nv; k += NW) {
-        const double x = STAGE == 3 ? fin_sys_sum(c, S, k, FIN_SUB * c.n_tiles, (maxmask >> k) & 1u)
+        const double x = STAGE == 3 ? fin_sys_sum(c, S, k, (maxmask >> k) & 1u)
                                     : warp_sys_sum(c, S, k, (maxmask >> k) & 1u);
         if (lane == 0) tot[k] = x;
     }
@@ -599,7 +605,7 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s) {
-    k_finalize<<<FIN_SUB * c.n_tiles, TI, 0, s>>>(c);
+    k_finalize<<<c.n_tiles, FIN_NT, 0, s>>>(c);
     return cudaGetLastError();
 }
 cudaError_t launch_update(const Ctx &c, cudaStream_t s) {

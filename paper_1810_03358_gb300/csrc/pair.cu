@@ -29,6 +29,7 @@
 
 #include "bonded.cuh"
 #include "ffmin_internal.cuh"
+#include "pair64.cuh"
 
 namespace ffm {
 
@@ -625,28 +626,44 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
     }
 }
 
-// Symmetric FP64 pair kernel: every unordered pair once.  The FP64 pipe
-// (2 FMA per clock per SM) is the limit of the FP64 terms, so the row sweep's
-// double evaluation of each pair is its largest cost; here an item (i-tile
-// I, chunk of j-tiles at or right of I) evaluates each pair (i, j) once,
-// adds the force to i's registers and its opposite to j's entry of a
-// warp-private shared-memory array (lanes of a warp take distinct j at every
-// step: lane t pairs with j = (t + k) mod TJ at step k; the diagonal tile runs
-// k = 1 .. TJ/2 and, at k = TJ/2, only its first half of the threads, so
-// every pair of the tile appears once).  No atomics: after each j-tile the
-// four warps' arrays are summed in warp order into the tile's j-side
-// partial rows, and the i-side rows are written once per item; the finalize
-// kernel sums an atom's j-side rows (tiles I <= its tile) and i-side rows in
-// a fixed order.  Row energies count each pair once.
+// Symmetric FP64 pair kernel: every unordered pair once.  An item (i-tile I,
+// chunk of j-tiles at or right of I, or a part of one j-tile) evaluates each
+// pair (i, j) once, adds the force to i's registers and its opposite to j's
+// entry of a warp-private shared-memory array (lanes of a warp take distinct
+// j at every step: thread t pairs with j = (t + k) mod W at step k, W the
+// j-atoms of the part).  The diagonal tile runs k = 1 .. TJ/2 and, at
+// k = TJ/2, only its first half of the threads, so every pair of the tile
+// appears once; in parts it takes the pairs with j > i.  No atomics: after
+// each j-tile the four warps' arrays are summed in warp order into the
+// tile's j-side partial row, and the i-side row is written once per item; the
+// finalize kernel sums an atom's rows in a fixed order.  Row energies count
+// each pair once.
+//
+// Bound: the FP64 pipe at 2 operations per SM and clock.  The terms are
+// formed on the integer pipes (pair64.cuh), which leaves 15 FP64
+// instructions of 31 a pair with forces and 6 of 18.5 for an energy.
 constexpr int NT_SYM = 128;
-// resident blocks per SM: 7 caps the kernel at 72 registers (a few spilled
-// stack bytes) and measured 1.5 % faster than 6 (80 registers, no spills)
 #ifndef FFMIN_SYM_MINBLOCKS
-#define FFMIN_SYM_MINBLOCKS 7
+#define FFMIN_SYM_MINBLOCKS 5
 #endif
+
+// the plain FP64 terms of a pair (coordinates or parameters outside the
+// range of the integer forms): e_cul, C6 r^-6, C12 r^-12, r^-2
+__device__ __noinline__ void terms64_plain(double dx, double dy, double dz, double qq, double c6, double c12,
+                                           double (&o)[4]) {
+    const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+    const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
+    o[0] = qq * ri;
+    o[1] = c6 * ri6;
+    o[2] = c12 * ri6 * ri6;
+    o[3] = ri2;
+}
+
 __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx c) {
-    __shared__ double4_32a sp[TJ];
-    __shared__ double2 sq[TJ];
+    // staged j-atoms: x, y | z, then q', c6, c12 as significands with their
+    // exponents and the charge's sign (forces), or as they are (energy only)
+    __shared__ ulonglong2 s_xy[TJ], s_zq[TJ], s_c[TJ];
+    __shared__ int2 s_e[TJ];
     __shared__ double jfx[NT_SYM / 32][TJ], jfy[NT_SYM / 32][TJ], jfz[NT_SYM / 32][TJ];
     __shared__ int s_item;
     const int32_t *A = c.act + 1 * (2 * c.n_sys + 2);
@@ -678,10 +695,12 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             bonded_item(c, I.j0, I.nj, 1);
             continue;
         }
-        const Tile tl = c.tiles[I.tile];
+        const Tile &tl = c.tiles[I.tile];
         const int kind = c.st[tl.sys].ev_kind;
         if (kind == EV_NONE || c.st[tl.sys].mode != 1) continue;
         const bool grad = kind == EV_EG;
+        const bool part = tl.r64.split > 1;
+        const int W = TJ / tl.r64.split;
         double4_32a pi;
         double2 ci;
         if (tid < tl.na) {
@@ -691,82 +710,125 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             pi = make_double4_32a(-1e6, -1e6, -1e6, 0.0);
             ci = make_double2(0.0, 0.0);
         }
+        u64 qm, c6m, c12m;
+        int qe, c6e, c12e;
+        bool in_range = split64(pi.w, qm, qe);
+        in_range = split64(ci.x, c6m, c6e) && in_range;
+        in_range = split64(ci.y, c12m, c12e) && in_range;
+        const int ce = (c6e << 16) | c12e;  // both biased: the sums of two stay below 2^16
+        const uint32_t qs = (uint32_t)(bits64(pi.w) >> 32) & 0x80000000u;
         double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
         double sc1 = 0.0, s6 = 0.0, s12 = 0.0;  // energy-only factored sums
         const int jend = I.j0 + I.nj;
         for (int jt = I.j0; jt < jend; jt += TJ) {
             const int jl = jt + tid;
-            if (jl < jend) {
-                sp[tid] = c.posd[jl];
-                sq[tid] = c.pard[jl];
-            } else {
-                sp[tid] = make_double4_32a(1e6, 1e6, 1e6, 0.0);
-                sq[tid] = make_double2(0.0, 0.0);
+            bool j_range = in_range;
+            if (tid < W) {
+                double4_32a pj = make_double4_32a(1e6, 1e6, 1e6, 0.0);
+                double2 cj = make_double2(0.0, 0.0);
+                if (jl < jend) {
+                    pj = c.posd[jl];
+                    cj = c.pard[jl];
+                }
+                s_xy[tid] = make_ulonglong2(bits64(pj.x), bits64(pj.y));
+                if (grad) {
+                    u64 m1, m6, m12;
+                    int e1, e6, e12;
+                    j_range = split64(pj.w, m1, e1) && j_range;
+                    j_range = split64(cj.x, m6, e6) && j_range;
+                    j_range = split64(cj.y, m12, e12) && j_range;
+                    s_zq[tid] = make_ulonglong2(bits64(pj.z), m1);
+                    s_c[tid] = make_ulonglong2(m6, m12);
+                    s_e[tid] = make_int2((int)((uint32_t)e1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
+                                         (e6 << 16) | e12);
+                } else {
+                    s_zq[tid] = make_ulonglong2(bits64(pj.z), bits64(pj.w));
+                    s_c[tid] = make_ulonglong2(bits64(cj.x), bits64(cj.y));
+                }
             }
             if (grad) {
 #pragma unroll
                 for (int q = lane; q < TJ; q += 32) { jfx[w][q] = 0.0; jfy[w][q] = 0.0; jfz[w][q] = 0.0; }
             }
-            __syncthreads();
-            // the diagonal tile (j-tile == i-tile) pairs t with t + k,
-            // k = 1 .. TJ/2 (at k = TJ/2 only t < TJ/2); other tiles every k
-            const bool diag = I.diag && jt == I.j0;
-            const int k0 = diag ? 1 : 0, k1 = diag ? TJ / 2 : TJ - 1;
+            // the diagonal tile (j-tile == i-tile): whole, thread t pairs with
+            // t + k, k = 1 .. TJ/2 (at k = TJ/2 only t < TJ/2); in parts,
+            // the pairs with j > i
+            const bool diag = I.diag && (part || jt == I.j0);
+            const bool half = diag && !part, mask = diag && part;
+            const int k0 = half ? 1 : 0;
+            const int k1 = half ? (tid < TJ / 2 ? TJ / 2 : TJ / 2 - 1)  // warp-uniform
+                                : (mask && I.joff + W <= (w << 5) + 1 ? -1 : W - 1);
+            const bool plain = __syncthreads_or(!j_range);  // some parameter out of range: FP64 terms
             if (!grad) {
                 // energy only: the i atom's factors leave the sums,
                 // E_i = q'_i sum q'_j / r + (c12_i sum c12_j r^-12 - c6_i sum c6_j r^-6) / 6
                 for (int k = k0; k <= k1; k++) {
-                    if (diag && k == TJ / 2 && tid >= TJ / 2) break;  // warp-uniform
-                    const int j = (tid + k) & (TJ - 1);
-                    const double4_32a pj = sp[j];
-                    const double2 qj = sq[j];
-                    const double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-                    const double r2 = dx * dx + dy * dy + dz * dz;
-                    const double ri = rsqrt(r2);
-                    const double ri2 = ri * ri;
-                    const double ri6 = ri2 * ri2 * ri2;
-                    sc1 = fma(pj.w, ri, sc1);
-                    s6 = fma(qj.x, ri6, s6);
-                    s12 = fma(qj.y, ri6 * ri6, s12);
+                    const int j = (tid + k) & (W - 1);
+                    const ulonglong2 xy = s_xy[j], zq = s_zq[j], cj = s_c[j];
+                    double dx = from_bits64(xy.x) - pi.x, dy = from_bits64(xy.y) - pi.y, dz = from_bits64(zq.x) - pi.z;
+                    const bool on = !mask || I.joff + j > tid;
+                    if (!on) { dx = 1.0; dy = 0.0; dz = 0.0; }
+                    Inv64 v;
+                    const bool ok = inv64(dx, dy, dz, v);
+                    double ri = inv64_r1(v), ri6 = inv64_r6(v), ri12 = inv64_r12(v);
+                    if (__any_sync(0xffffffffu, !ok)) {
+                        double o[4];
+                        terms64_plain(dx, dy, dz, 1.0, 1.0, 1.0, o);
+                        ri = o[0]; ri6 = o[1]; ri12 = o[2];
+                    }
+                    if (!on) ri = ri6 = ri12 = 0.0;
+                    sc1 = fma(from_bits64(zq.y), ri, sc1);
+                    s6 = fma(from_bits64(cj.x), ri6, s6);
+                    s12 = fma(from_bits64(cj.y), ri12, s12);
                 }
                 __syncthreads();
                 continue;
             }
             for (int k = k0; k <= k1; k++) {
-                if (diag && k == TJ / 2 && tid >= TJ / 2) break;  // warp-uniform
-                const int j = (tid + k) & (TJ - 1);
-                const double4_32a pj = sp[j];
-                const double2 qj = sq[j];
-                const double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                const double ri = rsqrt(r2);
-                const double ri2 = ri * ri;
-                const double e = pi.w * pj.w * ri;
-                const double ri6 = ri2 * ri2 * ri2;
-                const double c6 = ci.x * qj.x, c12 = ci.y * qj.y;
-                const double t1 = c12 * ri6 - c6;
-                ec += e;
-                lj += ri6 * t1;
-                if (grad) {
-                    const double t2 = c12 * ri6 + t1;
-                    const double f = (ri6 * t2 + e) * ri2;
-                    gx += f * dx;
-                    gy += f * dy;
-                    gz += f * dz;
-                    jfx[w][j] -= f * dx;
-                    jfy[w][j] -= f * dy;
-                    jfz[w][j] -= f * dz;
+                const int j = (tid + k) & (W - 1);
+                const ulonglong2 xy = s_xy[j], zq = s_zq[j], cj = s_c[j];
+                const int2 ej = s_e[j];
+                double dx = from_bits64(xy.x) - pi.x, dy = from_bits64(xy.y) - pi.y, dz = from_bits64(zq.x) - pi.z;
+                const bool on = !mask || I.joff + j > tid;
+                if (!on) { dx = 1.0; dy = 0.0; dz = 0.0; }
+                Inv64 v;
+                const bool ok = inv64(dx, dy, dz, v);
+                const int es = ce + ej.y;
+                double e = inv64_c1(v, qm, zq.y, qe + (ej.x & 0xffff));
+                e = from_bits64(bits64(e) ^ ((u64)(((uint32_t)ej.x & 0x80000000u) ^ qs) << 32));
+                double p6 = inv64_c6(v, c6m, cj.x, (int)((uint32_t)es >> 16));
+                double p12 = inv64_c12(v, c12m, cj.y, es & 0xffff);
+                double ri2 = inv64_r2(v);
+                if (__any_sync(0xffffffffu, !ok) || plain) {
+                    const int jg = jt + j;
+                    const double q_j = jg < jend ? c.posd[jg].w : 0.0;
+                    const double2 c_j = jg < jend ? c.pard[jg] : make_double2(0.0, 0.0);
+                    double o[4];
+                    terms64_plain(dx, dy, dz, pi.w * q_j, ci.x * c_j.x, ci.y * c_j.y, o);
+                    e = o[0]; p6 = o[1]; p12 = o[2]; ri2 = o[3];
                 }
+                if (!on) e = p6 = p12 = 0.0;
+                const double u = p12 - p6;
+                ec += e;
+                lj += u;
+                const double f = ((u + p12) + e) * ri2;
+                gx = fma(f, dx, gx);
+                gy = fma(f, dy, gy);
+                gz = fma(f, dz, gz);
+                jfx[w][j] = fma(-f, dx, jfx[w][j]);
+                jfy[w][j] = fma(-f, dy, jfy[w][j]);
+                jfz[w][j] = fma(-f, dz, jfz[w][j]);
                 __syncwarp();
             }
             __syncthreads();
-            if (grad) {  // j-side partial rows of this j-tile, warps summed in order
+            // j-side partial row of this j-tile, warps summed in order
+            if (tid < W && jl < jend) {
                 double4_32a o;
                 o.x = jfx[0][tid]; o.y = jfy[0][tid]; o.z = jfz[0][tid];
 #pragma unroll
                 for (int v = 1; v < NT_SYM / 32; v++) { o.x += jfx[v][tid]; o.y += jfy[v][tid]; o.z += jfz[v][tid]; }
                 o.w = 0.0;
-                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + tid] = o;
+                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + I.joff + tid] = o;
             }
             __syncthreads();
         }

@@ -1,0 +1,168 @@
+// FP64 pair terms with most of their arithmetic on the integer pipes.
+//
+// GB300 retires 2 FP64 operations per SM and clock, 16 cycles for a warp's
+// one, while a 64 x 64 -> high 64-bit product takes about 4 cycles.  A pair with
+// forces costs about 31 FP64 instructions (CUDA's rsqrt alone 5.7) when it
+// is written in FP64.  Here r^2, its reciprocal square root, the powers of r
+// and the products with the atoms' parameters are formed on 64-bit
+// significands with separate exponents and rounded once to FP64; FP64
+// instructions remain for the coordinate differences, the sums of the terms
+// and the accumulation (15 a pair with forces, 6 for an energy).  Every
+// significand below is good to 2^-57 or better and is rounded to 53 bits at
+// the end, so a term's error is no larger than that of the FP64 formula,
+// whose own roundings (each 2^-53) add up.
+//
+// r^-1 from the hardware's approximate FP32 reciprocal square root y and one
+// step of the series (1 - h)^(-1/2) = 1 + h/2 + 3 h^2/8 + O(h^3) with
+// h = 1 - r^2 y^2, |h| < 2^-20, so that the next term is below 2^-61.
+//
+// Ranges: |d|max in [2^-40, 2^41) A and parameters that are zero or within
+// 2^-200 .. 2^200; then no intermediate leaves the exponent range of FP64.
+// Anything else (coincident atoms, infinities, NaN) takes the FP64 formula.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDA_ARCH__
+#define FFM_P64 __device__ __forceinline__
+#else
+#define FFM_P64 __host__ __device__ inline
+#endif
+
+namespace ffm {
+
+typedef unsigned long long u64;
+
+// high 64 bits of a * b, at most 2 below; a, b <= 2^63 and not both 2^63
+FFM_P64 u64 mulh(u64 a, u64 b) {
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    const u64 mid = (u64)ah * bl + (u64)al * bh;
+    return (u64)ah * bh + (mid >> 32);
+}
+// high 64 bits of a * a, at most 2 below; a <= 2^63
+FFM_P64 u64 sqh(u64 a) {
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a;
+    return (u64)ah * ah + (((u64)ah * al) >> 31);
+}
+FFM_P64 int clz_hi(u64 v) {  // leading zeros of v >= 2^32
+#ifdef __CUDA_ARCH__
+    return __clz((int)(v >> 32));
+#else
+    return __builtin_clzll(v);
+#endif
+}
+FFM_P64 u64 bits64(double x) {
+#ifdef __CUDA_ARCH__
+    return (u64)__double_as_longlong(x);
+#else
+    u64 u;
+    __builtin_memcpy(&u, &x, 8);
+    return u;
+#endif
+}
+FFM_P64 double from_bits64(u64 u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)u);
+#else
+    double x;
+    __builtin_memcpy(&x, &u, 8);
+    return x;
+#endif
+}
+// y ~ x^-1/2 (relative error below 2^-21), x = xh 2^-30 in [1/4, 3), as an integer times 2^-30
+FFM_P64 uint32_t rsqrt_seed(uint32_t xh) {
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint2float_rn(xh)));
+    return __float2uint_rz(y * 0x1p45f);  // (xh)^-1/2 2^15 = y, times 2^30
+#else
+    const float y = 1.0f / __builtin_sqrtf((float)xh);
+    return (uint32_t)(y * 0x1p45f);
+#endif
+}
+
+// v 2^(b - 1023) rounded to FP64 (v in [2^55, 2^64)); ZERO: below the normal
+// range it is 0 (the exponent of a zero parameter puts it there)
+template <bool ZERO>
+FFM_P64 double pack64(u64 v, int b) {
+    const int n = clz_hi(v), s = 11 - n;
+    const u64 m = (v >> s) + ((uint32_t)((uint32_t)v >> (s - 1)) & 1u);  // 53 bits, or 2^53: carries into the exponent
+    const int ex = b + 63 - n;
+    const u64 r = m + ((u64)(uint32_t)((ex - 1) << 20) << 32);
+    return from_bits64(ZERO && ex < 1 ? 0 : r);
+}
+
+// a parameter's significand (top bit 62; value = m 2^(e - 62)) and biased
+// exponent e + P64_BIAS; zero: an exponent that every product flushes
+constexpr int P64_BIAS = 8192, P64_ZERO = P64_BIAS - 4000;
+FFM_P64 bool split64(double x, u64 &m, int &e) {  // |x|; false: out of the range of these forms
+    const u64 u = bits64(x);
+    const int ex = (int)((u >> 52) & 0x7ff);
+    m = ((u & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10;
+    if ((u << 1) == 0) {
+        e = P64_ZERO;
+        return true;
+    }
+    e = ex - 1023 + P64_BIAS;
+    return ex >= 1023 - 200 && ex <= 1023 + 200;
+}
+
+// r^-1 = m 2^(-63 - E), r^-2 = n2 2^(-62 - n - 2 E), r^-6 = n6 2^(-59 - 3 n - k - 6 E),
+// with m in [2^61, 2^63], n2 and n6 in [2^62, 2^63)
+struct Inv64 {
+    u64 m, n2, n6;
+    int E, n, k;
+};
+
+// from the coordinate differences; false: outside the range
+FFM_P64 bool inv64(double dx, double dy, double dz, Inv64 &o) {
+    const u64 ux = bits64(dx), uy = bits64(dy), uz = bits64(dz);
+    const int ex = (int)((uint32_t)(ux >> 32) >> 20) & 0x7ff, ey = (int)((uint32_t)(uy >> 32) >> 20) & 0x7ff,
+              ez = (int)((uint32_t)(uz >> 32) >> 20) & 0x7ff;
+    const int em = ex > ey ? (ex > ez ? ex : ez) : (ey > ez ? ey : ez);
+    // significands aligned to the largest exponent, top bit 62 (a zero's
+    // implicit bit is shifted out with the rest)
+    const u64 one = 0x10000000000000ULL, frac = one - 1;
+    const int sx = em - ex < 63 ? em - ex : 63, sy = em - ey < 63 ? em - ey : 63, sz = em - ez < 63 ? em - ez : 63;
+    const u64 ax = (((ux & frac) | one) << 10) >> sx, ay = (((uy & frac) | one) << 10) >> sy,
+              az = (((uz & frac) | one) << 10) >> sz;
+    const u64 R = sqh(ax) + sqh(ay) + sqh(az);  // r^2 = R 2^(2 E - 60), R in [2^60, 3 2^62)
+    o.E = em - 1023;
+    const uint32_t y = rsqrt_seed((uint32_t)(R >> 32));
+    // h = 1 - r^2 y^2 in units of 2^-57, then c = h/2 + 3 h^2/8 in units of 2^-58
+    const long long h = (long long)(1ULL << 57) - (long long)mulh(R >> 1, (u64)y * y);
+    const int hs = (int)(h >> 10);
+    const long long c = h + (((long long)hs * hs * 3) >> 39);
+    // m = y (1 + c), 62 fraction bits
+    const int ch = (int)(c >> 16);
+    const uint32_t cl = (uint32_t)c & 0xffffu;
+    o.m = ((u64)y << 32) + (u64)(((long long)((u64)y * cl) >> 26) + (((long long)(int)ch * (long long)y) >> 10));
+    const u64 q2 = sqh(o.m);  // 60 fraction bits, [2^58, 2^62]
+    o.n = clz_hi(q2) - 1;
+    o.n2 = q2 << o.n;
+    const u64 q6 = mulh(sqh(o.n2) << 1, o.n2);  // [2^59, 2^62), 53 + 3 n fraction bits
+    o.k = clz_hi(q6) - 1;
+    o.n6 = q6 << o.k;
+    return em >= 1023 - 40 && em <= 1023 + 40;
+}
+FFM_P64 double inv64_r1(const Inv64 &v) { return pack64<false>(v.m, 1023 - 63 - v.E); }
+FFM_P64 double inv64_r2(const Inv64 &v) { return pack64<false>(v.n2, 1023 - 62 - v.n - 2 * v.E); }
+FFM_P64 double inv64_r6(const Inv64 &v) { return pack64<false>(v.n6, 1023 - 59 - 3 * v.n - v.k - 6 * v.E); }
+FFM_P64 double inv64_r12(const Inv64 &v) {
+    return pack64<false>(sqh(v.n6), 1023 - 54 - 6 * v.n - 2 * v.k - 12 * v.E);
+}
+
+// products with a pair of parameters: significands a, b and the sum s of
+// their biased exponents
+FFM_P64 double inv64_c1(const Inv64 &v, u64 a, u64 b, int s) {
+    return pack64<true>(mulh(mulh(a, b) << 1, v.m), 1023 - 60 - 2 * P64_BIAS + s - v.E);
+}
+FFM_P64 double inv64_c6(const Inv64 &v, u64 a, u64 b, int s) {
+    return pack64<true>(mulh(mulh(a, b) << 1, v.n6), 1023 - 56 - 2 * P64_BIAS + s - 3 * v.n - v.k - 6 * v.E);
+}
+FFM_P64 double inv64_c12(const Inv64 &v, u64 a, u64 b, int s) {
+    return pack64<true>(mulh(mulh(a, b) << 1, sqh(v.n6) << 1),
+                        1023 - 52 - 2 * P64_BIAS + s - 6 * v.n - 2 * v.k - 12 * v.E);
+}
+
+}  // namespace ffm
