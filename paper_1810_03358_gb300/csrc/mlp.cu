@@ -7,8 +7,17 @@
 // Loss per sample: (z - t)^2; minibatch loss = mean.  Gradients:
 //   dz = 2 (z - t) / B,  dw2_k = dz h_k,  db2 = dz,
 //   dh_k = dz w2_k [a_k > 0],  dW1_ki = dh_k f_i,  db1_k = dh_k.
-// Per-block partial gradients are summed in block order by a second kernel,
+// Per-block partial gradients are summed in a fixed order by a second kernel,
 // so a step is deterministic.
+//
+// Bound: latency (a step of 16,384 rows is 44 MFLOP, under a microsecond of
+// FP32).  Forward with one thread per row, backward with one thread per two
+// hidden units, whose 14 gradient sums stay in registers; the start's form
+// kept all 449 sums per thread in local memory and added them over the block
+// one parameter at a time (320 us a step, 27 us for the Adam kernel).  The
+// two kernels of a step are launched programmatically dependent, so that the
+// next one's rows are gathered while this one ends, and the losses stay on
+// the device until the last step.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -19,8 +28,17 @@
 
 namespace ffm {
 
-constexpr int MT = 128;          // threads per training block
-constexpr int MLP_BLOCKS = 256;  // blocks per minibatch gradient
+constexpr int MT = 128;          // threads per training block, one row each
+constexpr int MLP_ROWS = 256;    // partial-gradient rows of the scratch
+constexpr int MLP_BLOCKS = 152;  // blocks per minibatch gradient, at most
+// the scratch rows that no block uses hold the losses of up to this many steps
+constexpr int MLP_LOSSES = (MLP_ROWS - MLP_BLOCKS) * MLP_NW;
+constexpr int AT = 1024, AP = 32;  // Adam kernel: threads, parameters per block
+
+// programmatic dependent launch: let the next kernel of the stream start /
+// wait for the previous one to have finished
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint64_t mix64(uint64_t seed, uint64_t k) {
     uint64_t z = seed + (k + 1) * 0x9E3779B97F4A7C15ULL;
@@ -35,79 +53,175 @@ __device__ __forceinline__ uint64_t mix64(uint64_t seed, uint64_t k) {
 __global__ void __launch_bounds__(MT) k_mlp_grad(const float *feat, const float *target, int64_t n,
                                                  const float *w32, int batch, uint64_t seed, uint64_t base,
                                                  int sample, float *part, float *loss_part) {
-    __shared__ float w[MLP_NW];
-    __shared__ float acc[MLP_NW];
-    __shared__ float lsum[MT];
-    for (int k = threadIdx.x; k < MLP_NW; k += MT) { w[k] = w32[k]; acc[k] = 0.f; }
-    __syncthreads();
-    float g[MLP_NW];  // per-thread gradient accumulator (registers / local)
-    for (int k = 0; k < MLP_NW; k++) g[k] = 0.f;
-    float loss = 0.f;
+    __shared__ float4 sw[MLP_H][2];        // per hidden unit: W1 (5), b1, w2
+    __shared__ float4 sf[MT / 32][32][2];  // per row of the warp: features (5), dz
+    __shared__ float acc[MT / 32][MLP_NW];
+    __shared__ float lsum[MT / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    pdl_trigger();
+    float f[MLP_IN], t = 0.f;
     const float inv_b = 1.0f / (float)batch;
-    for (int s = blockIdx.x * MT + threadIdx.x; s < batch; s += gridDim.x * MT) {
-        int64_t row = sample ? (int64_t)__umul64hi(mix64(seed, base + s), (uint64_t)n) : s;
-        float f[MLP_IN], h[MLP_H];
-        for (int i = 0; i < MLP_IN; i++) f[i] = feat[row * MLP_IN + i];
-        const float z = mlp_forward(w, f, h);
-        const float r = z - target[row];
+    float g[2][MLP_IN + 2] = {};  // of units lane, lane + 32: W1, b1, w2
+    float gb2 = 0.f, loss = 0.f;
+    float wu[2][MLP_IN + 2];
+    float b2 = 0.f;
+    for (int s0 = blockIdx.x * MT; s0 < batch; s0 += gridDim.x * MT) {
+        const int s = s0 + threadIdx.x;
+        const bool on = s < batch;
+#pragma unroll
+        for (int i = 0; i < MLP_IN; i++) f[i] = 0.f;
+        if (on) {
+            const int64_t row = sample ? (int64_t)__umul64hi(mix64(seed, base + s), (uint64_t)n) : s;
+#pragma unroll
+            for (int i = 0; i < MLP_IN; i++) f[i] = feat[row * MLP_IN + i];
+            t = target[row];
+        }
+        if (s0 == (int)blockIdx.x * MT) {  // the weights, once the previous step has written them
+            pdl_wait();
+            for (int k = threadIdx.x; k < MLP_H; k += MT) {
+                const float *w1 = w32 + MLP_W1 + k * MLP_IN;
+                sw[k][0] = make_float4(w1[0], w1[1], w1[2], w1[3]);
+                sw[k][1] = make_float4(w1[4], w32[MLP_B1 + k], w32[MLP_W2 + k], 0.f);
+            }
+            b2 = w32[MLP_B2];
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                const float4 p = sw[lane + 32 * u][0], q = sw[lane + 32 * u][1];
+                wu[u][0] = p.x; wu[u][1] = p.y; wu[u][2] = p.z; wu[u][3] = p.w;
+                wu[u][4] = q.x; wu[u][5] = q.y; wu[u][6] = q.z;
+            }
+        }
+        // forward: one row per thread
+        float z = b2;
+#pragma unroll 8
+        for (int k = 0; k < MLP_H; k++) {
+            const float4 p = sw[k][0], q = sw[k][1];
+            float a = fmaf(p.x, f[0], q.y);
+            a = fmaf(p.y, f[1], a);
+            a = fmaf(p.z, f[2], a);
+            a = fmaf(p.w, f[3], a);
+            a = fmaf(q.x, f[4], a);
+            z = fmaf(q.z, fmaxf(a, 0.f), z);
+        }
+        const float r = on ? z - t : 0.f;
         loss += r * r;
         const float dz = 2.f * r * inv_b;
-        g[MLP_B2] += dz;
-        for (int k = 0; k < MLP_H; k++) {
-            g[MLP_W2 + k] += dz * h[k];
-            const float dh = h[k] > 0.f ? dz * w[MLP_W2 + k] : 0.f;
-            g[MLP_B1 + k] += dh;
-            for (int i = 0; i < MLP_IN; i++) g[MLP_W1 + k * MLP_IN + i] += dh * f[i];
+        gb2 += dz;
+        sf[w][lane][0] = make_float4(f[0], f[1], f[2], f[3]);
+        sf[w][lane][1] = make_float4(f[4], dz, 0.f, 0.f);
+        __syncwarp();
+        // backward: two hidden units per thread, the warp's rows in order
+#pragma unroll 4
+        for (int m = 0; m < 32; m++) {
+            const float4 p = sf[w][m][0], q = sf[w][m][1];
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                float a = fmaf(wu[u][0], p.x, wu[u][5]);
+                a = fmaf(wu[u][1], p.y, a);
+                a = fmaf(wu[u][2], p.z, a);
+                a = fmaf(wu[u][3], p.w, a);
+                a = fmaf(wu[u][4], q.x, a);
+                const float h = fmaxf(a, 0.f);
+                const float dh = h > 0.f ? q.y * wu[u][6] : 0.f;
+                g[u][0] = fmaf(dh, p.x, g[u][0]);
+                g[u][1] = fmaf(dh, p.y, g[u][1]);
+                g[u][2] = fmaf(dh, p.z, g[u][2]);
+                g[u][3] = fmaf(dh, p.w, g[u][3]);
+                g[u][4] = fmaf(dh, q.x, g[u][4]);
+                g[u][5] += dh;
+                g[u][6] = fmaf(q.y, h, g[u][6]);
+            }
         }
+        __syncwarp();
     }
-    // block sum in thread order, one parameter at a time
-    for (int k = 0; k < MLP_NW; k++) {
-        lsum[threadIdx.x] = g[k];
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float t = 0.f;
-            for (int j = 0; j < MT; j++) t += lsum[j];
-            acc[k] = t;
-        }
-        __syncthreads();
+    // the warps' sums in warp order
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        const int k = lane + 32 * u;
+#pragma unroll
+        for (int i = 0; i < MLP_IN; i++) acc[w][MLP_W1 + k * MLP_IN + i] = g[u][i];
+        acc[w][MLP_B1 + k] = g[u][5];
+        acc[w][MLP_W2 + k] = g[u][6];
     }
-    lsum[threadIdx.x] = loss;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        gb2 += __shfl_xor_sync(0xffffffffu, gb2, o);
+        loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    }
+    if (lane == 0) {
+        acc[w][MLP_B2] = gb2;
+        lsum[w] = loss;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int j = 0; j < MT; j++) t += lsum[j];
-        loss_part[blockIdx.x] = t;
+    for (int k = threadIdx.x; k < MLP_NW; k += MT) {
+        float v = acc[0][k];
+#pragma unroll
+        for (int q = 1; q < MT / 32; q++) v += acc[q][k];
+        part[(int64_t)blockIdx.x * MLP_NW + k] = v;
     }
-    for (int k = threadIdx.x; k < MLP_NW; k += MT) part[(int64_t)blockIdx.x * MLP_NW + k] = acc[k];
+    if (threadIdx.x == 0) {
+        float v = lsum[0];
+#pragma unroll
+        for (int q = 1; q < MT / 32; q++) v += lsum[q];
+        loss_part[blockIdx.x] = v;
+    }
 }
 
-// sum of the block partials in block order; then one Adam step on the FP32
-// master weights (when lr > 0) and the FP16 copy for inference
-__global__ void k_mlp_adam(const float *part, const float *loss_part, int nblocks, int batch, float *w32,
-                           float *adam, int step, float lr, float *grad_out, float *loss_out,
-                           uint16_t *w16) {
+// Sum of the block partials (thread (q, k) of a block takes the blocks q,
+// q + 32, ... of parameter k, then the 32 sums in order); then one Adam step
+// on the FP32 master weights (when lr > 0) and the FP16 copy for inference
+__global__ void __launch_bounds__(AT) k_mlp_adam(const float *part, const float *loss_part, int nblocks, int batch,
+                                                 float *w32, float *adam, int step, float lr, float *grad_out,
+                                                 float *loss_out, uint16_t *w16) {
+    __shared__ float sums[AT / AP][AP + 1];
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    for (int k = threadIdx.x; k < MLP_NW; k += blockDim.x) {
-        float gk = 0.f;
-        for (int b = 0; b < nblocks; b++) gk += part[(int64_t)b * MLP_NW + k];
-        if (grad_out) grad_out[k] = gk;
-        if (lr > 0.f) {
-            float m = adam[k] = b1 * adam[k] + (1.f - b1) * gk;
-            float v = adam[MLP_NW + k] = b2 * adam[MLP_NW + k] + (1.f - b2) * gk * gk;
-            const float mh = m / (1.f - powf(b1, (float)step));
-            const float vh = v / (1.f - powf(b2, (float)step));
-            w32[k] -= lr * mh / (sqrtf(vh) + eps);
-        }
-        if (w16) {
-            __half hv = __float2half_rn(w32[k]);
-            w16[k] = *reinterpret_cast<uint16_t *>(&hv);
-        }
+    const int p = threadIdx.x & (AP - 1), q = threadIdx.x / AP, k = blockIdx.x * AP + p;
+    pdl_trigger();
+    pdl_wait();
+    // the loss counts as one more parameter, behind the last
+    float v = 0.f;
+    if (k < MLP_NW) {
+        for (int b = q; b < nblocks; b += AT / AP) v += part[(int64_t)b * MLP_NW + k];
+    } else if (k == MLP_NW) {
+        for (int b = q; b < nblocks; b += AT / AP) v += loss_part[b];
     }
-    if (threadIdx.x == 0 && loss_out) {
-        float t = 0.f;
-        for (int b = 0; b < nblocks; b++) t += loss_part[b];
-        *loss_out = t / (float)batch;
+    sums[q][p] = v;
+    __syncthreads();
+    if (q != 0 || k > MLP_NW) return;
+    float gk = 0.f;
+#pragma unroll
+    for (int r = 0; r < AT / AP; r++) gk += sums[r][p];
+    if (k == MLP_NW) {
+        if (loss_out) *loss_out = gk / (float)batch;
+        return;
     }
+    if (grad_out) grad_out[k] = gk;
+    if (lr > 0.f) {
+        float m = adam[k] = b1 * adam[k] + (1.f - b1) * gk;
+        float vv = adam[MLP_NW + k] = b2 * adam[MLP_NW + k] + (1.f - b2) * gk * gk;
+        const float mh = m / (1.f - powf(b1, (float)step));
+        const float vh = vv / (1.f - powf(b2, (float)step));
+        w32[k] -= lr * mh / (sqrtf(vh) + eps);
+    }
+    if (w16) {
+        __half hv = __float2half_rn(w32[k]);
+        w16[k] = *reinterpret_cast<uint16_t *>(&hv);
+    }
+}
+
+template <typename... A, typename... B>
+static cudaError_t launch_dependent(void (*kernel)(A...), int grid, int block, cudaStream_t s, bool dependent, B... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, A(args)...);
 }
 
 }  // namespace ffm
@@ -123,20 +237,32 @@ extern "C" ffmin_status ffmin_mlp_train(const float *feat_dev, const float *targ
     if (steps > 0 && (!adam_dev || !(lr > 0.f))) return FFMIN_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     float *part = work_dev;                                    // [MLP_BLOCKS][MLP_NW]
-    float *loss_part = work_dev + (size_t)MLP_BLOCKS * MLP_NW; // [MLP_BLOCKS]
-    float *loss_dev = loss_part + MLP_BLOCKS;                  // [1]
-    float *grad_dev = loss_dev + 1;                            // [MLP_NW]
+    float *losses = part + (size_t)MLP_BLOCKS * MLP_NW;        // [MLP_LOSSES]
+    float *loss_part = work_dev + (size_t)MLP_ROWS * MLP_NW;   // [MLP_ROWS]
+    float *grad_dev = loss_part + MLP_ROWS + 1;                // [MLP_NW]
     const int nsteps = steps > 0 ? steps : 1;
+    const int sample = steps > 0 ? 1 : 0;
+    const int b = steps > 0 ? batch : (int)std::min<int64_t>(batch, n_samples);
+    const int blocks = (int)std::min<int64_t>(MLP_BLOCKS, ((int64_t)b + MT - 1) / MT);
+    int kept = 0;  // steps whose losses have been copied
     for (int t = 0; t < nsteps; t++) {
-        const int sample = steps > 0 ? 1 : 0;
-        const int b = steps > 0 ? batch : (int)std::min<int64_t>(batch, n_samples);
-        k_mlp_grad<<<MLP_BLOCKS, MT, 0, s>>>(feat_dev, target_dev, n_samples, w32_dev, b, seed,
-                                             (uint64_t)t * (uint64_t)batch, sample, part, loss_part);
-        k_mlp_adam<<<1, 512, 0, s>>>(part, loss_part, MLP_BLOCKS, b, w32_dev, adam_dev, t + 1,
-                                     steps > 0 ? lr : 0.f, grad_dev, loss_dev, w16_dev);
-        if (loss_host) {
-            if (cudaMemcpyAsync(loss_host + t, loss_dev, sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+        // the first kernel waits for whatever the stream held before; the
+        // others depend on the kernel before them alone
+        if (launch_dependent(k_mlp_grad, blocks, MT, s, t > kept, feat_dev, target_dev, n_samples,
+                             (const float *)w32_dev, b, seed, (uint64_t)t * (uint64_t)batch, sample, part,
+                             loss_part) != cudaSuccess)
+            return FFMIN_ERR_CUDA;
+        const bool last = t == nsteps - 1;
+        if (launch_dependent(k_mlp_adam, (MLP_NW + AP) / AP, AT, s, true, (const float *)part,
+                             (const float *)loss_part, blocks, b, w32_dev, adam_dev, t + 1, steps > 0 ? lr : 0.f,
+                             last ? grad_dev : (float *)nullptr, losses + (t - kept),
+                             last ? w16_dev : (uint16_t *)nullptr) != cudaSuccess)
+            return FFMIN_ERR_CUDA;
+        if (last || t - kept + 1 == MLP_LOSSES) {
+            if (loss_host && cudaMemcpyAsync(loss_host + kept, losses, sizeof(float) * (size_t)(t - kept + 1),
+                                             cudaMemcpyDeviceToHost, s) != cudaSuccess)
                 return FFMIN_ERR_CUDA;
+            kept = t + 1;
         }
     }
     if (cudaStreamSynchronize(s) != cudaSuccess) return FFMIN_ERR_CUDA;
@@ -144,5 +270,5 @@ extern "C" ffmin_status ffmin_mlp_train(const float *feat_dev, const float *targ
 }
 
 extern "C" int64_t ffmin_mlp_work_floats(void) {
-    return (int64_t)MLP_BLOCKS * MLP_NW + MLP_BLOCKS + 1 + MLP_NW;
+    return (int64_t)MLP_ROWS * MLP_NW + MLP_ROWS + 1 + MLP_NW;
 }
