@@ -22,6 +22,7 @@ UNITS = {
     "pair.cu": ["-ftz=true"],
     "minimizer.cu": ["-fmad=false"],
     "parab.cu": ["-fmad=false"],
+    "moves.cu": ["-fmad=false"],
     "mlp.cu": [],
     "noalloc.cu": [],
     "peak.cu": [],

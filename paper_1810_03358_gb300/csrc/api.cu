@@ -39,7 +39,7 @@ namespace ffm {
 struct ParabState;
 cudaError_t launch_parab_move(const Ctx &c, ParabState *ps, int grid, cudaStream_t s);
 size_t parab_state_bytes();
-void parab_state_init(void *host_buf, int n, int atom0, int mode, int max_moves, uint64_t seed,
+void parab_state_init(void *host_buf, int n, int atom0, int max_moves, uint64_t seed,
                       double delta, double taylor_r);
 size_t parab_offset_move();
 size_t parab_offset_stop();
@@ -81,6 +81,8 @@ struct ffmin_system {
     int ep_parts = 0;
     double *ep_view = nullptr;
     float4 *ep_viewf = nullptr;
+    double *mv_view = nullptr;   // FP64 moves: private copies that do not fit in shared memory
+    int64_t mv_view_cap = 0;
     int32_t *ep_ints = nullptr;  // list [N], members [N], loff, moff [P + 1], allowed [P]
     // learned preconditioner
     bool have_precond = false;
@@ -1531,24 +1533,46 @@ ffmin_status ffmin_set_precond(ffmin_system *sys, const uint16_t *w, int32_t n_p
 // ---------------------------------------------------------------- parab
 static const int PARAB_MOVES = 64;  // moves per graph replay
 
+// private positions of a run of FP64 moves (kept for later runs)
+static ffmin_status moves_view(ffmin_system *sys, int n, int parts, int cs) {
+    const int64_t need = moves_view_doubles(n, parts, cs);
+    if (need <= sys->mv_view_cap) return FFMIN_OK;
+    if (sys->mv_view) {
+        cudaFree(sys->mv_view);
+        sys->allocs.erase(std::remove(sys->allocs.begin(), sys->allocs.end(), (void *)sys->mv_view),
+                          sys->allocs.end());
+        sys->mv_view = nullptr;
+        sys->mv_view_cap = 0;
+    }
+    CK(cudaMalloc(&sys->mv_view, sizeof(double) * (size_t)need));
+    sys->allocs.push_back(sys->mv_view);
+    sys->mv_view_cap = need;
+    return FFMIN_OK;
+}
+
 static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ffmin_result *res) {
     const Ctx &c = sys->c;
     const int n = sys->hst[0].natoms;
-    const int mode = sys->prec == FFMIN_MIXED ? 0 : 1;
-    if (!sys->parab_state) {
-        CK(cudaMalloc(&sys->parab_state, parab_state_bytes()));
-        sys->allocs.push_back(sys->parab_state);
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        sys->parab_grid = std::max(1, std::min((n + TI - 1) / TI, 2 * sms));
+    const bool fp64 = sys->prec != FFMIN_MIXED;
+    const double taylor_r2 = o->gradfree_taylor_r > 0.0 ? o->gradfree_taylor_r * o->gradfree_taylor_r : 0.0;
+    const int cs = moves_cluster(1, sys->sms);
+    ffm::ParabState *ps = nullptr;
+    ffmin_status st;
+    if (fp64) {
+        if ((st = moves_view(sys, n, 1, cs)) != FFMIN_OK) return st;
+    } else {
+        if (!sys->parab_state) {
+            CK(cudaMalloc(&sys->parab_state, parab_state_bytes()));
+            sys->allocs.push_back(sys->parab_state);
+            sys->parab_grid = std::max(1, std::min((n + TI - 1) / TI, 2 * sys->sms));
+        }
+        std::vector<char> hbuf(parab_state_bytes());
+        parab_state_init(hbuf.data(), n, (int)sys->atom_off[0], o->max_iter, o->seed, o->gradfree_delta,
+                         o->gradfree_taylor_r);
+        CK(cudaMemcpyAsync(sys->parab_state, hbuf.data(), hbuf.size(), cudaMemcpyHostToDevice, sys->stream));
+        ps = (ffm::ParabState *)sys->parab_state;
     }
-    std::vector<char> hbuf(parab_state_bytes());
-    parab_state_init(hbuf.data(), n, (int)sys->atom_off[0], mode, o->max_iter, o->seed, o->gradfree_delta,
-                     o->gradfree_taylor_r);
-    CK(cudaMemcpyAsync(sys->parab_state, hbuf.data(), hbuf.size(), cudaMemcpyHostToDevice, sys->stream));
-    ffm::ParabState *ps = (ffm::ParabState *)sys->parab_state;
-    if (!sys->parab_graph) {
+    if (!fp64 && !sys->parab_graph) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(sys->stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
@@ -1561,7 +1585,7 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
         if (e != cudaSuccess) return cuda_fail(sys, e, "parab instantiate");
     }
     // initial evaluation (also writes the pair-kernel positions of X)
-    ffmin_status st = eval_slot(sys, V_X, EV_EG);
+    st = eval_slot(sys, V_X, EV_EG);
     if (st != FFMIN_OK) return st;
     int32_t neg = 1, moves = 0, status = FFMIN_OK;
     double f = sys->hst[0].res_f, ginf = sys->hst[0].res_ginf;
@@ -1575,18 +1599,33 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
         if (!truncated) {
             const int32_t stop = (int32_t)std::min<int64_t>((int64_t)moves + n, o->max_iter);
             truncated = stop < moves + n;
-            CK(cudaMemcpyAsync((char *)sys->parab_state + parab_offset_stop(), &stop, sizeof(int32_t),
-                               cudaMemcpyHostToDevice, sys->stream));
-            for (int32_t k = moves; k < stop; k += PARAB_MOVES) {
-                CK(cudaGraphLaunch(sys->parab_graph, sys->stream));
-                launches += 2 * PARAB_MOVES;
-                ticks += PARAB_MOVES;
+            if (fp64) {  // the sweep's moves in one launch
+                MovesArgs ma{};
+                ma.view = sys->mv_view;
+                ma.n = n;
+                ma.moves = stop - moves;
+                ma.seed = o->seed;
+                ma.base = (uint64_t)moves;
+                ma.delta = o->gradfree_delta;
+                ma.taylor_r2 = taylor_r2;
+                CK(launch_moves64(c, ma, 1, cs, sys->stream));
+                launches += 1;
+                ticks += stop - moves;
+                moves = stop;
+            } else {
+                CK(cudaMemcpyAsync((char *)sys->parab_state + parab_offset_stop(), &stop, sizeof(int32_t),
+                                   cudaMemcpyHostToDevice, sys->stream));
+                for (int32_t k = moves; k < stop; k += PARAB_MOVES) {
+                    CK(cudaGraphLaunch(sys->parab_graph, sys->stream));
+                    launches += 2 * PARAB_MOVES;
+                    ticks += PARAB_MOVES;
+                }
+                CK(cudaMemcpyAsync(sys->h_nactive, (char *)sys->parab_state + parab_offset_move(), sizeof(int32_t),
+                                   cudaMemcpyDeviceToHost, sys->stream));
+                CK(cudaStreamSynchronize(sys->stream));
+                moves = *sys->h_nactive;
+                if (moves != stop) return fail(sys, FFMIN_ERR_CUDA, "gradient-free moves did not all run");
             }
-            CK(cudaMemcpyAsync(sys->h_nactive, (char *)sys->parab_state + parab_offset_move(), sizeof(int32_t),
-                               cudaMemcpyDeviceToHost, sys->stream));
-            CK(cudaStreamSynchronize(sys->stream));
-            moves = *sys->h_nactive;
-            if (moves != stop) return fail(sys, FFMIN_ERR_CUDA, "gradient-free moves did not all run");
         }
         st = eval_slot(sys, V_X, EV_EG);
         if (st != FFMIN_OK) return st;
@@ -1685,8 +1724,11 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
     Ctx &c = sys->c;
     const int n = sys->hst[0].natoms;
     const int P = std::min(o->gradfree_parts, n);
-    const int mode = sys->prec == FFMIN_MIXED ? 0 : 1;
-    if (sys->ep_parts < P) {  // per-part copies (kept for later runs)
+    const bool fp64 = sys->prec != FFMIN_MIXED;
+    const int cs = moves_cluster(P, sys->sms);
+    ffmin_status st;
+    if (fp64 && (st = moves_view(sys, n, P, cs)) != FFMIN_OK) return st;
+    if (sys->ep_parts < P) {  // per-part copies (FP64: the merged positions), kept for later runs
         for (void *p : {(void *)sys->ep_view, (void *)sys->ep_viewf, (void *)sys->ep_ints}) {
             if (!p) continue;
             cudaFree(p);
@@ -1695,7 +1737,7 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
         sys->ep_view = nullptr;
         sys->ep_viewf = nullptr;
         sys->ep_ints = nullptr;
-        CK(cudaMalloc(&sys->ep_view, sizeof(double) * 3 * (size_t)n * P));
+        CK(cudaMalloc(&sys->ep_view, sizeof(double) * 3 * (size_t)n * (fp64 ? 1 : P)));
         sys->allocs.push_back(sys->ep_view);
         if (sys->prec == FFMIN_MIXED) {
             CK(cudaMalloc(&sys->ep_viewf, sizeof(float4) * (size_t)n * P));
@@ -1707,7 +1749,7 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
     }
     int32_t *d_list = sys->ep_ints, *d_members = d_list + n, *d_loff = d_members + n;
     int32_t *d_moff = d_loff + P + 1, *d_allowed = d_moff + P + 1;
-    ffmin_status st = eval_slot(sys, V_X, EV_EG);
+    st = eval_slot(sys, V_X, EV_EG);
     if (st != FFMIN_OK) return st;
     int32_t neg = 1, moves = 0, status = FFMIN_OK;
     double f = sys->hst[0].res_f, ginf = sys->hst[0].res_ginf;
@@ -1759,10 +1801,19 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
         loff[P] = nl;
         CK(cudaMemcpyAsync(sys->ep_ints, ints.data(), sizeof(int32_t) * ints.size(), cudaMemcpyHostToDevice,
                            sys->stream));
-        EpochArgs ea{sys->ep_view, sys->ep_viewf, d_list, d_loff, d_allowed, d_members, d_moff,
-                     n, mode, o->seed, e, o->gradfree_delta,
-                     o->gradfree_taylor_r > 0.0 ? o->gradfree_taylor_r * o->gradfree_taylor_r : 0.0};
-        CK(launch_epoch(c, ea, P, sys->stream));
+        const double taylor_r2 = o->gradfree_taylor_r > 0.0 ? o->gradfree_taylor_r * o->gradfree_taylor_r : 0.0;
+        if (fp64) {
+            MovesArgs ma{sys->mv_view, sys->ep_view, d_list, d_loff, d_allowed, d_members, d_moff, n, 0, o->seed,
+                         e * (uint64_t)n, o->gradfree_delta, taylor_r2};
+            CK(launch_moves64(c, ma, P, cs, sys->stream));
+            // every atom belongs to one part: the merged positions are whole
+            CK(cudaMemcpyAsync(vslot(c, V_X), sys->ep_view, sizeof(double) * 3 * (size_t)n, cudaMemcpyDeviceToDevice,
+                               sys->stream));
+        } else {
+            EpochArgs ea{sys->ep_view, sys->ep_viewf, d_list, d_loff, d_allowed, d_members, d_moff,
+                         n, o->seed, e, o->gradfree_delta, taylor_r2};
+            CK(launch_epoch(c, ea, P, sys->stream));
+        }
         launches += 1;
         ticks += 1;
         moves += sum;

@@ -277,20 +277,33 @@ cudaError_t launch_mbh_accept(const Ctx &c, const int32_t *flags, const double *
 // 1 FP64 row sweep, 2 FP64 symmetric tiles, 3 FP32 energy only
 int pair_grid_size(int mode, int f32_ipt = 2);
 
-// arguments of one epoch of the parallel gradient-free search (one block
-// per part, each on its own copy of the positions)
+// arguments of one epoch of the parallel gradient-free search with FP32 terms
+// (one block per part, each on its own copy of the positions)
 struct EpochArgs {
     double *view;           // [P][3N] FP64 positions of each part's copy
-    float4 *viewf;          // [P][N] FP32 (x, y, z, q') copies (MIXED)
+    float4 *viewf;          // [P][N] FP32 (x, y, z, q') copies
     const int32_t *list;    // movable atoms of every part, concatenated
     const int32_t *loff;    // [P + 1] offsets into list
     const int32_t *allowed; // [P] moves of each part in this epoch
     const int32_t *members; // atoms of every part, concatenated
     const int32_t *moff;    // [P + 1] offsets into members
-    int n, mode;
+    int n;
     uint64_t seed, epoch;
     double delta;
     double taylor_r2;       // squared far-field radius of the linearised Coulomb rows, 0 = exact
 };
+
+// arguments of a run of gradient-free moves with FP64 terms (moves.cu)
+struct MovesArgs {
+    double *view;           // private positions of every block when they don't fit in shared memory
+    double *merged;         // [3N] out: the parts' atoms at the end of the epoch
+    const int32_t *list, *loff, *allowed, *members, *moff;  // as in EpochArgs; list == nullptr: the sequential search
+    int n, moves;           // moves: of the sequential search
+    uint64_t seed, base;    // atom picker: move m of part q takes output q 2^40 + base + m of the stream
+    double delta, taylor_r2;
+};
+int moves_cluster(int parts, int sms);
+int64_t moves_view_doubles(int n, int parts, int cs);
+cudaError_t launch_moves64(const Ctx &c, const MovesArgs &a, int parts, int cs, cudaStream_t s);
 
 }  // namespace ffm

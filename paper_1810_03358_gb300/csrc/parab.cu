@@ -15,10 +15,11 @@
 // SplitMix64 stream (Steele, Lea and Flood 2014) with the user's seed, scaled
 // to [0, N) by a 64x64 -> 128-bit multiply (high word).
 //
-// A move costs two launches over all j (7 rows, then the vertex row); the
-// last block of each launch reduces the block partials in a fixed order and
-// takes the move's decision, so the moves of a sweep replay as a CUDA graph
-// with no host involvement.
+// This file: FP32 terms (MIXED objects); moves.cu has the FP64 ones.  A move
+// costs two launches over all j (7 rows, then the vertex row); the last block
+// of each launch reduces the block partials in a fixed order and takes the
+// move's decision, so the moves of a sweep replay as a CUDA graph with no
+// host involvement.
 #include <cmath>
 #include <cstring>
 
@@ -32,7 +33,7 @@ namespace ffm {
 
 struct ParabState {
     int32_t move, stop_at, max_moves, n;
-    int32_t atom0, mode, atom, best;
+    int32_t atom0, pad, atom, best;
     uint64_t seed;
     double delta;
     double taylor_r2;  // r_far^2 of the linearised far field, 0 = exact rows
@@ -45,49 +46,13 @@ __device__ __forceinline__ int pick_atom(uint64_t seed, uint64_t k, int n) {
 }
 
 // Pair part of the row energy of atom i placed at each of NP positions,
-// this thread's share of the j atoms: j = j0, j0 + stride, ... (FP64
-// accumulation of FP64 terms, or FP32 sums of FP32 terms in the mixed form);
-// pos / posf give the other atoms, xi atom i's current position, tr2 the
-// squared far-field radius (0: exact rows).
+// this thread's share of the j atoms: j = j0, j0 + stride, ... (FP32 sums of
+// FP32 terms); posf gives the other atoms, xi atom i's current position, tr2
+// the squared far-field radius (0: exact rows).
 template <int NP>
-__device__ void row_sums(const Ctx &c, int mode, const double4_32a *pos, const float4 *posf,
-                         const double2 *par, const float2 *parf, int n, int i, const double (*p)[3],
+__device__ void row_sums(const float4 *posf, const float2 *parf, int n, int i, const double (*p)[3],
                          const double *xi, double tr2, int j0, int stride, double *acc) {
-    for (int q = 0; q < NP; q++) acc[q] = 0.0;
-    if (mode == 1) {
-        const double qi = pos[i].w;
-        const double2 ci = par[i];
-        for (int j = j0; j < n; j += stride) {
-            if (j == i) continue;
-            const double4_32a pj = pos[j];
-            const double2 cj = par[j];
-            const double c6 = ci.x * cj.x, c12 = ci.y * cj.y, qq = qi * pj.w;
-            bool far = false;
-            double e0 = 0.0, fac = 0.0;
-            const double d0x = pj.x - xi[0], d0y = pj.y - xi[1], d0z = pj.z - xi[2];
-            if (tr2 > 0.0) {
-                const double r02 = d0x * d0x + d0y * d0y + d0z * d0z;
-                if (r02 >= tr2) {
-                    far = true;
-                    e0 = qq * rsqrt(r02);
-                    fac = e0 / r02;
-                }
-            }
-            for (int q = 0; q < NP; q++) {
-                const double dx = pj.x - p[q][0], dy = pj.y - p[q][1], dz = pj.z - p[q][2];
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                const double ri = rsqrt(r2);
-                const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
-                const double lj = ri6 * (c12 * ri6 - c6) * (1.0 / 6.0);
-                if (far) {
-                    const double dd = d0x * (p[q][0] - xi[0]) + d0y * (p[q][1] - xi[1]) + d0z * (p[q][2] - xi[2]);
-                    acc[q] += e0 + fac * dd + lj;
-                } else {
-                    acc[q] += qq * ri + lj;
-                }
-            }
-        }
-    } else {
+    {
         const float qi = posf[i].w;
         const float2 ci = parf[i];
         float pf[NP][3], accf[NP];
@@ -138,8 +103,8 @@ template <int NP>
 __device__ void row_partial(const Ctx &c, const ParabState *ps, int i, const double (*p)[3], const double *xi,
                             double *acc) {
     const int a0 = ps->atom0;
-    row_sums<NP>(c, ps->mode, c.posd + a0, c.posf + a0, c.pard + a0, c.parf + a0, ps->n, i, p, xi, ps->taylor_r2,
-                 blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, acc);
+    row_sums<NP>(c.posf + a0, c.parf + a0, ps->n, i, p, xi, ps->taylor_r2, blockIdx.x * blockDim.x + threadIdx.x,
+                 gridDim.x * blockDim.x, acc);
 }
 
 // bonded terms containing atom i (global index a) with atom i at p
@@ -219,10 +184,7 @@ __global__ void __launch_bounds__(TI) k_parab_vertex(Ctx c, ParabState *ps) {
         double *X = vslot(c, V_X);
         for (int k = 0; k < 3; k++) X[3 * a + k] = ps->p[best][k];
         const double q = c.qs[a];
-        if (ps->mode == 1)
-            c.posd[a] = make_double4_32a(X[3 * a], X[3 * a + 1], X[3 * a + 2], q);
-        else
-            c.posf[a] = make_float4((float)X[3 * a], (float)X[3 * a + 1], (float)X[3 * a + 2], (float)q);
+        c.posf[a] = make_float4((float)X[3 * a], (float)X[3 * a + 1], (float)X[3 * a + 2], (float)q);
         ps->move = ps->move + 1;
         __threadfence();
         c.counters[CNT_PARAB2] = 0;
@@ -239,13 +201,12 @@ cudaError_t launch_parab_move(const Ctx &c, ParabState *ps, int grid, cudaStream
 
 size_t parab_state_bytes() { return sizeof(ParabState); }
 
-void parab_state_init(void *host_buf, int n, int atom0, int mode, int max_moves, uint64_t seed,
+void parab_state_init(void *host_buf, int n, int atom0, int max_moves, uint64_t seed,
                       double delta, double taylor_r) {
     ParabState ps;
     std::memset(&ps, 0, sizeof(ps));
     ps.n = n;
     ps.atom0 = atom0;
-    ps.mode = mode;
     ps.max_moves = max_moves;
     ps.stop_at = 0;
     ps.seed = seed;
@@ -261,7 +222,7 @@ size_t parab_offset_stop() { return offsetof(ParabState, stop_at); }
 // Parallel epochs of the gradient-free search (Section 3's proposal: cut the
 // molecule into parts, move atoms away from the cuts in every part at once,
 // merge, cut again).  One block per part q works on its own copy of the
-// epoch's starting positions (FP64 [3N] and, for MIXED, FP32 (x, y, z, q')),
+// epoch's starting positions (FP64 [3N] and FP32 (x, y, z, q')),
 // so it sees its own moves and the other parts as they were at the start of
 // the epoch; moves are those of the sequential method (7 rows, per-axis
 // parabola vertices, the best of 8) with row sums reduced by the block in a
@@ -270,49 +231,11 @@ size_t parab_offset_stop() { return offsetof(ParabState, stop_at); }
 constexpr int EPOCH_THREADS = 256;
 
 // row sums of NP positions of atom i over the part's copy: this thread's j
-// (the part's FP64 copy V is read through a double4-free view: positions
-// from V, charges q' from c.qs)
 template <int NP>
 __device__ void epoch_rows(const Ctx &c, const EpochArgs &a, const double *V, const float4 *Vf, int i,
                            const double (*p)[3], double *acc) {
-    for (int q = 0; q < NP; q++) acc[q] = 0.0;
     const double xi[3] = {V[3 * i], V[3 * i + 1], V[3 * i + 2]};  // current position
-    if (a.mode == 1) {
-        const double qi = c.qs[i];
-        const double2 ci = c.pard[i];
-        for (int j = threadIdx.x; j < a.n; j += blockDim.x) {
-            if (j == i) continue;
-            const double xj = V[3 * j], yj = V[3 * j + 1], zj = V[3 * j + 2];
-            const double2 cj = c.pard[j];
-            const double c6 = ci.x * cj.x, c12 = ci.y * cj.y, qq = qi * c.qs[j];
-            bool far = false;
-            double e0 = 0.0, fac = 0.0;
-            const double d0x = xj - xi[0], d0y = yj - xi[1], d0z = zj - xi[2];
-            if (a.taylor_r2 > 0.0) {
-                const double r02 = d0x * d0x + d0y * d0y + d0z * d0z;
-                if (r02 >= a.taylor_r2) {
-                    far = true;
-                    e0 = qq * rsqrt(r02);
-                    fac = e0 / r02;
-                }
-            }
-            for (int q = 0; q < NP; q++) {
-                const double dx = xj - p[q][0], dy = yj - p[q][1], dz = zj - p[q][2];
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                const double ri = rsqrt(r2);
-                const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
-                const double lj = ri6 * (c12 * ri6 - c6) * (1.0 / 6.0);
-                if (far) {
-                    const double dd = d0x * (p[q][0] - xi[0]) + d0y * (p[q][1] - xi[1]) + d0z * (p[q][2] - xi[2]);
-                    acc[q] += e0 + fac * dd + lj;
-                } else {
-                    acc[q] += qq * ri + lj;
-                }
-            }
-        }
-    } else {  // FP32 sums of this thread's j
-        row_sums<NP>(c, 0, nullptr, Vf, nullptr, c.parf, a.n, i, p, xi, a.taylor_r2, threadIdx.x, blockDim.x, acc);
-    }
+    row_sums<NP>(Vf, c.parf, a.n, i, p, xi, a.taylor_r2, threadIdx.x, blockDim.x, acc);
 }
 
 // fixed-order block sum of NP values (warp shuffles, then warps in order)
@@ -337,11 +260,11 @@ __device__ void block_sum_bcast(double (&v)[NP], double *out) {
 __global__ void __launch_bounds__(EPOCH_THREADS) k_epoch(Ctx c, EpochArgs a) {
     const int qp = blockIdx.x;
     double *V = a.view + (int64_t)qp * 3 * a.n;
-    float4 *Vf = a.mode == 0 ? a.viewf + (int64_t)qp * a.n : nullptr;
+    float4 *Vf = a.viewf + (int64_t)qp * a.n;
     const double *X = vslot(c, V_X);
     for (int j = threadIdx.x; j < a.n; j += blockDim.x) {
         for (int k = 0; k < 3; k++) V[3 * j + k] = X[3 * j + k];
-        if (Vf) Vf[j] = make_float4((float)X[3 * j], (float)X[3 * j + 1], (float)X[3 * j + 2], (float)c.qs[j]);
+        Vf[j] = make_float4((float)X[3 * j], (float)X[3 * j + 1], (float)X[3 * j + 2], (float)c.qs[j]);
     }
     __syncthreads();
     const int l0 = a.loff[qp], cnt = a.loff[qp + 1] - l0, moves = a.allowed[qp];
@@ -401,7 +324,7 @@ __global__ void __launch_bounds__(EPOCH_THREADS) k_epoch(Ctx c, EpochArgs a) {
             const double *pb = best < 7 ? p[best] : p7[0];
             if (f7 < fb) pb = p7[0];
             for (int k = 0; k < 3; k++) V[3 * i + k] = pb[k];
-            if (Vf) Vf[i] = make_float4((float)pb[0], (float)pb[1], (float)pb[2], Vf[i].w);
+            Vf[i] = make_float4((float)pb[0], (float)pb[1], (float)pb[2], Vf[i].w);
         }
         __syncthreads();
     }
