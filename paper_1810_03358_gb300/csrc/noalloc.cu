@@ -9,29 +9,42 @@
 // file-scope device array `g_noalloc_scratch` below, which every GPU that
 // loads this library holds until the process exits.
 //
-// Computation: the same FP64 row sweep as the main pair kernel, over all
-// i < j pairs of one system, Coulomb + Lennard-Jones, no bonded terms:
-// rows of 128 i-atoms against 8 j-chunks, partial rows to the scratch, then
-// one thread per atom sums its chunks in a fixed order and the last block
-// sums the block energies and flags a non-finite energy or gradient (two
-// coincident atoms), which the call reports after synchronising its stream.
+// Computation: an FP64 row sweep over all pairs of one system, Coulomb +
+// Lennard-Jones, no bonded terms: every pair in both of its rows, since the
+// fixed scratch has no room for the opposite forces.  Bound: the FP64 pipe;
+// the terms are formed on the integer pipes (pair64.cuh), which leaves 12 FP64
+// instructions an evaluated pair of about 28.  Blocks of 32 i-atoms against a
+// j-chunk, the chunk's atoms dealt to the four warps, give about 1,000 equal
+// blocks at 4,000 atoms (128 i-atoms per block: 256, 1.7 per SM).  4,000 atoms:
+// 1.10 -> 0.39 ms a call.  Partial rows go to the scratch, then one thread per atom
+// sums its chunks in a fixed order and the last block sums the block
+// energies and flags a non-finite energy or gradient (two coincident atoms),
+// which the call reports after synchronising its stream.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
 #include "ffmin.h"
+#include "pair64.cuh"
 
 namespace {
 
-constexpr int NA_TI = 128;      // i atoms per block (one per thread)
+using namespace ffm;
+
+constexpr int NA_TI = 32;       // i atoms per block (one per lane, the same for every warp)
 constexpr int NA_TJ = 128;      // j atoms staged per shared-memory tile
-constexpr int NA_CHUNKS = 8;    // j chunks per row
+constexpr int NA_NT = 128;      // threads per block
+constexpr int NA_CHUNKS = 16;   // j chunks per row, at most
 constexpr int NA_MAX_ATOMS = 8192;
-constexpr int NA_MAX_BLOCKS = (NA_MAX_ATOMS + NA_TI - 1) / NA_TI;
-// doubles: partial rows [chunk][atom][4], block energies, one 8-byte word
-// holding the last-block ticket and the non-finite flag (two uint32)
-constexpr size_t NA_SCRATCH = (size_t)NA_CHUNKS * NA_MAX_ATOMS * 4 + NA_MAX_BLOCKS + 1;
+constexpr int NA_FT = 64;       // atoms per block of the final sum
+constexpr int NA_MAX_BLOCKS = (NA_MAX_ATOMS + NA_FT - 1) / NA_FT;
+// doubles: the atoms' parameters [3][n], partial rows [chunk][n][4] (as many
+// chunks as fit), block energies, one 8-byte word holding the last-block
+// ticket and the non-finite flag (two uint32)
+constexpr size_t NA_ROWS = (size_t)8 * NA_MAX_ATOMS * 4;
+constexpr size_t NA_SCRATCH = NA_ROWS + NA_MAX_BLOCKS + 1;
 
 __device__ __align__(256) double g_noalloc_scratch[NA_SCRATCH];
 
@@ -44,100 +57,152 @@ std::mutex g_scratch_lock;
 
 struct NaArgs {
     const double *x, *q, *sigma, *eps;
-    int n;
+    int n, chunks;
     double sqrt_c;
     double *g, *e;
-    double *part;      // [NA_CHUNKS][NA_MAX_ATOMS][4]
+    double *par;       // [3][n] q sqrt(C), a sigma^3, a sigma^6 (a = sqrt(24 eps))
+    double *part;      // [chunks][n][4]
     double *eblock;    // [NA_MAX_BLOCKS]
     unsigned int *ticket;  // [0] last-block ticket, [1] non-finite flag
 };
 
-__device__ __forceinline__ void na_atom(const NaArgs &a, int j, double4_32a &p, double2 &c) {
+// per-atom parameters once per call; the ticket and the flag start at zero
+// (the array keeps the last call's contents)
+__global__ void __launch_bounds__(NA_NT) k_na_prepare(NaArgs a) {
+    const int i = blockIdx.x * NA_NT + threadIdx.x;
+    if (i == 0) a.ticket[0] = a.ticket[1] = 0u;
+    if (i >= a.n) return;
+    const double s3 = a.sigma[i] * a.sigma[i] * a.sigma[i];
+    const double w = sqrt(24.0 * a.eps[i]);
+    a.par[i] = a.q[i] * a.sqrt_c;
+    a.par[a.n + i] = w * s3;
+    a.par[2 * a.n + i] = w * s3 * s3;
+}
+
+__device__ __forceinline__ void na_atom(const NaArgs &a, int j, double far, double (&x)[3], double (&p)[3]) {
     if (j < a.n) {
-        const double s3 = a.sigma[j] * a.sigma[j] * a.sigma[j];
-        const double w = sqrt(24.0 * a.eps[j]);
-        p = make_double4_32a(a.x[3 * j], a.x[3 * j + 1], a.x[3 * j + 2], a.q[j] * a.sqrt_c);
-        c = make_double2(w * s3, w * s3 * s3);
+        for (int k = 0; k < 3; k++) {
+            x[k] = a.x[3 * j + k];
+            p[k] = a.par[k * a.n + j];
+        }
     } else {  // padding atom: far away, no charge, no Lennard-Jones
-        p = make_double4_32a(1e6, 1e6, 1e6, 0.0);
-        c = make_double2(0.0, 0.0);
+        x[0] = x[1] = x[2] = far;
+        p[0] = p[1] = p[2] = 0.0;
     }
 }
 
-__global__ void __launch_bounds__(NA_TI) k_na_rows(NaArgs a) {
-    __shared__ double4_32a sp[NA_TJ];
-    __shared__ double2 sc[NA_TJ];
-    const int i = blockIdx.x * NA_TI + threadIdx.x;
-    double4_32a pi;
-    double2 ci;
-    na_atom(a, i, pi, ci);
-    if (i >= a.n) pi = make_double4_32a(-1e6, -1e6, -1e6, 0.0);
-    const int chunk = blockIdx.y;
-    const int len = (a.n + NA_CHUNKS - 1) / NA_CHUNKS;
-    const int j0 = chunk * len, j1 = min(a.n, j0 + len);
-    double gx = 0.0, gy = 0.0, gz = 0.0, e = 0.0;
+__global__ void __launch_bounds__(NA_NT, 5) k_na_rows(NaArgs a) {
+    __shared__ ulonglong2 s_xy[NA_TJ], s_zq[NA_TJ], s_c[NA_TJ];
+    __shared__ int2 s_e[NA_TJ];
+    __shared__ double s_p[3][NA_TJ];  // the parameters as they are (the plain formula)
+    __shared__ double4_32a s_sum[NA_NT / 32][32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int i = blockIdx.x * NA_TI + lane;
+    double xi[3], pi[3];
+    na_atom(a, i, -1e6, xi, pi);
+    u64 m1, m6, m12;
+    int e1, e6, e12;
+    bool in_range = split64(pi[0], m1, e1);
+    in_range = split64(pi[1], m6, e6) && in_range && !(pi[1] < 0.0);  // the forms keep no sign of C6, C12
+    in_range = split64(pi[2], m12, e12) && in_range && !(pi[2] < 0.0);
+    const int ce = (e6 << 16) | e12;
+    const uint32_t qs = (uint32_t)(bits64(pi[0]) >> 32) & 0x80000000u;
+    const int len = (a.n + a.chunks - 1) / a.chunks;
+    const int j0 = blockIdx.y * len, j1 = min(a.n, j0 + len);
+    double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
     for (int jt = j0; jt < j1; jt += NA_TJ) {
-        const int jl = jt + threadIdx.x;
-        double4_32a pj;
-        double2 cj;
-        na_atom(a, jl < j1 ? jl : a.n, pj, cj);
-        sp[threadIdx.x] = pj;
-        sc[threadIdx.x] = cj;
-        __syncthreads();
-        for (int k = 0; k < NA_TJ; k++) {
-            if (jt + k == i) continue;
-            const double dx = sp[k].x - pi.x, dy = sp[k].y - pi.y, dz = sp[k].z - pi.z;
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const double ri = rsqrt(r2);
-            const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
-            const double ec = pi.w * sp[k].w * ri;
-            const double c6 = ci.x * sc[k].x, c12 = ci.y * sc[k].y;
-            const double t1 = c12 * ri6 - c6;
-            e += ec + ri6 * t1 * (1.0 / 6.0);
-            const double f = (ri6 * (c12 * ri6 + t1) + ec) * ri2;
-            gx += f * dx;
-            gy += f * dy;
-            gz += f * dz;
+        double xj[3], pj[3];
+        na_atom(a, jt + tid < j1 ? jt + tid : a.n, 1e6, xj, pj);
+        u64 u1, u6, u12;
+        int f1, f6, f12;
+        bool range = split64(pj[0], u1, f1) && in_range;
+        range = split64(pj[1], u6, f6) && range && !(pj[1] < 0.0);
+        range = split64(pj[2], u12, f12) && range && !(pj[2] < 0.0);
+        s_xy[tid] = make_ulonglong2(bits64(xj[0]), bits64(xj[1]));
+        s_zq[tid] = make_ulonglong2(bits64(xj[2]), u1);
+        s_c[tid] = make_ulonglong2(u6, u12);
+        s_e[tid] = make_int2((int)((uint32_t)f1 | ((uint32_t)(bits64(pj[0]) >> 32) & 0x80000000u)), (f6 << 16) | f12);
+        for (int k = 0; k < 3; k++) s_p[k][tid] = pj[k];
+        const bool plain = __syncthreads_or(!range);
+        const int kend = min(w * 32 + 32, j1 - jt);
+        for (int k = w * 32; k < kend; k++) {  // the same j for every lane
+            const ulonglong2 xy = s_xy[k], zq = s_zq[k], cj = s_c[k];
+            const int2 ej = s_e[k];
+            double dx = from_bits64(xy.x) - xi[0], dy = from_bits64(xy.y) - xi[1], dz = from_bits64(zq.x) - xi[2];
+            const bool on = jt + k != i;
+            if (!on) { dx = 1.0; dy = 0.0; dz = 0.0; }
+            Inv64 v;
+            const bool ok = inv64(dx, dy, dz, v);
+            const int es = ce + ej.y;
+            double e = inv64_c1(v, m1, zq.y, e1 + (ej.x & 0xffff));
+            e = from_bits64(bits64(e) ^ ((u64)(((uint32_t)ej.x & 0x80000000u) ^ qs) << 32));
+            double p6 = inv64_c6(v, m6, cj.x, (int)((uint32_t)es >> 16));
+            double p12 = inv64_c12(v, m12, cj.y, es & 0xffff);
+            double ri2 = inv64_r2(v);
+            if (__any_sync(0xffffffffu, !ok) || plain) {
+                const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+                ri2 = ri * ri;
+                const double ri6 = ri2 * ri2 * ri2;
+                e = pi[0] * s_p[0][k] * ri;
+                p6 = pi[1] * s_p[1][k] * ri6;
+                p12 = pi[2] * s_p[2][k] * ri6 * ri6;
+            }
+            if (!on) e = p6 = p12 = 0.0;
+            const double u = p12 - p6;
+            ec += e;
+            lj += u;
+            const double f = ((u + p12) + e) * ri2;
+            gx = fma(f, dx, gx);
+            gy = fma(f, dy, gy);
+            gz = fma(f, dz, gz);
         }
         __syncthreads();
     }
-    if (i < a.n) {
-        double *p = a.part + ((size_t)chunk * NA_MAX_ATOMS + i) * 4;
-        p[0] = gx; p[1] = gy; p[2] = gz; p[3] = e;
-    }
+    s_sum[w][lane] = make_double4_32a(gx, gy, gz, ec + lj * (1.0 / 6.0));
+    __syncthreads();
+    // component w of atom `lane`, the warps in order
+    const double *col = reinterpret_cast<const double *>(&s_sum[0][0]) + 4 * lane + w;
+    double sum = col[0];
+    for (int v = 1; v < NA_NT / 32; v++) sum += col[4 * 32 * v];
+    if (i < a.n) a.part[((size_t)blockIdx.y * a.n + i) * 4 + w] = sum;
 }
 
-__global__ void __launch_bounds__(NA_TI) k_na_final(NaArgs a) {
-    __shared__ double se[NA_TI];
-    const int i = blockIdx.x * NA_TI + threadIdx.x;
-    double e = 0.0;
+// four threads per atom (gradient components and energy)
+__global__ void __launch_bounds__(4 * NA_FT) k_na_final(NaArgs a) {
+    __shared__ double se[NA_FT];
+    const int i = blockIdx.x * NA_FT + threadIdx.x / 4, k = threadIdx.x % 4;
     bool bad = false;
+    double s = 0.0;
     if (i < a.n) {
-        double g0 = 0.0, g1 = 0.0, g2 = 0.0;
-        for (int ch = 0; ch < NA_CHUNKS; ch++) {
-            const double *p = a.part + ((size_t)ch * NA_MAX_ATOMS + i) * 4;
-            g0 += p[0]; g1 += p[1]; g2 += p[2]; e += p[3];
+#pragma unroll 4
+        for (int ch = 0; ch < a.chunks; ch++) s += a.part[((size_t)ch * a.n + i) * 4 + k];
+        if (k < 3) {
+            a.g[3 * i + k] = s;
+            bad = !isfinite(s);
+        } else {
+            s *= 0.5;  // each pair appears in two rows
         }
-        a.g[3 * i] = g0; a.g[3 * i + 1] = g1; a.g[3 * i + 2] = g2;
-        e *= 0.5;  // each pair appears in two rows
-        bad = !isfinite(g0) || !isfinite(g1) || !isfinite(g2);
     }
-    se[threadIdx.x] = e;
+    if (k == 3) se[threadIdx.x / 4] = s;
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(a.ticket + 1, 1u);
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < NA_TI; t++) s += se[t];
-        a.eblock[blockIdx.x] = s;
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    double t = se[lane] + se[lane + 32];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    unsigned last = 0u;
+    if (lane == 0) {
+        a.eblock[blockIdx.x] = t;
         __threadfence();
-        const unsigned t = atomicAdd(a.ticket, 1u);
-        if (t == gridDim.x - 1) {  // last block: total in block order
-            __threadfence();
-            double tot = 0.0;
-            for (int b = 0; b < (int)gridDim.x; b++) tot += __ldcg(&a.eblock[b]);
-            *a.e = tot;
-            if (!isfinite(tot)) atomicOr(a.ticket + 1, 1u);
-            *a.ticket = 0u;
-        }
+        last = atomicAdd(a.ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();  // last block: total over the blocks in a fixed order
+    double tot = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) tot += __ldcg(&a.eblock[b]);
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0) {
+        *a.e = tot;
+        if (!isfinite(tot)) atomicOr(a.ticket + 1, 1u);
     }
 }
 
@@ -170,15 +235,14 @@ extern "C" ffmin_status ffmin_pair_energy_grad_noalloc(const double *x_dev, cons
     a.sqrt_c = std::sqrt(coulomb_c == 0.0 ? 1389.38757 / 4.184 : coulomb_c);
     a.g = g_dev;
     a.e = e_dev;
-    a.part = scr;
-    a.eblock = scr + (size_t)NA_CHUNKS * NA_MAX_ATOMS * 4;
+    a.par = scr;
+    a.part = scr + (size_t)3 * n_atoms;
+    a.chunks = (int)std::min<size_t>(NA_CHUNKS, (NA_ROWS - (size_t)3 * n_atoms) / ((size_t)4 * n_atoms));
+    a.eblock = scr + NA_ROWS;
     a.ticket = (unsigned int *)(a.eblock + NA_MAX_BLOCKS);
-    // the ticket and the flag must start at zero on every call (the array
-    // keeps the last call's contents)
-    if (cudaMemsetAsync(a.ticket, 0, sizeof(double), s) != cudaSuccess) return FFMIN_ERR_CUDA;
-    const int blocks = (n_atoms + NA_TI - 1) / NA_TI;
-    k_na_rows<<<dim3(blocks, NA_CHUNKS), NA_TI, 0, s>>>(a);
-    k_na_final<<<blocks, NA_TI, 0, s>>>(a);
+    k_na_prepare<<<(n_atoms + NA_NT - 1) / NA_NT, NA_NT, 0, s>>>(a);
+    k_na_rows<<<dim3((n_atoms + NA_TI - 1) / NA_TI, a.chunks), NA_NT, 0, s>>>(a);
+    k_na_final<<<(n_atoms + NA_FT - 1) / NA_FT, 4 * NA_FT, 0, s>>>(a);
     if (cudaGetLastError() != cudaSuccess) return FFMIN_ERR_CUDA;
     // the status needs the flag: read it back (pageable host word) and wait
     unsigned int flag = 0u;

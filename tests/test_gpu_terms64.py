@@ -83,3 +83,43 @@ def test_out_of_range_and_special_values(ff, orc, what):
     else:                    # one difference far below the others
         x[1::2, 2] = x[::2, 2] + 1e-310
     check(ff, orc, dataclasses.replace(s, x=np.ascontiguousarray(x), charge=q, epsilon=ep))
+
+
+@pytest.mark.parametrize("what", ["plain", "zeros", "tiny", "huge", "far", "negative_sigma"])
+@pytest.mark.parametrize("n", [31, 32, 33, 150, 2049])
+def test_noalloc_special_values(ff, n, what):
+    """The allocation-free entry point against the same sums in numpy; it
+    takes parameters unchecked, a negative sigma among them."""
+    import torch
+    rng = np.random.default_rng(n)
+    x = synth.make_system(n, 5).x
+    q, sg, ep = rng.uniform(-0.8, 0.8, n), rng.uniform(2.5, 3.8, n), rng.uniform(0.02, 0.2, n)
+    if what == "zeros":
+        q[::3] = 0.0
+        ep[1::4] = 0.0
+    elif what == "tiny":
+        ep[9] = 1e-150
+    elif what == "huge":
+        q[5] = 1e62
+    elif what == "far":
+        x[n // 2:] += 1e13
+    elif what == "negative_sigma":
+        sg[::5] *= -1.0
+
+    def dev(a):
+        return torch.tensor(np.ascontiguousarray(a).reshape(-1), dtype=torch.float64, device="cuda")
+
+    g, e = torch.empty(3 * n, dtype=torch.float64, device="cuda"), torch.empty(1, dtype=torch.float64, device="cuda")
+    ff.ffmin_pair_energy_grad_noalloc(dev(x), dev(q), dev(sg), dev(ep), g, e, coulomb_c=332.0)
+    d = x[None] - x[:, None]
+    r2 = (d * d).sum(-1)
+    np.fill_diagonal(r2, 1.0)
+    w = 1.0 - np.eye(n)
+    ec = 332.0 * np.outer(q, q) / np.sqrt(r2) * w
+    s6, e4 = (np.outer(sg, sg) / r2) ** 3, 4.0 * np.sqrt(np.outer(ep, ep)) * w
+    e_ref = 0.5 * (ec + e4 * (s6 * s6 - s6)).sum()
+    f = (ec + e4 * (12.0 * s6 * s6 - 6.0 * s6)) / r2
+    g_ref = (f[:, :, None] * d).sum(1)
+    total = 0.5 * (np.abs(ec) + e4 * (s6 * s6 + np.abs(s6))).sum()
+    assert abs(e.item() - e_ref) <= 2e-11 * total
+    assert np.abs(g.cpu().numpy().reshape(n, 3) - g_ref).max() <= 1e-9 * np.abs(g_ref).max()
