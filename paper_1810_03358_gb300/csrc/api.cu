@@ -54,7 +54,7 @@ struct ffmin_system {
     int prec = 0;
     cudaStream_t user_stream = nullptr;
     cudaStream_t stream = nullptr;
-    cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+    cudaEvent_t ev_in = nullptr;
     Branches br{};  // side streams of a round's parallel branches
     bool broken = false;
     std::string err;
@@ -67,6 +67,7 @@ struct ffmin_system {
     int graph_ticks = 0;
     cudaGraphExec_t graph = nullptr;
     int32_t *h_nactive = nullptr;  // pinned
+    EvalOut *h_eval = nullptr;     // pinned, [n_sys]: written by the device
     // a minimization as one graph launch: a conditional WHILE node whose body
     // is TICKS_PER_GRAPH rounds and the loop-condition kernel; d_loop / h_loop
     // [2]: rounds run, round bound (device / pinned host)
@@ -391,12 +392,10 @@ ffmin_status ffmin_destroy(ffmin_system *sys) {
     if (sys->stream) cudaStreamSynchronize(sys->stream);
     if (sys->graph) cudaGraphExecDestroy(sys->graph);
     if (sys->loop_exec) cudaGraphExecDestroy(sys->loop_exec);
-    if (sys->h_loop) cudaFreeHost(sys->h_loop);
     if (sys->parab_graph) cudaGraphExecDestroy(sys->parab_graph);
     for (void *p : sys->allocs) cudaFree(p);
-    if (sys->h_nactive) cudaFreeHost(sys->h_nactive);
+    if (sys->h_eval) cudaFreeHost(sys->h_eval);  // with h_loop and h_nactive
     if (sys->ev_in) cudaEventDestroy(sys->ev_in);
-    if (sys->ev_out) cudaEventDestroy(sys->ev_out);
     for (int k = 0; k < 2; k++) {
         if (sys->br.side[k]) cudaStreamDestroy(sys->br.side[k]);
         if (sys->br.join[k]) cudaEventDestroy(sys->br.join[k]);
@@ -457,7 +456,6 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     cudaError_t e = cudaStreamCreateWithFlags(&sys->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) { ffmin_status st = cuda_fail(nullptr, e, "cudaStreamCreate"); delete sys; return st; }
     cudaEventCreateWithFlags(&sys->ev_in, cudaEventDisableTiming);
-    cudaEventCreateWithFlags(&sys->ev_out, cudaEventDisableTiming);
     e = cudaEventCreateWithFlags(&sys->br.fork, cudaEventDisableTiming);
     for (int k = 0; k < 2 && e == cudaSuccess; k++) {
         e = cudaStreamCreateWithFlags(&sys->br.side[k], cudaStreamNonBlocking);
@@ -468,11 +466,12 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
         ffmin_destroy(sys);
         return st;
     }
-    if (cudaMallocHost((void **)&sys->h_nactive, sizeof(int32_t)) != cudaSuccess ||
-        cudaMallocHost((void **)&sys->h_loop, 2 * sizeof(int64_t)) != cudaSuccess) {
+    if (cudaMallocHost((void **)&sys->h_eval, sizeof(EvalOut) * n_sys + 4 * sizeof(int64_t)) != cudaSuccess) {
         ffmin_destroy(sys);
         return fail(nullptr, FFMIN_ERR_OOM, "pinned allocation failed");
     }
+    sys->h_loop = (int64_t *)(sys->h_eval + n_sys);
+    sys->h_nactive = (int32_t *)(sys->h_loop + 2);
     sys->grid32 = pair_grid_size(0);
     sys->grid64 = pair_grid_size(1);
 
@@ -668,6 +667,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     sys->inc_off_h = inc_off;
 
     Ctx &c = sys->c;
+    c.eval_out = sys->h_eval;
     c.n_sys = n_sys;
     c.n_tiles = (int)tiles.size();
     set_item_counts(sys, (int)items.size());
@@ -832,10 +832,10 @@ static ffmin_status enter(ffmin_system *sys) {
     return FFMIN_OK;
 }
 
+// the work is done when the call returns, so the caller's stream needs no
+// event to wait for
 static ffmin_status leave(ffmin_system *sys) {
-    cudaError_t e = cudaEventRecord(sys->ev_out, sys->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(sys->user_stream, sys->ev_out, 0);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(sys->stream);
+    cudaError_t e = cudaStreamSynchronize(sys->stream);
     if (e != cudaSuccess) return cuda_fail(sys, e, "stream sync");
     return FFMIN_OK;
 }
@@ -968,40 +968,54 @@ static ffmin_status ensure_loop(ffmin_system *sys) {
     return FFMIN_OK;
 }
 
-// one evaluation (E or EG) of every system at the vector in `slot`, or at
-// slot + h * dir when dir >= 0; delta = 1 takes a MIXED energy-only trial
-// the way a line search does: pair terms as exact FP32 differences from the
-// pair energy of the last E + grad evaluation (at `slot`), bonded terms in FP64
-static ffmin_status eval_slot(ffmin_system *sys, int slot, int kind, int dir = -1, double h = 0.0,
-                              int delta = 0) {
+// one evaluation (E or EG) of every system at base (device), or at base + h *
+// dir; delta = true takes a MIXED energy-only trial the way a line search
+// does: pair terms as exact FP32 differences from the pair energy of the last
+// E + grad evaluation (at base), bonded terms in FP64.  Results in hst (res_f,
+// res_ginf, status, epair_last); g_out: also the gradient, on the device.
+static ffmin_status eval_at(ffmin_system *sys, const double *base, int kind, const double *dir = nullptr,
+                            double h = 0.0, bool delta = false, double *g_out = nullptr) {
+    const Ctx &c = sys->c;
+    EvalReq r{};
+    r.base = base;
+    r.dir = dir;
+    r.h = h;
+    r.kind = kind;
+    r.mode = sys->prec == FFMIN_MIXED ? 0 : 1;
+    r.delta = delta && r.mode == 0 && kind == EV_E && dir ? 1 : 0;
+    r.list = r.mode == 1 ? LIST_F64 : (kind == EV_E ? LIST_F32_E : LIST_F32_EG);
+    CK(launch_prepare_eval(c, r, sys->stream));
+    CK(launch_pair_list(c, r.list, r.list == LIST_F64 ? sys->grid64 : (r.list == LIST_F32_E ? sys->grid32e : sys->grid32),
+                        sys->stream));
+    CK(launch_finalize(c, sys->stream, g_out));
+    if (c.sep_reduce) CK(launch_sysreduce(c, 3, sys->stream));
+    CK(cudaStreamSynchronize(sys->stream));
     for (int b = 0; b < sys->n_sys; b++) {
         SysState &S = sys->hst[b];
-        S.active = 1;
-        S.phase = PH_EVAL_ONLY;
+        const EvalOut &o = sys->h_eval[b];
+        S.mode = r.mode;
+        S.phase = PH_DONE;
+        S.active = 0;
         S.upd.op = U_NONE;
         S.dir[0].on = S.dir[1].on = 0;
-        S.ev_kind = kind;
-        S.ev_base = slot;
-        S.ev_dir = dir;
-        S.ev_h = h;
-        S.ev_scale = 1.0;
-        S.ne = S.neg = 0;
-        S.mode = sys->prec == FFMIN_MIXED ? 0 : 1;
-        S.ev_delta = (delta && S.mode == 0 && kind == EV_E && dir >= 0) ? 1 : 0;
-        S.epair_base = S.epair_last;
+        S.ev_kind = EV_NONE;
+        S.ev_delta = 0;
+        S.res_f = o.f;
+        S.res_ginf = o.ginf;
+        S.epair_last = o.epair;
+        S.status = o.status;
     }
-    ffmin_status st = upload_states(sys);
-    if (st != FFMIN_OK) return st;
-    if ((st = set_counts(sys)) != FFMIN_OK) return st;
-    CK(launch_eval(sys, sys->stream));
-    return download_states(sys);
+    return FFMIN_OK;
 }
 
-// one evaluation (E or EG) of every system at x (device)
-static ffmin_status eval_all(ffmin_system *sys, const double *x_dev, int kind) {
-    CK(cudaMemcpyAsync(vslot(sys->c, V_XIN), x_dev, sizeof(double) * 3 * sys->n_atoms,
-                       cudaMemcpyDeviceToDevice, sys->stream));
-    return eval_slot(sys, V_XIN, kind);
+// energies of the last evaluation; NONFINITE when a system has none
+static ffmin_status eval_result(const ffmin_system *sys, double *e_host) {
+    ffmin_status res = FFMIN_OK;
+    for (int b = 0; b < sys->n_sys; b++) {
+        e_host[b] = sys->hst[b].res_f;
+        if (sys->hst[b].status == FFMIN_ERR_NONFINITE) res = FFMIN_ERR_NONFINITE;
+    }
+    return res;
 }
 
 extern "C" {
@@ -1011,15 +1025,8 @@ ffmin_status ffmin_energy(ffmin_system *sys, const double *x_dev, double *e_host
     ffmin_status st = enter(sys);
     if (st != FFMIN_OK) return st;
     if (!x_dev || !e_host) return fail(sys, FFMIN_ERR_INVALID_ARG, "NULL argument");
-    st = eval_all(sys, x_dev, EV_E);
-    if (st != FFMIN_OK) return st;
-    ffmin_status res = FFMIN_OK;
-    for (int b = 0; b < sys->n_sys; b++) {
-        e_host[b] = sys->hst[b].res_f;
-        if (sys->hst[b].status == FFMIN_ERR_NONFINITE) res = FFMIN_ERR_NONFINITE;
-    }
-    st = leave(sys);
-    return st != FFMIN_OK ? st : res;
+    st = eval_at(sys, x_dev, EV_E);
+    return st != FFMIN_OK ? st : eval_result(sys, e_host);
 }
 
 ffmin_status ffmin_energy_grad(ffmin_system *sys, const double *x_dev, double *e_host, double *g_dev) {
@@ -1027,17 +1034,8 @@ ffmin_status ffmin_energy_grad(ffmin_system *sys, const double *x_dev, double *e
     ffmin_status st = enter(sys);
     if (st != FFMIN_OK) return st;
     if (!x_dev || !e_host || !g_dev) return fail(sys, FFMIN_ERR_INVALID_ARG, "NULL argument");
-    st = eval_all(sys, x_dev, EV_EG);
-    if (st != FFMIN_OK) return st;
-    CK(cudaMemcpyAsync(g_dev, vslot(sys->c, V_GT), sizeof(double) * 3 * sys->n_atoms, cudaMemcpyDeviceToDevice,
-                       sys->stream));
-    ffmin_status res = FFMIN_OK;
-    for (int b = 0; b < sys->n_sys; b++) {
-        e_host[b] = sys->hst[b].res_f;
-        if (sys->hst[b].status == FFMIN_ERR_NONFINITE) res = FFMIN_ERR_NONFINITE;
-    }
-    st = leave(sys);
-    return st != FFMIN_OK ? st : res;
+    st = eval_at(sys, x_dev, EV_EG, nullptr, 0.0, false, g_dev);
+    return st != FFMIN_OK ? st : eval_result(sys, e_host);
 }
 
 ffmin_status ffmin_energy_grad_host(ffmin_system *sys, const double *x_host, double *e_host, double *g_host) {
@@ -1045,21 +1043,15 @@ ffmin_status ffmin_energy_grad_host(ffmin_system *sys, const double *x_host, dou
     if (st != FFMIN_OK) return st;
     if (!x_host || !e_host) return fail(sys, FFMIN_ERR_INVALID_ARG, "NULL argument");
     const size_t bytes = sizeof(double) * 3 * sys->n_atoms;
-    double *stage = vslot(sys->c, V_XT);  // scratch: overwritten by the evaluation anyway
+    double *stage = vslot(sys->c, V_XIN);
     CK(cudaMemcpyAsync(stage, x_host, bytes, cudaMemcpyHostToDevice, sys->stream));
-    st = eval_all(sys, stage, g_host ? EV_EG : EV_E);
+    st = eval_at(sys, stage, g_host ? EV_EG : EV_E);
     if (st != FFMIN_OK) return st;
     if (g_host) {
         CK(cudaMemcpyAsync(g_host, vslot(sys->c, V_GT), bytes, cudaMemcpyDeviceToHost, sys->stream));
         CK(cudaStreamSynchronize(sys->stream));
     }
-    ffmin_status res = FFMIN_OK;
-    for (int b = 0; b < sys->n_sys; b++) {
-        e_host[b] = sys->hst[b].res_f;
-        if (sys->hst[b].status == FFMIN_ERR_NONFINITE) res = FFMIN_ERR_NONFINITE;
-    }
-    st = leave(sys);
-    return st != FFMIN_OK ? st : res;
+    return eval_result(sys, e_host);
 }
 
 ffmin_status ffmin_energy_delta(ffmin_system *sys, const double *x_dev, const double *r_dev, double h,
@@ -1068,24 +1060,14 @@ ffmin_status ffmin_energy_delta(ffmin_system *sys, const double *x_dev, const do
     ffmin_status st = enter(sys);
     if (st != FFMIN_OK) return st;
     if (!x_dev || !r_dev || !de_host || !std::isfinite(h)) return fail(sys, FFMIN_ERR_INVALID_ARG, "bad argument");
-    const size_t bytes = sizeof(double) * 3 * sys->n_atoms;
-    CK(cudaMemcpyAsync(vslot(sys->c, V_XIN), x_dev, bytes, cudaMemcpyDeviceToDevice, sys->stream));
-    CK(cudaMemcpyAsync(vslot(sys->c, V_R), r_dev, bytes, cudaMemcpyDeviceToDevice, sys->stream));
     // the base of a line search is an E + grad evaluation
-    if ((st = eval_slot(sys, V_XIN, EV_EG)) != FFMIN_OK) return st;
-    ffmin_status res = FFMIN_OK;
     std::vector<double> base(sys->n_sys);
-    for (int b = 0; b < sys->n_sys; b++) {
-        base[b] = sys->hst[b].res_f;
-        if (sys->hst[b].status == FFMIN_ERR_NONFINITE) res = FFMIN_ERR_NONFINITE;
-    }
-    if ((st = eval_slot(sys, V_XIN, EV_E, V_R, h, 1)) != FFMIN_OK) return st;
-    for (int b = 0; b < sys->n_sys; b++) {
-        de_host[b] = sys->hst[b].res_f - base[b];
-        if (sys->hst[b].status == FFMIN_ERR_NONFINITE) res = FFMIN_ERR_NONFINITE;
-    }
-    st = leave(sys);
-    return st != FFMIN_OK ? st : res;
+    if ((st = eval_at(sys, x_dev, EV_EG)) != FFMIN_OK) return st;
+    ffmin_status res = eval_result(sys, base.data());
+    if ((st = eval_at(sys, x_dev, EV_E, r_dev, h, true)) != FFMIN_OK) return st;
+    st = eval_result(sys, de_host);
+    for (int b = 0; b < sys->n_sys; b++) de_host[b] -= base[b];
+    return res != FFMIN_OK ? res : st;
 }
 
 static ffmin_status check_options(ffmin_system *sys, const ffmin_options *o) {
@@ -1351,7 +1333,7 @@ ffmin_status ffmin_time_pair_kernel(ffmin_system *sys, const double *x_dev, int3
         (with_grad == 2 && sys->prec != FFMIN_MIXED))
         return fail(sys, FFMIN_ERR_INVALID_ARG, "bad argument");
     // one full evaluation leaves the positions of x in the pair-kernel inputs
-    st = eval_all(sys, x_dev, with_grad == 1 ? EV_EG : EV_E);
+    st = eval_at(sys, x_dev, with_grad == 1 ? EV_EG : EV_E);
     if (st != FFMIN_OK) return st;
     if (with_grad == 2) CK(cudaMemsetAsync(sys->c.dispf, 0, sizeof(float4) * sys->n_atoms, sys->stream));
     for (int b = 0; b < sys->n_sys; b++) {
@@ -1463,7 +1445,7 @@ ffmin_status ffmin_autotune(ffmin_system *sys, const double *x_dev, int32_t *den
         for (int k = 0; k < AUTOTUNE_N; k++) {
             const int dens = AUTOTUNE_DENSITIES[k];
             if ((st = install_layout(sys, dens, ipt)) != FFMIN_OK) return st;
-            if ((st = eval_all(sys, x_dev, EV_EG)) != FFMIN_OK) return st;
+            if ((st = eval_at(sys, x_dev, EV_EG)) != FFMIN_OK) return st;
             // score: one E + grad launch and three energy-only launches, the
             // mix of an L-BFGS step with LS_PAR (the row list serves the FP32
             // E + grad, the symmetric list the FP64 terms and every
@@ -1585,7 +1567,7 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
         if (e != cudaSuccess) return cuda_fail(sys, e, "parab instantiate");
     }
     // initial evaluation (also writes the pair-kernel positions of X)
-    st = eval_slot(sys, V_X, EV_EG);
+    st = eval_at(sys, vslot(c, V_X), EV_EG);
     if (st != FFMIN_OK) return st;
     int32_t neg = 1, moves = 0, status = FFMIN_OK;
     double f = sys->hst[0].res_f, ginf = sys->hst[0].res_ginf;
@@ -1627,7 +1609,7 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
                 if (moves != stop) return fail(sys, FFMIN_ERR_CUDA, "gradient-free moves did not all run");
             }
         }
-        st = eval_slot(sys, V_X, EV_EG);
+        st = eval_at(sys, vslot(c, V_X), EV_EG);
         if (st != FFMIN_OK) return st;
         neg++;
         launches += 3;
@@ -1749,7 +1731,7 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
     }
     int32_t *d_list = sys->ep_ints, *d_members = d_list + n, *d_loff = d_members + n;
     int32_t *d_moff = d_loff + P + 1, *d_allowed = d_moff + P + 1;
-    st = eval_slot(sys, V_X, EV_EG);
+    st = eval_at(sys, vslot(c, V_X), EV_EG);
     if (st != FFMIN_OK) return st;
     int32_t neg = 1, moves = 0, status = FFMIN_OK;
     double f = sys->hst[0].res_f, ginf = sys->hst[0].res_ginf;
@@ -1818,7 +1800,7 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
         ticks += 1;
         moves += sum;
         if (truncated) { status = FFMIN_ERR_MAX_ITER; report = true; break; }
-        st = eval_slot(sys, V_X, EV_EG);
+        st = eval_at(sys, vslot(c, V_X), EV_EG);
         if (st != FFMIN_OK) return st;
         neg++;
         launches += 3;
@@ -1829,7 +1811,7 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
         if (off == 0) { status = FFMIN_ERR_MAX_ITER; report = true; break; }
     }
     if (report) {
-        st = eval_slot(sys, V_X, EV_EG);
+        st = eval_at(sys, vslot(c, V_X), EV_EG);
         if (st != FFMIN_OK) return st;
         neg++;
         launches += 3;

@@ -420,7 +420,7 @@ __device__ void hb_step(SysState &S, int accept) {
 // reductions of the finalize kernel
 enum { RF_E = 0, RF_GG, RF_GINF, RF_GTG, RF_GTR, RF_BAD, RF_EPAIR, RF_N };
 
-__device__ void on_eval_done(const Ctx &c, SysState &S, const double *v) {
+__device__ void on_eval_done(const Ctx &c, SysState &S, int b, const double *v) {
     const double E = S.ev_delta ? S.epair_base + v[RF_E] : v[RF_E];
     const bool bad = v[RF_BAD] > 0.0 || !isfinite(E);
     const int kind = S.ev_kind;
@@ -436,6 +436,7 @@ __device__ void on_eval_done(const Ctx &c, SysState &S, const double *v) {
         S.status = bad ? FFMIN_ERR_NONFINITE : FFMIN_OK;
         S.phase = PH_DONE;
         deactivate(c, S);
+        c.eval_out[b] = EvalOut{S.res_f, S.res_ginf, S.epair_last, S.status, 0};
         return;
     }
     if (S.phase == PH_FINAL) {  // FGM report evaluation of the best point

@@ -161,6 +161,19 @@ constexpr double MIXED_SWITCH_RATIO = 1.0;
 // each per-tile kernel
 constexpr int LB_MAX_SYS = 8;
 
+// one evaluation of every system outside a minimization: the point is
+// base + h dir (dir may be nullptr), kind EV_E or EV_EG
+struct EvalReq {
+    const double *base, *dir;
+    double h;
+    int32_t kind, mode, delta, list;  // list: the work queue of (kind, mode)
+};
+// its result, written by the device to pinned host memory
+struct EvalOut {
+    double f, ginf, epair;
+    int32_t status, pad;
+};
+
 struct Ctx {
     int32_t n_sys, n_tiles, n_items, n_atoms;
     int64_t vstride;
@@ -221,6 +234,7 @@ struct Ctx {
     const float *feat;      // [n_atoms][3] (q, sigma, eps)
     int32_t *ncount;        // [n_atoms] neighbours within 8 A (pair kernel EG, optional)
     const uint16_t *mlp_w;  // 449 FP16 weights
+    EvalOut *eval_out;      // [n_sys] pinned host memory
 };
 
 inline __host__ __device__ double *vslot(const Ctx &c, int slot) { return c.vec + (int64_t)slot * c.vstride; }
@@ -261,7 +275,12 @@ cudaError_t launch_activelist(const Ctx &c, cudaStream_t s);
 // with br, the FP32 energy-only and FP64 kernels run on br's side streams
 cudaError_t launch_pair_kernels(const Ctx &c, int grid32, int grid32e, int grid64, cudaStream_t s,
                                 const Branches *br);
-cudaError_t launch_finalize(const Ctx &c, cudaStream_t s);
+// g_out: where EV_EG also writes the gradient (optional)
+cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out = nullptr);
+// states, work queue and trial point of one evaluation (in place of
+// launch_activelist and launch_prepare), and the one pair kernel it needs
+cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s);
+cudaError_t launch_pair_list(const Ctx &c, int list, int grid, cudaStream_t s);
 cudaError_t launch_update(const Ctx &c, cudaStream_t s);
 cudaError_t launch_dir(const Ctx &c, int which, cudaStream_t s);
 // per-system reduction + control step after a stage (only when sep_reduce):

@@ -33,35 +33,105 @@ __device__ __forceinline__ double dot3_fma(const double *a, const double *b) {
 }
 
 // ---------------------------------------------------------------- prepare
+// trial point of atom a: base + h (dir sc), and the pair-kernel positions
+__device__ __forceinline__ void prepare_atom(const Ctx &c, int a, const double *base, const double *dir, double h,
+                                             double sc, int mode, bool delta) {
+    double *xt = vslot(c, V_XT) + 3 * a;
+    double b[3], p[3];
+    for (int k = 0; k < 3; k++) b[k] = base[3 * a + k];
+    if (dir) {
+        for (int k = 0; k < 3; k++) p[k] = fma(h, dir[3 * a + k] * sc, b[k]);
+    } else {
+        for (int k = 0; k < 3; k++) p[k] = b[k];
+    }
+    for (int k = 0; k < 3; k++) xt[k] = p[k];
+    const double q = c.qs[a];
+    if (mode == 0 && delta) {
+        // difference trial: base position and the displacement, each rounded
+        // once to FP32 (the displacement keeps its full relative precision)
+        c.posf[a] = make_float4((float)b[0], (float)b[1], (float)b[2], (float)q);
+        c.dispf[a] = make_float4((float)(p[0] - b[0]), (float)(p[1] - b[1]), (float)(p[2] - b[2]), 0.f);
+    } else if (mode == 0) {
+        c.posf[a] = make_float4((float)p[0], (float)p[1], (float)p[2], (float)q);
+    } else {
+        c.posd[a] = make_double4_32a(p[0], p[1], p[2], q);
+    }
+}
+
 __global__ void __launch_bounds__(TI) k_prepare(Ctx c) {
     const Tile t = c.tiles[blockIdx.x];
     const SysState &S = c.st[t.sys];
     if (S.ev_kind == EV_NONE) return;
     const int i = threadIdx.x;
     if (i >= t.na) return;
-    const int a = t.a0 + i;
-    const double *base = vslot(c, S.ev_base) + 3 * a;
-    double *xt = vslot(c, V_XT) + 3 * a;
-    double p[3];
-    if (S.ev_dir >= 0) {
-        const double *d = vslot(c, S.ev_dir) + 3 * a;
-        const double h = S.ev_h, sc = S.ev_scale;
-        for (int k = 0; k < 3; k++) p[k] = fma(h, d[k] * sc, base[k]);
-    } else {
-        for (int k = 0; k < 3; k++) p[k] = base[k];
+    prepare_atom(c, t.a0 + i, vslot(c, S.ev_base), S.ev_dir >= 0 ? vslot(c, S.ev_dir) : nullptr, S.ev_h, S.ev_scale,
+                 S.mode, S.ev_delta);
+}
+
+// One evaluation outside a minimization in three launches (this, the pair
+// kernel of the kind, the finalize; one more for 8 systems and up): the point
+// is read where the caller has it, and block 0 sets every system's request
+// and the one work queue that the evaluation uses.  Uploading the states,
+// copying the point and the active lists were half of a small evaluation.
+__global__ void __launch_bounds__(TI) k_prepare_eval(Ctx c, EvalReq r) {
+    const Tile &t = c.tiles[blockIdx.x];
+    if (threadIdx.x < t.na) prepare_atom(c, t.a0 + threadIdx.x, r.base, r.dir, r.h, 1.0, r.mode, r.delta != 0);
+    if (blockIdx.x != 0) return;
+    __shared__ int wsum[NW];
+    __shared__ int base;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int2 *items = r.list == LIST_F64 ? (c.sym64 ? c.sys_items64 : c.sys_items)
+                                           : (r.list == LIST_F32_E && c.sym32 ? c.sys_items32 : c.sys_items);
+    int32_t *A = c.act + r.list * (2 * c.n_sys + 2);
+    if (threadIdx.x == 0) {
+        base = 0;
+        c.counters[r.list == LIST_F64 ? CNT_PAIR64 : (r.list == LIST_F32_E ? CNT_PAIR32E : CNT_PAIR)] = 0;
+        *c.nactive = c.n_sys;
+        c.nmode[0] = r.mode == 0 ? c.n_sys : 0;
+        c.nmode[1] = r.mode == 0 ? 0 : c.n_sys;
+        A[0] = c.n_sys;
     }
-    for (int k = 0; k < 3; k++) xt[k] = p[k];
-    const double q = c.qs[a];
-    if (S.mode == 0 && S.ev_delta) {
-        // difference trial: base position and the displacement, each rounded
-        // once to FP32 (the displacement keeps its full relative precision)
-        c.posf[a] = make_float4((float)base[0], (float)base[1], (float)base[2], (float)q);
-        c.dispf[a] = make_float4((float)(p[0] - base[0]), (float)(p[1] - base[1]), (float)(p[2] - base[2]), 0.f);
-    } else if (S.mode == 0) {
-        c.posf[a] = make_float4((float)p[0], (float)p[1], (float)p[2], (float)q);
-    } else {
-        c.posd[a] = make_double4_32a(p[0], p[1], p[2], q);
+    __syncthreads();
+    for (int b0 = 0; b0 < c.n_sys; b0 += TI) {
+        const int b = b0 + threadIdx.x;
+        int n = 0;
+        if (b < c.n_sys) {
+            SysState &S = c.st[b];
+            S.active = 1;
+            S.phase = PH_EVAL_ONLY;
+            S.upd.op = U_NONE;
+            S.dir[0].on = S.dir[1].on = 0;
+            S.ev_kind = r.kind;
+            S.ev_delta = r.delta;
+            S.ne = S.neg = 0;
+            S.mode = r.mode;
+            S.epair_base = S.epair_last;
+            n = items[b].y;
+        }
+        int sum = n;  // inclusive scan within the warp
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += u;
+        }
+        if (lane == 31) wsum[w] = sum;
+        __syncthreads();
+        int p = base + sum - n;
+        for (int v = 0; v < w; v++) p += wsum[v];
+        if (b < c.n_sys) {
+            A[2 + b] = p;
+            A[2 + c.n_sys + b] = b;
+        }
+        __syncthreads();
+        if (threadIdx.x == TI - 1) base = p + n;
+        __syncthreads();
     }
+    if (threadIdx.x == 0) A[1] = base;
+}
+
+cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) {
+    k_prepare_eval<<<c.n_tiles, TI, 0, s>>>(c, r);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- finalize
@@ -154,7 +224,7 @@ __device__ double fin_sys_sum(const Ctx &c, const SysState &S, int k, bool mx) {
     return x;
 }
 
-__global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c) {
+__global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
     const Tile &t = c.tiles[blockIdx.x];
     const SysState &S = c.st[t.sys];
     const int kind = S.ev_kind, mode = S.mode;
@@ -224,6 +294,7 @@ __global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c) {
                     const double g2 = ((r0.z + r1.z) + (r.z + r3.z)) + (bo.z + b1.z);
                     double *gt = vslot(c, V_GT) + 3 * a;
                     gt[0] = g0; gt[1] = g1; gt[2] = g2;
+                    if (g_out) { g_out[3 * a] = g0; g_out[3 * a + 1] = g1; g_out[3 * a + 2] = g2; }
                     const double *G = vslot(c, V_G) + 3 * a;
                     const double *R = vslot(c, V_R) + 3 * a;
                     v[RF_GG] = fma(g0, g0, fma(g1, g1, g2 * g2));
@@ -275,7 +346,7 @@ __global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c) {
         for (int b = 0; b < n; b++) {
             if (c.st[b].ev_kind == EV_NONE) continue;
             warp_copy_state(&sS, &c.st[b]);
-            if (lane == 0) on_eval_done(c, sS, tot[b]);
+            if (lane == 0) on_eval_done(c, sS, b, tot[b]);
             __syncwarp();
             warp_copy_state(&c.st[b], &sS);
         }
@@ -528,7 +599,7 @@ __global__ void __launch_bounds__(TI) k_sysreduce(Ctx c) {
         if (STAGE == 0) on_update_done(c, sS, tot);
         else if (STAGE == 1) on_dir_done(c, sS, 0, tot);
         else if (STAGE == 2) on_dir_done(c, sS, 1, tot);
-        else on_eval_done(c, sS, tot);
+        else on_eval_done(c, sS, blockIdx.x, tot);
     }
     __syncwarp();
     warp_copy_state(&S, &sS);
@@ -604,8 +675,8 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     k_prepare<<<c.n_tiles, TI, 0, s>>>(c);
     return cudaGetLastError();
 }
-cudaError_t launch_finalize(const Ctx &c, cudaStream_t s) {
-    k_finalize<<<c.n_tiles, FIN_NT, 0, s>>>(c);
+cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out) {
+    k_finalize<<<c.n_tiles, FIN_NT, 0, s>>>(c, g_out);
     return cudaGetLastError();
 }
 cudaError_t launch_update(const Ctx &c, cudaStream_t s) {

@@ -865,17 +865,29 @@ int pair_grid_size(int mode, int f32_ipt) {
     return sms * per;
 }
 
-// the FP32 E + grad and energy-only kernels of one shape
+// the FP32 E + grad (eonly false) or energy-only kernel in the object's shape
 template <int IPT>
-static void launch_f32(const Ctx &c, int grid32, int grid32e, cudaStream_t s, cudaStream_t se) {
+static void launch_f32_shape(const Ctx &c, bool eonly, int grid, cudaStream_t s) {
     constexpr int NT = TI / IPT;
     if (c.xs_off) {
-        k_pair<float, NT, IPT, true><<<grid32, NT, 0, s>>>(c);
-        k_pair<float, NT, IPT, true, true><<<grid32e, NT, 0, se>>>(c);
+        if (eonly) k_pair<float, NT, IPT, true, true><<<grid, NT, 0, s>>>(c);
+        else k_pair<float, NT, IPT, true><<<grid, NT, 0, s>>>(c);
     } else {
-        k_pair<float, NT, IPT><<<grid32, NT, 0, s>>>(c);
-        k_pair<float, NT, IPT, false, true><<<grid32e, NT, 0, se>>>(c);
+        if (eonly) k_pair<float, NT, IPT, false, true><<<grid, NT, 0, s>>>(c);
+        else k_pair<float, NT, IPT><<<grid, NT, 0, s>>>(c);
     }
+}
+
+cudaError_t launch_pair_list(const Ctx &c, int list, int grid, cudaStream_t s) {
+    if (list == LIST_F64) {
+        if (c.sym64) k_pair64_sym<<<grid, NT_SYM, 0, s>>>(c);
+        else K_F64<<<grid, NT_F64, 0, s>>>(c);
+    } else if (c.f32_ipt == 1) {
+        launch_f32_shape<1>(c, list == LIST_F32_E, grid, s);
+    } else {
+        launch_f32_shape<2>(c, list == LIST_F32_E, grid, s);
+    }
+    return cudaGetLastError();
 }
 
 // Active lists for the two pair kernels: for each precision mode, the
@@ -948,11 +960,7 @@ cudaError_t launch_activelist(const Ctx &c, cudaStream_t s) {
 cudaError_t launch_pair_kernels(const Ctx &c, int grid32, int grid32e, int grid64, cudaStream_t s,
                                 const Branches *br) {
     cudaError_t e;
-    if (c.prec != FFMIN_MIXED) {
-        if (c.sym64) k_pair64_sym<<<grid64, NT_SYM, 0, s>>>(c);
-        else K_F64<<<grid64, NT_F64, 0, s>>>(c);
-        return cudaGetLastError();
-    }
+    if (c.prec != FFMIN_MIXED) return launch_pair_list(c, LIST_F64, grid64, s);
     cudaStream_t se = s, s64 = s;
     if (br) {
         if ((e = cudaEventRecord(br->fork, s)) != cudaSuccess) return e;
@@ -961,11 +969,9 @@ cudaError_t launch_pair_kernels(const Ctx &c, int grid32, int grid32e, int grid6
         se = br->side[0];
         s64 = br->side[1];
     }
-    if (c.f32_ipt == 1) launch_f32<1>(c, grid32, grid32e, s, se);
-    else launch_f32<2>(c, grid32, grid32e, s, se);
-    if (c.sym64) k_pair64_sym<<<grid64, NT_SYM, 0, s64>>>(c);
-    else K_F64<<<grid64, NT_F64, 0, s64>>>(c);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pair_list(c, LIST_F32_EG, grid32, s)) != cudaSuccess) return e;
+    if ((e = launch_pair_list(c, LIST_F32_E, grid32e, se)) != cudaSuccess) return e;
+    if ((e = launch_pair_list(c, LIST_F64, grid64, s64)) != cudaSuccess) return e;
     if (br) {
         for (int k = 0; k < 2; k++) {
             if ((e = cudaEventRecord(br->join[k], br->side[k])) != cudaSuccess) return e;

@@ -215,17 +215,17 @@ def _dev_ptr(t, n_atoms):
     return C.c_void_p(t.data_ptr())
 
 
-def ffmin_energy(handle, x, n_sys=1):
+def ffmin_energy(handle, x, n_sys=1, n_atoms=None):
     e = np.zeros(n_sys)
-    st = lib().ffmin_energy(C.c_void_p(handle), _dev_ptr(x, ffmin_n_atoms(handle)),
-                            e.ctypes.data_as(_dp))
+    n = ffmin_n_atoms(handle) if n_atoms is None else n_atoms
+    st = lib().ffmin_energy(C.c_void_p(handle), _dev_ptr(x, n), e.ctypes.data_as(_dp))
     _check(st, handle)
     return e
 
 
-def ffmin_energy_grad(handle, x, g, n_sys=1):
+def ffmin_energy_grad(handle, x, g, n_sys=1, n_atoms=None):
     e = np.zeros(n_sys)
-    n = ffmin_n_atoms(handle)
+    n = ffmin_n_atoms(handle) if n_atoms is None else n_atoms
     st = lib().ffmin_energy_grad(C.c_void_p(handle), _dev_ptr(x, n), e.ctypes.data_as(_dp),
                                  _dev_ptr(g, n))
     _check(st, handle)
@@ -357,13 +357,13 @@ class System:
             pass
 
     def energy(self, x):
-        return ffmin_energy(self.handle, x, self.n_sys)
+        return ffmin_energy(self.handle, x, self.n_sys, self.n_atoms)
 
     def energy_grad(self, x, g=None):
         import torch
         if g is None:
             g = torch.empty_like(x)
-        e = ffmin_energy_grad(self.handle, x, g, self.n_sys)
+        e = ffmin_energy_grad(self.handle, x, g, self.n_sys, self.n_atoms)
         return e, g
 
     def energy_delta(self, x, r, h):
