@@ -60,6 +60,22 @@ __device__ __forceinline__ float pair_xscale(const Ctx &c, int i, int j) {
     return s;
 }
 
+// the scaled partners of the thread's i-atoms among the 32 atoms from j0 on,
+// one bit each: a pair without a bit has scale 1 and needs no lookup (the
+// lookup in global memory for every pair made a masked tile cost 10 plain ones)
+template <int IPT>
+__device__ __forceinline__ void xmask(const Ctx &c, const int *ig, int j0, unsigned (&m)[IPT]) {
+#pragma unroll
+    for (int u = 0; u < IPT; u++) {
+        m[u] = 0u;
+        if (ig[u] < 0) continue;
+        for (int k = c.xs_off[ig[u]]; k < c.xs_off[ig[u] + 1]; k++) {
+            const int d = c.xs_part[k] - j0;
+            if (d >= 0 && d < 32) m[u] |= 1u << d;
+        }
+    }
+}
+
 // IPT i-atoms per thread share every j load from shared memory.  DM: 0 an
 // off-diagonal tile; 1 the i-tile itself (j == i skipped); 2 the i-tile
 // itself on the symmetric list (only j > i: each pair once).  MASK: the j
@@ -75,8 +91,13 @@ __device__ __forceinline__ void sweep(const typename VT<T>::V4 *__restrict__ sp,
                                       T (&lj)[IPT], const Ctx *cx = nullptr, const int *ig = nullptr,
                                       int jt = 0) {
     // the masked form runs on a few tiles only: kept rolled (smaller kernel)
+    constexpr int KW = MASK ? 32 : TJ;
+    for (int kw = 0; kw < TJ; kw += KW) {
+    unsigned xm[IPT];
+    if (MASK) xmask<IPT>(*cx, ig, jt + kw, xm);
 #pragma unroll(MASK ? 1 : 8)
-    for (int k = 0; k < TJ; k++) {
+    for (int kk = 0; kk < KW; kk++) {
+        const int k = kw + kk;
         const typename VT<T>::V4 pj = sp[k];
         const typename VT<T>::V2 qj = sq[k];
 #pragma unroll
@@ -88,7 +109,7 @@ __device__ __forceinline__ void sweep(const typename VT<T>::V4 *__restrict__ sp,
             if (DM == 2) ri = (k <= dk[u]) ? T(0) : ri;
             T sc = T(1);
             if (MASK) {
-                if (ig[u] >= 0) sc = (T)pair_xscale(*cx, ig[u], jt + k);
+                if ((xm[u] >> kk) & 1u) sc = (T)pair_xscale(*cx, ig[u], jt + k);
             }
             const T ri2 = ri * ri;
             const T e = MASK ? pi[u].w * pj.w * sc * ri : pi[u].w * pj.w * ri;
@@ -106,6 +127,7 @@ __device__ __forceinline__ void sweep(const typename VT<T>::V4 *__restrict__ sp,
                 gz[u] += f * dz;
             }
         }
+    }
     }
 }
 
@@ -127,8 +149,13 @@ __device__ __forceinline__ void sweep_delta(const float4 *__restrict__ sp, const
                                             const float2 (&ci)[IPT], const float4 (&di)[IPT],
                                             const int (&dk)[IPT], float (&ec)[IPT], float (&lj)[IPT],
                                             const Ctx *cx = nullptr, const int *ig = nullptr, int jt = 0) {
+    constexpr int KW = MASK ? 32 : TJ;
+    for (int kw = 0; kw < TJ; kw += KW) {
+    unsigned xm[IPT];
+    if (MASK) xmask<IPT>(*cx, ig, jt + kw, xm);
 #pragma unroll(MASK ? 1 : 4)
-    for (int k = 0; k < TJ; k++) {
+    for (int kk = 0; kk < KW; kk++) {
+        const int k = kw + kk;
         const float4 pj = sp[k];
         const float2 qj = sq[k];
         const float4 dj = sd[k];
@@ -151,13 +178,14 @@ __device__ __forceinline__ void sweep_delta(const float4 *__restrict__ sp, const
             const float d12 = d6 * (rp4 * rp2 + ri4 * ri2);
             float sc = 1.f;
             if (MASK) {
-                if (ig[u] >= 0) sc = pair_xscale(*cx, ig[u], jt + k);
+                if ((xm[u] >> kk) & 1u) sc = pair_xscale(*cx, ig[u], jt + k);
             }
             const float c6 = MASK ? ci[u].x * qj.x * sc : ci[u].x * qj.x;
             const float c12 = MASK ? ci[u].y * qj.y * sc : ci[u].y * qj.y;
             ec[u] += MASK ? pi[u].w * pj.w * sc * d1 : pi[u].w * pj.w * d1;
             lj[u] += c12 * d12 - c6 * d6;
         }
+    }
     }
 }
 
