@@ -7,19 +7,22 @@
 // Loss per sample: (z - t)^2; minibatch loss = mean.  Gradients:
 //   dz = 2 (z - t) / B,  dw2_k = dz h_k,  db2 = dz,
 //   dh_k = dz w2_k [a_k > 0],  dW1_ki = dh_k f_i,  db1_k = dh_k.
-// Per-block partial gradients are summed in a fixed order by a second kernel,
-// so a step is deterministic.
+// Partial gradients are summed in a fixed order, so training is
+// deterministic.
 //
 // Bound: latency (a step of 16,384 rows is 44 MFLOP, under a microsecond of
-// FP32).  Forward with one thread per row, backward with one thread per two
-// hidden units, whose 14 gradient sums stay in registers; the start's form
-// kept all 449 sums per thread in local memory and added them over the block
-// one parameter at a time (320 us a step, 27 us for the Adam kernel).  The
-// two kernels of a step are launched programmatically dependent, so that the
-// next one's rows are gathered while this one ends, and the losses stay on
-// the device until the last step.
+// FP32).  A warp takes 32 rows, a thread two hidden units, whose weights,
+// activations and 14 gradient sums stay in registers.  All steps of a call run in one cooperative launch: a step's gradient is summed over a
+// cluster of 8 blocks through distributed shared memory, over the clusters
+// through global memory at one grid barrier, and every block takes the Adam
+// step for itself (same sums, same order), so that the weights never leave
+// the SM; the next step's rows are gathered while the barrier is pending.
+// 16,384 rows: 320 + 27 us a step with all 449 sums per thread in local memory,
+// 11.3 us as two kernels a step, 8.7 us now.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -28,17 +31,30 @@
 
 namespace ffm {
 
-constexpr int MT = 128;          // threads per training block, one row each
-constexpr int MLP_ROWS = 256;    // partial-gradient rows of the scratch
-constexpr int MLP_BLOCKS = 152;  // blocks per minibatch gradient, at most
-// the scratch rows that no block uses hold the losses of up to this many steps
-constexpr int MLP_LOSSES = (MLP_ROWS - MLP_BLOCKS) * MLP_NW;
-constexpr int AT = 1024, AP = 32;  // Adam kernel: threads, parameters per block
+namespace cg = cooperative_groups;
 
-// programmatic dependent launch: let the next kernel of the stream start /
-// wait for the previous one to have finished
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+constexpr int MT = 128;           // threads per training block, one row each
+constexpr int MLP_ROWS = 256;     // rows of MLP_NW floats that the scratch holds
+constexpr int MLP_CLUSTER = 8;    // blocks per cluster
+constexpr int MLP_CLUSTERS = 16;  // clusters, at most (128 blocks: all resident at once)
+constexpr int MLP_NV = MLP_NW + 1;                    // summed values: the gradient, the loss
+constexpr int MLP_SLICE = (MLP_NV + MLP_CLUSTER - 1) / MLP_CLUSTER;
+constexpr int MLP_STEPS = 4096;   // steps per launch (their losses wait in the scratch)
+constexpr long long MLP_SPIN = 1 << 22;  // polls of the grid barrier before a block gives up (about a second)
+
+// a run of training steps; lr == 0: one gradient, no update
+struct MlpRun {
+    const float *feat, *target;
+    int64_t n;
+    int batch, steps, step0, sample;  // step0: steps taken before; sample: minibatches from the stream
+    uint64_t seed;
+    float lr;
+    float *w32, *adam;
+    float *part;               // [2][MLP_CLUSTERS][MLP_NV]
+    unsigned int *sync;        // [0] barrier count, [1] set when a block gave up
+    float *losses, *grad_out;  // losses [steps]; grad_out optional
+    uint16_t *w16;             // optional: FP16 copy for inference
+};
 
 __device__ __forceinline__ uint64_t mix64(uint64_t seed, uint64_t k) {
     uint64_t z = seed + (k + 1) * 0x9E3779B97F4A7C15ULL;
@@ -47,181 +63,223 @@ __device__ __forceinline__ uint64_t mix64(uint64_t seed, uint64_t k) {
     return z ^ (z >> 31);
 }
 
-// partial gradient of one block over its share of the minibatch; samples of
-// the minibatch are index (base + k) of the SplitMix64 stream when sample
-// != 0, else rows [0, batch) of the data in order
-__global__ void __launch_bounds__(MT) k_mlp_grad(const float *feat, const float *target, int64_t n,
-                                                 const float *w32, int batch, uint64_t seed, uint64_t base,
-                                                 int sample, float *part, float *loss_part) {
+// Samples of minibatch t are index t batch + k of the SplitMix64 stream when
+// sample != 0, else rows [0, batch) of the data in order
+__global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(MlpRun o) {
+    cg::cluster_group cl = cg::this_cluster();
     __shared__ float4 sw[MLP_H][2];        // per hidden unit: W1 (5), b1, w2
     __shared__ float4 sf[MT / 32][32][2];  // per row of the warp: features (5), dz
-    __shared__ float acc[MT / 32][MLP_NW];
-    __shared__ float lsum[MT / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    pdl_trigger();
-    float f[MLP_IN], t = 0.f;
-    const float inv_b = 1.0f / (float)batch;
-    float g[2][MLP_IN + 2] = {};  // of units lane, lane + 32: W1, b1, w2
-    float gb2 = 0.f, loss = 0.f;
-    float wu[2][MLP_IN + 2];
-    float b2 = 0.f;
-    for (int s0 = blockIdx.x * MT; s0 < batch; s0 += gridDim.x * MT) {
-        const int s = s0 + threadIdx.x;
-        const bool on = s < batch;
+    __shared__ float acc[MT / 32][MLP_NV];
+    __shared__ float sum[MLP_NV];          // the block's sums, read by the cluster
+    __shared__ float wt[MLP_NW], am[MLP_NW], av[MLP_NW];
+    __shared__ float unbias[2];
+    __shared__ int failed;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int rank = (int)cl.block_rank(), cluster = blockIdx.x / MLP_CLUSTER, clusters = gridDim.x / MLP_CLUSTER;
+    const float be1 = 0.9f, be2 = 0.999f, eps = 1e-8f;
+    const float inv_b = 1.0f / (float)o.batch;
+    for (int k = tid; k < MLP_NW; k += MT) {
+        wt[k] = o.w32[k];
+        if (o.lr > 0.f) {
+            am[k] = o.adam[k];
+            av[k] = o.adam[MLP_NW + k];
+        }
+    }
+    if (tid == 0) failed = 0;
+    float f[MLP_IN], tg = 0.f;
+    auto gather = [&](int t, int s0) {  // this thread's row of minibatch t, from s0 on
+        const int s = s0 + tid;
 #pragma unroll
         for (int i = 0; i < MLP_IN; i++) f[i] = 0.f;
-        if (on) {
-            const int64_t row = sample ? (int64_t)__umul64hi(mix64(seed, base + s), (uint64_t)n) : s;
+        tg = 0.f;
+        if (s >= o.batch) return;
+        const uint64_t q = (uint64_t)(o.step0 + t) * (uint64_t)o.batch + (uint64_t)s;
+        const int64_t row = o.sample ? (int64_t)__umul64hi(mix64(o.seed, q), (uint64_t)o.n) : s;
 #pragma unroll
-            for (int i = 0; i < MLP_IN; i++) f[i] = feat[row * MLP_IN + i];
-            t = target[row];
+        for (int i = 0; i < MLP_IN; i++) f[i] = o.feat[row * MLP_IN + i];
+        tg = o.target[row];
+    };
+    gather(0, blockIdx.x * MT);
+    for (int t = 0; t < o.steps; t++) {
+        __syncthreads();  // wt of this step
+        if (tid < MLP_H) {
+            const float *w1 = wt + MLP_W1 + tid * MLP_IN;
+            sw[tid][0] = make_float4(w1[0], w1[1], w1[2], w1[3]);
+            sw[tid][1] = make_float4(w1[4], wt[MLP_B1 + tid], wt[MLP_W2 + tid], 0.f);
         }
-        if (s0 == (int)blockIdx.x * MT) {  // the weights, once the previous step has written them
-            pdl_wait();
-            for (int k = threadIdx.x; k < MLP_H; k += MT) {
-                const float *w1 = w32 + MLP_W1 + k * MLP_IN;
-                sw[k][0] = make_float4(w1[0], w1[1], w1[2], w1[3]);
-                sw[k][1] = make_float4(w1[4], w32[MLP_B1 + k], w32[MLP_W2 + k], 0.f);
+        __syncthreads();
+        const float b2 = wt[MLP_B2];
+        float g[2][MLP_IN + 2] = {};  // of units lane, lane + 32: W1, b1, w2
+        float wu[2][MLP_IN + 2], gb2 = 0.f, loss = 0.f;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const float4 p = sw[lane + 32 * u][0], q = sw[lane + 32 * u][1];
+            wu[u][0] = p.x; wu[u][1] = p.y; wu[u][2] = p.z; wu[u][3] = p.w;
+            wu[u][4] = q.x; wu[u][5] = q.y; wu[u][6] = q.z;
+        }
+        for (int s0 = blockIdx.x * MT; s0 < o.batch; s0 += gridDim.x * MT) {
+            if (s0 != (int)blockIdx.x * MT) gather(t, s0);
+            // The warp's 32 rows, two hidden units per thread: the units'
+            // activations stay in registers for the backward pass, and their
+            // shares of z are summed over the lanes by halving (31 exchanges
+            // for 32 rows), which leaves row `lane` in lane `lane`
+            sf[w][lane][0] = make_float4(f[0], f[1], f[2], f[3]);
+            sf[w][lane][1] = make_float4(f[4], 0.f, 0.f, 0.f);
+            __syncwarp();
+            float act[32][2], z[32];
+#pragma unroll
+            for (int m = 0; m < 32; m++) {
+                const float4 p = sf[w][m][0];
+                const float p4 = sf[w][m][1].x;
+                z[m] = 0.f;
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    float a = fmaf(wu[u][0], p.x, wu[u][5]);
+                    a = fmaf(wu[u][1], p.y, a);
+                    a = fmaf(wu[u][2], p.z, a);
+                    a = fmaf(wu[u][3], p.w, a);
+                    a = fmaf(wu[u][4], p4, a);
+                    act[m][u] = fmaxf(a, 0.f);
+                    z[m] = fmaf(wu[u][6], act[m][u], z[m]);
+                }
             }
-            b2 = w32[MLP_B2];
-            __syncthreads();
 #pragma unroll
-            for (int u = 0; u < 2; u++) {
-                const float4 p = sw[lane + 32 * u][0], q = sw[lane + 32 * u][1];
-                wu[u][0] = p.x; wu[u][1] = p.y; wu[u][2] = p.z; wu[u][3] = p.w;
-                wu[u][4] = q.x; wu[u][5] = q.y; wu[u][6] = q.z;
+            for (int q = 16; q > 0; q >>= 1) {
+                const bool up = lane & q;
+#pragma unroll
+                for (int m = 0; m < q; m++) {
+                    const float keep = up ? z[m + q] : z[m], send = up ? z[m] : z[m + q];
+                    z[m] = keep + __shfl_xor_sync(0xffffffffu, send, q);
+                }
+            }
+            const float r = s0 + tid < o.batch ? (z[0] + b2) - tg : 0.f;
+            loss += r * r;
+            const float dz = 2.f * r * inv_b;
+            gb2 += dz;
+            sf[w][lane][1].y = dz;
+            __syncwarp();
+#pragma unroll
+            for (int m = 0; m < 32; m++) {
+                const float4 p = sf[w][m][0];
+                const float2 q = *reinterpret_cast<const float2 *>(&sf[w][m][1]);
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const float h = act[m][u];
+                    const float dh = h > 0.f ? q.y * wu[u][6] : 0.f;
+                    g[u][0] = fmaf(dh, p.x, g[u][0]);
+                    g[u][1] = fmaf(dh, p.y, g[u][1]);
+                    g[u][2] = fmaf(dh, p.z, g[u][2]);
+                    g[u][3] = fmaf(dh, p.w, g[u][3]);
+                    g[u][4] = fmaf(dh, q.x, g[u][4]);
+                    g[u][5] += dh;
+                    g[u][6] = fmaf(q.y, h, g[u][6]);
+                }
+            }
+            __syncwarp();
+        }
+        // the block's sums, warps in order
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = lane + 32 * u;
+#pragma unroll
+            for (int i = 0; i < MLP_IN; i++) acc[w][MLP_W1 + k * MLP_IN + i] = g[u][i];
+            acc[w][MLP_B1 + k] = g[u][5];
+            acc[w][MLP_W2 + k] = g[u][6];
+        }
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) {
+            gb2 += __shfl_xor_sync(0xffffffffu, gb2, q);
+            loss += __shfl_xor_sync(0xffffffffu, loss, q);
+        }
+        if (lane == 0) {
+            acc[w][MLP_B2] = gb2;
+            acc[w][MLP_NW] = loss;
+        }
+        __syncthreads();
+        for (int k = tid; k < MLP_NV; k += MT) sum[k] = (acc[0][k] + acc[1][k]) + (acc[2][k] + acc[3][k]);
+        cl.sync();
+        // the cluster's sums, one slice per block, blocks in order
+        float *part = o.part + (int64_t)(t & 1) * MLP_CLUSTERS * MLP_NV;
+        {
+            const int k = rank * MLP_SLICE + tid;
+            if (tid < MLP_SLICE && k < MLP_NV) {
+                float x[MLP_CLUSTER];
+#pragma unroll
+                for (int r = 0; r < MLP_CLUSTER; r++) x[r] = *cl.map_shared_rank(&sum[k], r);
+                part[cluster * MLP_NV + k] = ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+                __threadfence();
             }
         }
-        // forward: one row per thread
-        float z = b2;
-#pragma unroll 8
-        for (int k = 0; k < MLP_H; k++) {
-            const float4 p = sw[k][0], q = sw[k][1];
-            float a = fmaf(p.x, f[0], q.y);
-            a = fmaf(p.y, f[1], a);
-            a = fmaf(p.z, f[2], a);
-            a = fmaf(p.w, f[3], a);
-            a = fmaf(q.x, f[4], a);
-            z = fmaf(q.z, fmaxf(a, 0.f), z);
+        cl.sync();
+        // grid barrier: every cluster has its sums of this step in memory
+        // (the two buffers alternate, so no cluster writes over sums that
+        // another still reads: it arrives here again only after reading them)
+        if (rank == 0 && tid == 0) atomicAdd(&o.sync[0], 1u);
+        if (t + 1 < o.steps) gather(t + 1, blockIdx.x * MT);
+        if (tid == MT - 1) {  // Adam's bias corrections of this step
+            const float step = (float)(o.step0 + t + 1);
+            unbias[0] = 1.f - powf(be1, step);
+            unbias[1] = 1.f - powf(be2, step);
         }
-        const float r = on ? z - t : 0.f;
-        loss += r * r;
-        const float dz = 2.f * r * inv_b;
-        gb2 += dz;
-        sf[w][lane][0] = make_float4(f[0], f[1], f[2], f[3]);
-        sf[w][lane][1] = make_float4(f[4], dz, 0.f, 0.f);
-        __syncwarp();
-        // backward: two hidden units per thread, the warp's rows in order
-#pragma unroll 4
-        for (int m = 0; m < 32; m++) {
-            const float4 p = sf[w][m][0], q = sf[w][m][1];
-#pragma unroll
-            for (int u = 0; u < 2; u++) {
-                float a = fmaf(wu[u][0], p.x, wu[u][5]);
-                a = fmaf(wu[u][1], p.y, a);
-                a = fmaf(wu[u][2], p.z, a);
-                a = fmaf(wu[u][3], p.w, a);
-                a = fmaf(wu[u][4], q.x, a);
-                const float h = fmaxf(a, 0.f);
-                const float dh = h > 0.f ? q.y * wu[u][6] : 0.f;
-                g[u][0] = fmaf(dh, p.x, g[u][0]);
-                g[u][1] = fmaf(dh, p.y, g[u][1]);
-                g[u][2] = fmaf(dh, p.z, g[u][2]);
-                g[u][3] = fmaf(dh, p.w, g[u][3]);
-                g[u][4] = fmaf(dh, q.x, g[u][4]);
-                g[u][5] += dh;
-                g[u][6] = fmaf(q.y, h, g[u][6]);
+        if (tid == 0) {
+            const unsigned want = (unsigned)(t + 1) * (unsigned)clusters;
+            long long polls = 0;
+            unsigned got;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&o.sync[0]) : "memory");
+            } while (got < want && ++polls < MLP_SPIN && *(volatile unsigned int *)&o.sync[1] == 0u);
+            if (got < want) {
+                failed = 1;
+                o.sync[1] = 1u;
             }
         }
-        __syncwarp();
-    }
-    // the warps' sums in warp order
+        __syncthreads();
+        if (failed) break;
+        // the gradient over the clusters, then one Adam step: every load of a
+        // thread's (up to four) parameters in flight together
+        constexpr int KT = (MLP_NV + MT - 1) / MT;
+        float x[KT][MLP_CLUSTERS];
 #pragma unroll
-    for (int u = 0; u < 2; u++) {
-        const int k = lane + 32 * u;
+        for (int h = 0; h < KT; h++) {
+            const int k = tid + h * MT;
 #pragma unroll
-        for (int i = 0; i < MLP_IN; i++) acc[w][MLP_W1 + k * MLP_IN + i] = g[u][i];
-        acc[w][MLP_B1 + k] = g[u][5];
-        acc[w][MLP_W2 + k] = g[u][6];
-    }
+            for (int q = 0; q < MLP_CLUSTERS; q++)
+                x[h][q] = q < clusters && k < MLP_NV ? __ldcg(part + q * MLP_NV + k) : 0.f;
+        }
+        const float d1 = unbias[0], d2 = unbias[1];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        gb2 += __shfl_xor_sync(0xffffffffu, gb2, o);
-        loss += __shfl_xor_sync(0xffffffffu, loss, o);
-    }
-    if (lane == 0) {
-        acc[w][MLP_B2] = gb2;
-        lsum[w] = loss;
+        for (int h = 0; h < KT; h++) {
+            const int k = tid + h * MT;
+#pragma unroll
+            for (int q = MLP_CLUSTERS / 2; q > 0; q >>= 1)
+#pragma unroll
+                for (int r = 0; r < q; r++) x[h][r] += x[h][r + q];
+            const float gk = x[h][0];
+            if (k == MLP_NW && blockIdx.x == 0) o.losses[t] = gk / (float)o.batch;
+            if (k >= MLP_NW) continue;
+            if (o.grad_out && blockIdx.x == 0 && t == o.steps - 1) o.grad_out[k] = gk;
+            if (o.lr > 0.f) {
+                const float m = am[k] = be1 * am[k] + (1.f - be1) * gk;
+                const float v = av[k] = be2 * av[k] + (1.f - be2) * gk * gk;
+                wt[k] -= o.lr * (m / d1) / (sqrtf(v / d2) + eps);
+            }
+        }
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < MLP_NW; k += MT) {
-        float v = acc[0][k];
-#pragma unroll
-        for (int q = 1; q < MT / 32; q++) v += acc[q][k];
-        part[(int64_t)blockIdx.x * MLP_NW + k] = v;
+    if (blockIdx.x == 0) {
+        for (int k = tid; k < MLP_NW; k += MT) {
+            if (o.lr > 0.f) {
+                o.w32[k] = wt[k];
+                o.adam[k] = am[k];
+                o.adam[MLP_NW + k] = av[k];
+            }
+            if (o.w16) {
+                __half hv = __float2half_rn(wt[k]);
+                o.w16[k] = *reinterpret_cast<uint16_t *>(&hv);
+            }
+        }
     }
-    if (threadIdx.x == 0) {
-        float v = lsum[0];
-#pragma unroll
-        for (int q = 1; q < MT / 32; q++) v += lsum[q];
-        loss_part[blockIdx.x] = v;
-    }
-}
-
-// Sum of the block partials (thread (q, k) of a block takes the blocks q,
-// q + 32, ... of parameter k, then the 32 sums in order); then one Adam step
-// on the FP32 master weights (when lr > 0) and the FP16 copy for inference
-__global__ void __launch_bounds__(AT) k_mlp_adam(const float *part, const float *loss_part, int nblocks, int batch,
-                                                 float *w32, float *adam, int step, float lr, float *grad_out,
-                                                 float *loss_out, uint16_t *w16) {
-    __shared__ float sums[AT / AP][AP + 1];
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const int p = threadIdx.x & (AP - 1), q = threadIdx.x / AP, k = blockIdx.x * AP + p;
-    pdl_trigger();
-    pdl_wait();
-    // the loss counts as one more parameter, behind the last
-    float v = 0.f;
-    if (k < MLP_NW) {
-        for (int b = q; b < nblocks; b += AT / AP) v += part[(int64_t)b * MLP_NW + k];
-    } else if (k == MLP_NW) {
-        for (int b = q; b < nblocks; b += AT / AP) v += loss_part[b];
-    }
-    sums[q][p] = v;
-    __syncthreads();
-    if (q != 0 || k > MLP_NW) return;
-    float gk = 0.f;
-#pragma unroll
-    for (int r = 0; r < AT / AP; r++) gk += sums[r][p];
-    if (k == MLP_NW) {
-        if (loss_out) *loss_out = gk / (float)batch;
-        return;
-    }
-    if (grad_out) grad_out[k] = gk;
-    if (lr > 0.f) {
-        float m = adam[k] = b1 * adam[k] + (1.f - b1) * gk;
-        float vv = adam[MLP_NW + k] = b2 * adam[MLP_NW + k] + (1.f - b2) * gk * gk;
-        const float mh = m / (1.f - powf(b1, (float)step));
-        const float vh = vv / (1.f - powf(b2, (float)step));
-        w32[k] -= lr * mh / (sqrtf(vh) + eps);
-    }
-    if (w16) {
-        __half hv = __float2half_rn(w32[k]);
-        w16[k] = *reinterpret_cast<uint16_t *>(&hv);
-    }
-}
-
-template <typename... A, typename... B>
-static cudaError_t launch_dependent(void (*kernel)(A...), int grid, int block, cudaStream_t s, bool dependent, B... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, A(args)...);
+    cl.sync();  // no block leaves while its sums may be read
 }
 
 }  // namespace ffm
@@ -236,36 +294,49 @@ extern "C" ffmin_status ffmin_mlp_train(const float *feat_dev, const float *targ
         return FFMIN_ERR_INVALID_ARG;
     if (steps > 0 && (!adam_dev || !(lr > 0.f))) return FFMIN_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    float *part = work_dev;                                    // [MLP_BLOCKS][MLP_NW]
-    float *losses = part + (size_t)MLP_BLOCKS * MLP_NW;        // [MLP_LOSSES]
-    float *loss_part = work_dev + (size_t)MLP_ROWS * MLP_NW;   // [MLP_ROWS]
-    float *grad_dev = loss_part + MLP_ROWS + 1;                // [MLP_NW]
+    MlpRun o{};
+    o.feat = feat_dev;
+    o.target = target_dev;
+    o.n = n_samples;
+    o.batch = steps > 0 ? batch : (int)std::min<int64_t>(batch, n_samples);
+    o.sample = steps > 0 ? 1 : 0;
+    o.seed = seed;
+    o.lr = steps > 0 ? lr : 0.f;
+    o.w32 = w32_dev;
+    o.adam = adam_dev;
+    o.part = work_dev;                                                // [2][MLP_CLUSTERS][MLP_NV]
+    o.losses = o.part + (size_t)2 * MLP_CLUSTERS * MLP_NV;            // [MLP_STEPS]
+    float *tail = work_dev + (size_t)MLP_ROWS * MLP_NW;               // [MLP_ROWS + 1], then the gradient
+    o.sync = reinterpret_cast<unsigned int *>(tail);
+    static_assert(2 * MLP_CLUSTERS * MLP_NV + MLP_STEPS <= MLP_ROWS * MLP_NW, "the losses fit in the scratch");
     const int nsteps = steps > 0 ? steps : 1;
-    const int sample = steps > 0 ? 1 : 0;
-    const int b = steps > 0 ? batch : (int)std::min<int64_t>(batch, n_samples);
-    const int blocks = (int)std::min<int64_t>(MLP_BLOCKS, ((int64_t)b + MT - 1) / MT);
-    int kept = 0;  // steps whose losses have been copied
-    for (int t = 0; t < nsteps; t++) {
-        // the first kernel waits for whatever the stream held before; the
-        // others depend on the kernel before them alone
-        if (launch_dependent(k_mlp_grad, blocks, MT, s, t > kept, feat_dev, target_dev, n_samples,
-                             (const float *)w32_dev, b, seed, (uint64_t)t * (uint64_t)batch, sample, part,
-                             loss_part) != cudaSuccess)
+    const int blocks = (o.batch + MT - 1) / MT;
+    const int clusters = std::min(MLP_CLUSTERS, (blocks + MLP_CLUSTER - 1) / MLP_CLUSTER);
+    for (int t = 0; t < nsteps; t += MLP_STEPS) {
+        o.step0 = t;
+        o.steps = std::min(MLP_STEPS, nsteps - t);
+        const bool last = t + o.steps == nsteps;
+        o.grad_out = last ? tail + MLP_ROWS + 1 : nullptr;
+        o.w16 = last ? w16_dev : nullptr;
+        if (cudaMemsetAsync(o.sync, 0, 2 * sizeof(unsigned int), s) != cudaSuccess) return FFMIN_ERR_CUDA;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(clusters * MLP_CLUSTER);
+        cfg.blockDim = dim3(MT);
+        cfg.stream = s;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeCooperative;  // all blocks resident: the grid barrier ends
+        at.val.cooperative = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, k_mlp_train, o) != cudaSuccess) return FFMIN_ERR_CUDA;
+        unsigned int gave_up[2] = {0u, 0u};
+        if (cudaMemcpyAsync(gave_up, o.sync, sizeof(gave_up), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            (loss_host && cudaMemcpyAsync(loss_host + t, o.losses, sizeof(float) * (size_t)o.steps,
+                                          cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+            cudaStreamSynchronize(s) != cudaSuccess)
             return FFMIN_ERR_CUDA;
-        const bool last = t == nsteps - 1;
-        if (launch_dependent(k_mlp_adam, (MLP_NW + AP) / AP, AT, s, true, (const float *)part,
-                             (const float *)loss_part, blocks, b, w32_dev, adam_dev, t + 1, steps > 0 ? lr : 0.f,
-                             last ? grad_dev : (float *)nullptr, losses + (t - kept),
-                             last ? w16_dev : (uint16_t *)nullptr) != cudaSuccess)
-            return FFMIN_ERR_CUDA;
-        if (last || t - kept + 1 == MLP_LOSSES) {
-            if (loss_host && cudaMemcpyAsync(loss_host + kept, losses, sizeof(float) * (size_t)(t - kept + 1),
-                                             cudaMemcpyDeviceToHost, s) != cudaSuccess)
-                return FFMIN_ERR_CUDA;
-            kept = t + 1;
-        }
+        if (gave_up[1]) return FFMIN_ERR_TIMEOUT;
     }
-    if (cudaStreamSynchronize(s) != cudaSuccess) return FFMIN_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? FFMIN_OK : FFMIN_ERR_CUDA;
 }
 
