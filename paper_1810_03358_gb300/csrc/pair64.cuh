@@ -6,8 +6,9 @@
 // is written in FP64.  Here r^2, its reciprocal square root, the powers of r
 // and the products with the atoms' parameters are formed on 64-bit
 // significands with separate exponents and rounded once to FP64; FP64
-// instructions remain for the coordinate differences, the sums of the terms
-// and the accumulation (15 a pair with forces, 6 for an energy).  Every
+// instructions remain for the sums of the terms and the accumulation (12 a
+// pair with forces, 3 for an energy) and, outside the fixed-point range, for
+// the coordinate differences (3 more).  Every
 // significand below is good to 2^-57 or better and is rounded to 53 bits at
 // the end, so a term's error is no larger than that of the FP64 formula,
 // whose own roundings (each 2^-53) add up.
@@ -15,6 +16,9 @@
 // r^-1 from the hardware's approximate FP32 reciprocal square root y and one
 // step of the series (1 - h)^(-1/2) = 1 + h/2 + 3 h^2/8 + O(h^3) with
 // h = 1 - r^2 y^2, |h| < 2^-20, so that the next term is below 2^-61.
+//
+// Coordinate differences come in as doubles (any range below) or, for the
+// coordinates of an ordinary system, as fixed-point integers.
 //
 // Ranges: |d|max in [2^-40, 2^41) A and parameters that are zero or within
 // 2^-200 .. 2^200; then no intermediate leaves the exponent range of FP64.
@@ -114,20 +118,9 @@ struct Inv64 {
     int E, n, k;
 };
 
-// from the coordinate differences; false: outside the range
-FFM_P64 bool inv64(double dx, double dy, double dz, Inv64 &o) {
-    const u64 ux = bits64(dx), uy = bits64(dy), uz = bits64(dz);
-    const int ex = (int)((uint32_t)(ux >> 32) >> 20) & 0x7ff, ey = (int)((uint32_t)(uy >> 32) >> 20) & 0x7ff,
-              ez = (int)((uint32_t)(uz >> 32) >> 20) & 0x7ff;
-    const int em = ex > ey ? (ex > ez ? ex : ez) : (ey > ez ? ey : ez);
-    // significands aligned to the largest exponent, top bit 62 (a zero's
-    // implicit bit is shifted out with the rest)
-    const u64 one = 0x10000000000000ULL, frac = one - 1;
-    const int sx = em - ex < 63 ? em - ex : 63, sy = em - ey < 63 ? em - ey : 63, sz = em - ez < 63 ? em - ez : 63;
-    const u64 ax = (((ux & frac) | one) << 10) >> sx, ay = (((uy & frac) | one) << 10) >> sy,
-              az = (((uz & frac) | one) << 10) >> sz;
-    const u64 R = sqh(ax) + sqh(ay) + sqh(az);  // r^2 = R 2^(2 E - 60), R in [2^60, 3 2^62)
-    o.E = em - 1023;
+// from r^2 = R 2^(2 E - 60), R in [2^60, 3 2^62)
+FFM_P64 void inv64_back(u64 R, int E, Inv64 &o) {
+    o.E = E;
     const uint32_t y = rsqrt_seed((uint32_t)(R >> 32));
     // h = 1 - r^2 y^2 in units of 2^-57, then c = h/2 + 3 h^2/8 in units of 2^-58
     const long long h = (long long)(1ULL << 57) - (long long)mulh(R >> 1, (u64)y * y);
@@ -143,7 +136,71 @@ FFM_P64 bool inv64(double dx, double dy, double dz, Inv64 &o) {
     const u64 q6 = mulh(sqh(o.n2) << 1, o.n2);  // [2^59, 2^62), 53 + 3 n fraction bits
     o.k = clz_hi(q6) - 1;
     o.n6 = q6 << o.k;
+}
+
+// from the coordinate differences; false: outside the range
+FFM_P64 bool inv64(double dx, double dy, double dz, Inv64 &o) {
+    const u64 ux = bits64(dx), uy = bits64(dy), uz = bits64(dz);
+    const int ex = (int)((uint32_t)(ux >> 32) >> 20) & 0x7ff, ey = (int)((uint32_t)(uy >> 32) >> 20) & 0x7ff,
+              ez = (int)((uint32_t)(uz >> 32) >> 20) & 0x7ff;
+    const int em = ex > ey ? (ex > ez ? ex : ez) : (ey > ez ? ey : ez);
+    // significands aligned to the largest exponent, top bit 62 (a zero's
+    // implicit bit is shifted out with the rest)
+    const u64 one = 0x10000000000000ULL, frac = one - 1;
+    const int sx = em - ex < 63 ? em - ex : 63, sy = em - ey < 63 ? em - ey : 63, sz = em - ez < 63 ? em - ez : 63;
+    const u64 ax = (((ux & frac) | one) << 10) >> sx, ay = (((uy & frac) | one) << 10) >> sy,
+              az = (((uz & frac) | one) << 10) >> sz;
+    inv64_back(sqh(ax) + sqh(ay) + sqh(az), em - 1023, o);
     return em >= 1023 - 40 && em <= 1023 + 40;
+}
+
+// ---- coordinates in fixed point, units of 2^-54 A, for |x| < FIX_MAX A.  A
+// double of at least 1/4 A converts exactly (its last place is 2^-54 or more),
+// a smaller one with an error of 2^-55 A at most, and differences are exact,
+// where an FP64 difference is rounded at 2^-53 of itself.  Pairs closer than
+// 1/4 A take the FP64 differences, so the error of a difference, relative to
+// the separation, stays below the two units that FP64 coordinates give.
+constexpr double FIX_MAX = 224.0;
+constexpr long long FIX_FAR = 255LL << 54;  // padding atoms: beyond any real one, differences still fit
+FFM_P64 bool fix64(double x, long long &o) {  // false: out of range (or NaN)
+#ifdef __CUDA_ARCH__
+    o = __double2ll_rn(x * 0x1p54);
+#else
+    o = (long long)__builtin_rint(x * 0x1p54);
+#endif
+    return x > -FIX_MAX && x < FIX_MAX;
+}
+FFM_P64 u64 abs64(long long v) {
+    const long long s = v >> 63;
+    return (u64)((v ^ s) - s);
+}
+// from fixed-point differences (|d| < 2^63); a* return |d| shifted left by the
+// returned n; false: below 1/4 A in every component
+FFM_P64 bool inv64_fix(long long dx, long long dy, long long dz, Inv64 &o, u64 &ax, u64 &ay, u64 &az, int &n) {
+    ax = abs64(dx);
+    ay = abs64(dy);
+    az = abs64(dz);
+    const u64 any = (ax | ay | az) | 1ULL << 32;  // at least one bit for the count
+    n = clz_hi(any) - 1;
+    const bool ok = ((ax | ay | az) >> 52) != 0ULL;
+    ax <<= n;
+    ay <<= n;
+    az <<= n;
+    inv64_back(sqh(ax) + sqh(ay) + sqh(az), 8 - n, o);
+    return ok;
+}
+// a 2^-(54 + n) with the sign of v, rounded to FP64
+FFM_P64 double fix_to_double(u64 a, int n, long long v) {
+    const uint32_t hi = (uint32_t)(a >> 32), lo = (uint32_t)a;
+#ifdef __CUDA_ARCH__
+    const int z = hi ? __clz((int)hi) : 32 + __clz((int)lo);
+#else
+    const int z = a ? __builtin_clzll(a) : 64;
+#endif
+    const u64 m = a << (z & 63);
+    const u64 r = ((m >> 11) + ((uint32_t)((uint32_t)m >> 10) & 1u)) +
+                  ((u64)(uint32_t)((1023 + 63 - 54 - 1 - n - z) << 20) << 32);
+    return from_bits64((a ? r : 0) | ((u64)v & 0x8000000000000000ULL));
 }
 FFM_P64 double inv64_r1(const Inv64 &v) { return pack64<false>(v.m, 1023 - 63 - v.E); }
 FFM_P64 double inv64_r2(const Inv64 &v) { return pack64<false>(v.n2, 1023 - 62 - v.n - 2 * v.E); }
