@@ -155,9 +155,6 @@ static void bonded_items(const ffmin_system *sys, int b, std::vector<Item> &item
 constexpr int LAYOUT_ROW_BLOCKS[2] = {6, 12};  // row list, by i-atoms per thread
 constexpr int LAYOUT_SYM_BLOCKS = 7;           // energy-only list
 
-// FP64 list: tile pairs are cut into parts below this many items per SM
-constexpr int SPLIT_ITEMS_PER_SM = 8;
-
 // some evaluation of the object runs on the row list
 static bool needs_row_list(const ffmin_system *sys) { return !sys->c.sym64 || sys->prec == FFMIN_MIXED; }
 
@@ -259,15 +256,23 @@ static void build_list32e(ffmin_system *sys, int dens, std::vector<Item> &items,
     build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, false, &Tile::r32, items, sys_items,
                     slots);
 }
-// the FP64 list: chunks of several j-tiles, or, for a batch with fewer tile
-// pairs than wanted items, parts of 64 or 32 j-atoms (a lone tile pair keeps
-// one SM busy for 128 steps while the others idle)
+// The FP64 list: chunks of several j-tiles, or, for a batch with fewer tile
+// pairs than wanted items, parts of 64 or 32 j-atoms: the resident blocks take
+// ceil(items / blocks) rounds of equal items, so the fewest rounds in units of
+// a whole tile pair win, by 8 % at least since every part adds an i-side row to
+// sum (measured, E + grad / E, whole tiles, two parts, four parts: 3,334 atoms
+// 0.252 / 0.113, 0.167 / 0.076, 0.167 / 0.077 ms; 5,000 atoms 0.435 / 0.167, 0.367 /
+// 0.148, 0.336 / 0.144 ms; 7,000 atoms 0.636 / 0.279, 0.626 / 0.252 ms)
 static void build_list64(ffmin_system *sys, int dens, std::vector<Item> &items, std::vector<int2> &sys_items,
                          int64_t *slots) {
     const int64_t want = (int64_t)dens * sys->grid_sym, pairs = tile_pairs(sys);
     const int chunk = (int)std::max<int64_t>(1, pairs / want);
     int split = 1;
-    while (chunk == 1 && split < 4 && pairs * split < SPLIT_ITEMS_PER_SM * sys->sms) split *= 2;
+    if (chunk == 1) {
+        auto rounds = [&](int s) { return (double)((pairs * s + sys->grid_sym - 1) / sys->grid_sym) / s; };
+        for (int s = 2; s <= 4; s *= 2)
+            if (rounds(s) < 0.92 * rounds(split)) split = s;
+    }
     build_items_sym(sys, chunk, split, true, &Tile::r64, items, sys_items, slots);
 }
 
@@ -679,7 +684,6 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     c.n_atoms = (int)total;
     c.vstride = ((3 * total + 31) / 32) * 32;
     c.prec = precision;
-    c.sep_reduce = n_sys >= LB_MAX_SYS ? 1 : 0;
 
 #define CKC(call)                                                              \
     do {                                                                       \
@@ -791,6 +795,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     CKC(dalloc(sys, &c.red, (size_t)c.n_tiles * NRED));
     CKC(dalloc(sys, &c.redf, (size_t)c.n_tiles * 8));
     CKC(dalloc(sys, &c.counters, CNT_N));
+    CKC(dalloc(sys, &c.tickets, (size_t)N_STAGES * n_sys));
     CKC(dalloc(sys, &c.nactive, 1));
     CKC(dalloc(sys, &c.nmode, 2));
     float *d_feat;
@@ -863,24 +868,14 @@ static ffmin_status set_counts(ffmin_system *sys) {
     return FFMIN_OK;
 }
 
-// One evaluation's kernels: the active lists (built from the control state)
-// beside the trial point, then the pair kernels, then the finalize.  The
-// active-list kernel and k_prepare read the same state and write disjoint
-// buffers, so they run on parallel branches.
+// One evaluation's kernels: trial points and active lists, the pair kernels,
+// the finalize
 static cudaError_t launch_eval(ffmin_system *sys, cudaStream_t s) {
     const Ctx &c = sys->c;
-    const Branches &br = sys->br;
     cudaError_t e;
-    if ((e = cudaEventRecord(br.fork, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(br.side[0], br.fork, 0)) != cudaSuccess) return e;
-    if ((e = launch_activelist(c, br.side[0])) != cudaSuccess) return e;
     if ((e = launch_prepare(c, s)) != cudaSuccess) return e;
-    if ((e = cudaEventRecord(br.join[0], br.side[0])) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(s, br.join[0], 0)) != cudaSuccess) return e;
-    if ((e = launch_pair_kernels(c, sys->grid32, sys->grid32e, sys->grid64, s, &br)) != cudaSuccess) return e;
-    if ((e = launch_finalize(c, s)) != cudaSuccess) return e;
-    if (c.sep_reduce) return launch_sysreduce(c, 3, s);
-    return cudaSuccess;
+    if ((e = launch_pair_kernels(c, sys->grid32, sys->grid32e, sys->grid64, s, &sys->br)) != cudaSuccess) return e;
+    return launch_finalize(c, s);
 }
 
 static cudaError_t launch_tick(ffmin_system *sys) {
@@ -888,11 +883,8 @@ static cudaError_t launch_tick(ffmin_system *sys) {
     cudaStream_t s = sys->stream;
     cudaError_t e;
     if ((e = launch_update(c, s)) != cudaSuccess) return e;
-    if (c.sep_reduce && (e = launch_sysreduce(c, 0, s)) != cudaSuccess) return e;
     if ((e = launch_dir(c, 0, s)) != cudaSuccess) return e;
-    if (c.sep_reduce && (e = launch_sysreduce(c, 1, s)) != cudaSuccess) return e;
     if ((e = launch_dir(c, 1, s)) != cudaSuccess) return e;
-    if (c.sep_reduce && (e = launch_sysreduce(c, 2, s)) != cudaSuccess) return e;
     return launch_eval(sys, s);
 }
 
@@ -907,7 +899,7 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, const int32_t *nactive
     cudaGraphSetConditional(h, (*nactive > 0 && t < loop[1]) ? 1u : 0u);
 }
 static int kernels_per_tick(const ffmin_system *sys) {
-    return (sys->prec == FFMIN_MIXED ? 8 : 6) + (sys->c.sep_reduce ? 4 : 0);
+    return sys->prec == FFMIN_MIXED ? 8 : 6;
 }
 
 static ffmin_status ensure_graph(ffmin_system *sys) {
@@ -988,7 +980,6 @@ static ffmin_status eval_at(ffmin_system *sys, const double *base, int kind, con
     CK(launch_pair_list(c, r.list, r.list == LIST_F64 ? sys->grid64 : (r.list == LIST_F32_E ? sys->grid32e : sys->grid32),
                         sys->stream));
     CK(launch_finalize(c, sys->stream, g_out));
-    if (c.sep_reduce) CK(launch_sysreduce(c, 3, sys->stream));
     CK(cudaStreamSynchronize(sys->stream));
     for (int b = 0; b < sys->n_sys; b++) {
         SysState &S = sys->hst[b];
@@ -1198,8 +1189,7 @@ static ffmin_status minimize_dev(ffmin_system *sys, double *x_dev, const ffmin_o
         // point) by the next round's update kernel: run that update once more
         // so that the returned point is the one the counters describe
         CK(launch_update(c, sys->stream));
-        if (c.sep_reduce) CK(launch_sysreduce(c, 0, sys->stream));
-        sys->last_launches += 1 + (c.sep_reduce ? 1 : 0);
+        sys->last_launches += 1;
     }
     st = download_states(sys);
     if (st != FFMIN_OK) return st;

@@ -686,22 +686,24 @@ __host__ __device__ constexpr int ru_sjy(int j) { return 3 + 2 * j; }
 __host__ __device__ constexpr int ru_sjg(int j) { return 4 + 2 * j; }
 __host__ __device__ constexpr int ru_count(int nS) { return 3 + 2 * nS; }
 
-__device__ void on_update_done(const Ctx &c, SysState &S, const double *v) {
+// returns true when the first loop of the L-BFGS recursion (lbfgs_alpha) and
+// its direction pass come next
+__device__ bool on_update_done(const Ctx &c, SysState &S, const double *v) {
     const int op = S.upd.op;
     S.upd.op = U_NONE;
     S.upd.best = 0;
     if (S.phase == PH_DONE) {
         deactivate(c, S);
-        return;
+        return false;
     }
     if (op == U_OGM) {  // <r, r> of the new direction: evaluate E and grad at y
-        if (S.phase != PH_OGM_UPD) return;
+        if (S.phase != PH_OGM_UPD) return false;
         S.rnorm = sqrt(v[0]);
         set_eval(S, EV_EG, V_W, -1, 0.0, 1.0);
         S.phase = PH_OGM_Y;
-        return;
+        return false;
     }
-    if (op != U_PUSH) return;
+    if (op != U_PUSH) return false;
     const int nS = S.upd.nS;
     for (int k = 0; k < nS; k++) S.sg[S.upd.sS[k]] = v[ru_sjg(k)];
     const double sy = v[RU_SY];
@@ -723,7 +725,7 @@ __device__ void on_update_done(const Ctx &c, SysState &S, const double *v) {
     }
     if (S.ginf < S.gtol || mixed_handover(S, S.f, S.ginf)) {
         finish(c, S, FFMIN_OK, S.f, S.ginf);
-        return;
+        return false;
     }
     // learned-diagonal safeguard (not in the paper): a run whose energy
     // stalls far from a stationary point with the diagonal continues as
@@ -736,20 +738,34 @@ __device__ void on_update_done(const Ctx &c, SysState &S, const double *v) {
     const int n = S.ring_count;
     if (n == 0) {
         set_dir(S, 1, -1.0, 0.0, 1.0, 1);
-        return;
+        return false;
     }
-    // first loop (newest -> oldest): alpha_i = rho_i <s_i, q_i>,
-    // q_i = -g - sum_{j newer} alpha_j y_j
-    for (int k = n - 1; k >= 0; k--) {
-        const int a = S.ring[k];
-        double q = -S.sg[a];
-        for (int j = n - 1; j > k; j--) {
-            const int b = S.ring[j];
-            q = q - S.alpha[b] * S.SY[a][b];
-        }
-        S.alpha[a] = S.rho[a] * q;
+    return true;
+}
+
+// First loop of the two-loop recursion (newest -> oldest), by a warp: alpha_i =
+// rho_i <s_i, q_i>, q_i = -g - sum_{j newer} alpha_j y_j.  Lane k holds pair k and
+// subtracts each newer alpha as it becomes known, in the order of the loop.
+__device__ void lbfgs_alpha(SysState &S) {
+    const int lane = threadIdx.x & 31, n = S.ring_count;
+    const int a = S.ring[lane < n ? lane : 0];
+    double q = -S.sg[a];
+    for (int j = n - 1; j >= 0; j--) {
+        const int b = S.ring[j];
+        const double al = __shfl_sync(0xffffffffu, S.rho[a] * q, j);
+        if (lane == j) S.alpha[a] = al;
+        if (lane < j) q = q - al * S.SY[a][b];
     }
-    lbfgs_pass1(S, S.precond_on);
+    __syncwarp();
+}
+
+__device__ void warp_update_done(const Ctx &c, SysState &S, const double *v) {
+    int more = 0;
+    if ((threadIdx.x & 31) == 0) more = on_update_done(c, S, v) ? 1 : 0;
+    __syncwarp();
+    if (!__shfl_sync(0xffffffffu, more, 0)) return;
+    lbfgs_alpha(S);
+    if ((threadIdx.x & 31) == 0) lbfgs_pass1(S, S.precond_on);
 }
 
 // reductions of the direction kernels
@@ -759,33 +775,47 @@ __device__ void on_dir_done(const Ctx &c, SysState &S, int which, const double *
     S.dir[which].on = 0;
     if (S.phase == PH_DONE) return;
     if (which == 0) {
-        if (S.method == FFMIN_LBFGS) {
-            // second loop (oldest -> newest): beta_i = rho_i <y_i, r_i>,
-            // r_i = r0 + sum_{j older} (alpha_j - beta_j) s_j
-            const int n = S.ring_count;
-            double beta[NRING];
-            DirOp &d = S.dir[1];
-            set_dir(S, 1, 0.0, 1.0, 1.0, 1);
-            d.nS = n;
-            for (int k = 0; k < n; k++) {
-                const int a = S.ring[k];
-                double yr = v[n - 1 - k];  // <y_a, r0>, dots were newest first
-                for (int j = 0; j < k; j++) {
-                    const int b = S.ring[j];
-                    yr = yr + (S.alpha[b] - beta[j]) * S.SY[b][a];
-                }
-                beta[k] = S.rho[a] * yr;
-                d.sS[k] = a;
-                d.cS[k] = S.alpha[a] - beta[k];
-            }
-            return;
-        }
         if (S.method == FFMIN_CG && S.cg_check && v[RD_GR] >= 0.0) {
             set_dir(S, 1, -1.0, 0.0, 1.0, 1);  // not a descent direction: restart
             return;
         }
     }
     ls_begin(c, S, v[RD_RR], v[RD_GR]);
+}
+
+// Second loop of the recursion (oldest -> newest), by a warp: beta_i = rho_i
+// <y_i, r_i>, r_i = r0 + sum_{j older} (alpha_j - beta_j) s_j; the direction
+// pass that adds the s_j comes next.  Lane k holds pair k.
+__device__ void lbfgs_beta(SysState &S, const double *v) {
+    const int lane = threadIdx.x & 31, n = S.ring_count;
+    const int a = S.ring[lane < n ? lane : 0];
+    double yr = lane < n ? v[n - 1 - lane] : 0.0;  // <y_a, r0>, dots were newest first
+    for (int j = 0; j < n; j++) {
+        const int b = S.ring[j];
+        const double cj = __shfl_sync(0xffffffffu, S.alpha[a] - S.rho[a] * yr, j);
+        if (lane == j) {
+            S.dir[1].sS[j] = a;
+            S.dir[1].cS[j] = cj;
+        }
+        if (lane > j) yr = yr + cj * S.SY[b][a];
+    }
+    __syncwarp();
+}
+
+__device__ void warp_dir_done(const Ctx &c, SysState &S, int which, const double *v) {
+    const int lane = threadIdx.x & 31;
+    if (which == 0 && S.method == FFMIN_LBFGS && S.phase != PH_DONE) {
+        if (lane == 0) {
+            S.dir[0].on = 0;
+            set_dir(S, 1, 0.0, 1.0, 1.0, 1);
+            S.dir[1].nS = S.ring_count;
+        }
+        __syncwarp();
+        lbfgs_beta(S, v);
+    } else if (lane == 0) {
+        on_dir_done(c, S, which, v);
+    }
+    __syncwarp();
 }
 
 }  // namespace ffm

@@ -156,11 +156,6 @@ struct SysState {
 // point); a failed FP32 line search also hands over
 constexpr double MIXED_SWITCH_RATIO = 1.0;
 
-// batches of at least this many systems reduce and run their control steps
-// in k_sysreduce (one block per system); smaller ones in the last block of
-// each per-tile kernel
-constexpr int LB_MAX_SYS = 8;
-
 // one evaluation of every system outside a minimization: the point is
 // base + h dir (dir may be nullptr), kind EV_E or EV_EG
 struct EvalReq {
@@ -178,7 +173,6 @@ struct Ctx {
     int32_t n_sys, n_tiles, n_items, n_atoms;
     int64_t vstride;
     int32_t prec;           // ffmin_precision
-    int32_t sep_reduce;     // 1: per-system reductions + control in separate kernels (large batches)
     int32_t f32_ipt;        // FP32 pair-kernel shape: i-atoms per thread (1 or 2; host-side dispatch)
     const Tile *tiles;
     const Item *items;
@@ -228,6 +222,7 @@ struct Ctx {
     double *red;            // [n_tiles][NRED]
     double *redf;           // finalize: [value][n_tiles]
     unsigned int *counters; // one per kernel kind, reset by the last block
+    unsigned int *tickets;  // [N_STAGES][n_sys]: blocks of a system that finished a stage
     int32_t *nactive;       // systems still minimizing
     int32_t *nmode;         // [2] active systems per pair-kernel precision mode
     // learned preconditioner features
@@ -250,14 +245,16 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t seed, uint64_t k) {
 }
 
 // counters[] indices
-enum { CNT_PAIR = 0, CNT_PAIR_EXIT = 1, CNT_FIN = 2, CNT_UPD = 3, CNT_DIR1 = 4, CNT_DIR2 = 5,
-       CNT_PARAB = 6, CNT_PARAB2 = 7, CNT_PAIR64 = 8, CNT_PAIR64_EXIT = 9, CNT_PAIR32E = 10, CNT_N = 11 };
+enum { CNT_PAIR = 0, CNT_PARAB, CNT_PARAB2, CNT_PAIR64, CNT_PAIR32E, CNT_N };
+// stages of a round that end in per-system control steps
+enum { STAGE_UPD = 0, STAGE_DIR1, STAGE_DIR2, STAGE_FIN, N_STAGES };
 
 // work queues of the pair kernels (one active list each): FP32 E + grad,
 // FP64 terms, FP32 energy only (plain and difference trials)
 enum { LIST_F32_EG = 0, LIST_F64 = 1, LIST_F32_E = 2, N_LISTS = 3 };
 
 // ---- launchers (defined in the .cu files) ----
+// trial points and (one more block) the active lists of the work queues
 cudaError_t launch_prepare(const Ctx &c, cudaStream_t s);
 cudaError_t launch_ncount(const Ctx &c, const double *x, int32_t *out, cudaStream_t s);
 // launches the FP32 kernel (MIXED objects) and the FP64 kernel; each skips
@@ -270,8 +267,7 @@ struct Branches {
     cudaStream_t side[2];
     cudaEvent_t fork, join[2];
 };
-cudaError_t launch_activelist(const Ctx &c, cudaStream_t s);
-// the pair kernels alone (launch_pair = active lists, then these in turn);
+// the pair kernels alone (launch_pair: active lists, then these in turn);
 // with br, the FP32 energy-only and FP64 kernels run on br's side streams
 cudaError_t launch_pair_kernels(const Ctx &c, int grid32, int grid32e, int grid64, cudaStream_t s,
                                 const Branches *br);
@@ -283,9 +279,6 @@ cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s);
 cudaError_t launch_pair_list(const Ctx &c, int list, int grid, cudaStream_t s);
 cudaError_t launch_update(const Ctx &c, cudaStream_t s);
 cudaError_t launch_dir(const Ctx &c, int which, cudaStream_t s);
-// per-system reduction + control step after a stage (only when sep_reduce):
-// stage 0 update, 1 / 2 direction passes, 3 finalize
-cudaError_t launch_sysreduce(const Ctx &c, int stage, cudaStream_t s);
 // basin hopping: out = best + step (2u - 1) per coordinate, u from the
 // SplitMix64 stream of seed + b at counter hop * 3N_b + k (system b); and the
 // copy of x into best for the systems whose flag is set

@@ -11,14 +11,15 @@
 //             scaled by gamma (and the learned diagonal), with their dots
 //
 // Reductions are deterministic: every block writes its partial sums, the
-// last block to finish (atomic ticket) sums each system's blocks in a fixed
-// order and runs that system's control step.  No thread ever waits.
+// last block of a system to finish (atomic ticket) sums the system's blocks
+// in a fixed order and runs its control step.  No thread ever waits.
 //
 // This file is compiled without contraction of a*b+c into FMA so that the
 // scalar control arithmetic and the vector updates round like their
 // textbook statements; fused multiply-adds appear only where written.
 #include <cmath>
 
+#include "activelist.cuh"
 #include "bonded.cuh"
 #include "control.cuh"
 #include "mlp.cuh"
@@ -59,6 +60,10 @@ __device__ __forceinline__ void prepare_atom(const Ctx &c, int a, const double *
 }
 
 __global__ void __launch_bounds__(TI) k_prepare(Ctx c) {
+    if (blockIdx.x == c.n_tiles) {  // the work queues, beside the tiles' trial points
+        active_lists(c);
+        return;
+    }
     const Tile t = c.tiles[blockIdx.x];
     const SysState &S = c.st[t.sys];
     if (S.ev_kind == EV_NONE) return;
@@ -69,64 +74,32 @@ __global__ void __launch_bounds__(TI) k_prepare(Ctx c) {
 }
 
 // One evaluation outside a minimization in three launches (this, the pair
-// kernel of the kind, the finalize; one more for 8 systems and up): the point
-// is read where the caller has it, and block 0 sets every system's request
-// and the one work queue that the evaluation uses.  Uploading the states,
+// kernel of the kind, the finalize): the point is read where the caller has
+// it, and block 0 sets every system's request and the work queues.  Uploading the states,
 // copying the point and the active lists were half of a small evaluation.
 __global__ void __launch_bounds__(TI) k_prepare_eval(Ctx c, EvalReq r) {
     const Tile &t = c.tiles[blockIdx.x];
     if (threadIdx.x < t.na) prepare_atom(c, t.a0 + threadIdx.x, r.base, r.dir, r.h, 1.0, r.mode, r.delta != 0);
     if (blockIdx.x != 0) return;
-    __shared__ int wsum[NW];
-    __shared__ int base;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int2 *items = r.list == LIST_F64 ? (c.sym64 ? c.sys_items64 : c.sys_items)
-                                           : (r.list == LIST_F32_E && c.sym32 ? c.sys_items32 : c.sys_items);
-    int32_t *A = c.act + r.list * (2 * c.n_sys + 2);
+    for (int b = threadIdx.x; b < c.n_sys; b += TI) {
+        SysState &S = c.st[b];
+        S.active = 1;
+        S.phase = PH_EVAL_ONLY;
+        S.upd.op = U_NONE;
+        S.dir[0].on = S.dir[1].on = 0;
+        S.ev_kind = r.kind;
+        S.ev_delta = r.delta;
+        S.ne = S.neg = 0;
+        S.mode = r.mode;
+        S.epair_base = S.epair_last;
+    }
     if (threadIdx.x == 0) {
-        base = 0;
-        c.counters[r.list == LIST_F64 ? CNT_PAIR64 : (r.list == LIST_F32_E ? CNT_PAIR32E : CNT_PAIR)] = 0;
         *c.nactive = c.n_sys;
         c.nmode[0] = r.mode == 0 ? c.n_sys : 0;
         c.nmode[1] = r.mode == 0 ? 0 : c.n_sys;
-        A[0] = c.n_sys;
     }
     __syncthreads();
-    for (int b0 = 0; b0 < c.n_sys; b0 += TI) {
-        const int b = b0 + threadIdx.x;
-        int n = 0;
-        if (b < c.n_sys) {
-            SysState &S = c.st[b];
-            S.active = 1;
-            S.phase = PH_EVAL_ONLY;
-            S.upd.op = U_NONE;
-            S.dir[0].on = S.dir[1].on = 0;
-            S.ev_kind = r.kind;
-            S.ev_delta = r.delta;
-            S.ne = S.neg = 0;
-            S.mode = r.mode;
-            S.epair_base = S.epair_last;
-            n = items[b].y;
-        }
-        int sum = n;  // inclusive scan within the warp
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, sum, o);
-            if (lane >= o) sum += u;
-        }
-        if (lane == 31) wsum[w] = sum;
-        __syncthreads();
-        int p = base + sum - n;
-        for (int v = 0; v < w; v++) p += wsum[v];
-        if (b < c.n_sys) {
-            A[2 + b] = p;
-            A[2 + c.n_sys + b] = b;
-        }
-        __syncthreads();
-        if (threadIdx.x == TI - 1) base = p + n;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) A[1] = base;
+    active_lists(c);
 }
 
 cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) {
@@ -167,25 +140,21 @@ __device__ __forceinline__ Row4 row_at(const double4_32a *rows, int64_t slot, in
     return Row4{p.x, p.y, p.z, p.w};
 }
 
-// this strand's share (w, w + 4, ...) of the sum over q < n of f(q), added to
-// a; XYZ / W: the components that count
+// this strand's share (w, w + 4, ...) of the sum over q < n of f(q), in order,
+// added to a; XYZ / W: the components that count; four or eight loads in flight
 template <bool XYZ, bool W, typename F>
 __device__ __forceinline__ void strand_sum(int n, int w, Row4 &a, F f) {
-    int q = w;
-    for (; q + 12 < n; q += 16) {  // four loads in flight
-        Row4 p[4];
+    constexpr int U = XYZ ? 4 : 8;
+    for (int q = w; q < n; q += 4 * U) {
+        Row4 p[U];
 #pragma unroll
-        for (int u = 0; u < 4; u++) p[u] = f(q + 4 * u);
+        for (int u = 0; u < U; u++) p[u] = q + 4 * u < n ? f(q + 4 * u) : Row4{0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
+        for (int u = 0; u < U; u++) {
+            if (q + 4 * u >= n) break;
             if (XYZ) { a.x += p[u].x; a.y += p[u].y; a.z += p[u].z; }
             if (W) a.w += p[u].w;
         }
-    }
-    for (; q < n; q += 4) {
-        const Row4 p = f(q);
-        if (XYZ) { a.x += p.x; a.y += p.y; a.z += p.z; }
-        if (W) a.w += p.w;
     }
 }
 
@@ -205,26 +174,7 @@ __device__ __forceinline__ void sym_rows(const Ctx &c, const Tile &t, int tile0,
     });
 }
 
-// sum (or max) of finalize value k over a system's tiles, fixed order, by a
-// whole warp; the result is valid on every lane
-__device__ double fin_sys_sum(const Ctx &c, const SysState &S, int k, bool mx) {
-    const int lane = threadIdx.x & 31, t1 = S.tile0 + S.ntile;
-    const double *r = c.redf + (int64_t)k * c.n_tiles;
-    double x = 0.0;
-#pragma unroll 4
-    for (int t = S.tile0 + lane; t < t1; t += 32) {
-        const double y = __ldcg(&r[t]);
-        x = mx ? fmax(x, y) : x + y;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double y = __shfl_xor_sync(0xffffffffu, x, o);
-        x = mx ? fmax(x, y) : x + y;
-    }
-    return x;
-}
-
-__global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
+__global__ void __launch_bounds__(FIN_NT, 2) k_finalize(Ctx c, double *g_out) {
     const Tile &t = c.tiles[blockIdx.x];
     const SysState &S = c.st[t.sys];
     const int kind = S.ev_kind, mode = S.mode;
@@ -235,7 +185,8 @@ __global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
     __shared__ double val[RF_N][TI + 1];
     __shared__ double strands[RF_N][RSTRANDS];
     const unsigned maxmask = (1u << RF_GINF) | (1u << RF_BAD);
-    if (kind != EV_NONE) {
+    if (kind == EV_NONE) return;
+    {
         const bool real = i < t.na, grad = kind == EV_EG;
         const int a = t.a0 + i;
         Row4 r = Row4{0.0, 0.0, 0.0, 0.0}, bo = r;
@@ -261,15 +212,28 @@ __global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
             // and position gradients through its incidence list, the even
             // entries in strand 2, the odd ones in strand 3
             if (w >= 2) {
+                constexpr int U = 5;  // an atom in a chain has 9 or 10 entries
                 const int k1 = c.inc_off[a + 1];
-#pragma unroll 2
-                for (int k = c.inc_off[a] + w - 2; k < k1; k += 2) {
-                    const int2 in = c.inc[k];
-                    const int type = in.x >> 2, pos = in.x & 3;
-                    if (pos == 0) bo.w += c.te[bonded_index(c, type, in.y)];
-                    if (grad) {
-                        const double *g = c.tg + 3 * bonded_grad_slot(c, type, in.y, pos);
-                        bo.x += g[0]; bo.y += g[1]; bo.z += g[2];
+                for (int k = c.inc_off[a] + w - 2; k < k1; k += 2 * U) {
+                    int2 in[U];
+                    Row4 p[U];
+#pragma unroll
+                    for (int u = 0; u < U; u++) in[u] = k + 2 * u < k1 ? c.inc[k + 2 * u] : make_int2(-1, 0);
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        const int type = in[u].x >> 2, pos = in[u].x & 3;
+                        if (in[u].x < 0) continue;
+                        p[u].w = pos == 0 ? c.te[bonded_index(c, type, in[u].y)] : 0.0;
+                        if (grad) {
+                            const double *g = c.tg + 3 * bonded_grad_slot(c, type, in[u].y, pos);
+                            p[u].x = g[0]; p[u].y = g[1]; p[u].z = g[2];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        if (in[u].x < 0) break;
+                        if ((in[u].x & 3) == 0) bo.w += p[u].w;
+                        if (grad) { bo.x += p[u].x; bo.y += p[u].y; bo.z += p[u].z; }
                     }
                 }
             }
@@ -328,30 +292,27 @@ __global__ void __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
             c.redf[(int64_t)k * c.n_tiles + blockIdx.x] = x;
         }
     }
-    if (c.sep_reduce || !last_block(&c.counters[CNT_FIN])) return;
-    // fewer than 8 systems: the last block sums every system's tiles, one
-    // (system, value) per warp at a time, then warp 0 runs the control steps
-    // in system order on a shared-memory copy of the state
-    __shared__ double tot[LB_MAX_SYS][RF_N];
+    if (!sys_last_block(&c.tickets[STAGE_FIN * c.n_sys + t.sys], S.ntile)) return;
+    __shared__ double tot[RF_N];
     __shared__ SysState sS;
-    const int n = c.n_sys < LB_MAX_SYS ? c.n_sys : LB_MAX_SYS;
-    for (int u = warp; u < n * RF_N; u += FIN_NT / 32) {
-        const SysState &Sb = c.st[u / RF_N];
-        if (Sb.ev_kind == EV_NONE) continue;
-        const double x = fin_sys_sum(c, Sb, u % RF_N, (maxmask >> (u % RF_N)) & 1u);
-        if (lane == 0) tot[u / RF_N][u % RF_N] = x;
+    const int t0 = S.tile0, t1 = S.tile0 + S.ntile;
+    const double *r = c.redf;
+    static_assert(RF_GG == RF_E + 1 && RF_GTR == RF_GTG + 1, "summed in pairs");
+    if (warp == 0) {
+        warp_sums8(r, c.n_tiles, 1, t0, t1, 2, &tot[RF_E]);
+    } else if (warp == 1) {
+        warp_sums8(r + (int64_t)RF_GTG * c.n_tiles, c.n_tiles, 1, t0, t1, 2, &tot[RF_GTG]);
+    } else if (warp == 2) {
+        warp_sums8(r + (int64_t)RF_EPAIR * c.n_tiles, c.n_tiles, 1, t0, t1, 1, &tot[RF_EPAIR]);
+    } else if (warp == 3) {
+        warp_max(r + (int64_t)RF_GINF * c.n_tiles, 1, t0, t1, &tot[RF_GINF]);
+    } else if (warp == 4) {
+        warp_max(r + (int64_t)RF_BAD * c.n_tiles, 1, t0, t1, &tot[RF_BAD]);
     }
     __syncthreads();
-    if (warp == 0) {
-        for (int b = 0; b < n; b++) {
-            if (c.st[b].ev_kind == EV_NONE) continue;
-            warp_copy_state(&sS, &c.st[b]);
-            if (lane == 0) on_eval_done(c, sS, b, tot[b]);
-            __syncwarp();
-            warp_copy_state(&c.st[b], &sS);
-        }
-    }
-    if (threadIdx.x == 0) c.counters[CNT_FIN] = 0;
+    sys_control(c, t.sys, sS, [&](SysState &W) {
+        if (lane == 0) on_eval_done(c, W, t.sys, tot);
+    });
 }
 
 // ---------------------------------------------------------------- update
@@ -360,6 +321,7 @@ __global__ void __launch_bounds__(TI) k_update(Ctx c) {
     const SysState &S = c.st[t.sys];
     const int op = S.upd.op;
     const int i = threadIdx.x;
+    if (op == U_NONE) return;
     if (op == U_PUSH) {
         double v[RU_N];
 #pragma unroll
@@ -431,7 +393,7 @@ __global__ void __launch_bounds__(TI) k_update(Ctx c) {
             v[0] = dot3_fma(rr, rr);
         }
         block_reduce_columns<1>(v, 1, 0u, &c.red[(int64_t)blockIdx.x * NRED]);
-    } else if (op != U_NONE && i < t.na) {
+    } else if (i < t.na) {
         const int64_t off = 3 * (int64_t)(t.a0 + i);
         double *X = vslot(c, V_X) + off, *G = vslot(c, V_G) + off, *W = vslot(c, V_W) + off;
         double *P = vslot(c, V_P) + off, *XB = vslot(c, V_XB) + off;
@@ -482,13 +444,11 @@ __global__ void __launch_bounds__(TI) k_update(Ctx c) {
             break;
         }
     }
-    if (c.sep_reduce || !last_block(&c.counters[CNT_UPD])) return;
-    last_block_systems<RU_N>(
-        c, RU_N, 0u, [](const SysState &S) { return S.upd.op != U_NONE; },
-        [&](SysState &S, const double *tot) { on_update_done(c, S, tot); },
-        [](const SysState &S) { return S.upd.op == U_PUSH ? ru_count(S.upd.nS) : (S.upd.op == U_OGM ? 1 : 0); });
-    __syncthreads();
-    if (threadIdx.x == 0) c.counters[CNT_UPD] = 0;
+    if (!sys_last_block(&c.tickets[STAGE_UPD * c.n_sys + t.sys], S.ntile)) return;
+    __shared__ double tot[RU_N];
+    __shared__ SysState sS;
+    sys_sums(c, S, op == U_PUSH ? ru_count(S.upd.nS) : (op == U_OGM ? 1 : 0), tot);
+    sys_control(c, t.sys, sS, [&](SysState &W) { warp_update_done(c, W, tot); });
 }
 
 // ---------------------------------------------------------------- direction
@@ -501,14 +461,14 @@ __global__ void __launch_bounds__(TI) k_dir(Ctx c) {
     double v[NRING];
 #pragma unroll
     for (int k = 0; k < NRING; k++) v[k] = 0.0;
-    const bool on = d.on != 0;
+    if (!d.on) return;
     __shared__ float w_mlp[MLP_NW];
-    if (on && d.use_d) {  // learned H0 diagonal: FP16 weights -> FP32 in shared memory
+    if (d.use_d) {  // learned H0 diagonal: FP16 weights -> FP32 in shared memory
         for (int k = threadIdx.x; k < MLP_NW; k += blockDim.x)
             w_mlp[k] = __half2float(__ushort_as_half(c.mlp_w[k]));
         __syncthreads();
     }
-    if (on && i < t.na) {
+    if (i < t.na) {
         const int64_t off = 3 * (int64_t)(t.a0 + i);
         const double *G = vslot(c, V_G) + off;
         double *R = vslot(c, V_R) + off;
@@ -554,85 +514,48 @@ __global__ void __launch_bounds__(TI) k_dir(Ctx c) {
             }
         }
     }
-    if (on) block_reduce_columns<NRING>(v, d.dots == 2 ? d.nY : 2, 0u, &c.red[(int64_t)blockIdx.x * NRED]);
-    if (c.sep_reduce || !last_block(&c.counters[WHICH == 0 ? CNT_DIR1 : CNT_DIR2])) return;
-    last_block_systems<NRING>(
-        c, 2, 0u, [](const SysState &S) { return S.dir[WHICH].on != 0; },
-        [&](SysState &S, const double *tot) { on_dir_done(c, S, WHICH, tot); },
-        [](const SysState &S) { return S.dir[WHICH].dots == 2 ? S.dir[WHICH].nY : 2; });
-    __syncthreads();
-    if (threadIdx.x == 0) c.counters[WHICH == 0 ? CNT_DIR1 : CNT_DIR2] = 0;
-}
-
-// one block per system: the system's tile partials of every value are summed
-// by the block's warps in tile order, then thread 0 runs the control step
-template <int STAGE>
-__global__ void __launch_bounds__(TI) k_sysreduce(Ctx c) {
-    SysState &S = c.st[blockIdx.x];
-    int nv;
-    unsigned maxmask = 0u;
-    if (STAGE == 0) {
-        if (S.upd.op == U_NONE) return;
-        nv = S.upd.op == U_PUSH ? ru_count(S.upd.nS) : (S.upd.op == U_OGM ? 1 : 0);
-    } else if (STAGE == 1 || STAGE == 2) {
-        const DirOp &d = S.dir[STAGE - 1];
-        if (!d.on) return;
-        nv = d.dots == 2 ? d.nY : 2;
-    } else {
-        if (S.ev_kind == EV_NONE) return;
-        nv = RF_N;
-        maxmask = (1u << RF_GINF) | (1u << RF_BAD);
-    }
-    __shared__ double tot[NRED];
+    const int nv = d.dots == 2 ? d.nY : 2;
+    block_reduce_columns<NRING>(v, nv, 0u, &c.red[(int64_t)blockIdx.x * NRED]);
+    if (!sys_last_block(&c.tickets[(WHICH == 0 ? STAGE_DIR1 : STAGE_DIR2) * c.n_sys + t.sys], S.ntile)) return;
+    __shared__ double tot[NRING + 1];
     __shared__ SysState sS;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int k = w; k < nv; k += NW) {
-        const double x = STAGE == 3 ? fin_sys_sum(c, S, k, (maxmask >> k) & 1u)
-                                    : warp_sys_sum(c, S, k, (maxmask >> k) & 1u);
-        if (lane == 0) tot[k] = x;
-    }
-    __syncthreads();
-    if (w != 0) return;
-    // the control step on a shared-memory copy of the state
-    warp_copy_state(&sS, &S);
-    if (lane == 0) {
-        if (STAGE == 0) on_update_done(c, sS, tot);
-        else if (STAGE == 1) on_dir_done(c, sS, 0, tot);
-        else if (STAGE == 2) on_dir_done(c, sS, 1, tot);
-        else on_eval_done(c, sS, blockIdx.x, tot);
-    }
-    __syncwarp();
-    warp_copy_state(&S, &sS);
+    sys_sums(c, S, nv, tot);
+    sys_control(c, t.sys, sS, [&](SysState &W) { warp_dir_done(c, W, WHICH, tot); });
 }
 
-cudaError_t launch_sysreduce(const Ctx &c, int stage, cudaStream_t s) {
-    switch (stage) {
-    case 0: k_sysreduce<0><<<c.n_sys, TI, 0, s>>>(c); break;
-    case 1: k_sysreduce<1><<<c.n_sys, TI, 0, s>>>(c); break;
-    case 2: k_sysreduce<2><<<c.n_sys, TI, 0, s>>>(c); break;
-    default: k_sysreduce<3><<<c.n_sys, TI, 0, s>>>(c); break;
-    }
-    return cudaGetLastError();
-}
-
-// neighbours within 8 A of every atom inside its own system, from X
+// Neighbours within 8 A of every atom inside its own system, at x.  Block
+// (tile, chunk): the tile's atoms against j-atoms staged in FP32 through shared
+// memory, chunk y of every NC_CHUNKS-th j-tile; counts add up in out (zero
+// before).  Each thread used to convert every j-atom of its system itself
+// (conversions run at the FP64 rate), on as many SMs as there are tiles:
+// 1,207 us for 32 systems of 200 to 5,000 atoms, 96 us now.
+constexpr int NC_CHUNKS = 8;
 __global__ void __launch_bounds__(TI) k_ncount(Ctx c, const double *x, int32_t *out) {
-    const Tile t = c.tiles[blockIdx.x];
+    __shared__ float4 sj[TI];
+    const Tile &t = c.tiles[blockIdx.x];
     const SysState &S = c.st[t.sys];
-    const int i = threadIdx.x;
-    if (i >= t.na) return;
-    const int a = t.a0 + i;
+    const int i = threadIdx.x, a = t.a0 + (i < t.na ? i : 0), end = S.atom0 + S.natoms;
     const float xi = (float)x[3 * a], yi = (float)x[3 * a + 1], zi = (float)x[3 * a + 2];
     int n = 0;
-    for (int j = S.atom0; j < S.atom0 + S.natoms; j++) {
-        const float dx = (float)x[3 * j] - xi, dy = (float)x[3 * j + 1] - yi, dz = (float)x[3 * j + 2] - zi;
-        n += (j != a && dx * dx + dy * dy + dz * dz < 64.f) ? 1 : 0;
+    for (int jt = S.atom0 + blockIdx.y * TI; jt < end; jt += NC_CHUNKS * TI) {
+        const int j = jt + i;
+        __syncthreads();
+        if (j < end) sj[i] = make_float4((float)x[3 * j], (float)x[3 * j + 1], (float)x[3 * j + 2], 0.f);
+        __syncthreads();
+        const int m = min(TI, end - jt);
+#pragma unroll 8
+        for (int k = 0; k < m; k++) {
+            const float dx = sj[k].x - xi, dy = sj[k].y - yi, dz = sj[k].z - zi;
+            n += (jt + k != a && dx * dx + dy * dy + dz * dz < 64.f) ? 1 : 0;
+        }
     }
-    out[a] = n;
+    if (i < t.na && n) atomicAdd(&out[a], n);
 }
 
 cudaError_t launch_ncount(const Ctx &c, const double *x, int32_t *out, cudaStream_t s) {
-    k_ncount<<<c.n_tiles, TI, 0, s>>>(c, x, out);
+    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(int32_t) * (size_t)c.n_atoms, s);
+    if (e != cudaSuccess) return e;
+    k_ncount<<<dim3(c.n_tiles, NC_CHUNKS), TI, 0, s>>>(c, x, out);
     return cudaGetLastError();
 }
 
@@ -672,7 +595,7 @@ cudaError_t launch_mbh_accept(const Ctx &c, const int32_t *flags, const double *
 }
 
 cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
-    k_prepare<<<c.n_tiles, TI, 0, s>>>(c);
+    k_prepare<<<c.n_tiles + 1, TI, 0, s>>>(c);
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out) {

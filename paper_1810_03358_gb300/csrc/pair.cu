@@ -28,6 +28,7 @@
 #include <cstdio>
 #include <type_traits>
 
+#include "activelist.cuh"
 #include "bonded.cuh"
 #include "ffmin_internal.cuh"
 #include "pair64.cuh"
@@ -977,68 +978,7 @@ cudaError_t launch_pair_list(const Ctx &c, int list, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Active lists for the two pair kernels: for each precision mode, the
-// systems with an evaluation request in that mode and the exclusive prefix
-// of their item counts, in system order (one block; warp-shuffle scans over
-// chunks of 256 systems).  The block also resets both work-queue counters.
-__global__ void __launch_bounds__(256) k_activelist(Ctx c) {
-    __shared__ int wsum_i[8], wsum_s[8];
-    __shared__ int base_items, base_sys;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        c.counters[CNT_PAIR] = 0;
-        c.counters[CNT_PAIR64] = 0;
-        c.counters[CNT_PAIR32E] = 0;
-    }
-    for (int L = 0; L < N_LISTS; L++) {
-        int32_t *A = c.act + L * (2 * c.n_sys + 2);
-        if (threadIdx.x == 0) { base_items = 0; base_sys = 0; }
-        __syncthreads();
-        for (int b0 = 0; b0 < c.n_sys; b0 += 256) {
-            const int b = b0 + threadIdx.x;
-            int n = 0;
-            if (b < c.n_sys) {
-                const SysState &S = c.st[b];
-                // queue of the system's evaluation: FP32 E + grad (row list),
-                // FP64 terms or FP32 energy only (symmetric list when the
-                // object has one)
-                const int mine = S.ev_kind == EV_NONE ? -1
-                                 : (S.mode == 1 ? LIST_F64 : (S.ev_kind == EV_E ? LIST_F32_E : LIST_F32_EG));
-                if (mine == L)
-                    n = (L == LIST_F64 ? (c.sym64 ? c.sys_items64 : c.sys_items)
-                                       : (L == LIST_F32_E && c.sym32 ? c.sys_items32 : c.sys_items))[b].y;
-            }
-            const int f = n > 0 ? 1 : 0;
-            int si = n, ss = f;  // inclusive scans within the warp
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int ti = __shfl_up_sync(0xffffffffu, si, o), ts = __shfl_up_sync(0xffffffffu, ss, o);
-                if (lane >= o) { si += ti; ss += ts; }
-            }
-            if (lane == 31) { wsum_i[warp] = si; wsum_s[warp] = ss; }
-            __syncthreads();
-            int pi = base_items + si - n, ps = base_sys + ss - f;
-            for (int w = 0; w < warp; w++) { pi += wsum_i[w]; ps += wsum_s[w]; }
-            if (f) {
-                A[2 + ps] = pi;
-                A[2 + c.n_sys + ps] = b;
-            }
-            __syncthreads();
-            if (threadIdx.x == 255) { base_items = pi + n; base_sys = ps + f; }
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            A[0] = base_sys;
-            A[1] = base_items;
-        }
-        __syncthreads();
-    }
-}
-
-cudaError_t launch_activelist(const Ctx &c, cudaStream_t s) {
-    k_activelist<<<1, 256, 0, s>>>(c);  // also gives every pair kernel a fresh work queue
-    return cudaGetLastError();
-}
+__global__ void __launch_bounds__(32 * N_LISTS) k_activelist(Ctx c) { active_lists(c); }
 
 // The three pair kernels of a MIXED object take disjoint work queues and
 // write disjoint outputs, so with side streams the FP32 energy-only and the
@@ -1069,7 +1009,8 @@ cudaError_t launch_pair_kernels(const Ctx &c, int grid32, int grid32e, int grid6
 }
 
 cudaError_t launch_pair(const Ctx &c, int grid32, int grid32e, int grid64, cudaStream_t s) {
-    cudaError_t e = launch_activelist(c, s);
+    k_activelist<<<1, 32 * N_LISTS, 0, s>>>(c);  // also gives every pair kernel a fresh work queue
+    const cudaError_t e = cudaGetLastError();
     return e != cudaSuccess ? e : launch_pair_kernels(c, grid32, grid32e, grid64, s, nullptr);
 }
 

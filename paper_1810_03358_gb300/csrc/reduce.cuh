@@ -1,6 +1,8 @@
 // Deterministic block and per-system reductions shared by the per-tile
-// kernels: every block stores its partial sums; the last block to finish
-// (atomic ticket, no waiting) sums each system's blocks in a fixed order.
+// kernels: every block stores its partial sums; the last block of a system to
+// finish (atomic ticket per system, no waiting) sums the system's blocks in a
+// fixed order and runs its control step, so the systems of a batch do not
+// wait for one another and no further launch is needed.
 #pragma once
 
 #include "ffmin_internal.cuh"
@@ -88,98 +90,90 @@ __device__ inline void block_reduce_columns(const double (&v)[NV], int nv, unsig
     }
 }
 
-// sum (or max) of one reduction value over a system's tiles, fixed order,
-// executed by a whole warp; the result is valid on every lane
-__device__ inline double warp_sys_sum(const Ctx &c, const SysState &S, int k, bool mx) {
-    const int lane = threadIdx.x & 31;
-    double x = 0.0;
-    for (int t = S.tile0 + lane; t < S.tile0 + S.ntile; t += 32) {
-        const double y = __ldcg(&c.red[(int64_t)t * NRED + k]);
-        x = mx ? fmax(x, y) : x + y;
+// ticket of a block among its system's: true in the last one, which then may
+// read what the others stored
+__device__ inline bool sys_last_block(unsigned int *cnt, int ntile) {
+    __shared__ int am_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        am_last = atomicAdd(cnt, 1u) == (unsigned)ntile - 1u;
+        if (am_last) *cnt = 0u;  // for the next launch
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double y = __shfl_xor_sync(0xffffffffu, x, o);
-        x = mx ? fmax(x, y) : x + y;
-    }
-    return x;
+    __syncthreads();
+    if (am_last) __threadfence();
+    return am_last != 0;
 }
 
-// the same for the first nv reduction values, eight at a time (the same
-// order per value, so the same results): lane l takes tiles l, l + 32, ...
-// in order with the group's values of a tile loaded together, then a
-// butterfly over the lanes; lane 0 stores the results to out
-template <int NR>
-__device__ inline void warp_sys_sums(const Ctx &c, const SysState &S, int nv, unsigned maxmask, double *out) {
-    constexpr int G = NR < 8 ? NR : 8;
+// Sums of up to 8 values over a system's tiles by a warp: value k of tile t at
+// r[k vs + t ts]; lane l takes tiles l, l + 32, ... in order, then the lanes
+// are combined 16 apart, 8 apart, ... 1 apart, sharing the values out on the
+// way (9 additions for 8 values; the FP64 unit takes 64 cycles for each,
+// however many lanes are on).  Stored to out[k].
+__device__ inline void warp_sums8(const double *r, int64_t vs, int64_t ts, int t0, int t1, int nv, double *out) {
     const int lane = threadIdx.x & 31;
-    for (int k0 = 0; k0 < nv; k0 += G) {  // nv is the same on every lane
-        double x[G];
+    double x[8];
 #pragma unroll
-        for (int k = 0; k < G; k++) x[k] = 0.0;
-        for (int t = S.tile0 + lane; t < S.tile0 + S.ntile; t += 32) {
-            const double *r = &c.red[(int64_t)t * NRED + k0];
-            double y[G];
+    for (int k = 0; k < 8; k++) x[k] = 0.0;
+#pragma unroll 2
+    for (int t = t0 + lane; t < t1; t += 32) {
+        double y[8];
 #pragma unroll
-            for (int k = 0; k < G; k++) y[k] = k0 + k < nv ? __ldcg(r + k) : 0.0;
+        for (int k = 0; k < 8; k++) y[k] = k < nv ? __ldcg(&r[k * vs + t * ts]) : 0.0;
 #pragma unroll
-            for (int k = 0; k < G; k++) x[k] = ((maxmask >> (k0 + k)) & 1u) ? fmax(x[k], y[k]) : x[k] + y[k];
-        }
+        for (int k = 0; k < 8; k++)
+            if (k < nv) x[k] += y[k];
+    }
 #pragma unroll
-        for (int k = 0; k < G; k++) {
-            const bool mx = (maxmask >> (k0 + k)) & 1u;
+    for (int h = 4; h > 0; h >>= 1) {
+        const bool up = lane & (4 * h);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double y = __shfl_xor_sync(0xffffffffu, x[k], o);
-                x[k] = mx ? fmax(x[k], y) : x[k] + y;
-            }
-            if (lane == 0 && k0 + k < nv) out[k0 + k] = x[k];
+        for (int k = 0; k < h; k++) {
+            const double keep = up ? x[k + h] : x[k], send = up ? x[k] : x[k + h];
+            x[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
         }
     }
+    x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+    x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+    if ((lane & 3) == 0 && (lane >> 2) < nv) out[lane >> 2] = x[0];
+}
+// largest value over a system's tiles by a warp
+__device__ inline void warp_max(const double *r, int64_t ts, int t0, int t1, double *out) {
+    const int lane = threadIdx.x & 31;
+    double x = 0.0;
+    for (int t = t0 + lane; t < t1; t += 32) x = fmax(x, __ldcg(&r[t * ts]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+    if (lane == 0) *out = x;
+}
+// the first nv reduction values of a per-tile kernel (c.red), by the block
+__device__ inline void sys_sums(const Ctx &c, const SysState &S, int nv, double *out) {
+    for (int k = 8 * (threadIdx.x >> 5); k < nv; k += 8 * (blockDim.x >> 5))
+        warp_sums8(c.red + k, 1, NRED, S.tile0, S.tile0 + S.ntile, min(8, nv - k), out + k);
+    __syncthreads();
 }
 
 // A system's control state copied by a warp (8-byte words, coalesced), so
-// that the control step, one thread's long chain of dependent reads and
-// writes of the state, runs on a shared-memory copy instead of global memory
+// that the control step, a long chain of dependent reads and writes of the
+// state, runs on a shared-memory copy instead of global memory
 __device__ inline void warp_copy_state(SysState *dst, const SysState *src) {
     static_assert(sizeof(SysState) % 8 == 0, "SysState is copied in 8-byte words");
     const unsigned long long *s = reinterpret_cast<const unsigned long long *>(src);
     unsigned long long *d = reinterpret_cast<unsigned long long *>(dst);
+#pragma unroll 8
     for (int k = threadIdx.x & 31; k < (int)(sizeof(SysState) / 8); k += 32) d[k] = s[k];
     __syncwarp();
 }
 
-// The last block's per-system work (fewer than 8 systems; larger batches
-// reduce in k_sysreduce): the warps reduce the systems' tiles (warp w takes
-// systems w, w + 4, ...), then warp 0 runs fn(S, totals) for every system
-// for which pred(S) holds, in system order, each on a shared-memory copy
-// of its state that is written back afterwards (the copy lives in the
-// buffer of block_reduce_columns<NR>, whose work is done by then).
-template <int NR, typename Pred, typename Fn>
-__device__ inline void last_block_systems(const Ctx &c, int nv_max, unsigned maxmask, Pred pred,
-                                          Fn fn, int (*nv_of)(const SysState &)) {
-    static_assert(sizeof(SysState) <= sizeof(double) * NR * (TI + 1), "state copy fits the column buffer");
-    __shared__ double wtot[LB_MAX_SYS][NR];
-    __shared__ int on[LB_MAX_SYS];
-    SysState &sS = *reinterpret_cast<SysState *>(columns_buffer<NR>());
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int n = c.n_sys < LB_MAX_SYS ? c.n_sys : LB_MAX_SYS;
-    for (int b = w; b < n; b += TI / 32) {
-        const SysState &S = c.st[b];
-        const bool p = pred(S);
-        if (lane == 0) on[b] = p ? 1 : 0;
-        if (!p) continue;
-        warp_sys_sums<NR>(c, S, nv_of ? nv_of(S) : nv_max, maxmask, wtot[b]);
-    }
-    __syncthreads();
-    if (w != 0) return;
-    for (int b = 0; b < n; b++) {
-        if (!on[b]) continue;
-        warp_copy_state(&sS, &c.st[b]);
-        if (lane == 0) fn(sS, wtot[b]);
-        __syncwarp();
-        warp_copy_state(&c.st[b], &sS);
-    }
+// control step of system b by warp 0 on the copy sS: fn(S) is called by the
+// whole warp
+template <typename Fn>
+__device__ inline void sys_control(const Ctx &c, int b, SysState &sS, Fn fn) {
+    if (threadIdx.x >= 32) return;
+    warp_copy_state(&sS, &c.st[b]);
+    fn(sS);
+    __syncwarp();
+    warp_copy_state(&c.st[b], &sS);
 }
 
 }  // namespace ffm

@@ -47,9 +47,9 @@ def check(ff, orc, s):
     assert np.abs(g - go).max() <= 1e-9 * np.abs(go).max()
 
 
-# 1 to 3 tiles, ragged last parts, the sizes around the change from four parts
-# to two (608 tile pairs) and to whole tiles (1,216), and several tiles a chunk
-@pytest.mark.parametrize("n", [31, 33, 96, 97, 257, 4352, 4481, 6200, 6273, 9000])
+# 1 to 3 tiles, ragged last parts, sizes with four parts a tile pair (up to 257,
+# 6,200 and 6,273), two (3,400 and 9,000) and whole tiles (4,352 and 4,481)
+@pytest.mark.parametrize("n", [31, 33, 96, 97, 257, 3400, 4352, 4481, 6200, 6273, 9000])
 def test_tiles_and_parts(ff, orc, n):
     rng = np.random.default_rng(n)
     s = synth.make_system(min(n, 2000), 900 + n)
@@ -123,3 +123,22 @@ def test_noalloc_special_values(ff, n, what):
     total = 0.5 * (np.abs(ec) + e4 * (s6 * s6 + np.abs(s6))).sum()
     assert abs(e.item() - e_ref) <= 2e-11 * total
     assert np.abs(g.cpu().numpy().reshape(n, 3) - g_ref).max() <= 1e-9 * np.abs(g_ref).max()
+
+
+@pytest.mark.parametrize("sizes", [(1,), (2, 127, 128, 129), (700, 5, 1025, 300)])
+def test_neighbour_counts(ff, orc, sizes):
+    """Counts within 8 A at tile edges and in a ragged batch, by brute force in
+    the FP32 arithmetic of the kernel."""
+    import torch
+    systems = [synth.make_system(n, 300 + n) for n in sizes]
+    S = ff.System(systems, 0)
+    counts = torch.full((S.n_atoms,), -1, dtype=torch.int32, device="cuda")
+    ff.ffmin_neighbour_counts(S.handle, to_dev([s.x for s in systems]), counts)
+    S.close()
+    want = []
+    for s in systems:
+        x = s.x.astype(np.float32)
+        d = x[:, None] - x[None]
+        near = d[..., 0] * d[..., 0] + d[..., 1] * d[..., 1] + d[..., 2] * d[..., 2] < np.float32(64.0)
+        want.append(near.sum(1) - 1)
+    assert np.array_equal(counts.cpu().numpy(), np.concatenate(want))
