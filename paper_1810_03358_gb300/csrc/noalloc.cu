@@ -12,8 +12,8 @@
 // Computation: an FP64 row sweep over all pairs of one system, Coulomb +
 // Lennard-Jones, no bonded terms: every pair in both of its rows, since the
 // fixed scratch has no room for the opposite forces.  Bound: the FP64 pipe;
-// the terms are formed on the integer pipes (pair64.cuh), which leaves 12 FP64
-// instructions an evaluated pair of about 28.  Blocks of 32 i-atoms against a
+// differences and terms are formed on the integer pipes (pair64.cuh), which
+// leaves 9 FP64 instructions an evaluated pair of about 28.  Blocks of 32 i-atoms against a
 // j-chunk, the chunk's atoms dealt to the four warps, give about 1,000 equal
 // blocks at 4,000 atoms (128 i-atoms per block: 256, 1.7 per SM).  4,000 atoms:
 // 1.10 -> 0.44 ms a call.  Partial rows go to the scratch, then one thread per atom
@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "ffmin.h"
 #include "pair64.cuh"
@@ -107,57 +108,101 @@ __global__ void __launch_bounds__(NA_NT, 5) k_na_rows(NaArgs a) {
     in_range = split64(pi[2], m12, e12) && in_range && !(pi[2] < 0.0);
     const int ce = (e6 << 16) | e12;
     const uint32_t qs = (uint32_t)(bits64(pi[0]) >> 32) & 0x80000000u;
+    long long fi[3];
+    bool i_fix = in_range;
+    for (int k = 0; k < 3; k++) i_fix = fix64(xi[k], fi[k]) && i_fix;
+    if (i >= a.n) {
+        fi[0] = fi[1] = fi[2] = -FIX_FAR;
+        i_fix = true;
+    }
     const int len = (a.n + a.chunks - 1) / a.chunks;
     const int j0 = blockIdx.y * len, j1 = min(a.n, j0 + len);
     double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
     for (int jt = j0; jt < j1; jt += NA_TJ) {
         double xj[3], pj[3];
-        na_atom(a, jt + tid < j1 ? jt + tid : a.n, 1e6, xj, pj);
+        const bool real = jt + tid < j1;
+        na_atom(a, real ? jt + tid : a.n, 1e6, xj, pj);
         u64 u1, u6, u12;
         int f1, f6, f12;
         bool range = split64(pj[0], u1, f1) && in_range;
         range = split64(pj[1], u6, f6) && range && !(pj[1] < 0.0);
         range = split64(pj[2], u12, f12) && range && !(pj[2] < 0.0);
-        s_xy[tid] = make_ulonglong2(bits64(xj[0]), bits64(xj[1]));
-        s_zq[tid] = make_ulonglong2(bits64(xj[2]), u1);
+        long long fj[3] = {FIX_FAR, FIX_FAR, FIX_FAR};
+        bool j_fix = i_fix;
+        if (real)
+            for (int k = 0; k < 3; k++) j_fix = fix64(xj[k], fj[k]) && j_fix;
+        // fixed-point coordinates for the tile when all of them fit (the
+        // barrier also ends the reads of the last tile)
+        const bool fix = __syncthreads_and(j_fix && range);
+        const bool plain = fix ? false : __syncthreads_or(!range);
+        s_xy[tid] = fix ? make_ulonglong2((u64)fj[0], (u64)fj[1]) : make_ulonglong2(bits64(xj[0]), bits64(xj[1]));
+        s_zq[tid] = make_ulonglong2(fix ? (u64)fj[2] : bits64(xj[2]), u1);
         s_c[tid] = make_ulonglong2(u6, u12);
         s_e[tid] = make_int2((int)((uint32_t)f1 | ((uint32_t)(bits64(pj[0]) >> 32) & 0x80000000u)), (f6 << 16) | f12);
         for (int k = 0; k < 3; k++) s_p[k][tid] = pj[k];
-        const bool plain = __syncthreads_or(!range);
-        const int kend = min(w * 32 + 32, j1 - jt);
-        for (int k = w * 32; k < kend; k++) {  // the same j for every lane
-            const ulonglong2 xy = s_xy[k], zq = s_zq[k], cj = s_c[k];
-            const int2 ej = s_e[k];
-            double dx = from_bits64(xy.x) - xi[0], dy = from_bits64(xy.y) - xi[1], dz = from_bits64(zq.x) - xi[2];
-            const bool on = jt + k != i;
-            if (!on) { dx = 1.0; dy = 0.0; dz = 0.0; }
-            Inv64 v;
-            const bool ok = inv64(dx, dy, dz, v);
-            const int es = ce + ej.y;
-            double e = inv64_c1(v, m1, zq.y, e1 + (ej.x & 0xffff));
-            e = from_bits64(bits64(e) ^ ((u64)(((uint32_t)ej.x & 0x80000000u) ^ qs) << 32));
-            double p6 = inv64_c6(v, m6, cj.x, (int)((uint32_t)es >> 16));
-            double p12 = inv64_c12(v, m12, cj.y, es & 0xffff);
-            double ri2 = inv64_r2(v);
-            if (__any_sync(0xffffffffu, !ok) || plain) {
-                const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
-                ri2 = ri * ri;
-                const double ri6 = ri2 * ri2 * ri2;
-                e = pi[0] * s_p[0][k] * ri;
-                p6 = pi[1] * s_p[1][k] * ri6;
-                p12 = pi[2] * s_p[2][k] * ri6 * ri6;
-            }
-            if (!on) e = p6 = p12 = 0.0;
-            const double u = p12 - p6;
-            ec += e;
-            lj += u;
-            const double f = ((u + p12) + e) * ri2;
-            gx = fma(f, dx, gx);
-            gy = fma(f, dy, gy);
-            gz = fma(f, dz, gz);
-        }
         __syncthreads();
+        const int kend = min(w * 32 + 32, j1 - jt);
+        auto rows = [&](auto FIX) {
+            for (int k = w * 32; k < kend; k++) {  // the same j for every lane
+                const ulonglong2 xy = s_xy[k], zq = s_zq[k], cj = s_c[k];
+                const int2 ej = s_e[k];
+                const bool on = jt + k != i;
+                Inv64 v;
+                bool ok;
+                double dx = 1.0, dy = 0.0, dz = 0.0;
+                if constexpr (decltype(FIX)::value) {
+                    const long long gx_ = (long long)xy.x - fi[0], gy_ = (long long)xy.y - fi[1],
+                                    gz_ = (long long)zq.x - fi[2];
+                    u64 ax, ay, az;
+                    int n;
+                    ok = inv64_fix(gx_, gy_, gz_, v, ax, ay, az, n) || !on;
+                    dx = fix_to_double(ax, n, gx_);
+                    dy = fix_to_double(ay, n, gy_);
+                    dz = fix_to_double(az, n, gz_);
+                } else {
+                    if (on) {
+                        dx = from_bits64(xy.x) - xi[0];
+                        dy = from_bits64(xy.y) - xi[1];
+                        dz = from_bits64(zq.x) - xi[2];
+                    }
+                    ok = inv64(dx, dy, dz, v);
+                }
+                const int es = ce + ej.y;
+                double e = inv64_c1(v, m1, zq.y, e1 + (ej.x & 0xffff));
+                e = from_bits64(bits64(e) ^ ((u64)(((uint32_t)ej.x & 0x80000000u) ^ qs) << 32));
+                double p6 = inv64_c6(v, m6, cj.x, (int)((uint32_t)es >> 16));
+                double p12 = inv64_c12(v, m12, cj.y, es & 0xffff);
+                double ri2 = inv64_r2(v);
+                if (__any_sync(0xffffffffu, !ok) || plain) {
+                    if (decltype(FIX)::value) {
+                        dx = 1.0; dy = dz = 0.0;
+                        if (on) {
+                            dx = a.x[3 * (jt + k)] - xi[0];
+                            dy = a.x[3 * (jt + k) + 1] - xi[1];
+                            dz = a.x[3 * (jt + k) + 2] - xi[2];
+                        }
+                    }
+                    const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+                    ri2 = ri * ri;
+                    const double ri6 = ri2 * ri2 * ri2;
+                    e = pi[0] * s_p[0][k] * ri;
+                    p6 = pi[1] * s_p[1][k] * ri6;
+                    p12 = pi[2] * s_p[2][k] * ri6 * ri6;
+                }
+                if (!on) e = p6 = p12 = ri2 = 0.0;
+                const double u = p12 - p6;
+                ec += e;
+                lj += u;
+                const double f = ((u + p12) + e) * ri2;
+                gx = fma(f, dx, gx);
+                gy = fma(f, dy, gy);
+                gz = fma(f, dz, gz);
+            }
+        };
+        if (fix) rows(std::true_type{});
+        else rows(std::false_type{});
     }
+    __syncthreads();
     s_sum[w][lane] = make_double4_32a(gx, gy, gz, ec + lj * (1.0 / 6.0));
     __syncthreads();
     // component w of atom `lane`, the warps in order
