@@ -256,6 +256,12 @@ static void build_list32e(ffmin_system *sys, int dens, std::vector<Item> &items,
     build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, false, &Tile::r32, items, sys_items,
                     slots);
 }
+// FP64 items per SM up to which a block of the symmetric kernel has two step
+// groups (four up to one item per SM): 312 items (1,500 atoms) E + grad 68 -> 53
+// us, 544 (2,000 atoms) 91 -> 82 us; beyond, the ordinary blocks already fill
+// the SMs.
+constexpr int KG2_ITEMS_PER_SM = 4;
+
 // The FP64 list: chunks of several j-tiles, or, for a batch with fewer tile
 // pairs than wanted items, parts of 64 or 32 j-atoms: the resident blocks take
 // ceil(items / blocks) rounds of equal items, so the fewest rounds in units of
@@ -273,6 +279,9 @@ static void build_list64(ffmin_system *sys, int dens, std::vector<Item> &items, 
         for (int s = 2; s <= 4; s *= 2)
             if (rounds(s) < 0.92 * rounds(split)) split = s;
     }
+    // more warps per item while the items leave SMs idle
+    const int64_t n = pairs * split;
+    sys->c.kg64 = split == 4 && n <= sys->sms ? 4 : (split >= 2 && n <= KG2_ITEMS_PER_SM * sys->sms ? 2 : 1);
     build_items_sym(sys, chunk, split, true, &Tile::r64, items, sys_items, slots);
 }
 

@@ -173,6 +173,7 @@ struct Ctx {
     int32_t n_sys, n_tiles, n_items, n_atoms;
     int64_t vstride;
     int32_t prec;           // ffmin_precision
+    int32_t kg64;           // FP64 symmetric kernel: step groups per block (1, 2 or 4; host-side dispatch)
     int32_t f32_ipt;        // FP32 pair-kernel shape: i-atoms per thread (1 or 2; host-side dispatch)
     const Tile *tiles;
     const Item *items;

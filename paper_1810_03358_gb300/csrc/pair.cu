@@ -693,20 +693,30 @@ __device__ __noinline__ void terms64_plain(double dx, double dy, double dz, doub
     o[3] = ri2;
 }
 
-__global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx c) {
+// KG > 1, for objects with fewer items than SMs (split >= KG): KG times the
+// warps, group g of four takes the steps k = g mod KG, and the groups' i-side
+// sums are added in order.  A lone warp needs about 2,500 cycles for a step (430
+// dependent instructions), 500 atoms kept every warp busy for 32 of them:
+// E + grad 45 -> 34 us with their queue.
+template <int KG>
+__global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (KG == 2 ? 2 : 1)) k_pair64_sym(Ctx c) {
     // staged j-atoms: x, y | z, then q', c6, c12 as significands with their
     // exponents and the charge's sign (forces), or as they are (energy only)
     __shared__ ulonglong2 s_xy[TJ], s_zq[TJ], s_c[TJ];
     __shared__ int2 s_e[TJ];
-    __shared__ double jfx[NT_SYM / 32][TJ], jfy[NT_SYM / 32][TJ], jfz[NT_SYM / 32][TJ];
+    // opposite forces, [warp][j of the part]: 4 KG warps, at most TJ / KG j-atoms
+    __shared__ double jfx[4 * TJ], jfy[4 * TJ], jfz[4 * TJ];
+    __shared__ double4_32a s_i[KG > 1 ? KG : 1][KG > 1 ? TI : 1];
     __shared__ int s_item;
     const int32_t *A = c.act + 1 * (2 * c.n_sys + 2);
     const int n_act = A[0], total = A[1];
     if (total == 0) return;
     const int32_t *aoff = A + 2, *asys = A + 2 + c.n_sys;
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    // i-atom, its warp among four, step group
+    const int tid = threadIdx.x % NT_SYM, lane = tid & 31, w = tid >> 5, kg = threadIdx.x / NT_SYM;
+    const int load = threadIdx.x;  // j-atom staged by this thread
     for (;;) {
-        if (tid == 0) {
+        if (threadIdx.x == 0) {
             const int q = (int)atomicAdd(&c.counters[CNT_PAIR64], 1u);
             if (q < total) {  // last active system whose first item is <= q
                 int lo = 0, hi = n_act - 1;
@@ -762,15 +772,16 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
         double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
         double sc1 = 0.0, s6 = 0.0, s12 = 0.0;  // energy-only factored sums
         const int jend = I.j0 + I.nj;
+        double *fx = jfx + (kg * 4 + w) * W, *fy = jfy + (kg * 4 + w) * W, *fz = jfz + (kg * 4 + w) * W;
         for (int jt = I.j0; jt < jend; jt += TJ) {
-            const int jl = jt + tid;
+            const int jl = jt + load;
             double4_32a pj = make_double4_32a(1e6, 1e6, 1e6, 0.0);
             double2 cj0 = make_double2(0.0, 0.0);
             long long xj = FIX_FAR, yj = FIX_FAR, zj = FIX_FAR;
             u64 m1 = 0, m6 = 0, m12 = 0;
             int e1 = P64_ZERO, e6 = P64_ZERO, e12 = P64_ZERO;
             bool j_range = in_range, j_fix = i_fix;
-            if (tid < W && jl < jend) {
+            if (load < W && jl < jend) {
                 pj = c.posd[jl];
                 cj0 = c.pard[jl];
                 j_range = split64(pj.w, m1, e1) && j_range;
@@ -784,17 +795,16 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             // the integer forms of the terms when every parameter is in range
             const bool fix = __syncthreads_and(j_fix && j_range);
             const bool plain = fix ? false : __syncthreads_or(!j_range);
-            if (tid < W) {
-                s_xy[tid] = fix ? make_ulonglong2((u64)xj, (u64)yj) : make_ulonglong2(bits64(pj.x), bits64(pj.y));
-                s_zq[tid] = make_ulonglong2(fix ? (u64)zj : bits64(pj.z), grad ? m1 : bits64(pj.w));
-                s_c[tid] = grad ? make_ulonglong2(m6, m12) : make_ulonglong2(bits64(cj0.x), bits64(cj0.y));
+            if (load < W) {
+                s_xy[load] = fix ? make_ulonglong2((u64)xj, (u64)yj) : make_ulonglong2(bits64(pj.x), bits64(pj.y));
+                s_zq[load] = make_ulonglong2(fix ? (u64)zj : bits64(pj.z), grad ? m1 : bits64(pj.w));
+                s_c[load] = grad ? make_ulonglong2(m6, m12) : make_ulonglong2(bits64(cj0.x), bits64(cj0.y));
                 if (grad)
-                    s_e[tid] = make_int2((int)((uint32_t)e1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
+                    s_e[load] = make_int2((int)((uint32_t)e1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
                                          (e6 << 16) | e12);
             }
             if (grad) {
-#pragma unroll
-                for (int q = lane; q < TJ; q += 32) { jfx[w][q] = 0.0; jfy[w][q] = 0.0; jfz[w][q] = 0.0; }
+                for (int q = lane; q < W; q += 32) { fx[q] = 0.0; fy[q] = 0.0; fz[q] = 0.0; }
             }
             __syncthreads();
             // the diagonal tile (j-tile == i-tile): whole, thread t pairs with
@@ -813,7 +823,7 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             auto energies = [&](auto FIX) {
                 // energy only: the i atom's factors leave the sums,
                 // E_i = q'_i sum q'_j / r + (c12_i sum c12_j r^-12 - c6_i sum c6_j r^-6) / 6
-                for (int k = k0; k <= k1; k++) {
+                for (int k = k0 + kg; k <= k1; k += KG) {
                     const int j = (tid + k) & (W - 1);
                     const ulonglong2 xy = s_xy[j], zq = s_zq[j], cj = s_c[j];
                     const bool on = !mask || I.joff + j > tid;
@@ -846,7 +856,7 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
                 }
             };
             auto forces = [&](auto FIX) {
-                for (int k = k0; k <= k1; k++) {
+                for (int k = k0 + kg; k <= k1; k += KG) {
                     const int j = (tid + k) & (W - 1);
                     const ulonglong2 xy = s_xy[j], zq = s_zq[j], cj = s_c[j];
                     const int2 ej = s_e[j];
@@ -896,9 +906,9 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
                     gx = fma(f, dx, gx);
                     gy = fma(f, dy, gy);
                     gz = fma(f, dz, gz);
-                    jfx[w][j] = fma(-f, dx, jfx[w][j]);
-                    jfy[w][j] = fma(-f, dy, jfy[w][j]);
-                    jfz[w][j] = fma(-f, dz, jfz[w][j]);
+                    fx[j] = fma(-f, dx, fx[j]);
+                    fy[j] = fma(-f, dy, fy[j]);
+                    fz[j] = fma(-f, dz, fz[j]);
                     __syncwarp();
                 }
             };
@@ -911,19 +921,30 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             else forces(std::false_type{});
             __syncthreads();
             // j-side partial row of this j-tile, warps summed in order
-            if (tid < W && jl < jend) {
+            if (load < W && jl < jend) {
                 double4_32a o;
-                o.x = jfx[0][tid]; o.y = jfy[0][tid]; o.z = jfz[0][tid];
+                o.x = jfx[load]; o.y = jfy[load]; o.z = jfz[load];
 #pragma unroll
-                for (int v = 1; v < NT_SYM / 32; v++) { o.x += jfx[v][tid]; o.y += jfy[v][tid]; o.z += jfz[v][tid]; }
+                for (int v = 1; v < 4 * KG; v++) { o.x += jfx[v * W + load]; o.y += jfy[v * W + load]; o.z += jfz[v * W + load]; }
                 o.w = 0.0;
-                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + I.joff + tid] = o;
+                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + I.joff + load] = o;
             }
         }
         double4_32a o;
         o.x = gx; o.y = gy; o.z = gz;
         o.w = grad ? ec + lj * (1.0 / 6.0) : pi.w * sc1 + (ci.y * s12 - ci.x * s6) * (1.0 / 6.0);
-        c.gpd[(int64_t)I.slot * TI + tid] = o;
+        if constexpr (KG > 1) {
+            s_i[kg][tid] = o;
+            __syncthreads();
+            if (kg == 0) {
+#pragma unroll
+                for (int v = 1; v < KG; v++) {
+                    const double4_32a q = s_i[v][tid];
+                    o.x += q.x; o.y += q.y; o.z += q.z; o.w += q.w;
+                }
+            }
+        }
+        if (kg == 0) c.gpd[(int64_t)I.slot * TI + tid] = o;
     }
 }
 
@@ -944,7 +965,7 @@ int pair_grid_size(int mode, int f32_ipt) {
     else if (mode == 1)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, K_F64, NT_F64, 0);
     else if (mode == 2)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair64_sym, NT_SYM, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair64_sym<1>, NT_SYM, 0);
     else if (one)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<float, TI, 1, false, true>, TI, 0);
     else
@@ -968,7 +989,9 @@ static void launch_f32_shape(const Ctx &c, bool eonly, int grid, cudaStream_t s)
 
 cudaError_t launch_pair_list(const Ctx &c, int list, int grid, cudaStream_t s) {
     if (list == LIST_F64) {
-        if (c.sym64) k_pair64_sym<<<grid, NT_SYM, 0, s>>>(c);
+        if (c.sym64 && c.kg64 == 4) k_pair64_sym<4><<<grid, NT_SYM * 4, 0, s>>>(c);
+        else if (c.sym64 && c.kg64 == 2) k_pair64_sym<2><<<grid, NT_SYM * 2, 0, s>>>(c);
+        else if (c.sym64) k_pair64_sym<1><<<grid, NT_SYM, 0, s>>>(c);
         else K_F64<<<grid, NT_F64, 0, s>>>(c);
     } else if (c.f32_ipt == 1) {
         launch_f32_shape<1>(c, list == LIST_F32_E, grid, s);
