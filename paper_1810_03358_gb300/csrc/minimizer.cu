@@ -1,5 +1,5 @@
 // Per-tile kernels of the minimizer pipeline (one 128-thread block per
-// 128-atom tile, one thread per atom) and the bonded terms.
+// 128-atom tile, one thread per atom; finalize: a cluster of four blocks).
 //
 //   prepare   trial point XT = base + h * dir * scale (FP64, fused multiply-add
 //             per component) and the pair-kernel positions (float4/double4_32a)
@@ -17,7 +17,10 @@
 // This file is compiled without contraction of a*b+c into FMA so that the
 // scalar control arithmetic and the vector updates round like their
 // textbook statements; fused multiply-adds appear only where written.
+#include <cooperative_groups.h>
+
 #include <cmath>
+#include <utility>
 
 #include "activelist.cuh"
 #include "bonded.cuh"
@@ -26,6 +29,8 @@
 #include "reduce.cuh"
 
 namespace ffm {
+
+namespace cg = cooperative_groups;
 
 // <a, b> of two 3-vectors with explicit FMA (this unit is compiled without
 // implicit contraction; the vector kernels are FP64-pipe bound)
@@ -108,15 +113,22 @@ cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) 
 }
 
 // ---------------------------------------------------------------- finalize
-// Bound: latency and the FP64 pipe (16 cycles per warp operation and SM).
-// One block per tile, four threads per atom: strand s of an atom sums its
-// partial rows s, s + 4, ..., the strands are combined through shared memory
-// as (0 + 1) + (2 + 3).  One thread per atom took 25 us for 500 atoms and 31 us
-// for 3,334 (cold caches).  The sums keep one order in every version of this
-// kernel (strands, then the columns of block_reduce_columns, then the tiles):
-// a MIXED minimization amplifies any other rounding.
+// Bound: latency (a chain of about ten loads, barriers and short FP64 sums; an
+// FP64 operation holds a quarter of an SM for 64 cycles however few of its
+// lanes are on).  A tile is a cluster of four blocks, 32 atoms each: warp w < 4
+// sums the atoms' partial rows w, w + 4, ... (strand w; combined as
+// (0 + 1) + (2 + 3)), warps 4 and 5 gather their bonded terms, then one warp
+// finishes each component; the first block receives the atoms' contributions
+// in its shared memory, forms the tile's sums and, in the system's last tile,
+// the control step.  One block of 512 threads a tile took 16.2 us for 500 atoms
+// and 22 us for 3,334 (FP64), half of them with one SM's FP64 pipe saturated and
+// a sixth in fences executed by every warp; now 12.4 and 14.6 us.  The sums keep one
+// order in every version of this kernel (strands, then the columns of
+// block_reduce_columns, then the tiles): a MIXED minimization amplifies any
+// other rounding.
 constexpr int FIN_STRANDS = 4;
-constexpr int FIN_NT = TI * FIN_STRANDS;
+constexpr int FIN_CLUSTER = TI / 32;
+constexpr int FIN_NT = 32 * (FIN_STRANDS + 2);
 
 // exact FP32 -> FP64 on the integer pipe (the conversion instruction runs at
 // the FP64 rate); the FP32 kernels flush denormals, which read as zero
@@ -174,140 +186,194 @@ __device__ __forceinline__ void sym_rows(const Ctx &c, const Tile &t, int tile0,
     });
 }
 
-__global__ void __launch_bounds__(FIN_NT, 2) k_finalize(Ctx c, double *g_out) {
-    const Tile &t = c.tiles[blockIdx.x];
+// the control step's value for each of finalize's sums
+__device__ __forceinline__ int fin_value(int k) {
+    return k == 0 ? RF_E : (k == 1 ? RF_EPAIR : (k == 2 ? RF_GG : (k == 3 ? RF_GTG : RF_GTR)));
+}
+
+__global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
+    const int tile = blockIdx.x / FIN_CLUSTER, rank = blockIdx.x % FIN_CLUSTER;
+    const Tile &t = c.tiles[tile];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;  // w: strand, then bonded terms
+    const int i = 32 * rank + lane, a = t.a0 + i;
+    const bool real = i < t.na;
+    constexpr int NSUM = 5;  // E, Epair and, with a gradient, g.g, g.G, g.R
+    __shared__ double part[FIN_STRANDS][4][32], bond[2][4][32];
+    __shared__ double sg[3 * 32], sr[3 * 32], sgt[3][32];  // current gradient, direction, new gradient
+    // first block of the cluster: the tile's contributions
+    __shared__ double val[NSUM][TI];
+    __shared__ unsigned long long gmax[3 * FIN_CLUSTER];
+    __shared__ int badf[4 * FIN_CLUSTER];
+    __shared__ double strands[NSUM][RSTRANDS], tot[RF_N];
+    __shared__ SysState sS;
+    cg::cluster_group cl = cg::this_cluster();
+    // bonded terms: the even entries of an atom's incidence list in warp 4,
+    // the odd ones in warp 5
+    constexpr int U = 5;  // an atom in a chain has 9 or 10 entries
+    int k1 = 0, kb = 0;
+    if (real && w >= FIN_STRANDS) {
+        k1 = c.inc_off[a + 1];
+        kb = c.inc_off[a] + w - FIN_STRANDS;
+    }
     const SysState &S = c.st[t.sys];
-    const int kind = S.ev_kind, mode = S.mode;
-    const int i = threadIdx.x % TI, w = threadIdx.x / TI;  // atom, strand
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ Row4 part[FIN_STRANDS][TI];
-    __shared__ Row4 bond[TI];
-    __shared__ double val[RF_N][TI + 1];
-    __shared__ double strands[RF_N][RSTRANDS];
-    const unsigned maxmask = (1u << RF_GINF) | (1u << RF_BAD);
-    if (kind == EV_NONE) return;
-    {
-        const bool real = i < t.na, grad = kind == EV_EG;
-        const int a = t.a0 + i;
-        Row4 r = Row4{0.0, 0.0, 0.0, 0.0}, bo = r;
+    const int kind = S.ev_kind, mode = S.mode, ntile = S.ntile, tile0 = S.tile0;
+    if (kind == EV_NONE) return;  // the whole cluster
+    auto started = cl.barrier_arrive();
+    const bool grad = kind == EV_EG;
+    if (rank == 0) prefetch_state(&sS, &S);
+    if (grad) {
+        const int64_t o = 3 * ((int64_t)t.a0 + 32 * rank);
+        const int n = 3 * min(32, max(0, t.na - 32 * rank));
+        for (int k = threadIdx.x; k < n; k += FIN_NT) {
+            async_copy8(&sg[k], vslot(c, V_G) + o + k);
+            async_copy8(&sr[k], vslot(c, V_R) + o + k);
+        }
+    }
+    if (w < FIN_STRANDS) {
+        Row4 r = Row4{0.0, 0.0, 0.0, 0.0};
         if (real) {
             if (mode == 0 && c.sym32 && !grad) {
                 // energies on the symmetric list, each pair counted once
                 const int C = t.r32.chunk;
-                strand_sum<false, true>((S.ntile - t.tloc + C - 1) / C, w, r, [&](int q) {
+                strand_sum<false, true>((ntile - t.tloc + C - 1) / C, w, r, [&](int q) {
                     return Row4{0.0, 0.0, 0.0, widen(c.gpf_sym[((int64_t)t.r32.slot + q) * TI + i])};
                 });
             } else if (mode == 0) {
                 strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpf, t.item0 + it, i); });
                 r.w *= 0.5;  // every pair was counted in both of its rows
             } else if (c.sym64) {
-                if (grad) sym_rows<true>(c, t, S.tile0, S.ntile, i, w, r);
-                else sym_rows<false>(c, t, S.tile0, S.ntile, i, w, r);
+                if (grad) sym_rows<true>(c, t, tile0, ntile, i, w, r);
+                else sym_rows<false>(c, t, tile0, ntile, i, w, r);
             } else {
                 strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpd, t.item0 + it, i); });
                 r.w *= 0.5;
             }
-            // bonded terms: evaluated once per term by the pair kernel's
-            // bonded items; every atom gathers its terms' energies (as owner)
-            // and position gradients through its incidence list, the even
-            // entries in strand 2, the odd ones in strand 3
-            if (w >= 2) {
-                constexpr int U = 5;  // an atom in a chain has 9 or 10 entries
-                const int k1 = c.inc_off[a + 1];
-                for (int k = c.inc_off[a] + w - 2; k < k1; k += 2 * U) {
-                    int2 in[U];
-                    Row4 p[U];
-#pragma unroll
-                    for (int u = 0; u < U; u++) in[u] = k + 2 * u < k1 ? c.inc[k + 2 * u] : make_int2(-1, 0);
-#pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        const int type = in[u].x >> 2, pos = in[u].x & 3;
-                        if (in[u].x < 0) continue;
-                        p[u].w = pos == 0 ? c.te[bonded_index(c, type, in[u].y)] : 0.0;
-                        if (grad) {
-                            const double *g = c.tg + 3 * bonded_grad_slot(c, type, in[u].y, pos);
-                            p[u].x = g[0]; p[u].y = g[1]; p[u].z = g[2];
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        if (in[u].x < 0) break;
-                        if ((in[u].x & 3) == 0) bo.w += p[u].w;
-                        if (grad) { bo.x += p[u].x; bo.y += p[u].y; bo.z += p[u].z; }
-                    }
-                }
-            }
         }
-        part[w][i] = r;
-        if (w == 3) bond[i] = bo;
-        __syncthreads();
-        if (w == 2) {  // the whole atom
-            double v[RF_N];
+        part[w][0][lane] = r.x; part[w][1][lane] = r.y; part[w][2][lane] = r.z; part[w][3][lane] = r.w;
+    } else {
+        // evaluated once per term by the pair kernel's bonded items; an atom
+        // takes its terms' energies (as owner) and position gradients
+        Row4 bo = Row4{0.0, 0.0, 0.0, 0.0};
+        for (; kb < k1; kb += 2 * U) {
+            int2 in[U];
+            Row4 p[U];
 #pragma unroll
-            for (int k = 0; k < RF_N; k++) v[k] = 0.0;
-            if (real) {
-                const Row4 r0 = part[0][i], r1 = part[1][i], r3 = part[3][i], b1 = bond[i];
-                const double ep = (r0.w + r1.w) + (r.w + r3.w);
-                const double e = ep + (bo.w + b1.w);
-                v[RF_EPAIR] = ep;
-                v[RF_E] = e;
-                bool bad = !isfinite(e);
+            for (int u = 0; u < U; u++) in[u] = kb + 2 * u < k1 ? c.inc[kb + 2 * u] : make_int2(-1, 0);
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int type = in[u].x >> 2, pos = in[u].x & 3;
+                if (in[u].x < 0) continue;
+                p[u].w = pos == 0 ? c.te[bonded_index(c, type, in[u].y)] : 0.0;
                 if (grad) {
-                    const double g0 = ((r0.x + r1.x) + (r.x + r3.x)) + (bo.x + b1.x);
-                    const double g1 = ((r0.y + r1.y) + (r.y + r3.y)) + (bo.y + b1.y);
-                    const double g2 = ((r0.z + r1.z) + (r.z + r3.z)) + (bo.z + b1.z);
-                    double *gt = vslot(c, V_GT) + 3 * a;
-                    gt[0] = g0; gt[1] = g1; gt[2] = g2;
-                    if (g_out) { g_out[3 * a] = g0; g_out[3 * a + 1] = g1; g_out[3 * a + 2] = g2; }
-                    const double *G = vslot(c, V_G) + 3 * a;
-                    const double *R = vslot(c, V_R) + 3 * a;
-                    v[RF_GG] = fma(g0, g0, fma(g1, g1, g2 * g2));
-                    v[RF_GINF] = fmax(fabs(g0), fmax(fabs(g1), fabs(g2)));
-                    v[RF_GTG] = fma(g0, G[0], fma(g1, G[1], g2 * G[2]));
-                    v[RF_GTR] = fma(g0, R[0], fma(g1, R[1], g2 * R[2]));
-                    bad = bad || !isfinite(g0) || !isfinite(g1) || !isfinite(g2);
+                    const double *g = c.tg + 3 * bonded_grad_slot(c, type, in[u].y, pos);
+                    p[u].x = g[0]; p[u].y = g[1]; p[u].z = g[2];
                 }
-                v[RF_BAD] = bad ? 1.0 : 0.0;
             }
 #pragma unroll
-            for (int k = 0; k < RF_N; k++) val[k][i] = v[k];
+            for (int u = 0; u < U; u++) {
+                if (in[u].x < 0) break;
+                if ((in[u].x & 3) == 0) bo.w += p[u].w;
+                if (grad) { bo.x += p[u].x; bo.y += p[u].y; bo.z += p[u].z; }
+            }
         }
-        __syncthreads();
-        // the tile's sums, in the order of block_reduce_columns
-        if (threadIdx.x < RF_N * RSTRANDS) {
-            const int k = threadIdx.x / RSTRANDS, s = threadIdx.x % RSTRANDS;
-            const bool mx = (maxmask >> k) & 1u;
-            double x = val[k][s];
-#pragma unroll
-            for (int u = s + RSTRANDS; u < TI; u += RSTRANDS) x = mx ? fmax(x, val[k][u]) : x + val[k][u];
-            strands[k][s] = x;
+        double (*b)[32] = bond[w - FIN_STRANDS];
+        b[0][lane] = bo.x; b[1][lane] = bo.y; b[2][lane] = bo.z; b[3][lane] = bo.w;
+    }
+    async_wait();
+    __syncthreads();
+    cl.barrier_wait(std::move(started));  // the first block's shared memory is there
+    double *tv = cl.map_shared_rank(&val[0][0], 0) + i;
+    auto finite = [](double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; };
+    if (w < 4 && (grad || w == 3)) {  // component w of the gradient, or the energy
+        double x = 0.0, q = 0.0;
+        if (real) {
+            q = (part[0][w][lane] + part[1][w][lane]) + (part[2][w][lane] + part[3][w][lane]);
+            x = q + (bond[0][w][lane] + bond[1][w][lane]);
         }
-        __syncthreads();
-        if (threadIdx.x < RF_N) {
-            const int k = threadIdx.x;
-            const bool mx = (maxmask >> k) & 1u;
-            double x = strands[k][0];
-#pragma unroll
-            for (int s = 1; s < RSTRANDS; s++) x = mx ? fmax(x, strands[k][s]) : x + strands[k][s];
-            c.redf[(int64_t)k * c.n_tiles + blockIdx.x] = x;
+        const unsigned bad = __ballot_sync(0xffffffffu, !finite(x));
+        if (lane == 0) cl.map_shared_rank(badf, 0)[4 * rank + w] = bad != 0u;
+        if (w == 3) {
+            tv[0] = x;
+            tv[TI] = q;
+        } else {
+            sgt[w][lane] = x;
+            if (real) {
+                vslot(c, V_GT)[3 * (int64_t)a + w] = x;
+                if (g_out) g_out[3 * (int64_t)a + w] = x;
+            }
+            // the largest |component|, as an integer (a NaN counts as 0)
+            const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+            const bool nan = hi > 0x7ff00000u || (hi == 0x7ff00000u && lo != 0u);
+            const unsigned mh = __reduce_max_sync(0xffffffffu, nan ? 0u : hi);
+            const unsigned ml = __reduce_max_sync(0xffffffffu, !nan && hi == mh ? lo : 0u);
+            if (lane == 0) cl.map_shared_rank(gmax, 0)[3 * rank + w] = (unsigned long long)mh << 32 | ml;
         }
     }
-    if (!sys_last_block(&c.tickets[STAGE_FIN * c.n_sys + t.sys], S.ntile)) return;
-    __shared__ double tot[RF_N];
-    __shared__ SysState sS;
-    const int t0 = S.tile0, t1 = S.tile0 + S.ntile;
-    const double *r = c.redf;
-    static_assert(RF_GG == RF_E + 1 && RF_GTR == RF_GTG + 1, "summed in pairs");
-    if (warp == 0) {
-        warp_sums8(r, c.n_tiles, 1, t0, t1, 2, &tot[RF_E]);
-    } else if (warp == 1) {
-        warp_sums8(r + (int64_t)RF_GTG * c.n_tiles, c.n_tiles, 1, t0, t1, 2, &tot[RF_GTG]);
-    } else if (warp == 2) {
-        warp_sums8(r + (int64_t)RF_EPAIR * c.n_tiles, c.n_tiles, 1, t0, t1, 1, &tot[RF_EPAIR]);
-    } else if (warp == 3) {
-        warp_max(r + (int64_t)RF_GINF * c.n_tiles, 1, t0, t1, &tot[RF_GINF]);
-    } else if (warp == 4) {
-        warp_max(r + (int64_t)RF_BAD * c.n_tiles, 1, t0, t1, &tot[RF_BAD]);
+    if (grad) {
+        __syncthreads();
+        if (w < 3) {
+            double x = 0.0;
+            if (real) {
+                const double g0 = sgt[0][lane], g1 = sgt[1][lane], g2 = sgt[2][lane];
+                const double *o = w == 1 ? sg : sr;
+                const double o0 = w == 0 ? g0 : o[3 * lane], o1 = w == 0 ? g1 : o[3 * lane + 1],
+                             o2 = w == 0 ? g2 : o[3 * lane + 2];
+                x = fma(g0, o0, fma(g1, o1, g2 * o2));
+            }
+            tv[(2 + w) * TI] = x;
+        }
+    }
+    cl.sync();
+    if (rank != 0) return;
+    // the tile's sums, in the order of block_reduce_columns: values 0 to 3 in
+    // warp 0, value 4 in warp 1
+    const int nsum = grad ? NSUM : 2;
+    if (w < 2) {
+        const int k = 4 * w + lane / RSTRANDS, s = lane % RSTRANDS;
+        if (k < nsum) {
+            double x = val[k][s];
+#pragma unroll
+            for (int u = s + RSTRANDS; u < TI; u += RSTRANDS) x += val[k][u];
+            strands[k][s] = x;
+        }
+        __syncwarp();
+        const int k1v = 4 * w + lane;
+        if (lane < 4 && k1v < NSUM) {
+            double x = 0.0;
+            if (k1v < nsum) {
+                x = strands[k1v][0];
+#pragma unroll
+                for (int q = 1; q < RSTRANDS; q++) x += strands[k1v][q];
+            }
+            c.redf[(int64_t)k1v * c.n_tiles + tile] = x;
+            tot[fin_value(k1v)] = 0.0 + x;  // of a system of one tile
+        }
+    } else if (w == 2) {
+        unsigned long long m = grad && lane < 3 * FIN_CLUSTER ? gmax[lane] : 0ULL;
+        const bool bad = lane < 4 * FIN_CLUSTER && (grad || (lane & 3) == 3) && badf[lane];
+        const unsigned any_bad = __ballot_sync(0xffffffffu, bad);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(0xffffffffu, m, o);
+            m = y > m ? y : m;
+        }
+        if (lane == 0) {
+            const double gi = __longlong_as_double((long long)m), fb = any_bad ? 1.0 : 0.0;
+            c.redf[(int64_t)5 * c.n_tiles + tile] = gi;
+            c.redf[(int64_t)6 * c.n_tiles + tile] = fb;
+            tot[RF_GINF] = gi;
+            tot[RF_BAD] = fb;
+        }
+    }
+    if (ntile > 1) {
+        if (!sys_last_block(&c.tickets[STAGE_FIN * c.n_sys + t.sys], ntile)) return;
+        const double *rd = c.redf + (int64_t)w * c.n_tiles;
+        if (w < NSUM) {
+            warp_sum1(rd, tile0, tile0 + ntile, &tot[fin_value(w)]);
+        } else {
+            warp_max(rd, tile0, tile0 + ntile, &tot[RF_GINF]);
+            warp_max(rd + c.n_tiles, tile0, tile0 + ntile, &tot[RF_BAD]);
+        }
     }
     __syncthreads();
     sys_control(c, t.sys, sS, [&](SysState &W) {
@@ -321,7 +387,9 @@ __global__ void __launch_bounds__(TI) k_update(Ctx c) {
     const SysState &S = c.st[t.sys];
     const int op = S.upd.op;
     const int i = threadIdx.x;
+    __shared__ SysState sS;
     if (op == U_NONE) return;
+    prefetch_state(&sS, &c.st[t.sys]);
     if (op == U_PUSH) {
         double v[RU_N];
 #pragma unroll
@@ -444,9 +512,9 @@ __global__ void __launch_bounds__(TI) k_update(Ctx c) {
             break;
         }
     }
+    async_wait();
     if (!sys_last_block(&c.tickets[STAGE_UPD * c.n_sys + t.sys], S.ntile)) return;
     __shared__ double tot[RU_N];
-    __shared__ SysState sS;
     sys_sums(c, S, op == U_PUSH ? ru_count(S.upd.nS) : (op == U_OGM ? 1 : 0), tot);
     sys_control(c, t.sys, sS, [&](SysState &W) { warp_update_done(c, W, tot); });
 }
@@ -461,7 +529,9 @@ __global__ void __launch_bounds__(TI) k_dir(Ctx c) {
     double v[NRING];
 #pragma unroll
     for (int k = 0; k < NRING; k++) v[k] = 0.0;
+    __shared__ SysState sS;
     if (!d.on) return;
+    prefetch_state(&sS, &c.st[t.sys]);
     __shared__ float w_mlp[MLP_NW];
     if (d.use_d) {  // learned H0 diagonal: FP16 weights -> FP32 in shared memory
         for (int k = threadIdx.x; k < MLP_NW; k += blockDim.x)
@@ -516,9 +586,9 @@ __global__ void __launch_bounds__(TI) k_dir(Ctx c) {
     }
     const int nv = d.dots == 2 ? d.nY : 2;
     block_reduce_columns<NRING>(v, nv, 0u, &c.red[(int64_t)blockIdx.x * NRED]);
+    async_wait();
     if (!sys_last_block(&c.tickets[(WHICH == 0 ? STAGE_DIR1 : STAGE_DIR2) * c.n_sys + t.sys], S.ntile)) return;
     __shared__ double tot[NRING + 1];
-    __shared__ SysState sS;
     sys_sums(c, S, nv, tot);
     sys_control(c, t.sys, sS, [&](SysState &W) { warp_dir_done(c, W, WHICH, tot); });
 }
@@ -599,7 +669,7 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out) {
-    k_finalize<<<c.n_tiles, FIN_NT, 0, s>>>(c, g_out);
+    k_finalize<<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
     return cudaGetLastError();
 }
 cudaError_t launch_update(const Ctx &c, cudaStream_t s) {

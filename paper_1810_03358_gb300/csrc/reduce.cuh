@@ -43,9 +43,9 @@ __device__ inline bool last_block(unsigned int *cnt) {
         __threadfence();
         const unsigned t = atomicAdd(cnt, 1u);
         am_last = (t == gridDim.x - 1);
+        if (am_last) __threadfence();
     }
     __syncthreads();
-    if (am_last) __threadfence();
     return am_last != 0;
 }
 
@@ -91,17 +91,21 @@ __device__ inline void block_reduce_columns(const double (&v)[NV], int nv, unsig
 }
 
 // ticket of a block among its system's: true in the last one, which then may
-// read what the others stored
+// read what the others stored (the thread with the ticket fences for the
+// block, the barrier passes it on: a fence in all of 16 warps took 5,000
+// cycles, during which the shuffles behind it waited)
 __device__ inline bool sys_last_block(unsigned int *cnt, int ntile) {
     __shared__ int am_last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         am_last = atomicAdd(cnt, 1u) == (unsigned)ntile - 1u;
-        if (am_last) *cnt = 0u;  // for the next launch
+        if (am_last) {
+            *cnt = 0u;  // for the next launch
+            __threadfence();
+        }
     }
     __syncthreads();
-    if (am_last) __threadfence();
     return am_last != 0;
 }
 
@@ -137,14 +141,36 @@ __device__ inline void warp_sums8(const double *r, int64_t vs, int64_t ts, int t
     x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
     if ((lane & 3) == 0 && (lane >> 2) < nv) out[lane >> 2] = x[0];
 }
-// largest value over a system's tiles by a warp
-__device__ inline void warp_max(const double *r, int64_t ts, int t0, int t1, double *out) {
+// the same for one value at r[t]
+__device__ inline void warp_sum1(const double *r, int t0, int t1, double *out) {
     const int lane = threadIdx.x & 31;
     double x = 0.0;
-    for (int t = t0 + lane; t < t1; t += 32) x = fmax(x, __ldcg(&r[t * ts]));
+    for (int t = t0 + lane; t < t1; t += 8 * 32) {
+        double y[8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+        for (int k = 0; k < 8; k++) y[k] = t + 32 * k < t1 ? __ldcg(&r[t + 32 * k]) : 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            if (t + 32 * k < t1) x += y[k];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     if (lane == 0) *out = x;
+}
+// largest of non-negative values (no NaN) over a system's tiles by a warp, as integers
+__device__ inline void warp_max(const double *r, int t0, int t1, double *out) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long x = 0ULL;
+    for (int t = t0 + lane; t < t1; t += 32) {
+        const unsigned long long y = (unsigned long long)__double_as_longlong(__ldcg(&r[t]));
+        x = y > x ? y : x;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = y > x ? y : x;
+    }
+    if (lane == 0) *out = __longlong_as_double((long long)x);
 }
 // the first nv reduction values of a per-tile kernel (c.red), by the block
 __device__ inline void sys_sums(const Ctx &c, const SysState &S, int nv, double *out) {
@@ -153,27 +179,32 @@ __device__ inline void sys_sums(const Ctx &c, const SysState &S, int nv, double 
     __syncthreads();
 }
 
-// A system's control state copied by a warp (8-byte words, coalesced), so
-// that the control step, a long chain of dependent reads and writes of the
-// state, runs on a shared-memory copy instead of global memory
-__device__ inline void warp_copy_state(SysState *dst, const SysState *src) {
-    static_assert(sizeof(SysState) % 8 == 0, "SysState is copied in 8-byte words");
-    const unsigned long long *s = reinterpret_cast<const unsigned long long *>(src);
-    unsigned long long *d = reinterpret_cast<unsigned long long *>(dst);
-#pragma unroll 8
-    for (int k = threadIdx.x & 31; k < (int)(sizeof(SysState) / 8); k += 32) d[k] = s[k];
-    __syncwarp();
+// A system's control state on its way to shared memory from the start of the
+// kernel (asynchronous copies by the whole block), so that the control step, a
+// long chain of dependent reads and writes of the state, runs on a copy that
+// is there when the last block gets to it.  async_wait, then a barrier, before
+// the first use.
+static_assert(sizeof(SysState) % 8 == 0, "SysState is copied in 8-byte words");
+__device__ inline void async_copy8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ inline void async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ inline void prefetch_state(SysState *dst, const SysState *src) {
+    for (int k = threadIdx.x; k < (int)(sizeof(SysState) / 8); k += blockDim.x)
+        async_copy8(reinterpret_cast<unsigned long long *>(dst) + k, reinterpret_cast<const unsigned long long *>(src) + k);
 }
 
-// control step of system b by warp 0 on the copy sS: fn(S) is called by the
-// whole warp
+// control step of system b by warp 0 on the prefetched copy sS: fn(sS) is
+// called by the whole warp
 template <typename Fn>
 __device__ inline void sys_control(const Ctx &c, int b, SysState &sS, Fn fn) {
     if (threadIdx.x >= 32) return;
-    warp_copy_state(&sS, &c.st[b]);
     fn(sS);
     __syncwarp();
-    warp_copy_state(&c.st[b], &sS);
+    const unsigned long long *s = reinterpret_cast<const unsigned long long *>(&sS);
+    unsigned long long *d = reinterpret_cast<unsigned long long *>(&c.st[b]);
+    for (int k = threadIdx.x; k < (int)(sizeof(SysState) / 8); k += 32) d[k] = s[k];
 }
 
 }  // namespace ffm
