@@ -144,6 +144,7 @@ static void bonded_items(const ffmin_system *sys, int b, std::vector<Item> &item
             it.j0 = starts[ty] + k;
             it.nj = std::min(BONDED_ITEM_TERMS, count - k);
             it.diag = b;
+            it.sys = b;
             items.push_back(it);
         }
     }
@@ -185,6 +186,7 @@ static void build_items(ffmin_system *sys, int density, std::vector<Item> &items
             for (int j0 = 0; j0 < n; j0 += L) {
                 Item it{};
                 it.tile = (int)t;
+                it.sys = b;
                 it.j0 = (int)(A + j0);
                 it.nj = std::min(L, n - j0);
                 it.diag = (a0 >= j0 && a0 < j0 + it.nj) ? 1 : 0;
@@ -224,6 +226,7 @@ static void build_items_sym(ffmin_system *sys, int chunk, int split, bool jrows,
                 for (int p = 0; p < split; p++) {
                     Item it{};
                     it.tile = (int)(t0 + I);
+                    it.sys = b;
                     it.joff = p * (TJ / split);
                     it.j0 = jf.a0 + it.joff;
                     it.nj = (split > 1 ? jf.a0 + std::min(jf.na, it.joff + TJ / split) : jl.a0 + jl.na) - it.j0;
@@ -256,11 +259,13 @@ static void build_list32e(ffmin_system *sys, int dens, std::vector<Item> &items,
     build_items_sym(sys, (int)std::max<int64_t>(1, tile_pairs(sys) / want), 1, false, &Tile::r32, items, sys_items,
                     slots);
 }
-// FP64 items per SM up to which a block of the symmetric kernel has two step
-// groups (four up to one item per SM): 312 items (1,500 atoms) E + grad 68 -> 53
-// us, 544 (2,000 atoms) 91 -> 82 us; beyond, the ordinary blocks already fill
-// the SMs.
-constexpr int KG2_ITEMS_PER_SM = 4;
+// FP64 blocks per SM up to which a part of a tile pair is shared by a cluster
+// of two, and of four or eight: the blocks that an SM holds at once are five,
+// a few more in a second wave still gain from the first doubling.  E + grad, us,
+// with 1, 2, 4, 8 blocks a part: 700 atoms (84 parts) -, -, 27, 25; 1,000
+// (144) 42, 35, 33, 39; 1,101 (180) 59, 39, 39, 45; 1,500 (312) 67, 51, 56, -;
+// 2,000 (544) 88, 82, 85, -.
+constexpr int CL64_PAIR_PER_SM = 8, CL64_BLOCKS_PER_SM = 5, CL64_MAX = 8;
 
 // The FP64 list: chunks of several j-tiles, or, for a batch with fewer tile
 // pairs than wanted items, parts of 64 or 32 j-atoms: the resident blocks take
@@ -279,10 +284,15 @@ static void build_list64(ffmin_system *sys, int dens, std::vector<Item> &items, 
         for (int s = 2; s <= 4; s *= 2)
             if (rounds(s) < 0.92 * rounds(split)) split = s;
     }
-    // more warps per item while the items leave SMs idle
-    const int64_t n = pairs * split;
-    sys->c.kg64 = split == 4 && n <= sys->sms ? 4 : (split >= 2 && n <= KG2_ITEMS_PER_SM * sys->sms ? 2 : 1);
     build_items_sym(sys, chunk, split, true, &Tile::r64, items, sys_items, slots);
+    // more blocks per part while the parts leave SMs idle
+    sys->c.cl64 = 1;
+    const int64_t parts = pairs * split;
+    if (split > 1 && 2 * parts <= (int64_t)CL64_PAIR_PER_SM * sys->sms) {
+        int cs = 2;
+        while (2 * cs <= CL64_MAX && 2 * cs * parts <= (int64_t)CL64_BLOCKS_PER_SM * sys->sms) cs *= 2;
+        sys->c.cl64 = cs;
+    }
 }
 
 // a symmetric list whose partial rows (which grow as the square of the atom

@@ -270,10 +270,11 @@ __device__ __forceinline__ int64_t bonded_grad_slot(const Ctx &c, int type, int 
 }
 
 // one bonded work item: every term of [t0, t0 + nt) whose system evaluates
-// in precision `mode`, energies to te[], position gradients to tg[]
-__device__ inline void bonded_item(const Ctx &c, int t0, int nt, int mode) {
+// in precision `mode`, energies to te[], position gradients to tg[]; thread
+// tid of nthreads
+__device__ inline void bonded_item(const Ctx &c, int t0, int nt, int mode, int tid, int nthreads) {
     const double *x = vslot(c, V_XT);
-    for (int t = t0 + threadIdx.x; t < t0 + nt; t += blockDim.x) {
+    for (int t = t0 + tid; t < t0 + nt; t += nthreads) {
         const SysState &S = c.st[c.term_sys[t]];
         if (S.ev_kind == EV_NONE || S.mode != mode) continue;
         int type, term;

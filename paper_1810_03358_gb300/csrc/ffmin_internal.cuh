@@ -66,7 +66,7 @@ enum Phase : int {
 // single j-tile (see SymRow; nj <= 0 for a part beyond a ragged tile).  slot:
 // the item's i-side slot, jslot: the j-side slot of its first j-tile, joff:
 // offset of j0 inside its j-tile.
-struct Item { int32_t tile, j0, nj, diag, slot, jslot, joff, pad; };
+struct Item { int32_t tile, j0, nj, diag, slot, jslot, joff, sys; };
 constexpr int BONDED_ITEM_TERMS = 64;
 
 // Row of a symmetric list: the items of one i-tile, by j.  Every `chunk`
@@ -173,7 +173,7 @@ struct Ctx {
     int32_t n_sys, n_tiles, n_items, n_atoms;
     int64_t vstride;
     int32_t prec;           // ffmin_precision
-    int32_t kg64;           // FP64 symmetric kernel: step groups per block (1, 2 or 4; host-side dispatch)
+    int32_t cl64;           // FP64 symmetric kernel: blocks per item (clusters; host-side dispatch)
     int32_t f32_ipt;        // FP32 pair-kernel shape: i-atoms per thread (1 or 2; host-side dispatch)
     const Tile *tiles;
     const Item *items;

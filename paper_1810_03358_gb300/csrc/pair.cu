@@ -25,6 +25,8 @@
 // the finalize kernel halves it.  The FP32 kernel flushes denormals (none
 // occur for separations above 1e-6 A) and takes r^-1 from the hardware
 // reciprocal square root (rsqrt.approx.ftz.f32).
+#include <cooperative_groups.h>
+
 #include <cstdio>
 #include <type_traits>
 
@@ -34,6 +36,8 @@
 #include "pair64.cuh"
 
 namespace ffm {
+
+namespace cg = cooperative_groups;
 
 __device__ __forceinline__ float rsqrt_approx(float x) {
     float y;
@@ -487,7 +491,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM
         if (it < 0) break;
         const Item I = sym ? c.items32[it] : c.items[it];
         if (I.tile < 0) {  // bonded terms (FP64), overlapping the pair items of other warps
-            bonded_item(c, I.j0, I.nj, MODE);
+            bonded_item(c, I.j0, I.nj, MODE, tid, NT);
             continue;
         }
         const Tile tl = c.tiles[I.tile];
@@ -693,55 +697,71 @@ __device__ __noinline__ void terms64_plain(double dx, double dy, double dz, doub
     o[3] = ri2;
 }
 
-// KG > 1, for objects with fewer items than SMs (split >= KG): KG times the
-// warps, group g of four takes the steps k = g mod KG, and the groups' i-side
-// sums are added in order.  A lone warp needs about 2,500 cycles for a step (430
-// dependent instructions), 500 atoms kept every warp busy for 32 of them:
-// E + grad 45 -> 34 us with their queue.
-template <int KG>
-__global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (KG == 2 ? 2 : 1)) k_pair64_sym(Ctx c) {
+// CL: for objects with fewer parts of tile pairs than the SMs hold, a part is
+// shared by a cluster of c.cl64 blocks: each takes a run of the part's steps,
+// and the blocks' sums are added in order through their shared memory.  A lone
+// warp needs about 2,500 cycles for a step (430 dependent instructions) and
+// 500 atoms kept every warp busy for 32 of them on 40 SMs.  The grid covers
+// every item of the object once (no work queue: its chain of dependent loads
+// and the atomic took 9,000 cycles).
+// E + grad with the queue's kernel before it, us: 500 atoms 45 (one block a part)
+// and 34 (four times the warps in a block) -> 22, 1,500 atoms 67 -> 51.
+template <bool CL>
+__global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx c) {
     // staged j-atoms: x, y | z, then q', c6, c12 as significands with their
     // exponents and the charge's sign (forces), or as they are (energy only)
     __shared__ ulonglong2 s_xy[TJ], s_zq[TJ], s_c[TJ];
     __shared__ int2 s_e[TJ];
-    // opposite forces, [warp][j of the part]: 4 KG warps, at most TJ / KG j-atoms
-    __shared__ double jfx[4 * TJ], jfy[4 * TJ], jfz[4 * TJ];
-    __shared__ double4_32a s_i[KG > 1 ? KG : 1][KG > 1 ? TI : 1];
+    __shared__ double jfx[4 * TJ], jfy[4 * TJ], jfz[4 * TJ];  // opposite forces, [warp][j of the part]
+    __shared__ double s_i[CL ? 4 : 1][CL ? TI : 1], s_j[CL ? 3 * TJ : 1];  // this block's sums
     __shared__ int s_item;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    cg::cluster_group cl = cg::this_cluster();
+    const int CS = CL ? (int)cl.num_blocks() : 1, rank = CL ? (int)cl.block_rank() : 0;
     const int32_t *A = c.act + 1 * (2 * c.n_sys + 2);
-    const int n_act = A[0], total = A[1];
-    if (total == 0) return;
+    int n_act = 0, total = 0;
+    if constexpr (!CL) {
+        n_act = A[0];
+        total = A[1];
+        if (total == 0) return;
+    }
     const int32_t *aoff = A + 2, *asys = A + 2 + c.n_sys;
-    // i-atom, its warp among four, step group
-    const int tid = threadIdx.x % NT_SYM, lane = tid & 31, w = tid >> 5, kg = threadIdx.x / NT_SYM;
-    const int load = threadIdx.x;  // j-atom staged by this thread
     for (;;) {
-        if (threadIdx.x == 0) {
-            const int q = (int)atomicAdd(&c.counters[CNT_PAIR64], 1u);
-            if (q < total) {  // last active system whose first item is <= q
-                int lo = 0, hi = n_act - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (aoff[mid] <= q) lo = mid;
-                    else hi = mid - 1;
+        int it = 0;
+        if constexpr (CL) {
+            it = blockIdx.x / CS;
+        } else {
+            if (tid == 0) {
+                const int q = (int)atomicAdd(&c.counters[CNT_PAIR64], 1u);
+                if (q < total) {  // last active system whose first item is <= q
+                    int lo = 0, hi = n_act - 1;
+                    while (lo < hi) {
+                        const int mid = (lo + hi + 1) >> 1;
+                        if (aoff[mid] <= q) lo = mid;
+                        else hi = mid - 1;
+                    }
+                    s_item = c.sys_items64[asys[lo]].x + (q - aoff[lo]);
+                } else {
+                    s_item = -1;
                 }
-                s_item = c.sys_items64[asys[lo]].x + (q - aoff[lo]);
-            } else {
-                s_item = -1;
             }
+            __syncthreads();
+            it = s_item;
+            __syncthreads();
+            if (it < 0) break;
         }
-        __syncthreads();
-        const int it = s_item;
-        __syncthreads();
-        if (it < 0) break;
         const Item I = c.items64[it];
         if (I.tile < 0) {
-            bonded_item(c, I.j0, I.nj, 1);
+            bonded_item(c, I.j0, I.nj, 1, rank * NT_SYM + tid, CS * NT_SYM);
+            if constexpr (CL) return;
             continue;
         }
         const Tile &tl = c.tiles[I.tile];
-        const int kind = c.st[tl.sys].ev_kind;
-        if (kind == EV_NONE || c.st[tl.sys].mode != 1) continue;
+        const int kind = c.st[I.sys].ev_kind;
+        if (kind == EV_NONE || c.st[I.sys].mode != 1) {
+            if constexpr (CL) return;  // every block of the cluster
+            continue;
+        }
         const bool grad = kind == EV_EG;
         const bool part = tl.r64.split > 1;
         const int W = TJ / tl.r64.split;
@@ -772,16 +792,16 @@ __global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (
         double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
         double sc1 = 0.0, s6 = 0.0, s12 = 0.0;  // energy-only factored sums
         const int jend = I.j0 + I.nj;
-        double *fx = jfx + (kg * 4 + w) * W, *fy = jfy + (kg * 4 + w) * W, *fz = jfz + (kg * 4 + w) * W;
+        double *fx = jfx + w * W, *fy = jfy + w * W, *fz = jfz + w * W;
         for (int jt = I.j0; jt < jend; jt += TJ) {
-            const int jl = jt + load;
+            const int jl = jt + tid;
             double4_32a pj = make_double4_32a(1e6, 1e6, 1e6, 0.0);
             double2 cj0 = make_double2(0.0, 0.0);
             long long xj = FIX_FAR, yj = FIX_FAR, zj = FIX_FAR;
             u64 m1 = 0, m6 = 0, m12 = 0;
             int e1 = P64_ZERO, e6 = P64_ZERO, e12 = P64_ZERO;
             bool j_range = in_range, j_fix = i_fix;
-            if (load < W && jl < jend) {
+            if (tid < W && jl < jend) {
                 pj = c.posd[jl];
                 cj0 = c.pard[jl];
                 j_range = split64(pj.w, m1, e1) && j_range;
@@ -795,12 +815,12 @@ __global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (
             // the integer forms of the terms when every parameter is in range
             const bool fix = __syncthreads_and(j_fix && j_range);
             const bool plain = fix ? false : __syncthreads_or(!j_range);
-            if (load < W) {
-                s_xy[load] = fix ? make_ulonglong2((u64)xj, (u64)yj) : make_ulonglong2(bits64(pj.x), bits64(pj.y));
-                s_zq[load] = make_ulonglong2(fix ? (u64)zj : bits64(pj.z), grad ? m1 : bits64(pj.w));
-                s_c[load] = grad ? make_ulonglong2(m6, m12) : make_ulonglong2(bits64(cj0.x), bits64(cj0.y));
+            if (tid < W) {
+                s_xy[tid] = fix ? make_ulonglong2((u64)xj, (u64)yj) : make_ulonglong2(bits64(pj.x), bits64(pj.y));
+                s_zq[tid] = make_ulonglong2(fix ? (u64)zj : bits64(pj.z), grad ? m1 : bits64(pj.w));
+                s_c[tid] = grad ? make_ulonglong2(m6, m12) : make_ulonglong2(bits64(cj0.x), bits64(cj0.y));
                 if (grad)
-                    s_e[load] = make_int2((int)((uint32_t)e1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
+                    s_e[tid] = make_int2((int)((uint32_t)e1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
                                          (e6 << 16) | e12);
             }
             if (grad) {
@@ -815,6 +835,7 @@ __global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (
             const int k0 = half ? 1 : 0;
             const int k1 = half ? (tid < TJ / 2 ? TJ / 2 : TJ / 2 - 1)  // warp-uniform
                                 : (mask && I.joff + W <= (w << 5) + 1 ? -1 : W - 1);
+            const int ka = CL ? rank * (W / CS) : k0, kb = CL ? min(k1, ka + W / CS - 1) : k1;
             // the FP64 differences of a pair whose fixed-point ones are too small
             auto differences = [&](int j, double &dx, double &dy, double &dz) {
                 const double4_32a q = jt + j < jend ? c.posd[jt + j] : make_double4_32a(1e6, 1e6, 1e6, 0.0);
@@ -823,7 +844,7 @@ __global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (
             auto energies = [&](auto FIX) {
                 // energy only: the i atom's factors leave the sums,
                 // E_i = q'_i sum q'_j / r + (c12_i sum c12_j r^-12 - c6_i sum c6_j r^-6) / 6
-                for (int k = k0 + kg; k <= k1; k += KG) {
+                for (int k = ka; k <= kb; k++) {
                     const int j = (tid + k) & (W - 1);
                     const ulonglong2 xy = s_xy[j], zq = s_zq[j], cj = s_c[j];
                     const bool on = !mask || I.joff + j > tid;
@@ -856,7 +877,7 @@ __global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (
                 }
             };
             auto forces = [&](auto FIX) {
-                for (int k = k0 + kg; k <= k1; k += KG) {
+                for (int k = ka; k <= kb; k++) {
                     const int j = (tid + k) & (W - 1);
                     const ulonglong2 xy = s_xy[j], zq = s_zq[j], cj = s_c[j];
                     const int2 ej = s_e[j];
@@ -921,30 +942,42 @@ __global__ void __launch_bounds__(NT_SYM * KG, KG == 1 ? FFMIN_SYM_MINBLOCKS : (
             else forces(std::false_type{});
             __syncthreads();
             // j-side partial row of this j-tile, warps summed in order
-            if (load < W && jl < jend) {
+            if constexpr (CL) {
+                for (int q = tid; q < 3 * W; q += NT_SYM) {
+                    const int j = q % W;
+                    const double *f = (q < W ? jfx : (q < 2 * W ? jfy : jfz)) + j;
+                    s_j[q] = ((f[0] + f[W]) + f[2 * W]) + f[3 * W];
+                }
+            } else if (tid < W && jl < jend) {
                 double4_32a o;
-                o.x = jfx[load]; o.y = jfy[load]; o.z = jfz[load];
+                o.x = jfx[tid]; o.y = jfy[tid]; o.z = jfz[tid];
 #pragma unroll
-                for (int v = 1; v < 4 * KG; v++) { o.x += jfx[v * W + load]; o.y += jfy[v * W + load]; o.z += jfz[v * W + load]; }
+                for (int v = 1; v < 4; v++) { o.x += jfx[v * W + tid]; o.y += jfy[v * W + tid]; o.z += jfz[v * W + tid]; }
                 o.w = 0.0;
-                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + I.joff + load] = o;
+                c.gpd[(int64_t)(I.jslot + (jt - I.j0) / TJ) * TI + I.joff + tid] = o;
             }
         }
         double4_32a o;
         o.x = gx; o.y = gy; o.z = gz;
         o.w = grad ? ec + lj * (1.0 / 6.0) : pi.w * sc1 + (ci.y * s12 - ci.x * s6) * (1.0 / 6.0);
-        if constexpr (KG > 1) {
-            s_i[kg][tid] = o;
-            __syncthreads();
-            if (kg == 0) {
-#pragma unroll
-                for (int v = 1; v < KG; v++) {
-                    const double4_32a q = s_i[v][tid];
-                    o.x += q.x; o.y += q.y; o.z += q.z; o.w += q.w;
-                }
+        if constexpr (CL) {
+            s_i[0][tid] = o.x; s_i[1][tid] = o.y; s_i[2][tid] = o.z; s_i[3][tid] = o.w;
+            cl.sync();
+            const int n = 4 * TI + (grad ? 3 * W : 0);
+            double *irow = reinterpret_cast<double *>(c.gpd + (int64_t)I.slot * TI);
+            double *jrow = reinterpret_cast<double *>(c.gpd + (int64_t)I.jslot * TI + I.joff);
+            for (int u = rank * NT_SYM + tid; u < n; u += CS * NT_SYM) {
+                const int v = u - 4 * TI;
+                double *mine = v < 0 ? &s_i[0][u] : &s_j[v];
+                double x = *cl.map_shared_rank(mine, 0);
+                for (int r = 1; r < CS; r++) x += *cl.map_shared_rank(mine, r);
+                if (v < 0) irow[4 * (u % TI) + u / TI] = x;
+                else if (v % W < I.nj) jrow[4 * (v % W) + v / W] = x;
             }
+            cl.sync();  // no block leaves while its shared memory is read
+            return;
         }
-        if (kg == 0) c.gpd[(int64_t)I.slot * TI + tid] = o;
+        c.gpd[(int64_t)I.slot * TI + tid] = o;
     }
 }
 
@@ -965,7 +998,7 @@ int pair_grid_size(int mode, int f32_ipt) {
     else if (mode == 1)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, K_F64, NT_F64, 0);
     else if (mode == 2)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair64_sym<1>, NT_SYM, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair64_sym<false>, NT_SYM, 0);
     else if (one)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<float, TI, 1, false, true>, TI, 0);
     else
@@ -987,11 +1020,24 @@ static void launch_f32_shape(const Ctx &c, bool eonly, int grid, cudaStream_t s)
     }
 }
 
+static cudaError_t launch_pair64_cl(const Ctx &c, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(c.n_items64 * c.cl64);
+    cfg.blockDim = dim3(NT_SYM);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = c.cl64;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_pair64_sym<true>, c);
+}
+
 cudaError_t launch_pair_list(const Ctx &c, int list, int grid, cudaStream_t s) {
     if (list == LIST_F64) {
-        if (c.sym64 && c.kg64 == 4) k_pair64_sym<4><<<grid, NT_SYM * 4, 0, s>>>(c);
-        else if (c.sym64 && c.kg64 == 2) k_pair64_sym<2><<<grid, NT_SYM * 2, 0, s>>>(c);
-        else if (c.sym64) k_pair64_sym<1><<<grid, NT_SYM, 0, s>>>(c);
+        if (c.sym64 && c.cl64 > 1) return launch_pair64_cl(c, s);
+        if (c.sym64) k_pair64_sym<false><<<grid, NT_SYM, 0, s>>>(c);
         else K_F64<<<grid, NT_F64, 0, s>>>(c);
     } else if (c.f32_ipt == 1) {
         launch_f32_shape<1>(c, list == LIST_F32_E, grid, s);

@@ -48,8 +48,8 @@ def check(ff, orc, s):
 
 
 # 1 to 3 tiles, ragged last parts, sizes with four parts a tile pair (up to 2,000,
-# 6,200 and 6,273), two (3,400 and 9,000) and whole tiles (4,352 and 4,481); four
-# step groups up to 1,000, two up to 2,000
+# 6,200 and 6,273), two (3,400 and 9,000) and whole tiles (4,352 and 4,481);
+# clusters of eight blocks a part up to 257, of four (1,000 and 1,101) and two (2,000)
 @pytest.mark.parametrize("n", [31, 33, 96, 97, 257, 1000, 1101, 2000, 3400, 4352, 4481, 6200, 6273, 9000])
 def test_tiles_and_parts(ff, orc, n):
     rng = np.random.default_rng(n)
