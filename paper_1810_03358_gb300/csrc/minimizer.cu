@@ -152,6 +152,40 @@ __device__ __forceinline__ Row4 row_at(const double4_32a *rows, int64_t slot, in
     return Row4{p.x, p.y, p.z, p.w};
 }
 
+// sum of m FP32 rows FIN_STRANDS * TI apart from p on, in order, added to a;
+// eight rows in flight (an object of 30,000 atoms has 20 a strand)
+__device__ __forceinline__ void rows_f32(const float4 *p, int m, Row4 &a) {
+    constexpr int U = 8, ST = FIN_STRANDS * TI;
+    for (int q = 0; q < m; q += U, p += U * ST) {
+        float4 v[U];
+        const bool full = q + U <= m;
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = full || q + u < m ? __ldcs(p + u * ST) : float4{0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (!full && q + u >= m) break;
+            a.x += widen(v[u].x);
+            a.y += widen(v[u].y);
+            a.z += widen(v[u].z);
+            a.w += widen(v[u].w);
+        }
+    }
+}
+// the same for energies alone
+__device__ __forceinline__ void rows_f32(const float *p, int m, double &a) {
+    constexpr int U = 16, ST = FIN_STRANDS * TI;
+    for (int q = 0; q < m; q += U, p += U * ST) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = q + u < m ? __ldcs(p + u * ST) : 0.f;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (q + u >= m) break;
+            a += widen(v[u]);
+        }
+    }
+}
+
 // this strand's share (w, w + 4, ...) of the sum over q < n of f(q), in order,
 // added to a; XYZ / W: the components that count; four or eight loads in flight
 template <bool XYZ, bool W, typename F>
@@ -234,12 +268,10 @@ __global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT) k_
         if (real) {
             if (mode == 0 && c.sym32 && !grad) {
                 // energies on the symmetric list, each pair counted once
-                const int C = t.r32.chunk;
-                strand_sum<false, true>((ntile - t.tloc + C - 1) / C, w, r, [&](int q) {
-                    return Row4{0.0, 0.0, 0.0, widen(c.gpf_sym[((int64_t)t.r32.slot + q) * TI + i])};
-                });
+                const int C = t.r32.chunk, n = (ntile - t.tloc + C - 1) / C;
+                rows_f32(c.gpf_sym + ((int64_t)t.r32.slot + w) * TI + i, (n - w + 3) / FIN_STRANDS, r.w);
             } else if (mode == 0) {
-                strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpf, t.item0 + it, i); });
+                rows_f32(c.gpf + ((int64_t)t.item0 + w) * TI + i, (t.nitem - w + 3) / FIN_STRANDS, r);
                 r.w *= 0.5;  // every pair was counted in both of its rows
             } else if (c.sym64) {
                 if (grad) sym_rows<true>(c, t, tile0, ntile, i, w, r);
