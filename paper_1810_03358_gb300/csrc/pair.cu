@@ -413,15 +413,29 @@ __device__ __forceinline__ void sweep2_delta(const J2 *__restrict__ sj, const ul
 // FP32 shapes: two i-atoms per thread (64-thread blocks: every j load from
 // shared memory serves two pairs) or one (128-thread blocks: twice the warps
 // per work item, which pays when an object has few items); the autotuner
-// picks one per object.  Register caps: FP32 kernels run 640 threads per SM
-// (10 blocks of 64 or 5 of 128, 96 registers; 768 at 80 registers: difference
-// trials 2 % slower at 30,000 atoms and 13 % at 3,334, 512: E + grad 8 %
-// slower), the FP64 kernel 8 blocks of 128 (64 registers); the rarely-run
-// bonded items may spill.  FFMIN_F32_THREADS_PER_SM overrides the FP32 cap
-// (registers per thread follow: 65536 / threads).
-#ifndef FFMIN_F32_THREADS_PER_SM
-#define FFMIN_F32_THREADS_PER_SM 640
+// picks one per object.  Register caps: the FP32 E + grad kernel runs 768
+// threads per SM (12 blocks of 64 or 6 of 128, 80 registers), the FP32
+// energy kernel 512 (128 registers: a difference trial keeps more values).  At
+// 30,000 atoms with 512, 640, 768, 896 threads: E + grad 744, 711, 682, 720 us;
+// difference trials 500, 532, 531, 537 us; plain energies 231, 223, 228, 232 us;
+// a minimization takes difference trials.  At 3,334 they are within 2 %, but
+// trials with 768 are 10 % slower.  With exclusions E + grad runs 640 (1,000
+// atoms 3 % faster than with 768, 20,000 the same).  The FP64 kernel runs 8 blocks of 128 (64
+// registers); the rarely-run bonded items may spill.  FFMIN_F32_EG_THREADS,
+// _XS_THREADS and _E_THREADS override the FP32 caps (registers per thread follow:
+// 65536 / threads).
+#ifndef FFMIN_F32_EG_THREADS
+#define FFMIN_F32_EG_THREADS 768
 #endif
+#ifndef FFMIN_F32_XS_THREADS
+#define FFMIN_F32_XS_THREADS 640
+#endif
+#ifndef FFMIN_F32_E_THREADS
+#define FFMIN_F32_E_THREADS 512
+#endif
+constexpr int f32_blocks(bool xs, bool eonly, int nt) {
+    return (eonly ? FFMIN_F32_E_THREADS : (xs ? FFMIN_F32_XS_THREADS : FFMIN_F32_EG_THREADS)) / nt;
+}
 // XS: the object carries the exclusion variant (FP32 sweeps scale the listed
 // pairs); a separate instantiation keeps the masked code out of the kernel
 // every other object runs
@@ -430,9 +444,9 @@ __device__ __forceinline__ void sweep2_delta(const J2 *__restrict__ sj, const ul
 // instantiation runs the E + grad row sweep only.  The FP64 row sweep (the
 // fallback of batches too large for the symmetric list) takes both kinds.
 template <typename T, int NT, int IPT, bool XS = false, bool EONLY = false>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM / NT : 8)) k_pair(Ctx c);
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? f32_blocks(XS, EONLY, NT) : 8)) k_pair(Ctx c);
 template <typename T, int NT, int IPT, bool XS, bool EONLY>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? FFMIN_F32_THREADS_PER_SM / NT : 8)) k_pair(Ctx c) {
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? f32_blocks(XS, EONLY, NT) : 8)) k_pair(Ctx c) {
     static_assert(NT * IPT == TI, "a block covers one i-tile");
     using V4 = typename VT<T>::V4;
     using V2 = typename VT<T>::V2;
