@@ -57,30 +57,45 @@ template <> struct VT<double> {
     static __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 };
 
-// scale of the pair (i, j) in the exclusion variant (1 for every pair not
-// listed); i must be a real atom
-__device__ __forceinline__ float pair_xscale(const Ctx &c, int i, int j) {
-    float s = 1.f;
-    for (int m = c.xs_off[i]; m < c.xs_off[i + 1]; m++)
-        if (c.xs_part[m] == j) s = c.xs_val[m];
-    return s;
-}
-
-// the scaled partners of the thread's i-atoms among the 32 atoms from j0 on,
-// one bit each: a pair without a bit has scale 1 and needs no lookup (the
-// lookup in global memory for every pair made a masked tile cost 10 plain ones)
+// The scaled partners of the thread's i-atoms (exclusion variant; sorted by
+// index), walked along a j tile 32 atoms at a time: one bit each, and the
+// scale of the partner at bit k from the number of bits below it.  A pair
+// without a bit has scale 1.  (A lookup of every pair in the atom's list made
+// a masked tile cost 10 plain ones; looking up only the pairs with a bit, still
+// a chain of dependent loads in nearly every step near the diagonal, kept it
+// at 900 cycles a step: 1,000 atoms E + grad 72 -> 45 us, 5,000 86 -> 61.)
 template <int IPT>
-__device__ __forceinline__ void xmask(const Ctx &c, const int *ig, int j0, unsigned (&m)[IPT]) {
+struct XCursor {
+    const Ctx *c;
+    int cur[IPT], end[IPT], base[IPT];
+    unsigned m[IPT];
+    __device__ __forceinline__ void begin(const Ctx *cx, const int *ig, int jt) {  // ig: -1 for padding
+        c = cx;
 #pragma unroll
-    for (int u = 0; u < IPT; u++) {
-        m[u] = 0u;
-        if (ig[u] < 0) continue;
-        for (int k = c.xs_off[ig[u]]; k < c.xs_off[ig[u] + 1]; k++) {
-            const int d = c.xs_part[k] - j0;
-            if (d >= 0 && d < 32) m[u] |= 1u << d;
+        for (int u = 0; u < IPT; u++) {
+            cur[u] = end[u] = 0;
+            if (ig[u] < 0) continue;
+            cur[u] = c->xs_off[ig[u]];
+            end[u] = c->xs_off[ig[u] + 1];
+            while (cur[u] < end[u] && c->xs_part[cur[u]] < jt) cur[u]++;
         }
     }
-}
+    __device__ __forceinline__ void window(int j0) {
+#pragma unroll
+        for (int u = 0; u < IPT; u++) {
+            m[u] = 0u;
+            base[u] = cur[u];
+            for (; cur[u] < end[u]; cur[u]++) {
+                const int d = c->xs_part[cur[u]] - j0;
+                if (d >= 32) break;
+                m[u] |= 1u << d;
+            }
+        }
+    }
+    __device__ __forceinline__ float scale(int u, int k) const {
+        return (m[u] >> k) & 1u ? c->xs_val[base[u] + __popc(m[u] & ((1u << k) - 1u))] : 1.f;
+    }
+};
 
 // IPT i-atoms per thread share every j load from shared memory.  DM: 0 an
 // off-diagonal tile; 1 the i-tile itself (j == i skipped); 2 the i-tile
@@ -98,9 +113,10 @@ __device__ __forceinline__ void sweep(const typename VT<T>::V4 *__restrict__ sp,
                                       int jt = 0) {
     // the masked form runs on a few tiles only: kept rolled (smaller kernel)
     constexpr int KW = MASK ? 32 : TJ;
+    XCursor<MASK ? IPT : 1> xs;
+    if constexpr (MASK) xs.begin(cx, ig, jt);
     for (int kw = 0; kw < TJ; kw += KW) {
-    unsigned xm[IPT];
-    if (MASK) xmask<IPT>(*cx, ig, jt + kw, xm);
+    if constexpr (MASK) xs.window(jt + kw);
 #pragma unroll(MASK ? 1 : 8)
     for (int kk = 0; kk < KW; kk++) {
         const int k = kw + kk;
@@ -114,9 +130,7 @@ __device__ __forceinline__ void sweep(const typename VT<T>::V4 *__restrict__ sp,
             if (DM == 1) ri = (k == dk[u]) ? T(0) : ri;
             if (DM == 2) ri = (k <= dk[u]) ? T(0) : ri;
             T sc = T(1);
-            if (MASK) {
-                if ((xm[u] >> kk) & 1u) sc = (T)pair_xscale(*cx, ig[u], jt + k);
-            }
+            if constexpr (MASK) sc = (T)xs.scale(u, kk);
             const T ri2 = ri * ri;
             const T e = MASK ? pi[u].w * pj.w * sc * ri : pi[u].w * pj.w * ri;
             const T ri6 = ri2 * ri2 * ri2;
@@ -156,9 +170,10 @@ __device__ __forceinline__ void sweep_delta(const float4 *__restrict__ sp, const
                                             const int (&dk)[IPT], float (&ec)[IPT], float (&lj)[IPT],
                                             const Ctx *cx = nullptr, const int *ig = nullptr, int jt = 0) {
     constexpr int KW = MASK ? 32 : TJ;
+    XCursor<MASK ? IPT : 1> xs;
+    if constexpr (MASK) xs.begin(cx, ig, jt);
     for (int kw = 0; kw < TJ; kw += KW) {
-    unsigned xm[IPT];
-    if (MASK) xmask<IPT>(*cx, ig, jt + kw, xm);
+    if constexpr (MASK) xs.window(jt + kw);
 #pragma unroll(MASK ? 1 : 4)
     for (int kk = 0; kk < KW; kk++) {
         const int k = kw + kk;
@@ -183,9 +198,7 @@ __device__ __forceinline__ void sweep_delta(const float4 *__restrict__ sp, const
             const float d6 = X * (rp4 + rp2 * ri2 + ri4);
             const float d12 = d6 * (rp4 * rp2 + ri4 * ri2);
             float sc = 1.f;
-            if (MASK) {
-                if ((xm[u] >> kk) & 1u) sc = pair_xscale(*cx, ig[u], jt + k);
-            }
+            if constexpr (MASK) sc = xs.scale(u, kk);
             const float c6 = MASK ? ci[u].x * qj.x * sc : ci[u].x * qj.x;
             const float c12 = MASK ? ci[u].y * qj.y * sc : ci[u].y * qj.y;
             ec[u] += MASK ? pi[u].w * pj.w * sc * d1 : pi[u].w * pj.w * d1;
