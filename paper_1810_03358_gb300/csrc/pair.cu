@@ -422,15 +422,52 @@ __device__ __forceinline__ void sweep2_delta(const J2 *__restrict__ sj, const ul
     }
 }
 
+// Item of position q of a work queue (the active systems' items in order), -1
+// past its end
+template <int LIST>
+__device__ __forceinline__ int queue_item(const Ctx &c, const int2 *items, int q) {
+    const int32_t *A = c.act + LIST * (2 * c.n_sys + 2);
+    const int n_act = A[0], total = A[1];
+    if (q >= total) return -1;
+    if (c.n_sys == 1) return q;
+    const int32_t *aoff = A + 2, *asys = A + 2 + c.n_sys;
+    int lo = 0, hi = n_act - 1;  // last active system whose first item is <= q
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (aoff[mid] <= q) lo = mid;
+        else hi = mid - 1;
+    }
+    return items[asys[lo]].x + (q - aoff[lo]);
+}
+// The next item of a block.  Its first position in the queue is its index and
+// is found by every thread; the following ones come from the counter, and a
+// block whose grid covers the queue takes none.  (Every position through one
+// thread and the counter was a chain of nine loads: E + grad kernel with its
+// list kernel at 3,334 atoms FP64 165 -> 160 us, energies 77 -> 73 us; MIXED trials of
+// 10,000 atoms 82 -> 76 us, of 5,000 with exclusions 54 -> 48 us.)
+template <int LIST>
+__device__ __forceinline__ int next_item(const Ctx &c, const int2 *items, unsigned *counter, bool first, int &s_item) {
+    if (first) return queue_item<LIST>(c, items, blockIdx.x);
+    if (threadIdx.x == 0)
+        s_item = c.act[LIST * (2 * c.n_sys + 2) + 1] <= (int)gridDim.x
+                     ? -1
+                     : queue_item<LIST>(c, items, gridDim.x + (int)atomicAdd(counter, 1u));
+    __syncthreads();
+    const int it = s_item;
+    __syncthreads();
+    return it;
+}
+
 // NT threads per block, IPT i-atoms per thread, NT * IPT == TI (one tile).
 // FP32 shapes: two i-atoms per thread (64-thread blocks: every j load from
 // shared memory serves two pairs) or one (128-thread blocks: twice the warps
 // per work item, which pays when an object has few items); the autotuner
-// picks one per object.  Register caps: the FP32 E + grad kernel runs 768
-// threads per SM (12 blocks of 64 or 6 of 128, 80 registers), the FP32
+// picks one per object.  Register caps: the FP32 E + grad kernel runs 832
+// threads per SM (13 blocks of 64 or 6 of 128, 72 registers or 80), the FP32
 // energy kernel 512 (128 registers: a difference trial keeps more values).  At
-// 30,000 atoms with 512, 640, 768, 896 threads: E + grad 744, 711, 682, 720 us;
-// difference trials 500, 532, 531, 537 us; plain energies 231, 223, 228, 232 us;
+// 30,000 atoms with 512, 640, 768, 832, 896 threads: E + grad 744, 711, 682, 667,
+// 668 us; with 512, 640, 768, 896 difference trials 500, 532, 531, 537 us and
+// plain energies 231, 223, 228, 232 us;
 // a minimization takes difference trials.  At 3,334 they are within 2 %, but
 // trials with 768 are 10 % slower.  With exclusions E + grad runs 640 (1,000
 // atoms 3 % faster than with 768, 20,000 the same).  The FP64 kernel runs 8 blocks of 128 (64
@@ -438,7 +475,7 @@ __device__ __forceinline__ void sweep2_delta(const J2 *__restrict__ sj, const ul
 // _XS_THREADS and _E_THREADS override the FP32 caps (registers per thread follow:
 // 65536 / threads).
 #ifndef FFMIN_F32_EG_THREADS
-#define FFMIN_F32_EG_THREADS 768
+#define FFMIN_F32_EG_THREADS 832
 #endif
 #ifndef FFMIN_F32_XS_THREADS
 #define FFMIN_F32_XS_THREADS 640
@@ -484,48 +521,25 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? f32_blocks(XS, EONLY, NT
     constexpr int LIST = MODE == 1 ? LIST_F64 : (EONLY ? LIST_F32_E : LIST_F32_EG);
     constexpr int CNT = MODE == 1 ? CNT_PAIR64 : (EONLY ? CNT_PAIR32E : CNT_PAIR);
     // the queue runs over the items of the systems evaluating in this
-    // precision and kind only (active list rebuilt before every launch)
-    const int32_t *A = c.act + LIST * (2 * c.n_sys + 2);
-    const int n_act = A[0], total = A[1];
-    if (total == 0) return;
-    const int32_t *aoff = A + 2, *asys = A + 2 + c.n_sys;
+    // precision and kind only (active list rebuilt before every launch).
+    // FP32 energy-only evaluations (plain or difference trials) run on the
+    // symmetric list: each pair once, no forces
+    const bool sym = MODE == 0 && EONLY && c.sym32;
     const int tid = threadIdx.x;
-    __shared__ int s_sym;
-    for (;;) {
-        if (tid == 0) {
-            const int q = (int)atomicAdd(&c.counters[CNT], 1u);
-            if (q < total) {  // last active system whose first item is <= q
-                int lo = 0, hi = n_act - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (aoff[mid] <= q) lo = mid;
-                    else hi = mid - 1;
-                }
-                // FP32 energy-only evaluations (plain or difference trials)
-                // run on the symmetric list: each pair once, no forces
-                const int b = asys[lo];
-                const int sym = MODE == 0 && EONLY && c.sym32;
-                s_item = (sym ? c.sys_items32 : c.sys_items)[b].x + (q - aoff[lo]);
-                s_sym = sym;
-            } else {
-                s_item = -1;
-            }
-        }
-        __syncthreads();
-        const int it = s_item;
-        const bool sym = MODE == 0 && s_sym;
-        __syncthreads();
+    for (bool first = true;; first = false) {
+        const int it = next_item<LIST>(c, sym ? c.sys_items32 : c.sys_items, &c.counters[CNT], first, s_item);
         if (it < 0) break;
-        const Item I = sym ? c.items32[it] : c.items[it];
+        const Item I = (sym ? c.items32 : c.items)[it];
         if (I.tile < 0) {  // bonded terms (FP64), overlapping the pair items of other warps
             bonded_item(c, I.j0, I.nj, MODE, tid, NT);
             continue;
         }
         const Tile tl = c.tiles[I.tile];
-        const int kind = c.st[tl.sys].ev_kind;
-        if (kind == EV_NONE || c.st[tl.sys].mode != MODE) continue;
+        const SysState &S = c.st[I.sys];
+        const int kind = S.ev_kind;
+        const bool delta = MODE == 0 && S.ev_delta;
+        if (kind == EV_NONE || S.mode != MODE) continue;
         if (MODE == 0 && (kind == EV_E) != EONLY) continue;  // the other FP32 queue's system
-        const bool delta = MODE == 0 && c.st[tl.sys].ev_delta;
         V4 pi[IPT];
         V2 ci[IPT];
         int ig[IPT];
@@ -729,8 +743,7 @@ __device__ __noinline__ void terms64_plain(double dx, double dy, double dz, doub
 // and the blocks' sums are added in order through their shared memory.  A lone
 // warp needs about 2,500 cycles for a step (430 dependent instructions) and
 // 500 atoms kept every warp busy for 32 of them on 40 SMs.  The grid covers
-// every item of the object once (no work queue: its chain of dependent loads
-// and the atomic took 9,000 cycles).
+// every item of the object once, without the queue.
 // E + grad with the queue's kernel before it, us: 500 atoms 45 (one block a part)
 // and 34 (four times the warps in a block) -> 22, 1,500 atoms 67 -> 51.
 template <bool CL>
@@ -745,38 +758,10 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     cg::cluster_group cl = cg::this_cluster();
     const int CS = CL ? (int)cl.num_blocks() : 1, rank = CL ? (int)cl.block_rank() : 0;
-    const int32_t *A = c.act + 1 * (2 * c.n_sys + 2);
-    int n_act = 0, total = 0;
-    if constexpr (!CL) {
-        n_act = A[0];
-        total = A[1];
-        if (total == 0) return;
-    }
-    const int32_t *aoff = A + 2, *asys = A + 2 + c.n_sys;
-    for (;;) {
-        int it = 0;
-        if constexpr (CL) {
-            it = blockIdx.x / CS;
-        } else {
-            if (tid == 0) {
-                const int q = (int)atomicAdd(&c.counters[CNT_PAIR64], 1u);
-                if (q < total) {  // last active system whose first item is <= q
-                    int lo = 0, hi = n_act - 1;
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (aoff[mid] <= q) lo = mid;
-                        else hi = mid - 1;
-                    }
-                    s_item = c.sys_items64[asys[lo]].x + (q - aoff[lo]);
-                } else {
-                    s_item = -1;
-                }
-            }
-            __syncthreads();
-            it = s_item;
-            __syncthreads();
-            if (it < 0) break;
-        }
+    for (bool first = true;; first = false) {
+        const int it = CL ? (int)blockIdx.x / CS
+                          : next_item<LIST_F64>(c, c.sys_items64, &c.counters[CNT_PAIR64], first, s_item);
+        if (it < 0) break;
         const Item I = c.items64[it];
         if (I.tile < 0) {
             bonded_item(c, I.j0, I.nj, 1, rank * NT_SYM + tid, CS * NT_SYM);
