@@ -643,7 +643,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
     }
     sys->grid_sym = pair_grid_size(2);
     for (int k = 0; k < 2; k++) {
-        sys->grid32_max_s[k] = pair_grid_size(0, k + 1);
+        sys->grid32_max_s[k] = pair_grid_size(0, k + 1, mixed && !xidx.empty());
         sys->grid32e_max_s[k] = pair_grid_size(3, k + 1);
     }
     // capacities: the densest layout the autotuner may choose, in the FP32

@@ -287,8 +287,9 @@ cudaError_t launch_mbh_perturb(const Ctx &c, const double *best, double *out, do
                                int64_t hop, cudaStream_t s);
 cudaError_t launch_mbh_accept(const Ctx &c, const int32_t *flags, const double *x, double *best, cudaStream_t s);
 // resident blocks of the pair kernel of a mode: 0 FP32 E + grad row sweep,
-// 1 FP64 row sweep, 2 FP64 symmetric tiles, 3 FP32 energy only
-int pair_grid_size(int mode, int f32_ipt = 2);
+// 1 FP64 row sweep, 2 FP64 symmetric tiles, 3 FP32 energy only; xs: of an
+// object with exclusions
+int pair_grid_size(int mode, int f32_ipt = 2, bool xs = false);
 
 // arguments of one epoch of the parallel gradient-free search with FP32 terms
 // (one block per part, each on its own copy of the positions)

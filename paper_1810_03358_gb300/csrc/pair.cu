@@ -998,12 +998,16 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
 constexpr int NT_F64 = 128;
 #define K_F64 k_pair<double, 128, 1>
 
-int pair_grid_size(int mode, int f32_ipt) {
+int pair_grid_size(int mode, int f32_ipt, bool xs) {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool one = f32_ipt == 1;
-    if (mode == 0 && one)
+    if (mode == 0 && xs && one)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<float, TI, 1, true>, TI, 0);
+    else if (mode == 0 && xs)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<float, TI / 2, 2, true>, TI / 2, 0);
+    else if (mode == 0 && one)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<float, TI, 1>, TI, 0);
     else if (mode == 0)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pair<float, TI / 2, 2>, TI / 2, 0);
