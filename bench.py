@@ -51,11 +51,12 @@ FLOPS_UNIQUE_E = 23.0
 FLOPS_PER_PAIR_EG = 32.0
 FLOPS_PER_PAIR_E = 21.0
 # hardware flops per unique pair of each kernel form: the FP64 symmetric
-# tiles evaluate a pair once and add its force to both atoms (32 + 6); the
-# FP32 E + grad row sweep evaluates it twice (2 x 32); the energy-only and
-# difference-trial forms run on the symmetric tiles once (21; ~40 for the
-# exact-difference identities)
-HW_SYM_EG, HW_SYM_E, HW_ROW_EG, HW_DELTA = 38.0, 21.0, 64.0, 40.0
+# tiles evaluate a pair once, form its terms on the integer pipes and execute
+# 12 FP64 instructions for it (sums, force, both atoms' accumulation), 3 for
+# an energy, two flops each; the FP32 E + grad row sweep evaluates it twice (2 x
+# 32); the FP32 energy-only and difference-trial forms run on the symmetric
+# tiles once (21; ~40 for the exact-difference identities)
+HW_FP64_EG, HW_FP64_E, HW_SYM_E, HW_ROW_EG, HW_DELTA = 24.0, 6.0, 21.0, 64.0, 40.0
 # ALU peaks derived from unit counts at the maximum SM clock: FP32 152 SMs x
 # 128 lanes x 2 flops; FP64 152 SMs x 2 FMA per clock x 2 flops (the GB300
 # nominal 1.25 TFLOP/s at 2,070 MHz)
@@ -305,8 +306,8 @@ def bench_gpu(args):
         return {"achieved": achieved, "frac": achieved / peak, "hw_achieved": hw, "hw_frac": hw / peak,
                 "ms_per_launch": ms, "unique_pairs_per_s": unique / (ms / 1e3)}
 
-    r64 = roof(ms_pair, FLOPS_UNIQUE_EG, HW_SYM_EG, fp64_derived)
-    r64e = roof(ms_pair_e, FLOPS_UNIQUE_E, HW_SYM_E, fp64_derived)
+    r64 = roof(ms_pair, FLOPS_UNIQUE_EG, HW_FP64_EG, fp64_derived)
+    r64e = roof(ms_pair_e, FLOPS_UNIQUE_E, HW_FP64_E, fp64_derived)
     r32 = roof(ms_pair32, FLOPS_UNIQUE_EG, HW_ROW_EG, fp32_derived)
     r32e = roof(ms_pair32_e, FLOPS_UNIQUE_E, HW_SYM_E, fp32_derived)
     r32d = roof(ms_pair32_d, FLOPS_UNIQUE_E, HW_DELTA, fp32_derived)
@@ -315,7 +316,7 @@ def bench_gpu(args):
     # weighted by the step's own launch mix (n_eg E + grad, n_e energy only)
     step_ms = n_eg * ms_pair + n_e * ms_pair_e
     step_alg = (n_eg * FLOPS_UNIQUE_EG + n_e * FLOPS_UNIQUE_E) * unique / (step_ms / 1e3) / 1e12
-    step_hw = (n_eg * HW_SYM_EG + n_e * HW_SYM_E) * unique / (step_ms / 1e3) / 1e12
+    step_hw = (n_eg * HW_FP64_EG + n_e * HW_FP64_E) * unique / (step_ms / 1e3) / 1e12
     step32_ms = ms_pair32 + 3 * ms_pair32_d  # a MIXED L-BFGS step: one E + grad, three trials
     step32_alg = (FLOPS_UNIQUE_EG + 3 * FLOPS_UNIQUE_E) * unique / (step32_ms / 1e3) / 1e12
     line = {
@@ -348,8 +349,9 @@ def bench_gpu(args):
                              f"unique pairs per launch (algorithmic); {n_eg} + {n_e} launches per step",
                      "ms_per_launch": step_ms / (n_eg + n_e),
                      "hw_achieved": step_hw, "hw_frac": step_hw / fp64_derived,
-                     "hw_work": f"{HW_SYM_EG:.0f} / {HW_SYM_E:.0f} flops per unique pair as executed "
-                                "(each pair once, force added to both atoms)",
+                     "hw_work": f"{HW_FP64_EG:.0f} / {HW_FP64_E:.0f} FP64 flops per unique pair as executed "
+                                "(12 / 3 instructions; r^2, r^-1 and the terms' products run on the integer "
+                                "pipes, so frac may pass 1)",
                      "peak_source": f"derived: 152 SMs x 2 FP64 FMA/clk x 2 flops x {sm_max_mhz:.0f} MHz",
                      "peak_probe": fp64_probe, "frac_of_probe": step_alg / fp64_probe,
                      "e_grad": {"ms_per_launch": ms_pair, "achieved": r64["achieved"], "frac": r64["frac"],

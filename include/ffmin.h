@@ -287,7 +287,10 @@ ffmin_status ffmin_neighbour_counts(ffmin_system *sys, const double *x_dev, int3
  * [ffmin_mlp_work_floats()] scratch, loss_host [steps] (optional) the
  * minibatch losses, w16_dev [449] (optional) FP16 weights out.  steps = 0
  * computes the mean-loss gradient over the first min(batch, n) rows into
- * work_dev[work - 449 .. work) without updating.  Synchronizes the stream. */
+ * work_dev[work - 449 .. work) without updating.  Synchronizes the stream.
+ * All steps run in one cooperative launch whose blocks wait for one another
+ * with a bounded poll; FFMIN_ERR_TIMEOUT when one gave up (weights and
+ * moments then hold some step's values). */
 ffmin_status ffmin_mlp_train(const float *feat_dev, const float *target_dev, int64_t n_samples,
                              int32_t steps, int32_t batch, float lr, uint64_t seed, float *w32_dev,
                              float *adam_dev, float *work_dev, float *loss_host, uint16_t *w16_dev,

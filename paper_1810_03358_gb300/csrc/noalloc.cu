@@ -16,7 +16,7 @@
 // leaves 9 FP64 instructions an evaluated pair of about 28.  Blocks of 32 i-atoms against a
 // j-chunk, the chunk's atoms dealt to the four warps, give about 1,000 equal
 // blocks at 4,000 atoms (128 i-atoms per block: 256, 1.7 per SM).  4,000 atoms:
-// 1.10 -> 0.44 ms a call.  Partial rows go to the scratch, then one thread per atom
+// 1.10 -> 0.37 ms a call.  Partial rows go to the scratch, then one thread per atom
 // sums its chunks in a fixed order and the last block sums the block
 // energies and flags a non-finite energy or gradient (two coincident atoms),
 // which the call reports after synchronising its stream.

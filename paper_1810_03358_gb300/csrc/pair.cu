@@ -7,8 +7,8 @@
 // evaluated in row i and again in row j, so no force is ever scattered and
 // no atomic touches a force (Newton's third law is not used).
 //
-// Work items are (i-tile, j-chunk) pairs taken from a device queue (reset by
-// a memset before each launch) by a persistent grid; each item writes its
+// Work items are (i-tile, j-chunk) pairs taken from a device queue (reset with
+// its active list before each launch) by a persistent grid; each item writes its
 // partial row sums (gx, gy, gz, row energy) to its own slot, and the
 // finalize kernel sums the slots of an atom in a fixed order, so results are
 // deterministic for a given chunking.  Bonded-term items share the queue.
