@@ -714,13 +714,14 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? f32_blocks(XS, EONLY, NT
 // finalize kernel sums an atom's rows in a fixed order.  Row energies count
 // each pair once.
 //
-// Bound: the FP64 pipe at 2 operations per SM and clock.  Differences (in
-// fixed point, when the tile pair's coordinates fit) and terms are formed on
-// the integer pipes (pair64.cuh), which leaves 12 FP64 instructions of 31 a pair
-// with forces and 3 of 18.5 for an energy.  30,000 atoms, E + grad / E: 24.46 /
-// 14.83 ms in plain FP64, 12.53 / 5.06 ms with FP64 differences, 10.20 / 4.00 ms
-// now.  Blocks per SM: 5 (4: 7 % slower energies, 6: 3 % slower E + grad at
-// 3,334 atoms, 2 % faster energies at 30,000).
+// Bound: the FP64 pipe at 2 operations per SM and clock, and issue.  Differences
+// (in fixed point, when the tile pair's coordinates fit), terms and their sums
+// are formed on the integer pipes (pair64.cuh), which leaves 7 FP64
+// instructions of 31 a pair with forces and 3 of 18.5 for an energy.  30,000
+// atoms, E + grad / E: 24.46 / 14.83 ms in plain FP64, 12.53 / 5.06 ms with FP64
+// differences, 10.14 / 3.98 ms with the sum of a pair's terms in FP64 (12
+// instructions, pipe 88 % busy), 8.66 / 3.98 ms now.  Blocks per SM: 5 (4: 4 % and
+// 7 % slower, 6: 3 % and 1 % faster at 30,000 atoms, 1 % and 2 % slower at 3,334).
 constexpr int NT_SYM = 128;
 #ifndef FFMIN_SYM_MINBLOCKS
 #define FFMIN_SYM_MINBLOCKS 5
@@ -801,7 +802,7 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             xi = yi = zi = -FIX_FAR;
             i_fix = true;
         }
-        double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
+        double gx = 0.0, gy = 0.0, gz = 0.0, e6 = 0.0;  // e6: six times the energy
         double sc1 = 0.0, s6 = 0.0, s12 = 0.0;  // energy-only factored sums
         const int jend = I.j0 + I.nj;
         double *fx = jfx + w * W, *fy = jfy + w * W, *fz = jfz + w * W;
@@ -811,14 +812,14 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
             double2 cj0 = make_double2(0.0, 0.0);
             long long xj = FIX_FAR, yj = FIX_FAR, zj = FIX_FAR;
             u64 m1 = 0, m6 = 0, m12 = 0;
-            int e1 = P64_ZERO, e6 = P64_ZERO, e12 = P64_ZERO;
+            int x1 = P64_ZERO, x6 = P64_ZERO, x12 = P64_ZERO;
             bool j_range = in_range, j_fix = i_fix;
             if (tid < W && jl < jend) {
                 pj = c.posd[jl];
                 cj0 = c.pard[jl];
-                j_range = split64(pj.w, m1, e1) && j_range;
-                j_range = split64(cj0.x, m6, e6) && j_range;
-                j_range = split64(cj0.y, m12, e12) && j_range;
+                j_range = split64(pj.w, m1, x1) && j_range;
+                j_range = split64(cj0.x, m6, x6) && j_range;
+                j_range = split64(cj0.y, m12, x12) && j_range;
                 j_fix = fix64(pj.x, xj) && j_fix;
                 j_fix = fix64(pj.y, yj) && j_fix;
                 j_fix = fix64(pj.z, zj) && j_fix;
@@ -832,8 +833,8 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
                 s_zq[tid] = make_ulonglong2(fix ? (u64)zj : bits64(pj.z), grad ? m1 : bits64(pj.w));
                 s_c[tid] = grad ? make_ulonglong2(m6, m12) : make_ulonglong2(bits64(cj0.x), bits64(cj0.y));
                 if (grad)
-                    s_e[tid] = make_int2((int)((uint32_t)e1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
-                                         (e6 << 16) | e12);
+                    s_e[tid] = make_int2((int)((uint32_t)x1 | ((uint32_t)(bits64(pj.w) >> 32) & 0x80000000u)),
+                                         (x6 << 16) | x12);
             }
             if (grad) {
                 for (int q = lane; q < W; q += 32) { fx[q] = 0.0; fy[q] = 0.0; fz[q] = 0.0; }
@@ -914,11 +915,9 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
                         ok = inv64(dx, dy, dz, v);
                     }
                     const int es = ce + ej.y;
-                    double e = inv64_c1(v, qm, zq.y, qe + (ej.x & 0xffff));
-                    e = from_bits64(bits64(e) ^ ((u64)(((uint32_t)ej.x & 0x80000000u) ^ qs) << 32));
-                    double p6 = inv64_c6(v, c6m, cj.x, (int)((uint32_t)es >> 16));
-                    double p12 = inv64_c12(v, c12m, cj.y, es & 0xffff);
-                    double ri2 = inv64_r2(v);
+                    double f, y;
+                    inv64_force(v, qm, zq.y, qe + (ej.x & 0xffff), ((uint32_t)ej.x ^ qs) & 0x80000000u, c6m, cj.x,
+                                (int)((uint32_t)es >> 16), c12m, cj.y, es & 0xffff, f, y);
                     if (__any_sync(0xffffffffu, !ok) || plain) {
                         if (decltype(FIX)::value) {
                             dx = 1.0; dy = dz = 0.0;
@@ -929,13 +928,12 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
                         const double2 c_j = jg < jend ? c.pard[jg] : make_double2(0.0, 0.0);
                         double o[4];
                         terms64_plain(dx, dy, dz, pi.w * q_j, ci.x * c_j.x, ci.y * c_j.y, o);
-                        e = o[0]; p6 = o[1]; p12 = o[2]; ri2 = o[3];
+                        const double u = o[2] - o[1];
+                        f = ((u + o[2]) + o[0]) * o[3];
+                        y = fma(6.0, o[0], u);
                     }
-                    if (!on) e = p6 = p12 = ri2 = 0.0;
-                    const double u = p12 - p6;
-                    ec += e;
-                    lj += u;
-                    const double f = ((u + p12) + e) * ri2;
+                    if (!on) f = y = 0.0;
+                    e6 += y;
                     gx = fma(f, dx, gx);
                     gy = fma(f, dy, gy);
                     gz = fma(f, dz, gz);
@@ -971,7 +969,7 @@ __global__ void __launch_bounds__(NT_SYM, FFMIN_SYM_MINBLOCKS) k_pair64_sym(Ctx 
         }
         double4_32a o;
         o.x = gx; o.y = gy; o.z = gz;
-        o.w = grad ? ec + lj * (1.0 / 6.0) : pi.w * sc1 + (ci.y * s12 - ci.x * s6) * (1.0 / 6.0);
+        o.w = grad ? e6 * (1.0 / 6.0) : pi.w * sc1 + (ci.y * s12 - ci.x * s6) * (1.0 / 6.0);
         if constexpr (CL) {
             s_i[0][tid] = o.x; s_i[1][tid] = o.y; s_i[2][tid] = o.z; s_i[3][tid] = o.w;
             cl.sync();

@@ -5,10 +5,10 @@
 // forces costs about 31 FP64 instructions (CUDA's rsqrt alone 5.7) when it
 // is written in FP64.  Here r^2, its reciprocal square root, the powers of r
 // and the products with the atoms' parameters are formed on 64-bit
-// significands with separate exponents and rounded once to FP64; FP64
-// instructions remain for the sums of the terms and the accumulation (12 a
-// pair with forces, 3 for an energy) and, outside the fixed-point range, for
-// the coordinate differences (3 more).  Every
+// significands with separate exponents, the terms of a pair are added as
+// integers, and the results rounded once to FP64; FP64 instructions remain for
+// the accumulation (7 a pair with forces, 3 for an energy) and, outside the
+// fixed-point range, for the coordinate differences (3 more).  Every
 // significand below is good to 2^-57 or better and is rounded to 53 bits at
 // the end, so a term's error is no larger than that of the FP64 formula,
 // whose own roundings (each 2^-53) add up.
@@ -220,6 +220,44 @@ FFM_P64 double inv64_c6(const Inv64 &v, u64 a, u64 b, int s) {
 FFM_P64 double inv64_c12(const Inv64 &v, u64 a, u64 b, int s) {
     return pack64<true>(mulh(mulh(a, b) << 1, sqh(v.n6) << 1),
                         1023 - 52 - 2 * P64_BIAS + s - 6 * v.n - 2 * v.k - 12 * v.E);
+}
+
+// The force over r and six times the energy of a pair,
+//   f = (e + 2 p12 - p6) r^-2,  y = 6 e + p12 - p6,
+// from the terms' significands (each in [2^58, 2^62)), aligned to the largest
+// exponent and added as integers, which leaves one FP64 addition (y) of a
+// pair's six besides the accumulation of the forces.  A term is cut at 2^-56
+// of the largest or better.  s1, s6, s12: sums of the parameters' biased
+// exponents; neg: sign of the charges' product in the top bit.
+FFM_P64 int clz64(u64 v) {  // v != 0
+#ifdef __CUDA_ARCH__
+    const uint32_t hi = (uint32_t)(v >> 32);
+    return hi ? __clz((int)hi) : 32 + __clz((int)(uint32_t)v);
+#else
+    return __builtin_clzll(v);
+#endif
+}
+FFM_P64 void inv64_force(const Inv64 &v, u64 q1, u64 q2, int s1, uint32_t neg, u64 a6, u64 b6, int s6, u64 a12, u64 b12,
+                         int s12, double &f, double &y) {
+    const u64 ve = mulh(mulh(q1, q2) << 1, v.m), v6 = mulh(mulh(a6, b6) << 1, v.n6),
+              v12 = mulh(mulh(a12, b12) << 1, sqh(v.n6) << 1);
+    const int k6 = 3 * v.n + v.k + 6 * v.E;
+    const int be = s1 - v.E - 60, be6 = s6 - k6 - 56, be12 = s12 - 2 * k6 - 52;
+    const int bm = be > be6 ? (be > be12 ? be : be12) : (be6 > be12 ? be6 : be12);
+    const int d = bm - be < 61 ? bm - be : 61, d6 = bm - be6 < 61 ? bm - be6 : 61, d12 = bm - be12 < 61 ? bm - be12 : 61;
+    const long long sg = (long long)(int)neg >> 63;
+    const long long e = ((long long)(ve >> (d + 2)) ^ sg) - sg, x6 = (long long)(v6 >> (d6 + 2)),
+                    x12 = (long long)(v12 >> (d12 + 2));
+    const long long u = x12 - x6, x = u + x12 + e, z = u + 6 * e;
+    const int b = bm + 2 + 1023 - 2 * P64_BIAS;  // biased exponent of a unit
+    const u64 ax = abs64(x), az = abs64(z);
+    const int n = clz64(ax | 1ULL) - 1, nz = clz64(az | 1ULL);
+    const double r = pack64<true>(mulh(ax << n, v.n2), b + 4 - 2 - n - v.n - 2 * v.E);
+    f = from_bits64(ax ? bits64(r) | ((u64)x & 0x8000000000000000ULL) : 0);
+    const u64 m = az << nz;
+    const int ex = b + 63 - nz;
+    const u64 w = ((m >> 11) + ((uint32_t)((uint32_t)m >> 10) & 1u)) + ((u64)(uint32_t)((ex - 1) << 20) << 32);
+    y = from_bits64(az && ex >= 1 ? w | ((u64)z & 0x8000000000000000ULL) : 0);
 }
 
 }  // namespace ffm
