@@ -12,11 +12,11 @@
 // Computation: an FP64 row sweep over all pairs of one system, Coulomb +
 // Lennard-Jones, no bonded terms: every pair in both of its rows, since the
 // fixed scratch has no room for the opposite forces.  Bound: the FP64 pipe;
-// differences and terms are formed on the integer pipes (pair64.cuh), which
-// leaves 9 FP64 instructions an evaluated pair of about 28.  Blocks of 32 i-atoms against a
+// differences, terms and their sums are formed on the integer pipes
+// (pair64.cuh), which leaves 4 FP64 instructions an evaluated pair of about 28.  Blocks of 32 i-atoms against a
 // j-chunk, the chunk's atoms dealt to the four warps, give about 1,000 equal
 // blocks at 4,000 atoms (128 i-atoms per block: 256, 1.7 per SM).  4,000 atoms:
-// 1.10 -> 0.37 ms a call.  Partial rows go to the scratch, then one thread per atom
+// 1.10 -> 0.37 ms a call with the terms added in FP64 (9 instructions), 0.34 ms now.  Partial rows go to the scratch, then one thread per atom
 // sums its chunks in a fixed order and the last block sums the block
 // energies and flags a non-finite energy or gradient (two coincident atoms),
 // which the call reports after synchronising its stream.
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(NA_NT, 5) k_na_rows(NaArgs a) {
     }
     const int len = (a.n + a.chunks - 1) / a.chunks;
     const int j0 = blockIdx.y * len, j1 = min(a.n, j0 + len);
-    double gx = 0.0, gy = 0.0, gz = 0.0, ec = 0.0, lj = 0.0;
+    double gx = 0.0, gy = 0.0, gz = 0.0, es6 = 0.0;  // es6: six times the energy
     for (int jt = j0; jt < j1; jt += NA_TJ) {
         double xj[3], pj[3];
         const bool real = jt + tid < j1;
@@ -168,11 +168,9 @@ __global__ void __launch_bounds__(NA_NT, 5) k_na_rows(NaArgs a) {
                     ok = inv64(dx, dy, dz, v);
                 }
                 const int es = ce + ej.y;
-                double e = inv64_c1(v, m1, zq.y, e1 + (ej.x & 0xffff));
-                e = from_bits64(bits64(e) ^ ((u64)(((uint32_t)ej.x & 0x80000000u) ^ qs) << 32));
-                double p6 = inv64_c6(v, m6, cj.x, (int)((uint32_t)es >> 16));
-                double p12 = inv64_c12(v, m12, cj.y, es & 0xffff);
-                double ri2 = inv64_r2(v);
+                double f, y;
+                inv64_force(v, m1, zq.y, e1 + (ej.x & 0xffff), ((uint32_t)ej.x ^ qs) & 0x80000000u, m6, cj.x,
+                            (int)((uint32_t)es >> 16), m12, cj.y, es & 0xffff, f, y);
                 if (__any_sync(0xffffffffu, !ok) || plain) {
                     if (decltype(FIX)::value) {
                         dx = 1.0; dy = dz = 0.0;
@@ -183,17 +181,14 @@ __global__ void __launch_bounds__(NA_NT, 5) k_na_rows(NaArgs a) {
                         }
                     }
                     const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
-                    ri2 = ri * ri;
-                    const double ri6 = ri2 * ri2 * ri2;
-                    e = pi[0] * s_p[0][k] * ri;
-                    p6 = pi[1] * s_p[1][k] * ri6;
-                    p12 = pi[2] * s_p[2][k] * ri6 * ri6;
+                    const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
+                    const double p12 = pi[2] * s_p[2][k] * ri6 * ri6, u = p12 - pi[1] * s_p[1][k] * ri6,
+                                 e = pi[0] * s_p[0][k] * ri;
+                    f = ((u + p12) + e) * ri2;
+                    y = fma(6.0, e, u);
                 }
-                if (!on) e = p6 = p12 = ri2 = 0.0;
-                const double u = p12 - p6;
-                ec += e;
-                lj += u;
-                const double f = ((u + p12) + e) * ri2;
+                if (!on) f = y = 0.0;
+                es6 += y;
                 gx = fma(f, dx, gx);
                 gy = fma(f, dy, gy);
                 gz = fma(f, dz, gz);
@@ -203,7 +198,7 @@ __global__ void __launch_bounds__(NA_NT, 5) k_na_rows(NaArgs a) {
         else rows(std::false_type{});
     }
     __syncthreads();
-    s_sum[w][lane] = make_double4_32a(gx, gy, gz, ec + lj * (1.0 / 6.0));
+    s_sum[w][lane] = make_double4_32a(gx, gy, gz, es6 * (1.0 / 6.0));
     __syncthreads();
     // component w of atom `lane`, the warps in order
     const double *col = reinterpret_cast<const double *>(&s_sum[0][0]) + 4 * lane + w;

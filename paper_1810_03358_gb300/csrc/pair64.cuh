@@ -209,19 +209,6 @@ FFM_P64 double inv64_r12(const Inv64 &v) {
     return pack64<false>(sqh(v.n6), 1023 - 54 - 6 * v.n - 2 * v.k - 12 * v.E);
 }
 
-// products with a pair of parameters: significands a, b and the sum s of
-// their biased exponents
-FFM_P64 double inv64_c1(const Inv64 &v, u64 a, u64 b, int s) {
-    return pack64<true>(mulh(mulh(a, b) << 1, v.m), 1023 - 60 - 2 * P64_BIAS + s - v.E);
-}
-FFM_P64 double inv64_c6(const Inv64 &v, u64 a, u64 b, int s) {
-    return pack64<true>(mulh(mulh(a, b) << 1, v.n6), 1023 - 56 - 2 * P64_BIAS + s - 3 * v.n - v.k - 6 * v.E);
-}
-FFM_P64 double inv64_c12(const Inv64 &v, u64 a, u64 b, int s) {
-    return pack64<true>(mulh(mulh(a, b) << 1, sqh(v.n6) << 1),
-                        1023 - 52 - 2 * P64_BIAS + s - 6 * v.n - 2 * v.k - 12 * v.E);
-}
-
 // The force over r and six times the energy of a pair,
 //   f = (e + 2 p12 - p6) r^-2,  y = 6 e + p12 - p6,
 // from the terms' significands (each in [2^58, 2^62)), aligned to the largest
