@@ -51,12 +51,12 @@ FLOPS_UNIQUE_E = 23.0
 FLOPS_PER_PAIR_EG = 32.0
 FLOPS_PER_PAIR_E = 21.0
 # hardware flops per unique pair of each kernel form: the FP64 symmetric
-# tiles evaluate a pair once, form its terms on the integer pipes and execute
-# 12 FP64 instructions for it (sums, force, both atoms' accumulation), 3 for
-# an energy, two flops each; the FP32 E + grad row sweep evaluates it twice (2 x
+# tiles evaluate a pair once, form its terms and their sums on the integer
+# pipes and execute 7 FP64 instructions for it (both atoms' accumulation), 3
+# for an energy, two flops each; the FP32 E + grad row sweep evaluates it twice (2 x
 # 32); the FP32 energy-only and difference-trial forms run on the symmetric
 # tiles once (21; ~40 for the exact-difference identities)
-HW_FP64_EG, HW_FP64_E, HW_SYM_E, HW_ROW_EG, HW_DELTA = 24.0, 6.0, 21.0, 64.0, 40.0
+HW_FP64_EG, HW_FP64_E, HW_SYM_E, HW_ROW_EG, HW_DELTA = 14.0, 6.0, 21.0, 64.0, 40.0
 # ALU peaks derived from unit counts at the maximum SM clock: FP32 152 SMs x
 # 128 lanes x 2 flops; FP64 152 SMs x 2 FMA per clock x 2 flops (the GB300
 # nominal 1.25 TFLOP/s at 2,070 MHz)
@@ -350,7 +350,7 @@ def bench_gpu(args):
                      "ms_per_launch": step_ms / (n_eg + n_e),
                      "hw_achieved": step_hw, "hw_frac": step_hw / fp64_derived,
                      "hw_work": f"{HW_FP64_EG:.0f} / {HW_FP64_E:.0f} FP64 flops per unique pair as executed "
-                                "(12 / 3 instructions; r^2, r^-1 and the terms' products run on the integer "
+                                "(7 / 3 instructions; r^2, r^-1 and the terms run on the integer "
                                 "pipes, so frac may pass 1)",
                      "peak_source": f"derived: 152 SMs x 2 FP64 FMA/clk x 2 flops x {sm_max_mhz:.0f} MHz",
                      "peak_probe": fp64_probe, "frac_of_probe": step_alg / fp64_probe,
