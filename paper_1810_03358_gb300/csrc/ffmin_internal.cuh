@@ -222,7 +222,7 @@ struct Ctx {
     // reductions
     double *red;            // [n_tiles][NRED]
     double *redf;           // finalize: [value][n_tiles]
-    unsigned int *counters; // one per kernel kind, reset by the last block
+    unsigned int *counters; // per work queue (reset with its active list), MIXED moves (by the last block)
     unsigned int *tickets;  // [N_STAGES][n_sys]: blocks of a system that finished a stage
     int32_t *nactive;       // systems still minimizing
     int32_t *nmode;         // [2] active systems per pair-kernel precision mode

@@ -143,10 +143,6 @@ __device__ __forceinline__ double widen(float x) {
 struct Row4 {
     double x, y, z, w;
 };
-__device__ __forceinline__ Row4 row_at(const float4 *rows, int64_t slot, int i) {
-    const float4 p = rows[slot * TI + i];
-    return Row4{widen(p.x), widen(p.y), widen(p.z), widen(p.w)};
-}
 __device__ __forceinline__ Row4 row_at(const double4_32a *rows, int64_t slot, int i) {
     const double4_32a p = rows[slot * TI + i];
     return Row4{p.x, p.y, p.z, p.w};
