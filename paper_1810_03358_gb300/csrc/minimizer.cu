@@ -129,6 +129,7 @@ cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) 
 constexpr int FIN_STRANDS = 4;
 constexpr int FIN_CLUSTER = TI / 32;
 constexpr int FIN_NT = 32 * (FIN_STRANDS + 2);
+constexpr int FIN_DENSE_TILES = 152;  // k_finalize<6> above it
 
 // exact FP32 -> FP64 on the integer pipe (the conversion instruction runs at
 // the FP64 rate); the FP32 kernels flush denormals, which read as zero
@@ -221,7 +222,13 @@ __device__ __forceinline__ int fin_value(int k) {
     return k == 0 ? RF_E : (k == 1 ? RF_EPAIR : (k == 2 ? RF_GG : (k == 3 ? RF_GTG : RF_GTR)));
 }
 
-__global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT) k_finalize(Ctx c, double *g_out) {
+// BLOCKS: resident blocks per SM, 4 (80 registers, the shortest chain) or 6 (56
+// registers) for objects of more tiles than SMs, which run in waves.  Us with 4
+// and 6: 79 tiles 19.7, 19.8 (with gradient) and 11.7, 14.1; 157 tiles 33.9, 29.8
+// and 17.3, 17.1; batches, 13 rounds: 119 tiles 193, 193; 186 tiles 246, 216; 399
+// tiles 362, 331; 1,533 tiles (16 rounds) 1,007, 860.
+template <int BLOCKS>
+__global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT, BLOCKS) k_finalize(Ctx c, double *g_out) {
     const int tile = blockIdx.x / FIN_CLUSTER, rank = blockIdx.x % FIN_CLUSTER;
     const Tile &t = c.tiles[tile];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;  // w: strand, then bonded terms
@@ -697,7 +704,8 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out) {
-    k_finalize<<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
+    if (c.n_tiles > FIN_DENSE_TILES) k_finalize<6><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
+    else k_finalize<4><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
     return cudaGetLastError();
 }
 cudaError_t launch_update(const Ctx &c, cudaStream_t s) {
