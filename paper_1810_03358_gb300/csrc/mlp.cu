@@ -207,14 +207,18 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
 #pragma unroll
                 for (int r = 0; r < MLP_CLUSTER; r++) x[r] = *cl.map_shared_rank(&sum[k], r);
                 part[cluster * MLP_NV + k] = ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
-                __threadfence();
             }
         }
         cl.sync();
         // grid barrier: every cluster has its sums of this step in memory
         // (the two buffers alternate, so no cluster writes over sums that
-        // another still reads: it arrives here again only after reading them)
-        if (rank == 0 && tid == 0) atomicAdd(&o.sync[0], 1u);
+        // another still reads: it arrives here again only after reading them).
+        // The cluster barrier orders every block's slice before this thread,
+        // whose fence releases them with its arrival to the pollers' acquire
+        if (rank == 0 && tid == 0) {
+            __threadfence();
+            atomicAdd(&o.sync[0], 1u);
+        }
         if (t + 1 < o.steps) gather(t + 1, blockIdx.x * MT);
         if (tid == MT - 1) {  // Adam's bias corrections of this step
             const float step = (float)(o.step0 + t + 1);
