@@ -40,7 +40,10 @@ constexpr int MLP_CLUSTERS = 16;  // clusters, at most (128 blocks: all resident
 constexpr int MLP_NV = MLP_NW + 1;                    // summed values: the gradient, the loss
 constexpr int MLP_SLICE = (MLP_NV + MLP_CLUSTER - 1) / MLP_CLUSTER;
 constexpr int MLP_STEPS = 4096;   // steps per launch (their losses wait in the scratch)
-constexpr long long MLP_SPIN = 1 << 22;  // polls of the grid barrier before a block gives up (about a second)
+// polls of the grid barrier before a block gives up (about a second)
+#ifndef FFMIN_MLP_POLLS
+#define FFMIN_MLP_POLLS (1 << 22)
+#endif
 
 // a run of training steps; lr == 0: one gradient, no update
 struct MlpRun {
@@ -73,7 +76,7 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
     __shared__ float sum[MLP_NV];          // the block's sums, read by the cluster
     __shared__ float wt[MLP_NW], am[MLP_NW], av[MLP_NW];
     __shared__ float unbias[2];
-    __shared__ int failed;
+    __shared__ int gave_up, failed;  // this block at the last grid barrier; some block of the cluster
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int rank = (int)cl.block_rank(), cluster = blockIdx.x / MLP_CLUSTER, clusters = gridDim.x / MLP_CLUSTER;
     const float be1 = 0.9f, be2 = 0.999f, eps = 1e-8f;
@@ -198,6 +201,7 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
         __syncthreads();
         for (int k = tid; k < MLP_NV; k += MT) sum[k] = (acc[0][k] + acc[1][k]) + (acc[2][k] + acc[3][k]);
         cl.sync();
+        if (failed) break;  // the whole cluster: no block reads the sums of one that has left
         // the cluster's sums, one slice per block, blocks in order
         float *part = o.part + (int64_t)(t & 1) * MLP_CLUSTERS * MLP_NV;
         {
@@ -231,14 +235,18 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
             unsigned got;
             do {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&o.sync[0]) : "memory");
-            } while (got < want && ++polls < MLP_SPIN && *(volatile unsigned int *)&o.sync[1] == 0u);
+            } while (got < want && ++polls < FFMIN_MLP_POLLS && *(volatile unsigned int *)&o.sync[1] == 0u);
+            gave_up = got < want;
             if (got < want) {
-                failed = 1;
-                o.sync[1] = 1u;
+                // its cluster leaves together behind the next cluster barrier
+                // (another block of it may have seen the count in time); the
+                // other clusters run out of arrivals or see the word
+                *(volatile unsigned int *)&o.sync[1] = 1u;
+                for (int r = 0; r < MLP_CLUSTER; r++) *cl.map_shared_rank(&failed, r) = 1;
             }
         }
         __syncthreads();
-        if (failed) break;
+        if (gave_up) continue;
         // the gradient over the clusters, then one Adam step: every load of a
         // thread's (up to four) parameters in flight together
         constexpr int KT = (MLP_NV + MT - 1) / MT;

@@ -1,0 +1,81 @@
+"""The preconditioner network's training kernel in forms that a plain call on a
+whole GPU does not reach: mlp.cu compiled by itself with other values of its
+build-time constants.
+
+A wait that runs out: with a single poll at the grid barrier some block gives
+up within a few steps (the first cluster to arrive finds the other 15 missing),
+while blocks of the same cluster that poll later see the count complete.  The
+call reports the timeout, the weights are those of some step (a step moves a
+weight by at most about lr), and the context still computes what it did."""
+import ctypes as C
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1810_03358_gb300 import build, learn
+from tests.gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def ff():
+    return need_gpu()
+
+
+@pytest.fixture(scope="module")
+def variant(ff, tmp_path_factory):
+    """variant(FFMIN_X=1, ...) -> a train function like ffmin.ffmin_mlp_train
+    that returns (status, losses), from mlp.cu with those constants"""
+    def make(**macros):
+        out = str(tmp_path_factory.mktemp("mlp") / "libmlp.so")
+        cmd = [build.nvcc(), "-O3", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", build.ROOT + "/include", "-I",
+               build.CSRC] + build.ARCH + [f"-D{k}={v}" for k, v in macros.items()] + ["-o", out, build.CSRC + "/mlp.cu"]
+        subprocess.run(cmd, check=True, capture_output=True, text=True)
+        L = C.CDLL(out)
+        L.ffmin_mlp_train.argtypes = ff.lib().ffmin_mlp_train.argtypes
+
+        def train(feat, target, steps, batch, lr, seed, w, adam, work):
+            losses = np.zeros(max(steps, 1), dtype=np.float32)
+            st = L.ffmin_mlp_train(feat.data_ptr(), target.data_ptr(), target.numel(), steps, batch, lr, seed,
+                                   w.data_ptr(), adam.data_ptr(), work.data_ptr(),
+                                   losses.ctypes.data_as(C.POINTER(C.c_float)), None,
+                                   torch.cuda.current_stream().cuda_stream)
+            return st, losses
+        return train
+    return make
+
+
+def inputs(rows, seed=3):
+    rng = np.random.default_rng(seed)
+    feat = rng.normal(size=(rows, 5)).astype(np.float32)
+    target = np.sin(feat.sum(axis=1)).astype(np.float32)
+    dev = dict(dtype=torch.float32, device="cuda")
+    return torch.tensor(feat, **dev), torch.tensor(target, **dev)
+
+
+def fresh(ff):
+    dev = dict(dtype=torch.float32, device="cuda")
+    return (torch.tensor(learn.init_weights(5).astype(np.float32), **dev), torch.zeros(2 * learn.N_PARAMS, **dev),
+            torch.zeros(ff.ffmin_mlp_work_floats(), **dev))
+
+
+def test_a_wait_that_runs_out_is_reported(ff, variant):
+    feat, target = inputs(50000)
+    lr, steps = 3e-3, 50
+
+    def plain():
+        w, adam, work = fresh(ff)
+        return ff.ffmin_mlp_train(feat, target, 5, 16384, lr, 9, w, adam, work), w.cpu().numpy()
+    before = plain()
+    impatient = variant(FFMIN_MLP_POLLS=1)
+    for _ in range(3):
+        w, adam, work = fresh(ff)
+        w0 = w.cpu().numpy()
+        st, _ = impatient(feat, target, steps, 16384, lr, 9, w, adam, work)
+        assert st == ff.FFMIN_ERR_TIMEOUT
+        assert np.abs(w.cpu().numpy() - w0).max() <= 2 * steps * lr
+    after = plain()
+    assert np.array_equal(before[0], after[0]) and np.array_equal(before[1], after[1])
