@@ -90,8 +90,11 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
     }
     if (tid == 0) failed = 0;
     float f[MLP_IN], tg = 0.f;
-    auto gather = [&](int t, int s0) {  // this thread's row of minibatch t, from s0 on
-        const int s = s0 + tid;
+    // rows are counted in 64 bits: a 32-bit index of a batch near 2^31 would
+    // wrap before it reached the end, and the loop would never end
+    const int64_t first = (int64_t)blockIdx.x * MT, stride = (int64_t)gridDim.x * MT;
+    auto gather = [&](int t, int64_t s0) {  // this thread's row of minibatch t, from s0 on
+        const int64_t s = s0 + tid;
 #pragma unroll
         for (int i = 0; i < MLP_IN; i++) f[i] = 0.f;
         tg = 0.f;
@@ -102,7 +105,7 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
         for (int i = 0; i < MLP_IN; i++) f[i] = o.feat[row * MLP_IN + i];
         tg = o.target[row];
     };
-    gather(0, blockIdx.x * MT);
+    gather(0, first);
     for (int t = 0; t < o.steps; t++) {
         __syncthreads();  // wt of this step
         if (tid < MLP_H) {
@@ -120,8 +123,8 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
             wu[u][0] = p.x; wu[u][1] = p.y; wu[u][2] = p.z; wu[u][3] = p.w;
             wu[u][4] = q.x; wu[u][5] = q.y; wu[u][6] = q.z;
         }
-        for (int s0 = blockIdx.x * MT; s0 < o.batch; s0 += gridDim.x * MT) {
-            if (s0 != (int)blockIdx.x * MT) gather(t, s0);
+        for (int64_t s0 = first; s0 < o.batch; s0 += stride) {
+            if (s0 != first) gather(t, s0);
             // The warp's 32 rows, two hidden units per thread: the units'
             // activations stay in registers for the backward pass, and their
             // shares of z are summed over the lanes by halving (31 exchanges
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
             __threadfence();
             atomicAdd(&o.sync[0], 1u);
         }
-        if (t + 1 < o.steps) gather(t + 1, blockIdx.x * MT);
+        if (t + 1 < o.steps) gather(t + 1, first);
         if (tid == MT - 1) {  // Adam's bias corrections of this step
             const float step = (float)(o.step0 + t + 1);
             unbias[0] = 1.f - powf(be1, step);
@@ -322,8 +325,8 @@ extern "C" ffmin_status ffmin_mlp_train(const float *feat_dev, const float *targ
     o.sync = reinterpret_cast<unsigned int *>(tail);
     static_assert(2 * MLP_CLUSTERS * MLP_NV + MLP_STEPS <= MLP_ROWS * MLP_NW, "the losses fit in the scratch");
     const int nsteps = steps > 0 ? steps : 1;
-    const int blocks = (o.batch + MT - 1) / MT;
-    const int clusters = std::min(MLP_CLUSTERS, (blocks + MLP_CLUSTER - 1) / MLP_CLUSTER);
+    const int64_t blocks = ((int64_t)o.batch + MT - 1) / MT;
+    const int clusters = (int)std::min<int64_t>(MLP_CLUSTERS, (blocks + MLP_CLUSTER - 1) / MLP_CLUSTER);
     for (int t = 0; t < nsteps; t += MLP_STEPS) {
         o.step0 = t;
         o.steps = std::min(MLP_STEPS, nsteps - t);

@@ -6,7 +6,12 @@ A wait that runs out: with a single poll at the grid barrier some block gives
 up within a few steps (the first cluster to arrive finds the other 15 missing),
 while blocks of the same cluster that poll later see the count complete.  The
 call reports the timeout, the weights are those of some step (a step moves a
-weight by at most about lr), and the context still computes what it did."""
+weight by at most about lr), and the context still computes what it did.
+
+The largest batch, 2^31 - 1 samples (of one row): every thread adds up 2^17 equal
+terms in FP32, each addition off by at most 2^-24 of the sum, so the loss is
+within 2^17 2^-24 = 1 % of the row's; the first Adam step moves a weight by lr
+towards the gradient's sign, whatever its size."""
 import ctypes as C
 import subprocess
 
@@ -79,3 +84,21 @@ def test_a_wait_that_runs_out_is_reported(ff, variant):
         assert np.abs(w.cpu().numpy() - w0).max() <= 2 * steps * lr
     after = plain()
     assert np.array_equal(before[0], after[0]) and np.array_equal(before[1], after[1])
+
+
+def test_largest_batch(ff):
+    feat, target = inputs(1)
+    lr = 3e-3
+    w, adam, work = fresh(ff)
+    w[384:448] = 0.1  # every unit reaches the output
+    y = w.double().requires_grad_(True)
+    h = torch.relu(feat[0].double() @ y[:320].view(64, 5).T + y[320:384])
+    loss = (h @ y[384:448] + y[448] - target[0]) ** 2
+    loss.backward()
+    got = ff.ffmin_mlp_train(feat, target, 1, 2 ** 31 - 1, lr, 9, w, adam, work)
+    assert abs(got[0] - float(loss.detach())) <= 0.01 * float(loss.detach())
+    step, sign = w.double() - y.detach(), y.grad.sign()
+    big = y.grad.abs() > 1e-4  # beside Adam's epsilon of 1e-8
+    assert int(big.sum()) > 100
+    assert (step + lr * sign)[big].abs().max() <= 1e-3 * lr
+    assert step[y.grad == 0].abs().max() == 0.0
