@@ -290,7 +290,9 @@ ffmin_status ffmin_neighbour_counts(ffmin_system *sys, const double *x_dev, int3
  * work_dev[work - 449 .. work) without updating.  Synchronizes the stream.
  * All steps run in one cooperative launch whose blocks wait for one another
  * with a bounded poll; FFMIN_ERR_TIMEOUT when one gave up (weights and
- * moments then hold some step's values). */
+ * moments then hold some step's values).  Up to 128 blocks of 128 threads, on
+ * clusters of eight; where the SMs at hand (a share of the GPU) hold fewer at
+ * once, fewer run (the sums then have another rounding). */
 ffmin_status ffmin_mlp_train(const float *feat_dev, const float *target_dev, int64_t n_samples,
                              int32_t steps, int32_t batch, float lr, uint64_t seed, float *w32_dev,
                              float *adam_dev, float *work_dev, float *loss_host, uint16_t *w16_dev,

@@ -35,10 +35,17 @@ namespace cg = cooperative_groups;
 
 constexpr int MT = 128;           // threads per training block, one row each
 constexpr int MLP_ROWS = 256;     // rows of MLP_NW floats that the scratch holds
-constexpr int MLP_CLUSTER = 8;    // blocks per cluster
-constexpr int MLP_CLUSTERS = 16;  // clusters, at most (128 blocks: all resident at once)
+#ifndef FFMIN_MLP_CLUSTER
+#define FFMIN_MLP_CLUSTER 8
+#endif
+constexpr int MLP_CLUSTER = FFMIN_MLP_CLUSTER;  // blocks per cluster
+// clusters, at most; all of a launch's blocks have to be resident at once, and
+// a launch that finds too few SMs (128 blocks need 43) is repeated with fewer
+#ifndef FFMIN_MLP_CLUSTERS
+#define FFMIN_MLP_CLUSTERS 16
+#endif
+constexpr int MLP_CLUSTERS = FFMIN_MLP_CLUSTERS;
 constexpr int MLP_NV = MLP_NW + 1;                    // summed values: the gradient, the loss
-constexpr int MLP_SLICE = (MLP_NV + MLP_CLUSTER - 1) / MLP_CLUSTER;
 constexpr int MLP_STEPS = 4096;   // steps per launch (their losses wait in the scratch)
 // polls of the grid barrier before a block gives up (about a second)
 #ifndef FFMIN_MLP_POLLS
@@ -67,8 +74,11 @@ __device__ __forceinline__ uint64_t mix64(uint64_t seed, uint64_t k) {
 }
 
 // Samples of minibatch t are index t batch + k of the SplitMix64 stream when
-// sample != 0, else rows [0, batch) of the data in order
-__global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(MlpRun o) {
+// sample != 0, else rows [0, batch) of the data in order.  CS: blocks per
+// cluster; 1 where the SMs at hand cannot hold a cluster
+template <int CS>
+__global__ void __launch_bounds__(MT) k_mlp_train(MlpRun o) {
+    constexpr int SLICE = (MLP_NV + CS - 1) / CS;  // sums per block of a cluster
     cg::cluster_group cl = cg::this_cluster();
     __shared__ float4 sw[MLP_H][2];        // per hidden unit: W1 (5), b1, w2
     __shared__ float4 sf[MT / 32][32][2];  // per row of the warp: features (5), dz
@@ -78,7 +88,7 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
     __shared__ float unbias[2];
     __shared__ int gave_up, failed;  // this block at the last grid barrier; some block of the cluster
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int rank = (int)cl.block_rank(), cluster = blockIdx.x / MLP_CLUSTER, clusters = gridDim.x / MLP_CLUSTER;
+    const int rank = (int)cl.block_rank(), cluster = blockIdx.x / CS, clusters = gridDim.x / CS;
     const float be1 = 0.9f, be2 = 0.999f, eps = 1e-8f;
     const float inv_b = 1.0f / (float)o.batch;
     for (int k = tid; k < MLP_NW; k += MT) {
@@ -207,13 +217,18 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
         if (failed) break;  // the whole cluster: no block reads the sums of one that has left
         // the cluster's sums, one slice per block, blocks in order
         float *part = o.part + (int64_t)(t & 1) * MLP_CLUSTERS * MLP_NV;
-        {
-            const int k = rank * MLP_SLICE + tid;
-            if (tid < MLP_SLICE && k < MLP_NV) {
-                float x[MLP_CLUSTER];
 #pragma unroll
-                for (int r = 0; r < MLP_CLUSTER; r++) x[r] = *cl.map_shared_rank(&sum[k], r);
-                part[cluster * MLP_NV + k] = ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+        for (int u = 0; u < SLICE; u += MT) {
+            const int k = rank * SLICE + u + tid;
+            if (u + tid < SLICE && k < MLP_NV) {
+                float x[CS];
+#pragma unroll
+                for (int r = 0; r < CS; r++) x[r] = *cl.map_shared_rank(&sum[k], r);
+#pragma unroll
+                for (int q = 1; q < CS; q *= 2)
+#pragma unroll
+                    for (int r = 0; r < CS; r += 2 * q) x[r] += x[r + q];
+                part[cluster * MLP_NV + k] = x[0];
             }
         }
         cl.sync();
@@ -245,7 +260,7 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
                 // (another block of it may have seen the count in time); the
                 // other clusters run out of arrivals or see the word
                 *(volatile unsigned int *)&o.sync[1] = 1u;
-                for (int r = 0; r < MLP_CLUSTER; r++) *cl.map_shared_rank(&failed, r) = 1;
+                for (int r = 0; r < CS; r++) *cl.map_shared_rank(&failed, r) = 1;
             }
         }
         __syncthreads();
@@ -297,6 +312,23 @@ __global__ void __launch_bounds__(MT) __cluster_dims__(MLP_CLUSTER) k_mlp_train(
     cl.sync();  // no block leaves while its sums may be read
 }
 
+// all blocks resident (cooperative): the grid barrier ends
+static cudaError_t launch_train(const MlpRun &o, int clusters, int cs, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(clusters * cs);
+    cfg.blockDim = dim3(MT);
+    cfg.stream = s;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cs;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cs == 1 ? cudaLaunchKernelEx(&cfg, k_mlp_train<1>, o) : cudaLaunchKernelEx(&cfg, k_mlp_train<MLP_CLUSTER>, o);
+}
+
 }  // namespace ffm
 
 using namespace ffm;
@@ -326,7 +358,7 @@ extern "C" ffmin_status ffmin_mlp_train(const float *feat_dev, const float *targ
     static_assert(2 * MLP_CLUSTERS * MLP_NV + MLP_STEPS <= MLP_ROWS * MLP_NW, "the losses fit in the scratch");
     const int nsteps = steps > 0 ? steps : 1;
     const int64_t blocks = ((int64_t)o.batch + MT - 1) / MT;
-    const int clusters = (int)std::min<int64_t>(MLP_CLUSTERS, (blocks + MLP_CLUSTER - 1) / MLP_CLUSTER);
+    int cs = MLP_CLUSTER, clusters = (int)std::min<int64_t>(MLP_CLUSTERS, (blocks + cs - 1) / cs);
     for (int t = 0; t < nsteps; t += MLP_STEPS) {
         o.step0 = t;
         o.steps = std::min(MLP_STEPS, nsteps - t);
@@ -334,16 +366,22 @@ extern "C" ffmin_status ffmin_mlp_train(const float *feat_dev, const float *targ
         o.grad_out = last ? tail + MLP_ROWS + 1 : nullptr;
         o.w16 = last ? w16_dev : nullptr;
         if (cudaMemsetAsync(o.sync, 0, 2 * sizeof(unsigned int), s) != cudaSuccess) return FFMIN_ERR_CUDA;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(clusters * MLP_CLUSTER);
-        cfg.blockDim = dim3(MT);
-        cfg.stream = s;
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeCooperative;  // all blocks resident: the grid barrier ends
-        at.val.cooperative = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, k_mlp_train, o) != cudaSuccess) return FFMIN_ERR_CUDA;
+        cudaError_t e;
+        while ((e = launch_train(o, clusters, cs, s)) != cudaSuccess) {
+            // refused: too few SMs at hand (a share of the GPU) for so many
+            // blocks, or, at the end, for a cluster
+            if ((clusters == 1 && cs == 1) ||
+                (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources &&
+                 e != cudaErrorInvalidClusterSize))
+                return FFMIN_ERR_CUDA;
+            (void)cudaGetLastError();
+            if (clusters > 1) {
+                clusters = (clusters + 1) / 2;
+            } else {
+                cs = 1;
+                clusters = (int)std::min<int64_t>(MLP_CLUSTER, blocks);
+            }
+        }
         unsigned int gave_up[2] = {0u, 0u};
         if (cudaMemcpyAsync(gave_up, o.sync, sizeof(gave_up), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             (loss_host && cudaMemcpyAsync(loss_host + t, o.losses, sizeof(float) * (size_t)o.steps,

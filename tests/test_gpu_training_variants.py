@@ -8,6 +8,14 @@ while blocks of the same cluster that poll later see the count complete.  The
 call reports the timeout, the weights are those of some step (a step moves a
 weight by at most about lr), and the context still computes what it did.
 
+A grid that is not resident at once: with 64 clusters (512 blocks, of which the
+SMs hold two each) the first launch is refused, and the call goes on with fewer
+clusters; so it goes where a process has a share of the SMs, down to blocks
+without clusters.  The gradient over all rows against FP64: a thread adds 128
+rows' terms in FP32 (2,048 in the 16 blocks without clusters), the rest is a
+tree, so at the worst 2^11 2^-24 = 1.2e-4 of the terms' magnitudes: a bar of 2e-4
+of the largest component, where a lost block would show as 1 / 512.
+
 The largest batch, 2^31 - 1 samples (of one row): every thread adds up 2^17 equal
 terms in FP32, each addition off by at most 2^-24 of the sum, so the loss is
 within 2^17 2^-24 = 1 % of the row's; the first Adam step moves a weight by lr
@@ -84,6 +92,22 @@ def test_a_wait_that_runs_out_is_reported(ff, variant):
         assert np.abs(w.cpu().numpy() - w0).max() <= 2 * steps * lr
     after = plain()
     assert np.array_equal(before[0], after[0]) and np.array_equal(before[1], after[1])
+
+
+@pytest.mark.parametrize("macros", [dict(FFMIN_MLP_CLUSTERS=64), dict(FFMIN_MLP_CLUSTER=1)])
+def test_other_grids(ff, variant, macros):
+    feat, target = inputs(1 << 17)
+    w, adam, work = fresh(ff)
+    w[384:448] = 0.1
+    y = w.double().requires_grad_(True)
+    h = torch.relu(feat.double() @ y[:320].view(64, 5).T + y[320:384])
+    loss = ((h @ y[384:448] + y[448] - target.double()) ** 2).mean()
+    loss.backward()
+    st, got = variant(**macros)(feat, target, 0, 1 << 17, 0.0, 0, w, adam, work)
+    assert st == ff.FFMIN_OK
+    assert abs(got[0] - float(loss.detach())) <= 2e-4 * float(loss.detach())
+    g = work[-learn.N_PARAMS:].double()
+    assert (g - y.grad).abs().max() <= 2e-4 * y.grad.abs().max()
 
 
 def test_largest_batch(ff):
