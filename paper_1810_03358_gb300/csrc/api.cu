@@ -1549,7 +1549,16 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
     const int cs = moves_cluster(1, sys->sms);
     ffm::ParabState *ps = nullptr;
     ffmin_status st;
+    bool gen = false, on_cluster = false;
     if (fp64) {
+        std::vector<double> xh(3 * (size_t)n);
+        CK(cudaMemcpyAsync(xh.data(), vslot(c, V_X), sizeof(double) * xh.size(), cudaMemcpyDeviceToHost,
+                           sys->stream));
+        CK(cudaStreamSynchronize(sys->stream));
+        gen = moves_general(xh.data(), n, o->gradfree_delta, taylor_r2);
+        on_cluster = !moves_on_grid(n, gen);
+    }
+    if (on_cluster) {
         if ((st = moves_view(sys, n, 1, cs)) != FFMIN_OK) return st;
     } else {
         if (!sys->parab_state) {
@@ -1563,7 +1572,7 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
         CK(cudaMemcpyAsync(sys->parab_state, hbuf.data(), hbuf.size(), cudaMemcpyHostToDevice, sys->stream));
         ps = (ffm::ParabState *)sys->parab_state;
     }
-    if (!fp64 && !sys->parab_graph) {
+    if (!on_cluster && !sys->parab_graph) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(sys->stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
@@ -1590,7 +1599,7 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
         if (!truncated) {
             const int32_t stop = (int32_t)std::min<int64_t>((int64_t)moves + n, o->max_iter);
             truncated = stop < moves + n;
-            if (fp64) {  // the sweep's moves in one launch
+            if (on_cluster) {  // the sweep's moves in one launch
                 MovesArgs ma{};
                 ma.view = sys->mv_view;
                 ma.n = n;
@@ -1599,7 +1608,7 @@ static ffmin_status parab_minimize(ffmin_system *sys, const ffmin_options *o, ff
                 ma.base = (uint64_t)moves;
                 ma.delta = o->gradfree_delta;
                 ma.taylor_r2 = taylor_r2;
-                CK(launch_moves64(c, ma, 1, cs, sys->stream));
+                CK(launch_moves64(c, ma, gen, 1, cs, sys->stream));
                 launches += 1;
                 ticks += stop - moves;
                 moves = stop;
@@ -1796,7 +1805,7 @@ static ffmin_status epoch_minimize(ffmin_system *sys, const ffmin_options *o, ff
         if (fp64) {
             MovesArgs ma{sys->mv_view, sys->ep_view, d_list, d_loff, d_allowed, d_members, d_moff, n, 0, o->seed,
                          e * (uint64_t)n, o->gradfree_delta, taylor_r2};
-            CK(launch_moves64(c, ma, P, cs, sys->stream));
+            CK(launch_moves64(c, ma, moves_general(xh.data(), n, ma.delta, taylor_r2), P, cs, sys->stream));
             // every atom belongs to one part: the merged positions are whole
             CK(cudaMemcpyAsync(vslot(c, V_X), sys->ep_view, sizeof(double) * 3 * (size_t)n, cudaMemcpyDeviceToDevice,
                                sys->stream));

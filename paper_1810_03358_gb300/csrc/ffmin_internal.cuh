@@ -318,6 +318,8 @@ struct MovesArgs {
 };
 int moves_cluster(int parts, int sms);
 int64_t moves_view_doubles(int n, int parts, int cs);
-cudaError_t launch_moves64(const Ctx &c, const MovesArgs &a, int parts, int cs, cudaStream_t s);
+bool moves_general(const double *x, int n, double delta, double taylor_r2);
+bool moves_on_grid(int n, bool gen);
+cudaError_t launch_moves64(const Ctx &c, const MovesArgs &a, bool gen, int parts, int cs, cudaStream_t s);
 
 }  // namespace ffm

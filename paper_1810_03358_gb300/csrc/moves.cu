@@ -25,6 +25,8 @@
 // positions and the far-field test round like their statements.
 #include <cooperative_groups.h>
 
+#include <cmath>
+
 #include "bonded.cuh"
 #include "ffmin_internal.cuh"
 #include "pair64.cuh"
@@ -41,6 +43,9 @@ constexpr int MV_CLUSTER = 8;      // largest (portable) cluster
 // fast rows: coordinates within this (differences below 2^62 units), an axis
 // offset of at most 0.2 A, and pairs at least 1/2 A apart along some axis
 constexpr double MV_FIX_MAX = 112.0, MV_DELTA_MAX = 0.2;
+// fixed-point coordinate of one beyond: its difference from any in range is at
+// least 2^62 (and below 2^63)
+constexpr long long MV_FAR = 3LL << 61;
 // arc tangents: sine and cosine at multiples of pi / MV_ATAN
 constexpr int MV_ATAN = 128;
 
@@ -194,8 +199,12 @@ __device__ __forceinline__ bool in_fix(const double *x) {
 }
 
 // SH: positions and this block's share of the parameters in shared memory;
-// otherwise a private copy in global memory and the object's arrays
-template <bool SH>
+// otherwise a private copy in global memory and the object's arrays.
+// GEN: rows from FP64 differences, for what the fixed-point rows leave out: a
+// larger offset, the far field, systems beyond the range.  A kernel of its own,
+// since its code beside the other rows cost those 3 % (4.54 -> 4.71 ms for 500
+// moves of 500 atoms).
+template <bool SH, bool GEN>
 __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
     cg::cluster_group cl = cg::this_cluster();
     const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank(), part = blockIdx.x / CS;
@@ -208,18 +217,16 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
     __shared__ double pos[8][3];                           // the 7 positions and the vertex
     __shared__ double buf[MV_BOND_WARPS][32];
     __shared__ double s_f[8];
-    __shared__ int s_slow;
     double *V = SH ? dyn : a.view + (int64_t)blockIdx.x * (3 * (int64_t)n + 3 * sh);
     long long *F = reinterpret_cast<long long *>(V + 3 * n);             // the share in fixed point
     double *pq = V + 3 * n + 3 * sh, *p6 = pq + sh, *p12 = p6 + sh;      // SH: the share's parameters
     const double *X = vslot(c, V_X);
-    if (tid == 0) s_slow = !(a.delta <= MV_DELTA_MAX) || a.taylor_r2 > 0.0;
-    __syncthreads();
     for (int t = tid; t < 3 * n; t += MV_THREADS) V[t] = X[t];
     for (int t = tid; t < 3 * nj; t += MV_THREADS) {
         const double x = X[3 * j0 + t];
-        fix64(x, F[t]);
-        if (!(fabs(x) < MV_FIX_MAX)) s_slow = 1;
+        long long f;
+        fix64(x, f);
+        F[t] = fabs(x) < MV_FIX_MAX ? f : MV_FAR;
     }
     if (SH) {
         for (int t = tid; t < nj; t += MV_THREADS) {
@@ -241,7 +248,7 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
     cl.sync();  // every block has its copy (and started: its shared memory may be written)
 
     // FP64 form of the pair term of atoms i (at p, current position x0) and
-    // j0 + t, with the far field; for what the integer forms leave out
+    // j0 + t, with the far field; for the pairs that the integer forms leave out
     auto pair_plain = [&](int i, const double *p, const double *x0, int t) -> double {
         const int j = j0 + t;
         const double dx = V[3 * j] - p[0], dy = V[3 * j + 1] - p[1], dz = V[3 * j + 2] - p[2];
@@ -249,7 +256,7 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
         const double qq = c.qs[i] * c.qs[j];
         const double c6 = c.pard[i].x * c.pard[j].x, c12 = c.pard[i].y * c.pard[j].y;
         const double lj = ri6 * (c12 * ri6 - c6) * (1.0 / 6.0);
-        if (a.taylor_r2 > 0.0) {
+        if (GEN && a.taylor_r2 > 0.0) {
             const double ex = V[3 * j] - x0[0], ey = V[3 * j + 1] - x0[1], ez = V[3 * j + 2] - x0[2];
             const double r02 = ex * ex + ey * ey + ez * ez;
             if (r02 >= a.taylor_r2) {
@@ -258,6 +265,67 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
             }
         }
         return qq * ri + lj;
+    };
+
+    // the linearised far field of atom j about the moving atom's current position
+    // x0: Coulomb energy e0 + fac (d . displacement), d = x_j - x0; false: near
+    auto far_field = [&](const double *x0, int j, double w1, double (&d)[3], double &e0, double &fac) -> bool {
+        if (!(a.taylor_r2 > 0.0)) return false;
+        for (int k = 0; k < 3; k++) d[k] = V[3 * j + k] - x0[k];
+        const double r02 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        if (!(r02 >= a.taylor_r2)) return false;
+        Inv64 v;
+        if (inv64(d[0], d[1], d[2], v)) {
+            e0 = w1 * inv64_r1(v);
+            fac = e0 * inv64_r2(v);
+        } else {
+            e0 = w1 * rsqrt(r02);
+            fac = e0 / r02;
+        }
+        return true;
+    };
+    // plain terms of one pair at the positions of a mask
+    auto plain_rows = [&](int i, const double *x0, int t, unsigned mask, double (&acc)[8]) {
+#pragma unroll 1
+        for (int q = 0; q < 7; q++) {
+            if (!((mask >> q) & 1u)) continue;
+            const double e = pair_plain(i, pos[q], x0, t);
+#pragma unroll
+            for (int k = 0; k < 7; k++)
+                if (k == q) acc[k] += e;
+        }
+    };
+    // GEN: the 7 rows of one pair, 9 FP64 differences (the positions share two
+    // coordinates of three) and 21 accumulations
+    auto general_rows = [&](int i, const double *x0, int t, double w1, double w6, double w12, double (&acc)[8]) {
+        const int j = j0 + t;
+        double e0, fac, ex[3];
+        const bool far = far_field(x0, j, w1, ex, e0, fac);
+        double d0[3], dp[3], dm[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const double x = V[3 * j + k];
+            d0[k] = x - pos[0][k];
+            dp[k] = x - pos[1 + 2 * k][k];
+            dm[k] = x - pos[2 + 2 * k][k];
+        }
+        unsigned out = 0u;
+#pragma unroll
+        for (int q = 0; q < 7; q++) {
+            double d[3] = {d0[0], d0[1], d0[2]};
+            const int k = q > 0 ? (q - 1) / 2 : 0;
+            if (q > 0) d[k] = q & 1 ? dp[k] : dm[k];
+            Inv64 v;
+            if (!inv64(d[0], d[1], d[2], v)) {
+                out |= 1u << q;
+                continue;
+            }
+            if (far) acc[q] += q > 0 ? e0 + fac * (ex[k] * (pos[q][k] - x0[k])) : e0;
+            else acc[q] = fma(w1, inv64_r1(v), acc[q]);
+            acc[q] = fma(w6, inv64_r6(v), acc[q]);
+            acc[q] = fma(w12, inv64_r12(v), acc[q]);
+        }
+        if (out) plain_rows(i, x0, t, out, acc);
     };
 
     for (int m = 0; m < moves; m++) {
@@ -274,11 +342,18 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
         const double qi = c.qs[i], c6i = c.pard[i].x * (1.0 / 6.0), c12i = c.pard[i].y * (1.0 / 6.0);
         __syncthreads();
         const double x0[3] = {pos[0][0], pos[0][1], pos[0][2]};
-        const bool slow = s_slow || !in_fix(x0);
+        const bool fix = !GEN && in_fix(x0);
         // ---- the 7 rows
         if (w < MV_PAIR_WARPS) {
             double acc[8] = {};
-            if (w * 32 < nj && !slow) {
+            if (GEN) {
+                for (int t = w * 32 + lane; t < nj; t += 32 * MV_PAIR_WARPS) {
+                    const int j = j0 + t;
+                    if (j == i) continue;
+                    general_rows(i, x0, t, qi * (SH ? pq[t] : c.qs[j]), -(c6i * (SH ? p6[t] : c.pard[j].x)),
+                                 c12i * (SH ? p12[t] : c.pard[j].y), acc);
+                }
+            } else if (w * 32 < nj && fix) {
                 long long f0[3], fp[3], fm[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
@@ -298,12 +373,8 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
                         sm[k] = abs64(x - fm[k]);
                         any |= s0[k];
                     }
-                    if (!(any >> 53)) {  // closer than 1/2 A along every axis
-#pragma unroll 1
-                        for (int q = 0; q < 7; q++) {
-                            const double e = pair_plain(i, pos[q], x0, t);
-                            for (int k = 0; k < 7; k++) acc[k] += k == q ? e : 0.0;
-                        }
+                    if ((unsigned)(any >> 53) - 1u >= 511u) {  // closer than 1/2 A along every axis, or MV_FAR
+                        plain_rows(i, x0, t, 127u, acc);
                         continue;
                     }
                     const double w1 = qi * (SH ? pq[t] : c.qs[j]);
@@ -331,15 +402,9 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
                         acc[q] = fma(w12, inv64_r12(v), acc[q]);
                     }
                 }
-            } else if (slow) {
+            } else if (!fix) {  // an atom beyond the range moves
                 for (int t = w * 32 + lane; t < nj; t += 32 * MV_PAIR_WARPS)
-                    if (j0 + t != i) {
-#pragma unroll 1
-                        for (int q = 0; q < 7; q++) {
-                            const double e = pair_plain(i, pos[q], x0, t);
-                            for (int k = 0; k < 7; k++) acc[k] += k == q ? e : 0.0;
-                        }
-                    }
+                    if (j0 + t != i) plain_rows(i, x0, t, 127u, acc);
             }
             __syncwarp();
             double s = 0.0;
@@ -387,20 +452,28 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
         if (w < MV_PAIR_WARPS) {
             if (w * 32 < nj) {
                 long long f[3];
-                const bool fit = !slow && in_fix(pv);
+                const bool fit = fix && in_fix(pv);
 #pragma unroll
                 for (int k = 0; k < 3; k++) fix64(pv[k], f[k]);
                 for (int t = w * 32 + lane; t < nj; t += 32 * MV_PAIR_WARPS) {
                     const int j = j0 + t;
                     if (j == i) continue;
+                    const double w1 = qi * (SH ? pq[t] : c.qs[j]);
                     Inv64 v;
                     u64 ax, ay, az;
                     int nz;
-                    if (!fit || !inv64_fix(F[3 * t] - f[0], F[3 * t + 1] - f[1], F[3 * t + 2] - f[2], v, ax, ay, az, nz)) {
+                    if (GEN ? !inv64(V[3 * j] - pv[0], V[3 * j + 1] - pv[1], V[3 * j + 2] - pv[2], v)
+                            : (!fit ||
+                               !inv64_fix(F[3 * t] - f[0], F[3 * t + 1] - f[1], F[3 * t + 2] - f[2], v, ax, ay, az, nz) ||
+                               nz == 0)) {  // nz: MV_FAR
                         e += pair_plain(i, pv, x0, t);
                         continue;
                     }
-                    e = fma(qi * (SH ? pq[t] : c.qs[j]), inv64_r1(v), e);
+                    double e0, fac, d[3];
+                    if (GEN && far_field(x0, j, w1, d, e0, fac))
+                        e += e0 + fac * (d[0] * (pv[0] - x0[0]) + d[1] * (pv[1] - x0[1]) + d[2] * (pv[2] - x0[2]));
+                    else
+                        e = fma(w1, inv64_r1(v), e);
                     e = fma(-(c6i * (SH ? p6[t] : c.pard[j].x)), inv64_r6(v), e);
                     e = fma(c12i * (SH ? p12[t] : c.pard[j].y), inv64_r12(v), e);
                 }
@@ -450,8 +523,9 @@ __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
                 const double x = pos[best][lane];
                 V[3 * i + lane] = x;
                 if (i >= j0 && i < j0 + nj) {
-                    fix64(x, F[3 * (i - j0) + lane]);
-                    if (!(fabs(x) < MV_FIX_MAX)) s_slow = 1;
+                    long long f;
+                    fix64(x, f);
+                    F[3 * (i - j0) + lane] = fabs(x) < MV_FIX_MAX ? f : MV_FAR;
                 }
             }
         }
@@ -491,10 +565,38 @@ int64_t moves_view_doubles(int n, int parts, int cs) {
     return moves_smem(n, cs) ? 0 : (int64_t)parts * cs * (3 * (int64_t)n + 3 * ((n + cs - 1) / cs));
 }
 
-cudaError_t launch_moves64(const Ctx &c, const MovesArgs &a, int parts, int cs, cudaStream_t s) {
+// whether a run takes the GEN rows; x: the positions, on the host.  A pair with
+// an atom beyond the range costs the fixed-point rows a plain evaluation, so a
+// few such atoms (one that a move has thrown out) are no reason
+bool moves_general(const double *x, int n, double delta, double taylor_r2) {
+    if (!(delta <= MV_DELTA_MAX) || taylor_r2 > 0.0) return true;
+    int far = 0;
+    for (int i = 0; i < n; i++) {
+        const double *p = x + 3 * (size_t)i;
+        far += !(std::fabs(p[0]) < MV_FIX_MAX && std::fabs(p[1]) < MV_FIX_MAX && std::fabs(p[2]) < MV_FIX_MAX);
+    }
+    return far > n / 256;
+}
+
+// Whether a sequential search of n atoms moves by launches over all SMs
+// (parab.cu) instead of on one cluster: a move there costs two launches however
+// small it is, here the time of eight SMs.  Us a move there, fixed-point rows, GEN
+// (offset 0.3 A), and with the far field there and GEN: 7,000 atoms 32, 17, 27, and
+// 37, 33; 10,000 36, 22, 35, and 39, 45; 14,000 34, 26, 44, and 38, 56; 30,000 54, 46,
+// 86, and 62, 111; 60,000 70, 82, 164, and 85, 214.
+bool moves_on_grid(int n, bool gen) { return n > (gen ? 8000 : 40000); }
+
+template <bool SH>
+static cudaError_t launch_moves(const Ctx &c, const MovesArgs &a, bool gen, const cudaLaunchConfig_t &cfg) {
+    return gen ? cudaLaunchKernelEx(&cfg, k_moves64<SH, true>, c, a) : cudaLaunchKernelEx(&cfg, k_moves64<SH, false>, c, a);
+}
+
+cudaError_t launch_moves64(const Ctx &c, const MovesArgs &a, bool gen, int parts, int cs, cudaStream_t s) {
     const size_t smem = moves_smem(a.n, cs);
     cudaError_t e = cudaSuccess;
-    if (smem) e = cudaFuncSetAttribute(k_moves64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MV_SMEM);
+    if (smem)
+        e = cudaFuncSetAttribute(gen ? k_moves64<true, true> : k_moves64<true, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MV_SMEM);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(parts * cs);
@@ -507,7 +609,7 @@ cudaError_t launch_moves64(const Ctx &c, const MovesArgs &a, int parts, int cs, 
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return smem ? cudaLaunchKernelEx(&cfg, k_moves64<true>, c, a) : cudaLaunchKernelEx(&cfg, k_moves64<false>, c, a);
+    return smem ? launch_moves<true>(c, a, gen, cfg) : launch_moves<false>(c, a, gen, cfg);
 }
 
 }  // namespace ffm

@@ -15,11 +15,13 @@
 // SplitMix64 stream (Steele, Lea and Flood 2014) with the user's seed, scaled
 // to [0, N) by a 64x64 -> 128-bit multiply (high word).
 //
-// This file: FP32 terms (MIXED objects); moves.cu has the FP64 ones.  A move
-// costs two launches over all j (7 rows, then the vertex row); the last block
-// of each launch reduces the block partials in a fixed order and takes the
-// move's decision, so the moves of a sweep replay as a CUDA graph with no
-// host involvement.
+// This file: FP32 terms (MIXED objects), and the sequential search with FP64
+// terms for systems that keep a cluster of eight SMs busy for longer than two
+// launches over all of them take (see moves_on_grid); moves.cu has the other
+// FP64 moves.  A move costs two launches over all j (7 rows, then the vertex
+// row); the last block of each launch reduces the block partials in a fixed
+// order and takes the move's decision, so the moves of a sweep replay as a CUDA
+// graph with no host involvement.
 #include <cmath>
 #include <cstring>
 
@@ -98,13 +100,51 @@ __device__ void row_sums(const float4 *posf, const float2 *parf, int n, int i, c
     }
 }
 
-// the grid's share of one row evaluation over the system's atoms
+// the same with FP64 terms
 template <int NP>
+__device__ void row_sums64(const double4_32a *pos, const double2 *par, int n, int i, const double (*p)[3],
+                           const double *xi, double tr2, int j0, int stride, double *acc) {
+    for (int q = 0; q < NP; q++) acc[q] = 0.0;
+    const double qi = pos[i].w;
+    const double2 ci = par[i];
+    for (int j = j0; j < n; j += stride) {
+        if (j == i) continue;
+        const double4_32a pj = pos[j];
+        const double2 cj = par[j];
+        const double c6 = ci.x * cj.x, c12 = ci.y * cj.y, qq = qi * pj.w;
+        bool far = false;
+        double e0 = 0.0, fac = 0.0;
+        const double ex = pj.x - xi[0], ey = pj.y - xi[1], ez = pj.z - xi[2];
+        if (tr2 > 0.0) {
+            const double r02 = ex * ex + ey * ey + ez * ez;
+            if (r02 >= tr2) {
+                far = true;
+                e0 = qq * rsqrt(r02);
+                fac = e0 / r02;
+            }
+        }
+        for (int q = 0; q < NP; q++) {
+            const double dx = pj.x - p[q][0], dy = pj.y - p[q][1], dz = pj.z - p[q][2];
+            const double ri = rsqrt(dx * dx + dy * dy + dz * dz);
+            const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
+            const double lj = ri6 * (c12 * ri6 - c6) * (1.0 / 6.0);
+            if (far) {  // a branch: selected, its FP64 work took 10 % of every exact row
+                const double dd = ex * (p[q][0] - xi[0]) + ey * (p[q][1] - xi[1]) + ez * (p[q][2] - xi[2]);
+                acc[q] += e0 + fac * dd + lj;
+            } else {
+                acc[q] += qq * ri + lj;
+            }
+        }
+    }
+}
+
+// the grid's share of one row evaluation over the system's atoms
+template <int NP, bool F64>
 __device__ void row_partial(const Ctx &c, const ParabState *ps, int i, const double (*p)[3], const double *xi,
                             double *acc) {
-    const int a0 = ps->atom0;
-    row_sums<NP>(c.posf + a0, c.parf + a0, ps->n, i, p, xi, ps->taylor_r2, blockIdx.x * blockDim.x + threadIdx.x,
-                 gridDim.x * blockDim.x, acc);
+    const int a0 = ps->atom0, j0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (F64) row_sums64<NP>(c.posd + a0, c.pard + a0, ps->n, i, p, xi, ps->taylor_r2, j0, stride, acc);
+    else row_sums<NP>(c.posf + a0, c.parf + a0, ps->n, i, p, xi, ps->taylor_r2, j0, stride, acc);
 }
 
 // bonded terms containing atom i (global index a) with atom i at p
@@ -119,6 +159,7 @@ __device__ double row_bonded(const Ctx &c, int a, const double *p) {
 }
 
 // 7 row energies: current position and +-delta along x, y, z
+template <bool F64>
 __global__ void __launch_bounds__(TI) k_parab_rows(Ctx c, ParabState *ps) {
     if (ps->move >= ps->stop_at) return;
     const int n = ps->n, atom0 = ps->atom0;
@@ -132,7 +173,7 @@ __global__ void __launch_bounds__(TI) k_parab_rows(Ctx c, ParabState *ps) {
         p[2 + 2 * a][a] = p[2 + 2 * a][a] - ps->delta;
     }
     double acc[7];
-    row_partial<7>(c, ps, i, p, p[0], acc);  // p[0]: the current position
+    row_partial<7, F64>(c, ps, i, p, p[0], acc);  // p[0]: the current position
     double v[7];
     for (int q = 0; q < 7; q++) v[q] = acc[q];
     block_reduce_store<7>(v, 0u, &c.red[(int64_t)blockIdx.x * NRED]);
@@ -162,13 +203,14 @@ __global__ void __launch_bounds__(TI) k_parab_rows(Ctx c, ParabState *ps) {
 }
 
 // the vertex row, the decision and the move
+template <bool F64>
 __global__ void __launch_bounds__(TI) k_parab_vertex(Ctx c, ParabState *ps) {
     if (ps->move >= ps->stop_at) return;
     const int atom0 = ps->atom0, i = ps->atom;
     double p[1][3];
     for (int a = 0; a < 3; a++) p[0][a] = ps->p[7][a];
     double acc[1];
-    row_partial<1>(c, ps, i, p, ps->p[0], acc);  // ps->p[0]: the current position
+    row_partial<1, F64>(c, ps, i, p, ps->p[0], acc);  // ps->p[0]: the current position
     double v[1] = {acc[0]};
     block_reduce_store<1>(v, 0u, &c.red[(int64_t)blockIdx.x * NRED]);
     if (!last_block(&c.counters[CNT_PARAB2])) return;
@@ -184,7 +226,8 @@ __global__ void __launch_bounds__(TI) k_parab_vertex(Ctx c, ParabState *ps) {
         double *X = vslot(c, V_X);
         for (int k = 0; k < 3; k++) X[3 * a + k] = ps->p[best][k];
         const double q = c.qs[a];
-        c.posf[a] = make_float4((float)X[3 * a], (float)X[3 * a + 1], (float)X[3 * a + 2], (float)q);
+        if (F64) c.posd[a] = make_double4_32a(X[3 * a], X[3 * a + 1], X[3 * a + 2], q);
+        else c.posf[a] = make_float4((float)X[3 * a], (float)X[3 * a + 1], (float)X[3 * a + 2], (float)q);
         ps->move = ps->move + 1;
         __threadfence();
         c.counters[CNT_PARAB2] = 0;
@@ -192,10 +235,13 @@ __global__ void __launch_bounds__(TI) k_parab_vertex(Ctx c, ParabState *ps) {
 }
 
 cudaError_t launch_parab_move(const Ctx &c, ParabState *ps, int grid, cudaStream_t s) {
-    k_parab_rows<<<grid, TI, 0, s>>>(c, ps);
+    const bool f64 = c.prec != FFMIN_MIXED;
+    if (f64) k_parab_rows<true><<<grid, TI, 0, s>>>(c, ps);
+    else k_parab_rows<false><<<grid, TI, 0, s>>>(c, ps);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_parab_vertex<<<grid, TI, 0, s>>>(c, ps);
+    if (f64) k_parab_vertex<true><<<grid, TI, 0, s>>>(c, ps);
+    else k_parab_vertex<false><<<grid, TI, 0, s>>>(c, ps);
     return cudaGetLastError();
 }
 
