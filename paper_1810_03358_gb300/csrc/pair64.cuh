@@ -8,10 +8,13 @@
 // significands with separate exponents, the terms of a pair are added as
 // integers, and the results rounded once to FP64; FP64 instructions remain for
 // the accumulation (7 a pair with forces, 3 for an energy) and, outside the
-// fixed-point range, for the coordinate differences (3 more).  Every
-// significand below is good to 2^-57 or better and is rounded to 53 bits at
-// the end, so a term's error is no larger than that of the FP64 formula,
-// whose own roundings (each 2^-53) add up.
+// fixed-point range, for the coordinate differences (3 more).  The relative
+// errors of the significands (largest of millions of differences, host side,
+// against long double) are 2^-56.8 for r^-1, 2^-55.8 for r^-2, 2^-54.2 for r^-6 and
+// 2^-53.2 for r^-12 (each product's cuts and the power's multiple of r^-1's), and
+// a result is rounded to 53 bits once, so a term is within two units of 2^-53,
+// where the roundings of the FP64 formula (2^-53 each, raised to the same powers)
+// add up to more.
 //
 // r^-1 from the hardware's approximate FP32 reciprocal square root y and one
 // step of the series (1 - h)^(-1/2) = 1 + h/2 + 3 h^2/8 + O(h^3) with
