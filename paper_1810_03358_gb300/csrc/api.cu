@@ -640,6 +640,7 @@ ffmin_status ffmin_create(const ffmin_topology *tops, int32_t n_sys, int32_t pre
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sys->sms, cudaDevAttrMultiProcessorCount, dev);
+        sys->c.sms = sys->sms;
     }
     sys->grid_sym = pair_grid_size(2);
     for (int k = 0; k < 2; k++) {

@@ -174,6 +174,7 @@ struct Ctx {
     int64_t vstride;
     int32_t prec;           // ffmin_precision
     int32_t cl64;           // FP64 symmetric kernel: blocks per item (clusters; host-side dispatch)
+    int32_t sms;            // SMs of the device (host-side dispatch)
     int32_t f32_ipt;        // FP32 pair-kernel shape: i-atoms per thread (1 or 2; host-side dispatch)
     const Tile *tiles;
     const Item *items;

@@ -129,7 +129,6 @@ cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) 
 constexpr int FIN_STRANDS = 4;
 constexpr int FIN_CLUSTER = TI / 32;
 constexpr int FIN_NT = 32 * (FIN_STRANDS + 2);
-constexpr int FIN_DENSE_TILES = 152;  // k_finalize<6> above it
 
 // exact FP32 -> FP64 on the integer pipe (the conversion instruction runs at
 // the FP64 rate); the FP32 kernels flush denormals, which read as zero
@@ -704,7 +703,7 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out) {
-    if (c.n_tiles > FIN_DENSE_TILES) k_finalize<6><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
+    if (c.n_tiles > c.sms) k_finalize<6><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
     else k_finalize<4><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
     return cudaGetLastError();
 }
