@@ -46,7 +46,10 @@ constexpr int MLP_CLUSTER = FFMIN_MLP_CLUSTER;  // blocks per cluster
 #endif
 constexpr int MLP_CLUSTERS = FFMIN_MLP_CLUSTERS;
 constexpr int MLP_NV = MLP_NW + 1;                    // summed values: the gradient, the loss
-constexpr int MLP_STEPS = 4096;   // steps per launch (their losses wait in the scratch)
+#ifndef FFMIN_MLP_STEPS
+#define FFMIN_MLP_STEPS 4096
+#endif
+constexpr int MLP_STEPS = FFMIN_MLP_STEPS;  // steps per launch (their losses wait in the scratch)
 // polls of the grid barrier before a block gives up (about a second)
 #ifndef FFMIN_MLP_POLLS
 #define FFMIN_MLP_POLLS (1 << 22)

@@ -8,6 +8,10 @@ while blocks of the same cluster that poll later see the count complete.  The
 call reports the timeout, the weights are those of some step (a step moves a
 weight by at most about lr), and the context still computes what it did.
 
+Runs of several launches (more than 4,096 steps): weights, moments, the sample
+stream and the bias corrections go on where the launch before ended, so the
+losses and weights have the bits of one launch, and of launches of seven steps.
+
 A grid that is not resident at once: with 64 clusters (512 blocks, of which the
 SMs hold two each) the first launch is refused, and the call goes on with fewer
 clusters; so it goes where a process has a share of the SMs, down to blocks
@@ -126,3 +130,15 @@ def test_largest_batch(ff):
     assert int(big.sum()) > 100
     assert (step + lr * sign)[big].abs().max() <= 1e-3 * lr
     assert step[y.grad == 0].abs().max() == 0.0
+
+
+@pytest.mark.parametrize("steps,split", [(4100, 8192), (50, 7)])
+def test_runs_of_several_launches(ff, variant, steps, split):
+    feat, target = inputs(5000)
+    one, two = fresh(ff), fresh(ff)
+    st, la = variant(FFMIN_MLP_STEPS=split)(feat, target, steps, 300, 1e-3, 21, *one)
+    lb = ff.ffmin_mlp_train(feat, target, steps, 300, 1e-3, 21, *two)
+    assert st == ff.FFMIN_OK and np.isfinite(la).all() and la[-5:].mean() < la[:5].mean()
+    assert np.array_equal(la, lb)
+    for a, b in zip(one[:2], two[:2]):
+        assert torch.equal(a, b)
