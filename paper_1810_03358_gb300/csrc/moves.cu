@@ -19,7 +19,7 @@
 // warps of their own, one per kind, lane = (term, position), in forms of their
 // own: 10 instructions for a bond, about 35 for an angle, 45 for a torsion.
 // 500 atoms: 66 us a move as two launches, 16 us with the terms in plain FP64
-// and a warp per position, 9.2 us now.
+// and a warp per position, 8.7 us now; 3,334 atoms 68 and 14.3 us.
 //
 // This file is compiled without implicit contraction (as parab.cu), so that
 // positions and the far-field test round like their statements.
@@ -201,9 +201,11 @@ __device__ __forceinline__ bool in_fix(const double *x) {
 // SH: positions and this block's share of the parameters in shared memory;
 // otherwise a private copy in global memory and the object's arrays.
 // GEN: rows from FP64 differences, for what the fixed-point rows leave out: a
-// larger offset, the far field, systems beyond the range.  A kernel of its own,
-// since its code beside the other rows cost those 3 % (4.54 -> 4.71 ms for 500
-// moves of 500 atoms).
+// larger offset, the far field, systems beyond the range.  Nine FP64 instructions
+// more for an atom's 7 rows (with the far field about 35), and the alignment of
+// the significands: 3,334 atoms 19.4 us a move (22.6), 41 (70) in plain FP64 terms.
+// A kernel of its own, since its code beside the other rows cost those 3 % (4.54
+// -> 4.71 ms for 500 moves of 500 atoms).
 template <bool SH, bool GEN>
 __global__ void __launch_bounds__(MV_THREADS, 1) k_moves64(Ctx c, MovesArgs a) {
     cg::cluster_group cl = cg::this_cluster();

@@ -462,12 +462,13 @@ __device__ __forceinline__ int next_item(const Ctx &c, const int2 *items, unsign
 // FP32 shapes: two i-atoms per thread (64-thread blocks: every j load from
 // shared memory serves two pairs) or one (128-thread blocks: twice the warps
 // per work item, which pays when an object has few items); the autotuner
-// picks one per object.  Register caps: the FP32 E + grad kernel runs 832
-// threads per SM (13 blocks of 64 or 6 of 128, 72 registers or 80), the FP32
-// energy kernel 512 (128 registers: a difference trial keeps more values).  At
-// 30,000 atoms with 512, 640, 768, 832, 896 threads: E + grad 744, 711, 682, 667,
-// 668 us; with 512, 640, 768, 896 difference trials 500, 532, 531, 537 us and
-// plain energies 231, 223, 228, 232 us;
+// picks one per object.  Register caps: the FP32 E + grad kernel is compiled
+// for 832 threads per SM (13 blocks of 64, whose 72 registers let 14 be
+// resident, or 6 of 128 with 80; it spills 148 bytes), the FP32
+// energy kernel for 512 (128 registers: a difference trial keeps more values).  At
+// 30,000 atoms with 512, 640, 768, 832 threads: E + grad 744, 711, 682, 667
+// us (896 is the same kernel in blocks of 64); with 512, 640, 768, 896 difference
+// trials 500, 532, 531, 537 us and plain energies 231, 223, 228, 232 us;
 // a minimization takes difference trials.  At 3,334 they are within 2 %, but
 // trials with 768 are 10 % slower.  With exclusions E + grad runs 640 (1,000
 // atoms 3 % faster than with 768, 20,000 the same).  The FP64 kernel runs 8 blocks of 128 (64

@@ -54,50 +54,48 @@ __device__ __forceinline__ int pick_atom(uint64_t seed, uint64_t k, int n) {
 template <int NP>
 __device__ void row_sums(const float4 *posf, const float2 *parf, int n, int i, const double (*p)[3],
                          const double *xi, double tr2, int j0, int stride, double *acc) {
-    {
-        const float qi = posf[i].w;
-        const float2 ci = parf[i];
-        float pf[NP][3], accf[NP];
-        for (int q = 0; q < NP; q++) {
-            accf[q] = 0.f;
-            for (int a = 0; a < 3; a++) pf[q][a] = (float)p[q][a];
-        }
-        const float xf[3] = {(float)xi[0], (float)xi[1], (float)xi[2]};
-        const float tr2f = (float)tr2;
-        // FP32 sums of this thread's j (tile-local FP32 accumulation of the
-        // mixed form), FP64 from the block reduction on
-        for (int j = j0; j < n; j += stride) {
-            if (j == i) continue;
-            const float4 pj = posf[j];
-            const float2 cj = parf[j];
-            const float c6 = ci.x * cj.x, c12 = ci.y * cj.y, qq = qi * pj.w;
-            bool far = false;
-            float e0 = 0.f, fac = 0.f;
-            const float d0x = pj.x - xf[0], d0y = pj.y - xf[1], d0z = pj.z - xf[2];
-            if (tr2f > 0.f) {
-                const float r02 = d0x * d0x + d0y * d0y + d0z * d0z;
-                if (r02 >= tr2f) {
-                    far = true;
-                    e0 = qq * rsqrtf(r02);
-                    fac = e0 / r02;
-                }
-            }
-            for (int q = 0; q < NP; q++) {
-                const float dx = pj.x - pf[q][0], dy = pj.y - pf[q][1], dz = pj.z - pf[q][2];
-                const float r2 = dx * dx + dy * dy + dz * dz;
-                const float ri = rsqrtf(r2);
-                const float ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
-                const float lj = ri6 * (c12 * ri6 - c6) * (1.0f / 6.0f);
-                if (far) {
-                    const float dd = d0x * (pf[q][0] - xf[0]) + d0y * (pf[q][1] - xf[1]) + d0z * (pf[q][2] - xf[2]);
-                    accf[q] += e0 + fac * dd + lj;
-                } else {
-                    accf[q] += qq * ri + lj;
-                }
-            }
-        }
-        for (int q = 0; q < NP; q++) acc[q] = (double)accf[q];
+    const float qi = posf[i].w;
+    const float2 ci = parf[i];
+    float pf[NP][3], accf[NP];
+    for (int q = 0; q < NP; q++) {
+        accf[q] = 0.f;
+        for (int a = 0; a < 3; a++) pf[q][a] = (float)p[q][a];
     }
+    const float xf[3] = {(float)xi[0], (float)xi[1], (float)xi[2]};
+    const float tr2f = (float)tr2;
+    // FP32 sums of this thread's j (tile-local FP32 accumulation of the
+    // mixed form), FP64 from the block reduction on
+    for (int j = j0; j < n; j += stride) {
+        if (j == i) continue;
+        const float4 pj = posf[j];
+        const float2 cj = parf[j];
+        const float c6 = ci.x * cj.x, c12 = ci.y * cj.y, qq = qi * pj.w;
+        bool far = false;
+        float e0 = 0.f, fac = 0.f;
+        const float d0x = pj.x - xf[0], d0y = pj.y - xf[1], d0z = pj.z - xf[2];
+        if (tr2f > 0.f) {
+            const float r02 = d0x * d0x + d0y * d0y + d0z * d0z;
+            if (r02 >= tr2f) {
+                far = true;
+                e0 = qq * rsqrtf(r02);
+                fac = e0 / r02;
+            }
+        }
+        for (int q = 0; q < NP; q++) {
+            const float dx = pj.x - pf[q][0], dy = pj.y - pf[q][1], dz = pj.z - pf[q][2];
+            const float r2 = dx * dx + dy * dy + dz * dz;
+            const float ri = rsqrtf(r2);
+            const float ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
+            const float lj = ri6 * (c12 * ri6 - c6) * (1.0f / 6.0f);
+            if (far) {
+                const float dd = d0x * (pf[q][0] - xf[0]) + d0y * (pf[q][1] - xf[1]) + d0z * (pf[q][2] - xf[2]);
+                accf[q] += e0 + fac * dd + lj;
+            } else {
+                accf[q] += qq * ri + lj;
+            }
+        }
+    }
+    for (int q = 0; q < NP; q++) acc[q] = (double)accf[q];
 }
 
 // the same with FP64 terms
