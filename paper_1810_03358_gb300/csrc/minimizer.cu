@@ -115,7 +115,8 @@ cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) 
 // ---------------------------------------------------------------- finalize
 // Bound: latency (a chain of about ten loads, barriers and short FP64 sums; an
 // FP64 operation holds a quarter of an SM for 64 cycles however few of its
-// lanes are on).  A tile is a cluster of four blocks, 32 atoms each: warp w < 4
+// lanes are on).  A tile is a cluster of four blocks, 32 atoms each (or one block,
+// 32 atoms after 32): warp w < 4
 // sums the atoms' partial rows w, w + 4, ... (strand w; combined as
 // (0 + 1) + (2 + 3)), warps 4 and 5 gather their bonded terms, then one warp
 // finishes each component; the first block receives the atoms' contributions
@@ -127,7 +128,7 @@ cudaError_t launch_prepare_eval(const Ctx &c, const EvalReq &r, cudaStream_t s) 
 // block_reduce_columns, then the tiles): a MIXED minimization amplifies any
 // other rounding.
 constexpr int FIN_STRANDS = 4;
-constexpr int FIN_CLUSTER = TI / 32;
+constexpr int FIN_PARTS = TI / 32;
 constexpr int FIN_NT = 32 * (FIN_STRANDS + 2);
 
 // exact FP32 -> FP64 on the integer pipe (the conversion instruction runs at
@@ -221,25 +222,29 @@ __device__ __forceinline__ int fin_value(int k) {
     return k == 0 ? RF_E : (k == 1 ? RF_EPAIR : (k == 2 ? RF_GG : (k == 3 ? RF_GTG : RF_GTR)));
 }
 
-// BLOCKS: resident blocks per SM, 4 (80 registers, the shortest chain) or 6 (56
-// registers) for objects of more tiles than SMs, which run in waves.  Us with 4
-// and 6: 79 tiles 19.7, 19.8 (with gradient) and 11.7, 14.1; 157 tiles 33.9, 29.8
-// and 17.3, 17.1; batches, 13 rounds: 119 tiles 193, 193; 186 tiles 246, 216; 399
-// tiles 362, 331; 1,533 tiles (16 rounds) 1,007, 860.
-template <int BLOCKS>
-__global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT, BLOCKS) k_finalize(Ctx c, double *g_out) {
-    const int tile = blockIdx.x / FIN_CLUSTER, rank = blockIdx.x % FIN_CLUSTER;
+// CS: blocks per tile, four, or one that takes the tile's 32 atoms in turn, for
+// objects of so many tiles that only the work of a block counts (its chain of
+// loads, the state that it fetches, its ticket).  BLOCKS: resident blocks per SM, 4
+// (80 registers, the shortest chain), 6 (56) for objects of more tiles than SMs,
+// which run in waves, or 8 (40).  Us with 4 and 6 blocks of four per tile: 79 tiles
+// 19.7, 19.8 (with gradient) and 11.7, 14.1; 157 tiles 33.9, 29.8 and 17.3, 17.1.
+// Whole L-BFGS runs of batches, MIXED, ms, with four per tile at 6, one per tile at 6
+// and at 8: 660 tiles 6.08, 6.13, 6.19; 1,024 tiles (500 atoms each) 8.85, 8.89, 8.39,
+// (2,000) 11.19, 11.28, 10.78, (60) 11.99, 11.02, 10.29; 4,096 tiles 30.5, 28.8, 28.2.
+template <int CS, int BLOCKS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(FIN_NT, BLOCKS) k_finalize(Ctx c, double *g_out) {
+    const int tile = blockIdx.x / CS, rank = blockIdx.x % CS;
     const Tile &t = c.tiles[tile];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;  // w: strand, then bonded terms
-    const int i = 32 * rank + lane, a = t.a0 + i;
-    const bool real = i < t.na;
+    int i = 32 * rank + lane, a = t.a0 + i;
+    bool real = i < t.na;
     constexpr int NSUM = 5;  // E, Epair and, with a gradient, g.g, g.G, g.R
     __shared__ double part[FIN_STRANDS][4][32], bond[2][4][32];
     __shared__ double sg[3 * 32], sr[3 * 32], sgt[3][32];  // current gradient, direction, new gradient
     // first block of the cluster: the tile's contributions
     __shared__ double val[NSUM][TI];
-    __shared__ unsigned long long gmax[3 * FIN_CLUSTER];
-    __shared__ int badf[4 * FIN_CLUSTER];
+    __shared__ unsigned long long gmax[3 * FIN_PARTS];
+    __shared__ int badf[4 * FIN_PARTS];
     __shared__ double strands[NSUM][RSTRANDS], tot[RF_N];
     __shared__ SysState sS;
     cg::cluster_group cl = cg::this_cluster();
@@ -254,110 +259,129 @@ __global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT, BL
     const SysState &S = c.st[t.sys];
     const int kind = S.ev_kind, mode = S.mode, ntile = S.ntile, tile0 = S.tile0;
     if (kind == EV_NONE) return;  // the whole cluster
-    auto started = cl.barrier_arrive();
+    cg::cluster_group::arrival_token started{};
+    if constexpr (CS > 1) started = cl.barrier_arrive();
     const bool grad = kind == EV_EG;
     if (rank == 0) prefetch_state(&sS, &S);
-    if (grad) {
-        const int64_t o = 3 * ((int64_t)t.a0 + 32 * rank);
-        const int n = 3 * min(32, max(0, t.na - 32 * rank));
-        for (int k = threadIdx.x; k < n; k += FIN_NT) {
-            async_copy8(&sg[k], vslot(c, V_G) + o + k);
-            async_copy8(&sr[k], vslot(c, V_R) + o + k);
-        }
-    }
-    if (w < FIN_STRANDS) {
-        Row4 r = Row4{0.0, 0.0, 0.0, 0.0};
-        if (real) {
-            if (mode == 0 && c.sym32 && !grad) {
-                // energies on the symmetric list, each pair counted once
-                const int C = t.r32.chunk, n = (ntile - t.tloc + C - 1) / C;
-                rows_f32(c.gpf_sym + ((int64_t)t.r32.slot + w) * TI + i, (n - w + 3) / FIN_STRANDS, r.w);
-            } else if (mode == 0) {
-                rows_f32(c.gpf + ((int64_t)t.item0 + w) * TI + i, (t.nitem - w + 3) / FIN_STRANDS, r);
-                r.w *= 0.5;  // every pair was counted in both of its rows
-            } else if (c.sym64) {
-                if (grad) sym_rows<true>(c, t, tile0, ntile, i, w, r);
-                else sym_rows<false>(c, t, tile0, ntile, i, w, r);
-            } else {
-                strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpd, t.item0 + it, i); });
-                r.w *= 0.5;
+    for (int part32 = rank;; part32 += CS) {  // 32 atoms of the tile
+        if (grad) {
+            const int64_t o = 3 * ((int64_t)t.a0 + 32 * part32);
+            const int n = 3 * min(32, max(0, t.na - 32 * part32));
+            for (int k = threadIdx.x; k < n; k += FIN_NT) {
+                async_copy8(&sg[k], vslot(c, V_G) + o + k);
+                async_copy8(&sr[k], vslot(c, V_R) + o + k);
             }
         }
-        part[w][0][lane] = r.x; part[w][1][lane] = r.y; part[w][2][lane] = r.z; part[w][3][lane] = r.w;
-    } else {
-        // evaluated once per term by the pair kernel's bonded items; an atom
-        // takes its terms' energies (as owner) and position gradients
-        Row4 bo = Row4{0.0, 0.0, 0.0, 0.0};
-        for (; kb < k1; kb += 2 * U) {
-            int2 in[U];
-            Row4 p[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) in[u] = kb + 2 * u < k1 ? c.inc[kb + 2 * u] : make_int2(-1, 0);
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int type = in[u].x >> 2, pos = in[u].x & 3;
-                if (in[u].x < 0) continue;
-                p[u].w = pos == 0 ? c.te[bonded_index(c, type, in[u].y)] : 0.0;
-                if (grad) {
-                    const double *g = c.tg + 3 * bonded_grad_slot(c, type, in[u].y, pos);
-                    p[u].x = g[0]; p[u].y = g[1]; p[u].z = g[2];
+        if (w < FIN_STRANDS) {
+            Row4 r = Row4{0.0, 0.0, 0.0, 0.0};
+            if (real) {
+                if (mode == 0 && c.sym32 && !grad) {
+                    // energies on the symmetric list, each pair counted once
+                    const int C = t.r32.chunk, n = (ntile - t.tloc + C - 1) / C;
+                    rows_f32(c.gpf_sym + ((int64_t)t.r32.slot + w) * TI + i, (n - w + 3) / FIN_STRANDS, r.w);
+                } else if (mode == 0) {
+                    rows_f32(c.gpf + ((int64_t)t.item0 + w) * TI + i, (t.nitem - w + 3) / FIN_STRANDS, r);
+                    r.w *= 0.5;  // every pair was counted in both of its rows
+                } else if (c.sym64) {
+                    if (grad) sym_rows<true>(c, t, tile0, ntile, i, w, r);
+                    else sym_rows<false>(c, t, tile0, ntile, i, w, r);
+                } else {
+                    strand_sum<true, true>(t.nitem, w, r, [&](int it) { return row_at(c.gpd, t.item0 + it, i); });
+                    r.w *= 0.5;
                 }
             }
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                if (in[u].x < 0) break;
-                if ((in[u].x & 3) == 0) bo.w += p[u].w;
-                if (grad) { bo.x += p[u].x; bo.y += p[u].y; bo.z += p[u].z; }
-            }
-        }
-        double (*b)[32] = bond[w - FIN_STRANDS];
-        b[0][lane] = bo.x; b[1][lane] = bo.y; b[2][lane] = bo.z; b[3][lane] = bo.w;
-    }
-    async_wait();
-    __syncthreads();
-    cl.barrier_wait(std::move(started));  // the first block's shared memory is there
-    double *tv = cl.map_shared_rank(&val[0][0], 0) + i;
-    auto finite = [](double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; };
-    if (w < 4 && (grad || w == 3)) {  // component w of the gradient, or the energy
-        double x = 0.0, q = 0.0;
-        if (real) {
-            q = (part[0][w][lane] + part[1][w][lane]) + (part[2][w][lane] + part[3][w][lane]);
-            x = q + (bond[0][w][lane] + bond[1][w][lane]);
-        }
-        const unsigned bad = __ballot_sync(0xffffffffu, !finite(x));
-        if (lane == 0) cl.map_shared_rank(badf, 0)[4 * rank + w] = bad != 0u;
-        if (w == 3) {
-            tv[0] = x;
-            tv[TI] = q;
+            part[w][0][lane] = r.x; part[w][1][lane] = r.y; part[w][2][lane] = r.z; part[w][3][lane] = r.w;
         } else {
-            sgt[w][lane] = x;
-            if (real) {
-                vslot(c, V_GT)[3 * (int64_t)a + w] = x;
-                if (g_out) g_out[3 * (int64_t)a + w] = x;
+            // evaluated once per term by the pair kernel's bonded items; an atom
+            // takes its terms' energies (as owner) and position gradients
+            Row4 bo = Row4{0.0, 0.0, 0.0, 0.0};
+            for (; kb < k1; kb += 2 * U) {
+                int2 in[U];
+                Row4 p[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) in[u] = kb + 2 * u < k1 ? c.inc[kb + 2 * u] : make_int2(-1, 0);
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int type = in[u].x >> 2, pos = in[u].x & 3;
+                    if (in[u].x < 0) continue;
+                    p[u].w = pos == 0 ? c.te[bonded_index(c, type, in[u].y)] : 0.0;
+                    if (grad) {
+                        const double *g = c.tg + 3 * bonded_grad_slot(c, type, in[u].y, pos);
+                        p[u].x = g[0]; p[u].y = g[1]; p[u].z = g[2];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (in[u].x < 0) break;
+                    if ((in[u].x & 3) == 0) bo.w += p[u].w;
+                    if (grad) { bo.x += p[u].x; bo.y += p[u].y; bo.z += p[u].z; }
+                }
             }
-            // the largest |component|, as an integer (a NaN counts as 0)
-            const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
-            const bool nan = hi > 0x7ff00000u || (hi == 0x7ff00000u && lo != 0u);
-            const unsigned mh = __reduce_max_sync(0xffffffffu, nan ? 0u : hi);
-            const unsigned ml = __reduce_max_sync(0xffffffffu, !nan && hi == mh ? lo : 0u);
-            if (lane == 0) cl.map_shared_rank(gmax, 0)[3 * rank + w] = (unsigned long long)mh << 32 | ml;
+            double (*b)[32] = bond[w - FIN_STRANDS];
+            b[0][lane] = bo.x; b[1][lane] = bo.y; b[2][lane] = bo.z; b[3][lane] = bo.w;
         }
-    }
-    if (grad) {
+        async_wait();
         __syncthreads();
-        if (w < 3) {
-            double x = 0.0;
+        if constexpr (CS > 1) cl.barrier_wait(std::move(started));  // the first block's shared memory is there
+        // the first block's shared memory
+        auto first = [&](auto *p) {
+            if constexpr (CS > 1) return cl.map_shared_rank(p, 0);
+            else return p;
+        };
+        double *tv = first(&val[0][0]) + i;
+        auto finite = [](double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; };
+        if (w < 4 && (grad || w == 3)) {  // component w of the gradient, or the energy
+            double x = 0.0, q = 0.0;
             if (real) {
-                const double g0 = sgt[0][lane], g1 = sgt[1][lane], g2 = sgt[2][lane];
-                const double *o = w == 1 ? sg : sr;
-                const double o0 = w == 0 ? g0 : o[3 * lane], o1 = w == 0 ? g1 : o[3 * lane + 1],
-                             o2 = w == 0 ? g2 : o[3 * lane + 2];
-                x = fma(g0, o0, fma(g1, o1, g2 * o2));
+                q = (part[0][w][lane] + part[1][w][lane]) + (part[2][w][lane] + part[3][w][lane]);
+                x = q + (bond[0][w][lane] + bond[1][w][lane]);
             }
-            tv[(2 + w) * TI] = x;
+            const unsigned bad = __ballot_sync(0xffffffffu, !finite(x));
+            if (lane == 0) first(&badf[0])[4 * part32 + w] = bad != 0u;
+            if (w == 3) {
+                tv[0] = x;
+                tv[TI] = q;
+            } else {
+                sgt[w][lane] = x;
+                if (real) {
+                    vslot(c, V_GT)[3 * (int64_t)a + w] = x;
+                    if (g_out) g_out[3 * (int64_t)a + w] = x;
+                }
+                // the largest |component|, as an integer (a NaN counts as 0)
+                const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+                const bool nan = hi > 0x7ff00000u || (hi == 0x7ff00000u && lo != 0u);
+                const unsigned mh = __reduce_max_sync(0xffffffffu, nan ? 0u : hi);
+                const unsigned ml = __reduce_max_sync(0xffffffffu, !nan && hi == mh ? lo : 0u);
+                if (lane == 0) first(&gmax[0])[3 * part32 + w] = (unsigned long long)mh << 32 | ml;
+            }
         }
+        if (grad) {
+            __syncthreads();
+            if (w < 3) {
+                double x = 0.0;
+                if (real) {
+                    const double g0 = sgt[0][lane], g1 = sgt[1][lane], g2 = sgt[2][lane];
+                    const double *o = w == 1 ? sg : sr;
+                    const double o0 = w == 0 ? g0 : o[3 * lane], o1 = w == 0 ? g1 : o[3 * lane + 1],
+                                 o2 = w == 0 ? g2 : o[3 * lane + 2];
+                    x = fma(g0, o0, fma(g1, o1, g2 * o2));
+                }
+                tv[(2 + w) * TI] = x;
+            }
+        }
+        if (CS == FIN_PARTS || part32 + CS >= FIN_PARTS) break;
+        i += 32 * CS;
+        a += 32 * CS;
+        real = i < t.na;
+        k1 = kb = 0;
+        if (real && w >= FIN_STRANDS) {
+            k1 = c.inc_off[a + 1];
+            kb = c.inc_off[a] + w - FIN_STRANDS;
+        }
+        __syncthreads();  // the buffers of the next 32 atoms
     }
-    cl.sync();
+    if constexpr (CS == 1) __syncthreads();
+    if constexpr (CS > 1) cl.sync();
     if (rank != 0) return;
     // the tile's sums, in the order of block_reduce_columns: values 0 to 3 in
     // warp 0, value 4 in warp 1
@@ -383,8 +407,8 @@ __global__ void __cluster_dims__(FIN_CLUSTER, 1, 1) __launch_bounds__(FIN_NT, BL
             tot[fin_value(k1v)] = 0.0 + x;  // of a system of one tile
         }
     } else if (w == 2) {
-        unsigned long long m = grad && lane < 3 * FIN_CLUSTER ? gmax[lane] : 0ULL;
-        const bool bad = lane < 4 * FIN_CLUSTER && (grad || (lane & 3) == 3) && badf[lane];
+        unsigned long long m = grad && lane < 3 * FIN_PARTS ? gmax[lane] : 0ULL;
+        const bool bad = lane < 4 * FIN_PARTS && (grad || (lane & 3) == 3) && badf[lane];
         const unsigned any_bad = __ballot_sync(0xffffffffu, bad);
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) {
@@ -703,8 +727,9 @@ cudaError_t launch_prepare(const Ctx &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 cudaError_t launch_finalize(const Ctx &c, cudaStream_t s, double *g_out) {
-    if (c.n_tiles > c.sms) k_finalize<6><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
-    else k_finalize<4><<<c.n_tiles * FIN_CLUSTER, FIN_NT, 0, s>>>(c, g_out);
+    if (c.n_tiles <= c.sms) k_finalize<FIN_PARTS, 4><<<c.n_tiles * FIN_PARTS, FIN_NT, 0, s>>>(c, g_out);
+    else if (c.n_tiles <= 5 * c.sms) k_finalize<FIN_PARTS, 6><<<c.n_tiles * FIN_PARTS, FIN_NT, 0, s>>>(c, g_out);
+    else k_finalize<1, 8><<<c.n_tiles, FIN_NT, 0, s>>>(c, g_out);
     return cudaGetLastError();
 }
 cudaError_t launch_update(const Ctx &c, cudaStream_t s) {
